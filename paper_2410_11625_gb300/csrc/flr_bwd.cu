@@ -13,6 +13,7 @@
 //             dz_j = Abar_j g_j                                    (the applied guide)
 // j in T_k <=> k in T_j for clipped square windows of one radius, so every adjoint of a
 // window sum is the same clipped box sum.
+#include <algorithm>
 #include <cstring>
 
 #include "flr_internal.cuh"
@@ -100,14 +101,15 @@ __global__ void __launch_bounds__(kBThreads) box_sum_kernel(const float *__restr
     }
 }
 
-// The same clipped box sum over many planes with TMA staging (rows 16-byte aligned): one CTA
-// per 64 x 32 output tile walks every plane; each plane's tile + halo arrives by one TMA box
-// copy (the copy engine zero-fills outside the image) into a double-buffered ring, so the
-// next plane loads while the current one is summed.  Waits are bounded (1 s).
+// The same clipped box sum over many planes with TMA staging (rows 16-byte aligned): a CTA
+// walks the planes [p0, p1) of one 64 x 32 output tile, p0 = blockIdx.z * per_cta; each plane's
+// tile + halo arrives by one TMA box copy (the copy engine zero-fills outside the image) into
+// a double-buffered ring, so the next plane loads while the current one is summed.  Waits are
+// bounded (1 s).
 struct alignas(128) BoxKArgs {
     CUtensorMap tm;  // [nplanes][H][W] float32, box (TS, THh, 1)
     float *out;
-    int H, W, rad, nplanes;
+    int H, W, rad, nplanes, per_cta;
     int *status;
 };
 
@@ -141,11 +143,12 @@ __global__ void __launch_bounds__(kBThreads, 4) box_sum_tma_kernel(const __grid_
     const int tid = threadIdx.x, lane = tid & 31;
     const int tx0 = blockIdx.x * kBW, ty0 = blockIdx.y * kBH;
     const size_t plane = (size_t)k.H * k.W;
+    const int p0 = blockIdx.z * k.per_cta, np = min(k.per_cta, k.nplanes - p0);  // p below counts from p0
     auto stage = [&](float *T, int p) {
         if (tid == 0) {
             uint64_t *b = bar + (p & 1);
             tma::mbar_expect_tx(b, (unsigned)(g.THh * g.TS * 4));
-            tma::load_3d(T, &k.tm, tx0 - g.RCA, ty0 - rad, p, b);
+            tma::load_3d(T, &k.tm, tx0 - g.RCA, ty0 - rad, p0 + p, b);
         }
     };
     if (tid == 0) {
@@ -158,16 +161,16 @@ __global__ void __launch_bounds__(kBThreads, 4) box_sum_tma_kernel(const __grid_
     stage(T0, 0);
     const int x = tid % kBW, run = tid / kBW;
     const int gx = tx0 + x;
-    for (int p = 0; p < k.nplanes; ++p) {
+    for (int p = 0; p < np; ++p) {
         float *Tc = (p & 1) ? T1 : T0;
-        if (p + 1 < k.nplanes) stage((p & 1) ? T0 : T1, p + 1);
+        if (p + 1 < np) stage((p & 1) ? T0 : T1, p + 1);
         if (!tma::wait_warp(bar + (p & 1), (uint32_t)((p >> 1) & 1), kBoxTimeoutNs) && lane == 0) {
             s_abort = 1;
             if (k.status) atomicExch(k.status, 1);
         }
         __syncthreads();
         if (s_abort) {  // let a copy still in flight land before the CTA exits, then stop
-            if (p + 1 < k.nplanes && tid < 32)
+            if (p + 1 < np && tid < 32)
                 tma::wait_warp(bar + ((p + 1) & 1), (uint32_t)(((p + 1) >> 1) & 1), kBoxTimeoutNs);
             return;
         }
@@ -216,7 +219,7 @@ __global__ void __launch_bounds__(kBThreads, 4) box_sum_tma_kernel(const __grid_
         const float *q = Hb + (run * 8) * g.HS + x;
         float s = 0.f;
         for (int kk = 0; kk <= 2 * rad; ++kk) s += q[kk * g.HS];
-        float *dst = k.out + (size_t)p * plane;
+        float *dst = k.out + (size_t)(p0 + p) * plane;
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
             if (t > 0) s += q[(t + 2 * rad) * g.HS] - q[(t - 1) * g.HS];
@@ -295,7 +298,9 @@ __global__ void __launch_bounds__(256) bwd_contract_kernel(const BwdArgs a)
 // 4-byte loads, and each output channel's gradient formed from its own planes in turn, so
 // that a thread holds four pixels' inputs and one channel's operands at a time.  Every
 // pixel's arithmetic (operands, order of the fused multiply-adds) is that of
-// bwd_contract_kernel, so the results are the same bit for bit.
+// bwd_contract_kernel, so the results are the same bit for bit.  With gridDim.y = Q + 3 a
+// thread forms only output channel blockIdx.y (guide channels, then radiance): a small frame
+// has too few pixels to fill the chip, and its planes stay in L2 for the second reading.
 __device__ __forceinline__ float4 ld4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
 __device__ __forceinline__ void st4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
 __device__ __forceinline__ float4 fma4(float4 a, float4 b, float4 c)
@@ -338,8 +343,10 @@ __global__ void __launch_bounds__(256) bwd_contract4_kernel(const BwdArgs a)
             }
         }
         const float *BS = a.BS;
+        const bool all = gridDim.y == 1;
+        const int one = blockIdx.y;
 #pragma unroll 1
-        for (int i = 0; i < Q; ++i) {  // one guide channel's 15 planes in flight at a time
+        for (int i = all ? 0 : min(one, Q); i < (all ? Q : min(one + 1, Q)); ++i) {  // one channel's 15 planes in flight
             float4 d = ld4(BS + (C::X0 + i) * plane + p);
 #pragma unroll
             for (int j = 0; j < Q; ++j) {
@@ -361,13 +368,21 @@ __global__ void __launch_bounds__(256) bwd_contract4_kernel(const BwdArgs a)
             }
         }
 #pragma unroll 1
-        for (int c = 0; c < 3; ++c) {
+        for (int c = all ? 0 : max(one - Q, 0); c < (all ? 3 : one - Q + 1); ++c) {
             float4 d = ld4(BS + (C::Y0 + c) * plane + p);
 #pragma unroll
             for (int i = 0; i < Q; ++i) d = fma4(ld4(BS + C::xy(i, c) * plane + p), xs[i], d);
             st4(a.grad_rad + c * plane + p, d);
         }
     }
+}
+
+int sm_count()
+{
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 1;
+    return n;
 }
 
 int elem_grid(size_t n) { return (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096); }
@@ -403,7 +418,7 @@ cudaError_t launch_box_sum_tma(const BoxKArgs &k, cudaStream_t st)
     e = cudaFuncSetAttribute(box_sum_tma_kernel<RT>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
-    dim3 grid((k.W + kBW - 1) / kBW, (k.H + kBH - 1) / kBH);
+    dim3 grid((k.W + kBW - 1) / kBW, (k.H + kBH - 1) / kBH, (k.nplanes + k.per_cta - 1) / k.per_cta);
     box_sum_tma_kernel<RT><<<grid, kBThreads, smem, st>>>(k);
     return cudaGetLastError();
 }
@@ -421,6 +436,14 @@ cudaError_t launch_box_sum(const float *in, float *out, int nplanes, int H, int 
             k.rad = rad;
             k.nplanes = nplanes;
             k.status = status;
+            // Planes per CTA: about eight waves of four CTAs per SM, so that the last wave
+            // costs little, and one plane per CTA on frames with fewer tile-planes than that.
+            // One CTA walking every plane of a tile left a 128 x 128 frame on 8 SMs (its three
+            // box sums 105 us, split 10 us) and a 1080p frame with a second wave two thirds
+            // full (the backward pass 1.066 ms, split 1.029 ms).
+            const long long tiles = (long long)((W + kBW - 1) / kBW) * ((H + kBH - 1) / kBH);
+            const long long target = 8LL * 4 * sm_count();
+            k.per_cta = (int)std::min<long long>(nplanes, std::max<long long>(1, tiles * nplanes / target));
             return rad == 8 ? launch_box_sum_tma<8>(k, st) : launch_box_sum_tma<-1>(k, st);
         }
     }
@@ -437,7 +460,10 @@ cudaError_t launch_bwd_contract(int q, const BwdArgs &a, cudaStream_t st)
     auto al = [](const void *p) { return ((uintptr_t)p & 15) == 0; };
     if ((a.W & 3) == 0 && al(a.guide) && al(a.rad) && al(a.g) && al(a.BS) && al(a.BA) && al(a.grad_guide) &&
         al(a.grad_map) && al(a.grad_rad)) {
-        const int grid4 = (int)(((size_t)a.H * a.W / 4 + 255) / 256);  // one thread per four pixels
+        // one thread per four pixels; below two CTAs per SM (about 311k pixels, whose planes fit
+        // in L2) also one output channel per thread: 128 x 128 takes 14.8 us without, 4.0 us with
+        const int ctas = (int)(((size_t)a.H * a.W / 4 + 255) / 256);
+        const dim3 grid4(ctas, ctas < 2 * sm_count() ? q + 3 : 1);
         switch (q) {
         case 1: bwd_contract4_kernel<1><<<grid4, 256, 0, st>>>(a); break;
         case 2: bwd_contract4_kernel<2><<<grid4, 256, 0, st>>>(a); break;
