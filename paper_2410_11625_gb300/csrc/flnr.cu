@@ -12,8 +12,14 @@
 //   up(f2) ++ f1, d1a 3x3 96->32 ReLU, d1b 3x3 32->32 ReLU                     d1 (H/2)
 //   up(d1) ++ f0, d0a 3x3 48->16 ReLU, d0b 3x3 16->16 ReLU                     d0 (H)
 //   o0 3x3 16->16 ReLU, o1 1x1 16->8, sigmoid                                  X' (8 ch)
-// Activations are NHWC BF16 (channels innermost; the 11 inputs padded to 16, the 8 outputs
-// of o1 computed as 16 with zero weights); the enhanced guides leave as planar FP32 for FLR.
+// Activations are BF16 in planes of eight channels, [N][C/8][H][W][8] (the 11 inputs padded
+// to 16 channels, the 8 outputs of o1 computed as 16 with zero weights): a row of a plane is
+// contiguous, so a tile with its halo arrives in rows of 8 (NT + 1/4) x 16 bytes per TMA request
+// instead of 16 bytes (the eight channels of one pixel of an NHWC map; a 3x3 16->16 layer of a
+// 1920x1080 frame: 49 us with NHWC tiles, 32 us with plane tiles).  The outputs of e1a and
+// e2a, which stride-2 convolutions read, are additionally split by row and column parity,
+// [N][C/8][2][2][H/2][W/2][8].  flnr_layer's tensors are NHWC; the kernels take either.  The
+// enhanced guides leave as planar FP32 for FLR.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -23,6 +29,7 @@
 #include <cstdint>
 #include <cstring>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "flr.h"
@@ -42,6 +49,34 @@ constexpr LayerDef kLayers[kNL] = {
 __host__ __device__ constexpr int pad16(int c) { return (c + 15) / 16 * 16; }
 
 // ---------------------------------------------------------------------------------------
+// Programmatic dependent launch.  The network is a chain of short kernels, each reading what the
+// one before wrote, and at 16 x 128^2 a training pass lost 120 us of 690 between them.  A kernel
+// launched with launch_pdl may start when every CTA of its predecessor has called pdl_trigger (or
+// exited); it must call pdl_wait, which returns when the predecessor has finished and its writes
+// are visible, before it touches global memory.  Only the set-up of barriers and tensor memory
+// runs ahead.  A kernel that allocates tensor memory triggers after its allocation: its
+// successor's CTAs, which may be resident beside it and hold columns while they wait, then cannot
+// keep it from allocating.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
+
+// ---------------------------------------------------------------------------------------
 // Asynchronous 16-byte global -> shared copies (zero fill when !valid).
 __device__ __forceinline__ void cp_async16(void *dst, const void *src, bool valid)
 {
@@ -53,24 +88,49 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
 
 // Arguments of the convolution kernels (stride 1, zero padding KS/2, implicit GEMM on the
-// tensor cores).  x [N][H][W][CIN] bf16, w [taps][COUT][CIN] bf16, bias [COUT] fp32.  The
-// kernels' template parameters select the epilogue:
-//   OUTM 0 -> y [N][H][W][ystride] bf16 at channel offset 0 (ACT 1 = ReLU);
-//   OUTM 1 -> yf planar fp32 [N][8][H][W], sigmoid of channels 0..7;
-//   MASK   -> the result times (mask > 0), mask [N][H][W][COUT] bf16 (the ReLU of the
-//             layer input, for input gradients);
-// The decoder kernel reads x as the half-resolution map [N][H/2][W/2][CA] and x2 as the
-// skip [N][H][W][CIN-CA] of the concatenated input up2(x) ++ x2.
+// tensor cores).  x: CIN channels, w [taps][COUT][CIN] bf16, bias [COUT] fp32.  The kernels'
+// template parameters select the epilogue:
+//   OUTM 0 -> y: COUT channels bf16 (ACT 1 = ReLU);
+//   OUTM 1 -> yf planar fp32 [N][nbias][H][W] (may be NULL), sigmoid of the true outputs;
+//   OUTM 2 -> y: the gradient g s (1 - s) at the sigmoid's input, s the sigmoid of the result
+//             and g planar fp32 [N][nbias][H][W] (zero for the padding channels);
+//   MASK   -> the result times (mask > 0), mask: COUT channels bf16 (the ReLU of the layer
+//             input, for input gradients);
+// The decoder kernel reads x as the half-resolution map (CA channels) and x2 as the skip
+// (CIN - CA channels) of the concatenated input up2(x) ++ x2.  Every bf16 tensor has one of
+// these layouts:
+enum Layout {
+    kNHWC = 0,    // [N][H][W][C]
+    kPlanes = 1,  // [N][C/8][H][W][8]
+    kParity = 2   // [N][C/8][2][2][H/2][W/2][8]: planes split by row and column parity, H and W even
+};
 struct ConvArgs {
     const bf16 *x, *w, *mask;
     const float *bias;
     bf16 *y;
     float *yf;
-    int N, H, W, ystride;
-    int nbias;  // valid bias entries (the true output channels); 0 without bias
+    const float *g;
+    int N, H, W;
+    int lx, ly, lm;  // layouts of x and x2, y, mask
+    int nbias;       // valid bias entries (the true output channels); 0 without bias
     const bf16 *x2;
     int *status;  // tensor-core path: set to FLNR_STATUS_TIMEOUT if a completion wait ran out
 };
+
+// Address of pixel (n, y, x)'s first eight channels in a C-channel tensor of an H x W map;
+// the further channel groups are *chunk elements apart.
+__device__ __forceinline__ size_t pixel_at(int layout, int C, int H, int W, int n, int y, int x, size_t *chunk)
+{
+    const size_t hw = (size_t)H * W;
+    if (layout == kNHWC) {
+        *chunk = 8;
+        return ((size_t)n * hw + (size_t)y * W + x) * C;
+    }
+    *chunk = hw * 8;
+    const size_t q = layout == kPlanes ? (size_t)y * W + x
+                                       : ((size_t)(2 * (y & 1) + (x & 1)) * (H / 2) + (y >> 1)) * (W / 2) + (x >> 1);
+    return ((size_t)n * (C / 8) * hw + q) * 8;
+}
 
 // ---------------------------------------------------------------------------------------
 // The same convolution on the fifth-generation tensor cores (tcgen05): BF16 operands in shared
@@ -160,7 +220,8 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t mbar, uint32_t parity)
 template <int N>
 constexpr int tmem_cols()
 {
-    return N <= 32 ? 32 : N <= 64 ? 64 : N <= 128 ? 128 : 256;
+    static_assert(N <= 512, "tensor memory has 512 columns");
+    return N <= 32 ? 32 : N <= 64 ? 64 : N <= 128 ? 128 : N <= 256 ? 256 : 512;
 }
 
 // Kernel parameters: the tensor map (4-D: channels, W, H, N) of the operand that TMA stages
@@ -211,23 +272,24 @@ __device__ __forceinline__ void tc_load_acc(uint32_t taddr, float (&v)[COUT])
     asm volatile("tcgen05.fence::before_thread_sync;\n");
 }
 
-// tc_store: bias, activation, optional ReLU mask, then bf16 NHWC stores, or sigmoid into
-// planar fp32 (OUTM 1).  (n, yy, xx): the output pixel of an [N][a.H][a.W] map.
+// tc_store: bias, activation, optional ReLU mask, then bf16 stores, or sigmoid into planar
+// fp32 (OUTM 1).  (n, yy, xx): the output pixel of an [N][a.H][a.W] map.
 template <int COUT, int ACT, int OUTM, bool MASK>
 __device__ __forceinline__ void tc_store(const ConvArgs &a, float (&v)[COUT], const float (&bias)[COUT], int n,
                                          int yy, int xx)
 {
     const bool in = yy < a.H && xx < a.W;
-    const size_t pix = ((size_t)n * a.H + yy) * a.W + xx;
 #pragma unroll
     for (int c = 0; c < COUT; ++c) {
         v[c] += bias[c];
         if (ACT == 1) v[c] = fmaxf(v[c], 0.f);
     }
     if (MASK && in) {
+        size_t mc;
+        const bf16 *mp = a.mask + pixel_at(a.lm, COUT, a.H, a.W, n, yy, xx, &mc);
 #pragma unroll
         for (int c8 = 0; c8 < COUT / 8; ++c8) {
-            const uint4 m = *reinterpret_cast<const uint4 *>(a.mask + pix * COUT + c8 * 8);
+            const uint4 m = *reinterpret_cast<const uint4 *>(mp + c8 * mc);
             const __nv_bfloat162 *mh = reinterpret_cast<const __nv_bfloat162 *>(&m);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -236,52 +298,80 @@ __device__ __forceinline__ void tc_store(const ConvArgs &a, float (&v)[COUT], co
             }
         }
     }
-    if (OUTM == 0) {
+    const size_t hw = (size_t)a.H * a.W, off = (size_t)yy * a.W + xx;  // planar fp32 (OUTM 1, 2)
+    if (OUTM == 1) {
+        if (in && a.yf) {
 #pragma unroll
-        for (int c8 = 0; c8 < COUT / 8; ++c8) {
-            uint4 o;
-            __nv_bfloat162 *oh = reinterpret_cast<__nv_bfloat162 *>(&o);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) oh[i] = __floats2bfloat162_rn(v[c8 * 8 + 2 * i], v[c8 * 8 + 2 * i + 1]);
-            if (in) *reinterpret_cast<uint4 *>(a.y + pix * a.ystride + c8 * 8) = o;
+            for (int c = 0; c < COUT; ++c)  // a.nbias planes: the head's true outputs
+                if (c < a.nbias) a.yf[((size_t)n * a.nbias + c) * hw + off] = 1.f / (1.f + expf(-v[c]));
         }
-    } else if (in) {
-        const size_t hw = (size_t)a.H * a.W, off = (size_t)yy * a.W + xx;
+        return;
+    }
+    if (OUTM == 2 && in) {
 #pragma unroll
-        for (int c = 0; c < COUT; ++c)  // a.nbias planes: the head's true outputs
-            if (c < a.nbias) a.yf[((size_t)n * a.nbias + c) * hw + off] = 1.f / (1.f + expf(-v[c]));
+        for (int c = 0; c < COUT; ++c) {
+            const float sv = 1.f / (1.f + expf(-v[c]));
+            v[c] = c < a.nbias ? a.g[((size_t)n * a.nbias + c) * hw + off] * sv * (1.f - sv) : 0.f;
+        }
+    }
+    size_t yc;
+    bf16 *yp = a.y + pixel_at(a.ly, COUT, a.H, a.W, n, yy, xx, &yc);
+#pragma unroll
+    for (int c8 = 0; c8 < COUT / 8; ++c8) {
+        uint4 o;
+        __nv_bfloat162 *oh = reinterpret_cast<__nv_bfloat162 *>(&o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) oh[i] = __floats2bfloat162_rn(v[c8 * 8 + 2 * i], v[c8 * 8 + 2 * i + 1]);
+        if (in) *reinterpret_cast<uint4 *>(yp + c8 * yc) = o;
     }
 }
 
 // ---------------------------------------------------------------------------------------
 // Warp-specialised tensor-core convolution (layers whose input is one tensor): no CTA-wide
-// barrier in the main loop.  Warp 4 (one lane) is the producer: it loads tile j into ring
+// barrier in the main loop.  The next warp (one lane) is the producer: it loads tile j into ring
 // stage j % NBUF with one TMA box copy per channel chunk once the MMAs of tile j - NBUF have
-// released the stage.  Warp 5 (one lane) issues tile j's MMAs into accumulator j & 1 once the
+// released the stage.  The last warp (one lane) issues tile j's MMAs into accumulator j & 1 once the
 // stage has landed and the epilogue has drained that accumulator, then commits them to the
-// stage's "empty" barrier and the accumulator's "full" barrier.  Warps 0-3 read the
-// accumulator rows of their TMEM lane quarter, release the accumulator, and run the epilogue.
-// The tile geometry and operand layouts are those described above.  Every wait is bounded.
-template <int CIN, int COUT, int KS>
+// stage's "empty" barrier and the accumulator's "full" barrier.  The epilogue warps read the
+// accumulator rows of their TMEM lane quarter, release the accumulator, and run the epilogue
+// (with several tiles per stage eight warps: the sigmoid of the head keeps four busy longer than
+// the MMAs take; o0 + o1 at 1920x1080 101 us with four, 81 us with eight).
+// The operand layouts are those described above.  A stage covers NT MMA tiles side by side
+// (16 rows x 8 NT pixels): one halo and one hand-over of the barriers for NT accumulators, which
+// pays where there are enough stages to go round (conv_ws_launch).  Every wait is bounded.
+template <int CIN, int COUT, int KS, int NT>
 struct WsGeom {
-    static constexpr int TH = 16, TW = 8, P = KS / 2, SH = TH + 2 * P, SW = TW + 2 * P, C8 = CIN / 8;
-    static constexpr int NBUF = 4;
+    static constexpr int TH = 16, TW = 8 * NT, P = KS / 2, SH = TH + 2 * P, SW = TW + 2 * P, C8 = CIN / 8;
+    static constexpr int NBUF = NT == 1 ? 4 : (C8 <= 2 ? 3 : 2);
     static constexpr int PS = (SH * SW * 16 + 127) / 128 * 128;
     static constexpr int XBYTES = C8 * PS;
     static constexpr int WBYTES = (KS * KS * C8 * COUT * 16 + 127) / 128 * 128;
     static constexpr int TMA_BYTES = C8 * SH * SW * 16;
+    static constexpr int EW = NT == 1 ? 4 : 8;  // epilogue warps: warp w takes tiles w / 4, + EW / 4, ...
+    static constexpr int THREADS = 32 * (EW + 2);
     static constexpr int NBAR = 2 * NBUF + 4;  // full[NBUF], empty[NBUF], accf[2], acce[2]
     static constexpr int SMEM = 128 + WBYTES + NBUF * XBYTES + NBAR * 8 + 16;
-    static constexpr int COLS = tmem_cols<2 * COUT>();
+    static constexpr int COLS = tmem_cols<2 * NT * COUT>();
 };
 constexpr int kWsThreads = 192;
 
-template <int CIN, int COUT, int KS, int ACT, int OUTM, bool MASK = false>
-__global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(const __grid_constant__ TcArgs args)
+// One stage's input planes: channel chunk k of columns x.., rows y.. of image n
+template <int C8, int PS>
+__device__ __forceinline__ void load_planes(uint32_t dst, const CUtensorMap *tm, int layout, int x, int y, int n, uint32_t bar)
 {
-    using G = WsGeom<CIN, COUT, KS>;
+#pragma unroll
+    for (int k = 0; k < C8; ++k) {
+        if (layout == kNHWC) tma_load_4d(dst + k * PS, tm, k * 8, x, y, n, bar);
+        else tma_load_4d(dst + k * PS, tm, 4 * x, y, k, n, bar);  // 32-bit elements: four per pixel
+    }
+}
+
+template <int CIN, int COUT, int KS, int ACT, int OUTM, bool MASK, int NT>
+__global__ void __launch_bounds__(WsGeom<CIN, COUT, KS, NT>::THREADS) conv_ws_kernel(const __grid_constant__ TcArgs args)
+{
+    using G = WsGeom<CIN, COUT, KS, NT>;
     constexpr int TH = G::TH, TW = G::TW, P = G::P, SW = G::SW, C8 = G::C8, NBUF = G::NBUF, PS = G::PS;
-    static_assert(CIN % 16 == 0 && COUT % 16 == 0 && 2 * COUT <= 256, "UMMA shape");
+    static_assert(CIN % 16 == 0 && COUT % 16 == 0 && COUT <= 256, "UMMA shape");
     const ConvArgs &a = args.c;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char *base = smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127);
@@ -308,14 +398,18 @@ __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(const __grid_consta
         }
         for (int i = 0; i < 2; ++i) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(accf + i)));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;\n" ::"r"(smem_u32(acce + i)));  // 4 epilogue warps
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(acce + i)), "r"(G::EW));
         }
         asm volatile("fence.mbarrier_init.release.cluster;\n");
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&args.tm)) : "memory");
         s_issued = 0;
         s_consumed = 0;
     }
-    for (int i = tid; i < KS * KS * COUT * C8; i += kWsThreads) {
+    asm volatile("tcgen05.fence::before_thread_sync;\n");
+    __syncthreads();  // tensor memory allocated
+    pdl_trigger();
+    pdl_wait();
+    for (int i = tid; i < KS * KS * COUT * C8; i += G::THREADS) {
         const int c8 = i % C8, row = i / C8, tap = row / COUT, co = row % COUT;
         cp_async16(sw + ((tap * C8 + c8) * COUT + co) * 16, a.w + (size_t)row * CIN + c8 * 8, true);
     }
@@ -337,7 +431,7 @@ __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(const __grid_consta
         tx0 = (r % tiles_x) * TW;
     };
 
-    if (warp == 4) {
+    if (warp == G::EW) {
         if (lane == 0) {  // producer
             for (int j = 0; j < mine; ++j) {
                 const int st = j % NBUF;
@@ -350,12 +444,11 @@ __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(const __grid_consta
                 const uint32_t bar = smem_u32(full + st);
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(G::TMA_BYTES) : "memory");
                 const uint32_t dst = smem_u32(sx0 + st * G::XBYTES);
-#pragma unroll
-                for (int k = 0; k < C8; ++k) tma_load_4d(dst + k * PS, &args.tm, k * 8, tx0 - P, ty0 - P, n, bar);
+                load_planes<C8, PS>(dst, &args.tm, a.lx, tx0 - P, ty0 - P, n, bar);
                 s_issued = j + 1;
             }
         }
-    } else if (warp == 5) {
+    } else if (warp == G::EW + 1) {
         if (lane == 0) {  // MMA issuer
             constexpr uint32_t idesc = umma_idesc(COUT);
             const uint64_t adesc0 = umma_sdesc(smem_u32(sx0), PS, SW * 16);
@@ -373,14 +466,17 @@ __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(const __grid_consta
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;\n");
                 const uint64_t ab = adesc0 + (uint64_t)((st * G::XBYTES) >> 4);
-                const uint32_t d = tmem + (uint32_t)(acc * COUT);
 #pragma unroll
-                for (int tap = 0; tap < KS * KS; ++tap) {
+                for (int t = 0; t < NT; ++t) {
+                    const uint32_t d = tmem + (uint32_t)((acc * NT + t) * COUT);
 #pragma unroll
-                    for (int kk = 0; kk < C8 / 2; ++kk) {
-                        const uint32_t aoff = (uint32_t)((2 * kk * PS + ((tap / KS) * SW + tap % KS) * 16) >> 4);
-                        const uint32_t boff = (uint32_t)(((tap * C8 + 2 * kk) * COUT * 16) >> 4);
-                        umma_bf16(d, ab + aoff, bdesc0 + boff, idesc, (tap | kk) ? 1u : 0u);
+                    for (int tap = 0; tap < KS * KS; ++tap) {
+#pragma unroll
+                        for (int kk = 0; kk < C8 / 2; ++kk) {
+                            const uint32_t aoff = (uint32_t)((2 * kk * PS + ((tap / KS) * SW + tap % KS + 8 * t) * 16) >> 4);
+                            const uint32_t boff = (uint32_t)(((tap * C8 + 2 * kk) * COUT * 16) >> 4);
+                            umma_bf16(d, ab + aoff, bdesc0 + boff, idesc, (tap | kk) ? 1u : 0u);
+                        }
                     }
                 }
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
@@ -389,7 +485,7 @@ __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(const __grid_consta
                     smem_u32(accf + acc)));
             }
         }
-    } else {  // epilogue warps 0-3: TMEM lane quarter = warp
+    } else {  // epilogue warps: TMEM lane quarter = warp % 4
         float bias[COUT];
 #pragma unroll
         for (int c = 0; c < COUT; ++c) bias[c] = c < a.nbias ? a.bias[c] : 0.f;
@@ -400,19 +496,24 @@ __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(const __grid_consta
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;\n");
-            float v[COUT];
-            tc_load_acc<COUT>(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(acc * COUT), v);
-            __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(acce + acc)) : "memory");
             int n, ty0, tx0;
             origin(j, n, ty0, tx0);
-            tc_store<COUT, ACT, OUTM, MASK>(a, v, bias, n, ty0 + 4 * warp + (lane >> 3), tx0 + (lane & 7));
+#pragma unroll 1
+            for (int t = warp / 4; t < NT; t += G::EW / 4) {
+                float v[COUT];
+                tc_load_acc<COUT>(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((acc * NT + t) * COUT), v);
+                if (t + G::EW / 4 >= NT) {
+                    __syncwarp();
+                    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(acce + acc)) : "memory");
+                }
+                tc_store<COUT, ACT, OUTM, MASK>(a, v, bias, n, ty0 + 4 * (warp & 3) + (lane >> 3), tx0 + 8 * t + (lane & 7));
+            }
         }
     }
     __syncwarp();  // the single-lane roles rejoin their warps before the CTA barrier
     asm volatile("tcgen05.fence::before_thread_sync;\n");
     __syncthreads();
-    if (tid == 4 * 32) {  // after a failure: let copies still in flight land before the CTA exits
+    if (tid == G::EW * 32) {  // after a failure: let copies still in flight land before the CTA exits
         for (int j = s_consumed; j < s_issued; ++j) mbar_wait_thread(smem_u32(full + j % NBUF), (uint32_t)((j / NBUF) & 1));
     }
     __syncthreads();
@@ -429,42 +530,46 @@ __global__ void __launch_bounds__(kWsThreads) conv_ws_kernel(const __grid_consta
 // A operand of the 1x1 MMA ([chunk][128 pixels][8 channels]), the MMA lane issues that one
 // MMA into a second pair of accumulators, and the epilogue warps finish the tile from it
 // (ReLU and BF16 for in1, sigmoid into planar FP32 for o1).  Roles as
-// conv_ws_kernel; the MMA lane issues tile j's convolution, then tile j - 1's 1x1.
-// Barriers: full/empty per input stage, accf/acce per first accumulator, a2full (the A
-// operand of the 1x1 written, four epilogue warps), acc2f (1x1 committed) and acc2e (its
-// accumulator drained, four warps), all per accumulator slot j & 1.
+// conv_ws_kernel; the MMA lane issues stage j's convolution, then stage j - 1's 1x1, and the
+// epilogue warps write stage j's A operands before they finish stage j - 1, so that neither
+// waits for the other's round trip.
+// Barriers: full/empty per input stage, accf/acce per first accumulator set, a2full (the A
+// operands of the 1x1 written, four epilogue warps), acc2f (1x1 committed) and acc2e (its
+// accumulators drained, four warps), all per accumulator slot j & 1.
 struct alignas(128) TailArgs {
     CUtensorMap tm;
-    ConvArgs c;   // first layer: x, w, bias, nbias, N, H, W, status; y (may be NULL), ystride
-    ConvArgs c2;  // 1x1 layer: w, bias, nbias, N, H, W and the outputs (y, ystride / yf)
+    ConvArgs c;   // first layer: x, w, bias, nbias, N, H, W, status; y (may be NULL)
+    ConvArgs c2;  // 1x1 layer: w, bias, nbias, N, H, W and the outputs (y / yf)
+    bf16 *w2_kept;   // when given: a copy of the 1x1 layer's weights and biases as this pass used
+    float *b2_kept;  // them (the backward pass forms the sigmoid again from the stored a5)
 };
 
-template <int CIN, int COUT, int KS, int COUT2>
+template <int CIN, int COUT, int KS, int COUT2, int NT>
 struct TailGeom {
-    using G1 = WsGeom<CIN, COUT, KS>;
+    using G1 = WsGeom<CIN, COUT, KS, NT>;
     static constexpr int NBUF = G1::NBUF;
-    static constexpr int A2BYTES = (COUT / 8) * 128 * 16;             // one 1x1 A operand
+    static constexpr int A2BYTES = (COUT / 8) * 128 * 16;             // one tile's 1x1 A operand
     static constexpr int W2BYTES = ((COUT / 8) * COUT2 * 16 + 127) / 128 * 128;
     static constexpr int NBAR = 2 * NBUF + 10;  // full, empty, accf, acce, a2full, acc2f, acc2e
-    static constexpr int SMEM = 128 + G1::WBYTES + W2BYTES + NBUF * G1::XBYTES + 2 * A2BYTES + NBAR * 8 + 16;
-    static constexpr int COLS = tmem_cols<2 * COUT + 2 * COUT2>();
+    static constexpr int SMEM = 128 + G1::WBYTES + W2BYTES + NBUF * G1::XBYTES + 2 * NT * A2BYTES + NBAR * 8 + 16;
+    static constexpr int COLS = tmem_cols<2 * NT * (COUT + COUT2)>();
 };
 
-template <int CIN, int COUT, int KS, int COUT2, int ACT2, int OUTM2>
-__global__ void __launch_bounds__(kWsThreads) conv_tail_kernel(const __grid_constant__ TailArgs args)
+template <int CIN, int COUT, int KS, int COUT2, int ACT2, int OUTM2, int NT>
+__global__ void __launch_bounds__(WsGeom<CIN, COUT, KS, NT>::THREADS) conv_tail_kernel(const __grid_constant__ TailArgs args)
 {
-    using T = TailGeom<CIN, COUT, KS, COUT2>;
+    using T = TailGeom<CIN, COUT, KS, COUT2, NT>;
     using G = typename T::G1;
     constexpr int TH = G::TH, TW = G::TW, P = G::P, SW = G::SW, C8 = G::C8, NBUF = G::NBUF, PS = G::PS;
-    static_assert(CIN % 16 == 0 && COUT % 16 == 0 && COUT2 % 16 == 0 && 2 * COUT + 2 * COUT2 <= 256, "UMMA shape");
+    static_assert(CIN % 16 == 0 && COUT % 16 == 0 && COUT2 % 16 == 0, "UMMA shape");
     const ConvArgs &a = args.c;
     const ConvArgs &a2 = args.c2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char *base = smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127);
     unsigned char *sw = base;
     unsigned char *sw2 = sw + G::WBYTES;
-    unsigned char *sa2 = sw2 + T::W2BYTES;                   // [2][COUT/8][128][8] 1x1 A operands
-    unsigned char *sx0 = sa2 + 2 * T::A2BYTES;
+    unsigned char *sa2 = sw2 + T::W2BYTES;                   // [2][NT][COUT/8][128][8] 1x1 A operands
+    unsigned char *sx0 = sa2 + 2 * NT * T::A2BYTES;
     uint64_t *full = reinterpret_cast<uint64_t *>(sx0 + NBUF * G::XBYTES);
     uint64_t *empty = full + NBUF, *accf = empty + NBUF, *acce = accf + 2;
     uint64_t *a2full = acce + 2, *acc2f = a2full + 2, *acc2e = acc2f + 2;
@@ -487,21 +592,29 @@ __global__ void __launch_bounds__(kWsThreads) conv_tail_kernel(const __grid_cons
         }
         for (int i = 0; i < 2; ++i) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(accf + i)));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;\n" ::"r"(smem_u32(acce + i)));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;\n" ::"r"(smem_u32(a2full + i)));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(acce + i)), "r"(G::EW));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(a2full + i)), "r"(G::EW));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(acc2f + i)));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 4;\n" ::"r"(smem_u32(acc2e + i)));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(acc2e + i)), "r"(G::EW));
         }
         asm volatile("fence.mbarrier_init.release.cluster;\n");
         asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(&args.tm)) : "memory");
         s_issued = 0;
         s_consumed = 0;
     }
-    for (int i = tid; i < KS * KS * COUT * C8; i += kWsThreads) {
+    asm volatile("tcgen05.fence::before_thread_sync;\n");
+    __syncthreads();  // tensor memory allocated
+    pdl_trigger();
+    pdl_wait();
+    for (int i = tid; i < KS * KS * COUT * C8; i += G::THREADS) {
         const int c8 = i % C8, row = i / C8, tap = row / COUT, co = row % COUT;
         cp_async16(sw + ((tap * C8 + c8) * COUT + co) * 16, a.w + (size_t)row * CIN + c8 * 8, true);
     }
-    for (int i = tid; i < COUT2 * (COUT / 8); i += kWsThreads) {  // 1x1 weights [COUT2][COUT] -> [c8][COUT2][8]
+    if (args.w2_kept && blockIdx.x == 0) {
+        for (int i = tid; i < COUT2 * COUT; i += G::THREADS) args.w2_kept[i] = a2.w[i];
+        if (tid < a2.nbias) args.b2_kept[tid] = a2.bias[tid];
+    }
+    for (int i = tid; i < COUT2 * (COUT / 8); i += G::THREADS) {  // 1x1 weights [COUT2][COUT] -> [c8][COUT2][8]
         const int c8 = i % (COUT / 8), co = i / (COUT / 8);
         cp_async16(sw2 + (c8 * COUT2 + co) * 16, a2.w + (size_t)co * COUT + c8 * 8, true);
     }
@@ -512,7 +625,7 @@ __global__ void __launch_bounds__(kWsThreads) conv_tail_kernel(const __grid_cons
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n");
     const uint32_t tmem = *tslot;
-    const uint32_t tmem2 = tmem + (uint32_t)(2 * COUT);  // the 1x1 accumulators
+    const uint32_t tmem2 = tmem + (uint32_t)(2 * NT * COUT);  // the 1x1 accumulators
     auto fail = [&]() {
         if (a.status) atomicExch(a.status, FLNR_STATUS_TIMEOUT);
     };
@@ -524,7 +637,7 @@ __global__ void __launch_bounds__(kWsThreads) conv_tail_kernel(const __grid_cons
         tx0 = (r % tiles_x) * TW;
     };
 
-    if (warp == 4) {
+    if (warp == G::EW) {
         if (lane == 0) {  // producer
             for (int j = 0; j < mine; ++j) {
                 const int st = j % NBUF;
@@ -537,12 +650,11 @@ __global__ void __launch_bounds__(kWsThreads) conv_tail_kernel(const __grid_cons
                 const uint32_t bar = smem_u32(full + st);
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(G::TMA_BYTES) : "memory");
                 const uint32_t dst = smem_u32(sx0 + st * G::XBYTES);
-#pragma unroll
-                for (int k = 0; k < C8; ++k) tma_load_4d(dst + k * PS, &args.tm, k * 8, tx0 - P, ty0 - P, n, bar);
+                load_planes<C8, PS>(dst, &args.tm, a.lx, tx0 - P, ty0 - P, n, bar);
                 s_issued = j + 1;
             }
         }
-    } else if (warp == 5) {
+    } else if (warp == G::EW + 1) {
         if (lane == 0) {  // MMA issuer
             constexpr uint32_t idesc = umma_idesc(COUT), idesc2 = umma_idesc(COUT2);
             const uint64_t adesc0 = umma_sdesc(smem_u32(sx0), PS, SW * 16);
@@ -555,12 +667,15 @@ __global__ void __launch_bounds__(kWsThreads) conv_tail_kernel(const __grid_cons
                 if (!mbar_wait_thread(smem_u32(a2full + sl), (uint32_t)((t >> 1) & 1))) return false;
                 if (t >= 2 && !mbar_wait_thread(smem_u32(acc2e + sl), (uint32_t)(((t >> 1) - 1) & 1))) return false;
                 asm volatile("tcgen05.fence::after_thread_sync;\n");
-                const uint32_t d = tmem2 + (uint32_t)(sl * COUT2);
-                const uint64_t ab = a2desc0 + (uint64_t)((sl * T::A2BYTES) >> 4);
 #pragma unroll
-                for (int kk = 0; kk < COUT / 16; ++kk)
-                    umma_bf16(d, ab + (uint64_t)((2 * kk * 128 * 16) >> 4), b2desc0 + (uint64_t)((2 * kk * COUT2 * 16) >> 4),
-                              idesc2, kk ? 1u : 0u);
+                for (int i = 0; i < NT; ++i) {
+                    const uint32_t d = tmem2 + (uint32_t)((sl * NT + i) * COUT2);
+                    const uint64_t ab = a2desc0 + (uint64_t)(((sl * NT + i) * T::A2BYTES) >> 4);
+#pragma unroll
+                    for (int kk = 0; kk < COUT / 16; ++kk)
+                        umma_bf16(d, ab + (uint64_t)((2 * kk * 128 * 16) >> 4), b2desc0 + (uint64_t)((2 * kk * COUT2 * 16) >> 4),
+                                  idesc2, kk ? 1u : 0u);
+                }
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
                     smem_u32(acc2f + sl)));
                 return true;
@@ -579,14 +694,17 @@ __global__ void __launch_bounds__(kWsThreads) conv_tail_kernel(const __grid_cons
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;\n");
                 const uint64_t ab = adesc0 + (uint64_t)((st * G::XBYTES) >> 4);
-                const uint32_t d = tmem + (uint32_t)(acc * COUT);
 #pragma unroll
-                for (int tap = 0; tap < KS * KS; ++tap) {
+                for (int t = 0; t < NT; ++t) {
+                    const uint32_t d = tmem + (uint32_t)((acc * NT + t) * COUT);
 #pragma unroll
-                    for (int kk = 0; kk < C8 / 2; ++kk) {
-                        const uint32_t aoff = (uint32_t)((2 * kk * PS + ((tap / KS) * SW + tap % KS) * 16) >> 4);
-                        const uint32_t boff = (uint32_t)(((tap * C8 + 2 * kk) * COUT * 16) >> 4);
-                        umma_bf16(d, ab + aoff, bdesc0 + boff, idesc, (tap | kk) ? 1u : 0u);
+                    for (int tap = 0; tap < KS * KS; ++tap) {
+#pragma unroll
+                        for (int kk = 0; kk < C8 / 2; ++kk) {
+                            const uint32_t aoff = (uint32_t)((2 * kk * PS + ((tap / KS) * SW + tap % KS + 8 * t) * 16) >> 4);
+                            const uint32_t boff = (uint32_t)(((tap * C8 + 2 * kk) * COUT * 16) >> 4);
+                            umma_bf16(d, ab + aoff, bdesc0 + boff, idesc, (tap | kk) ? 1u : 0u);
+                        }
                     }
                 }
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
@@ -598,62 +716,81 @@ __global__ void __launch_bounds__(kWsThreads) conv_tail_kernel(const __grid_cons
             if (ok && mine > 0) ok = tail(mine - 1);
             if (!ok) fail();
         }
-    } else {  // epilogue warps 0-3: TMEM lane quarter = warp; row 32w + l = pixel (4w + l/8, l%8)
+    } else {  // epilogue warps: TMEM lane quarter q = warp % 4; row 32q + l = pixel (4q + l/8, l%8)
         float bias[COUT], bias2[COUT2];
 #pragma unroll
         for (int c = 0; c < COUT; ++c) bias[c] = c < a.nbias ? a.bias[c] : 0.f;
 #pragma unroll
         for (int c = 0; c < COUT2; ++c) bias2[c] = c < a2.nbias ? a2.bias[c] : 0.f;
-        const int m = 32 * warp + lane;
-        for (int j = 0; j < mine; ++j) {
+        const int m = 32 * (warp & 3) + lane;
+        // the 1x1's accumulators of stage t: false if the wait ran out
+        auto finish = [&](int t) -> bool {
+            const int sl = t & 1;
+            if (!mbar_wait_warp(smem_u32(acc2f + sl), (uint32_t)((t / 2) & 1))) return false;
+            asm volatile("tcgen05.fence::after_thread_sync;\n");
+            int n, ty0, tx0;
+            origin(t, n, ty0, tx0);
+#pragma unroll 1
+            for (int i = warp / 4; i < NT; i += G::EW / 4) {
+                float v2[COUT2];
+                tc_load_acc<COUT2>(tmem2 + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((sl * NT + i) * COUT2), v2);
+                if (i + G::EW / 4 >= NT) {
+                    __syncwarp();
+                    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(acc2e + sl)) : "memory");
+                }
+                tc_store<COUT2, ACT2, OUTM2, false>(a2, v2, bias2, n, ty0 + 4 * (warp & 3) + (lane >> 3), tx0 + 8 * i + (lane & 7));
+            }
+            return true;
+        };
+        bool ok = true;
+        for (int j = 0; j < mine && ok; ++j) {
             const int acc = j & 1;
             if (!mbar_wait_warp(smem_u32(accf + acc), (uint32_t)((j / 2) & 1))) {
-                if (lane == 0) fail();
+                ok = false;
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;\n");
-            float v[COUT];
-            tc_load_acc<COUT>(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(acc * COUT), v);
-            __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(acce + acc)) : "memory");
             int n, ty0, tx0;
             origin(j, n, ty0, tx0);
-            const int yy = ty0 + 4 * warp + (lane >> 3), xx = tx0 + (lane & 7);
-            const bool in = yy < a.H && xx < a.W;
-            const size_t pix = ((size_t)n * a.H + yy) * a.W + xx;
-            // first layer's bias + ReLU, rounded to bfloat16: the 1x1's A operand row m, and
-            // (when a.y is set) the first layer's stored output, which the backward pass reads
-            unsigned char *arow = sa2 + acc * T::A2BYTES + m * 16;
+#pragma unroll 1
+            for (int t = warp / 4; t < NT; t += G::EW / 4) {
+                float v[COUT];
+                tc_load_acc<COUT>(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((acc * NT + t) * COUT), v);
+                if (t + G::EW / 4 >= NT) {
+                    __syncwarp();
+                    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(acce + acc)) : "memory");
+                }
+                const int yy = ty0 + 4 * (warp & 3) + (lane >> 3), xx = tx0 + 8 * t + (lane & 7);
+                const bool in = yy < a.H && xx < a.W;
+                size_t yc;
+                bf16 *yp = a.y + pixel_at(a.ly, COUT, a.H, a.W, n, yy, xx, &yc);
+                // first layer's bias + ReLU, rounded to bfloat16: the 1x1's A operand row m, and
+                // (when a.y is set) the first layer's stored output, which the backward pass reads
+                unsigned char *arow = sa2 + (acc * NT + t) * T::A2BYTES + m * 16;
 #pragma unroll
-            for (int c8 = 0; c8 < COUT / 8; ++c8) {
-                uint4 o;
-                __nv_bfloat162 *oh = reinterpret_cast<__nv_bfloat162 *>(&o);
+                for (int c8 = 0; c8 < COUT / 8; ++c8) {
+                    uint4 o;
+                    __nv_bfloat162 *oh = reinterpret_cast<__nv_bfloat162 *>(&o);
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    oh[i] = __floats2bfloat162_rn(fmaxf(v[c8 * 8 + 2 * i] + bias[c8 * 8 + 2 * i], 0.f),
-                                                  fmaxf(v[c8 * 8 + 2 * i + 1] + bias[c8 * 8 + 2 * i + 1], 0.f));
-                *reinterpret_cast<uint4 *>(arow + c8 * 128 * 16) = o;
-                if (a.y && in) *reinterpret_cast<uint4 *>(a.y + pix * a.ystride + c8 * 8) = o;
+                    for (int i = 0; i < 4; ++i)
+                        oh[i] = __floats2bfloat162_rn(fmaxf(v[c8 * 8 + 2 * i] + bias[c8 * 8 + 2 * i], 0.f),
+                                                      fmaxf(v[c8 * 8 + 2 * i + 1] + bias[c8 * 8 + 2 * i + 1], 0.f));
+                    *reinterpret_cast<uint4 *>(arow + c8 * 128 * 16) = o;
+                    if (a.y && in) *reinterpret_cast<uint4 *>(yp + c8 * yc) = o;
+                }
             }
             asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // visible to the tensor core
             __syncwarp();
             if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(a2full + acc)) : "memory");
-            if (!mbar_wait_warp(smem_u32(acc2f + acc), (uint32_t)((j / 2) & 1))) {
-                if (lane == 0) fail();
-                break;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;\n");
-            float v2[COUT2];
-            tc_load_acc<COUT2>(tmem2 + ((uint32_t)(32 * warp) << 16) + (uint32_t)(acc * COUT2), v2);
-            __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(acc2e + acc)) : "memory");
-            tc_store<COUT2, ACT2, OUTM2, false>(a2, v2, bias2, n, yy, xx);
+            if (j >= 1) ok = finish(j - 1);
         }
+        if (ok && mine > 0) ok = finish(mine - 1);
+        if (!ok && lane == 0) fail();
     }
     __syncwarp();  // the single-lane roles rejoin their warps before the CTA barrier
     asm volatile("tcgen05.fence::before_thread_sync;\n");
     __syncthreads();
-    if (tid == 4 * 32) {  // after a failure: let copies still in flight land before the CTA exits
+    if (tid == G::EW * 32) {  // after a failure: let copies still in flight land before the CTA exits
         for (int j = s_consumed; j < s_issued; ++j) mbar_wait_thread(smem_u32(full + j % NBUF), (uint32_t)((j / NBUF) & 1));
     }
     __syncthreads();
@@ -676,8 +813,8 @@ __global__ void __launch_bounds__(kWsThreads) conv_tail_kernel(const __grid_cons
 //         box copy each;
 //   skip  its four parity planes (a', b') x CB/8 chunks [18][10][8] (rows i0 - 1 .. i0 + 16
 //         of row parity a', columns j0 - 1 .. j0 + 8 of column parity b'), one TMA box copy
-//         each from a 5-D view (channels of a column pair, column pairs, row parity, row
-//         pairs, images) in which the start channel b' * CB + 8k selects the column parity.
+//         each from a 5-D view (a column pair's channels, column pairs, row parity, row
+//         pairs, images or chunk planes) in which the start channel selects the column parity.
 // The products are those of the convolution on the concatenated map; only their order of
 // accumulation differs.  Roles and waits as conv_ws_kernel; the MMA lane issues the four
 // classes of a stage into one of two accumulator sets (4 * COUT columns each).
@@ -697,7 +834,7 @@ struct UpGeom {
 
 struct alignas(128) UpArgs {
     CUtensorMap tlo, tskip;
-    ConvArgs c;  // x = lo [N][H/2][W/2][CA], x2 = skip [N][H][W][CB], H and W even
+    ConvArgs c;  // x = lo (CA channels, H/2 x W/2), x2 = skip (CB channels, H x W), H and W even
 };
 
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *tm, int c0, int c1, int c2, int c3,
@@ -750,6 +887,10 @@ __global__ void __launch_bounds__(kWsThreads) conv_up_kernel(const __grid_consta
         s_issued = 0;
         s_consumed = 0;
     }
+    asm volatile("tcgen05.fence::before_thread_sync;\n");
+    __syncthreads();  // tensor memory allocated
+    pdl_trigger();
+    pdl_wait();
     // weights: global [tap][COUT][CA + CB] -> shared [tap][c8][COUT][8] (lo chunks first)
     for (int i = tid; i < 9 * COUT * C8; i += kWsThreads) {
         const int c8 = i % C8, row = i / C8, tap = row / COUT, co = row % COUT;
@@ -786,14 +927,14 @@ __global__ void __launch_bounds__(kWsThreads) conv_up_kernel(const __grid_consta
                 const uint32_t bar = smem_u32(full + st);
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(G::TMA_BYTES) : "memory");
                 const uint32_t dst = smem_u32(sx0 + st * G::XBYTES);
-#pragma unroll
-                for (int k = 0; k < CA8; ++k) tma_load_4d(dst + k * PS, &args.tlo, 8 * k, j0 - 1, i0 - 1, n, bar);
+                load_planes<CA8, PS>(dst, &args.tlo, a.lx, j0 - 1, i0 - 1, n, bar);
+                const bool nhwc = a.lx == kNHWC;
 #pragma unroll
                 for (int pp = 0; pp < 4; ++pp) {
 #pragma unroll
                     for (int k = 0; k < CB8; ++k)
-                        tma_load_5d(dst + (CA8 + pp * CB8 + k) * PS, &args.tskip, (pp & 1) * CB + 8 * k, j0 - 1, pp >> 1,
-                                    i0 - 1, n, bar);
+                        tma_load_5d(dst + (CA8 + pp * CB8 + k) * PS, &args.tskip, (pp & 1) * (nhwc ? CB : 8) + (nhwc ? 8 * k : 0),
+                                    j0 - 1, pp >> 1, i0 - 1, nhwc ? n : n * CB8 + k, bar);
                 }
                 s_issued = j + 1;
             }
@@ -895,9 +1036,10 @@ __global__ void __launch_bounds__(kWsThreads) conv_up_kernel(const __grid_consta
 // column parity pc = (v != 1) at column offset (v == 2) of its plane.  Consecutive output
 // pixels step by one pair, so every tap's operand is a plain K-major tile of the staged
 // planes: 9 taps x CIN/16 MMAs per tile, no products for the dropped positions.  The planes
-// come from two 5-D views of the NHWC input (channels of a column pair, column pairs, row
-// parity, row pairs, images), boxes 8 and 9 pairs wide; the start channel pc * CIN + 8k
-// selects the column parity.  Roles, waits and epilogue as conv_ws_kernel.
+// are those of a kParity input (boxes 8 and 9 columns wide of its parity planes: contiguous
+// rows), or come from two 5-D views of an NHWC input (channels of a column pair, column pairs,
+// row parity, row pairs, images) whose start channel pc * CIN + 8k selects the column parity.
+// Roles, waits and epilogue as conv_ws_kernel.
 template <int CIN, int COUT, int NBUF_>
 struct S2Geom {
     static constexpr int TH = 16, TW = 8, SH = TH + 1, WE = TW, WO = TW + 1, C8 = CIN / 8, NBUF = NBUF_;
@@ -915,7 +1057,7 @@ struct S2Geom {
 
 struct alignas(128) S2Args {
     CUtensorMap te, to;  // even-column and odd-column views of the input
-    ConvArgs c;          // x [N][H][W][CIN] (H, W: the input's size), y [N][H/2][W/2][ystride]
+    ConvArgs c;          // x: CIN channels (H, W: the input's size), kNHWC or kParity; y at H/2 x W/2
 };
 
 template <int CIN, int COUT, int NBUF>
@@ -961,6 +1103,10 @@ __global__ void __launch_bounds__(kWsThreads) conv_s2_kernel(const __grid_consta
         s_issued = 0;
         s_consumed = 0;
     }
+    asm volatile("tcgen05.fence::before_thread_sync;\n");
+    __syncthreads();  // tensor memory allocated
+    pdl_trigger();
+    pdl_wait();
     for (int i = tid; i < 9 * COUT * C8; i += kWsThreads) {
         const int c8 = i % C8, row = i / C8, tap = row / COUT, co = row % COUT;
         cp_async16(sw + ((tap * C8 + c8) * COUT + co) * 16, a.w + (size_t)row * CIN + c8 * 8, true);
@@ -999,11 +1145,16 @@ __global__ void __launch_bounds__(kWsThreads) conv_s2_kernel(const __grid_consta
 #pragma unroll
                 for (int pr = 0; pr < 2; ++pr) {
 #pragma unroll
-                    for (int k = 0; k < C8; ++k)
-                        tma_load_5d(dst + pr * ROWP + k * PSE, &args.te, 8 * k, ox0, pr, oy0 - 1, n, bar);
-#pragma unroll
-                    for (int k = 0; k < C8; ++k)
-                        tma_load_5d(dst + pr * ROWP + C8 * PSE + k * PSO, &args.to, CIN + 8 * k, ox0 - 1, pr, oy0 - 1, n, bar);
+                    for (int k = 0; k < C8; ++k) {
+                        const uint32_t de = dst + pr * ROWP + k * PSE, dd = dst + pr * ROWP + C8 * PSE + k * PSO;
+                        if (a.lx == kNHWC) {
+                            tma_load_5d(de, &args.te, 8 * k, ox0, pr, oy0 - 1, n, bar);
+                            tma_load_5d(dd, &args.to, CIN + 8 * k, ox0 - 1, pr, oy0 - 1, n, bar);
+                        } else {
+                            tma_load_4d(de, &args.te, 4 * ox0, oy0 - 1, 4 * k + 2 * pr, n, bar);
+                            tma_load_4d(dd, &args.to, 4 * (ox0 - 1), oy0 - 1, 4 * k + 2 * pr + 1, n, bar);
+                        }
+                    }
                 }
                 s_issued = j + 1;
             }
@@ -1081,228 +1232,225 @@ __global__ void __launch_bounds__(kWsThreads) conv_s2_kernel(const __grid_consta
 }
 
 // ---------------------------------------------------------------------------------------
-// Weight gradient on the tensor cores (tcgen05): for every tap and channel pair
-//   dW[o][i][tap] = sum_p dz[p][o] x[p + off(tap)][i],
-// one GEMM D[(tap, i)][o] = sum_p A[(tap, i)][p] B[o][p] with the pixels as K: A is the
-// im2col of x (M = KS^2 * CIN rows, split into MT accumulators of 128 rows), B = dz^T
-// (N = COUT).  A CTA walks a contiguous range of 8 x 8 pixel tiles (K = 64 per tile) and keeps
-// its MT accumulators in tensor memory across the whole range:
-//   1. x (with a KS/2 halo, zero outside the image) and dz of the tile land in shared memory
-//      by cp.async as 16-byte pixel rows [chunk][row][col][8 channels], double-buffered;
-//   2. the four warps build the K-major operands from them with ldmatrix.trans: an 8 x 8
-//      block of (8 pixels of one tile row) x (8 channels) becomes one 128-byte core matrix
-//      (8 channels x 8 pixels); the tap's offset is applied in the ldmatrix row addresses;
-//   3. one thread issues MT x 4 MMAs (K = 16 each) and commits them to an mbarrier, which
-//      the warps wait on (bounded) before they overwrite the operands with the next tile.
-// Operand layouts (no swizzle): A tile mt at mt * 16 KB, core matrix (row group rg, pixel
-// row kg) at (16 kg + rg) * 128 (LBO 2048 between K groups, SBO 128 between row groups);
-// B core matrix (channel group og, kg) at (kg * COUT/8 + og) * 128 (LBO COUT * 16, SBO 128).
-// Rows of A past KS^2 * CIN are never written and their accumulator rows are discarded.
-// At the end each thread writes its accumulator row (one (tap, i)) to the CTA's slot of a
-// partials buffer; wgrad_reduce_kernel then adds the CTAs' partials in CTA order to the FP32
-// master gradient [Cout][Cin][k][k] (padding channels skipped), so the result does not depend
-// on the order in which CTAs finish.
-struct WgradArgs {
-    const bf16 *x, *dz;
-    float *gw;    // master layout
-    float *part;  // per-CTA partial products [grid][KS^2 CIN][COUT]
-    int N, H, W, cin_true, cout_true, tiles_per_cta;
+// Weight and bias gradients (tcgen05):
+//   dW[o][i][tap] = sum_p dz[p][o] x[p + off(tap)][i],   db[o] = sum_p dz[p][o],
+// as D[o][(tap, i)] += A[o][p] B[(tap, i)][p] with the pixels as K.  Eight pixels of a row by
+// eight channels, 128 bytes, are a core matrix of an MN-major operand as they lie (channels
+// contiguous, pixels 16 bytes apart), so neither x nor dz is transposed or copied.  x is staged
+// row by row, [row][chunk][col][8]: the channel chunks of consecutive rows are then one sequence
+// of N groups, XW * 16 bytes apart, and one MMA takes three taps of a column kx (ky = 0, 1, 2)
+// at N = 3 CIN.  An MMA costs about 60 clocks whatever its N up to there, so that is three times
+// fewer clocks than a tap each (16 -> 16 channels on a 16 x 128^2 batch: 28.8 us, now 13.6).
+// M = 64 rows of A are read: COUT of dz, the rest whatever the shared memory after it holds, rows
+// of D that nothing reads.
+// A tile is 16 rows x 8 pixels, K = 128.  A CTA walks tiles blockIdx.x, + gridDim.x, ...: one lane
+// loads them by TMA into a ring, one lane issues a tile's MMAs, warp 3 adds up the bias gradient
+// from the staged dz, and the accumulators stay in tensor memory to the end.  Where nine taps do
+// not fit (CIN = 64, 96), blockIdx.y takes a column of taps each.  MODE 1 is the stride-2 layer:
+// dz at the output's size and x as parity planes (conv_s2_kernel's taps: rows ky = 0 and 2 of
+// parity 1, ky = 1 of parity 0), so that no product is spent on dropped positions.  Every CTA
+// writes its accumulators to its slice of the layer's partials and wgrad_reduce_kernel adds the
+// slices in a fixed order.
+// The form before built both operands with ldmatrix and shared stores from NHWC pixels and took
+// its bias sums in kernels of their own: the backward pass of a 16 x 128^2 batch spent 343 us in
+// weight gradients, 158 us in bias gradients and 110 us in twelve reductions; now 145 us with the bias and one reduction
+// of 27 us.
+struct alignas(128) WgradArgs {
+    CUtensorMap tx, tdz;
+    float *part;  // [gridDim.x][COUT][KS^2 CIN + 8]
+    int N, H, W;  // the size of dz
+    int layout;   // of dz (and, MODE 0, of x): kNHWC or kPlanes
     int *status;
 };
 
-// gw[o][i][tap] += sum over the CTAs, in CTA order, of their partial (tap CIN + i, o): the
-// weight gradient without atomics, the same every run.  Thread f takes element f of the
-// partials' own layout ((tap CIN + i) COUT + o), so that the threads of a warp read
-// consecutive addresses of each CTA's partial; the loads of several CTAs are in flight at once
-// while the additions keep CTA order.
-template <int CIN, int COUT, int KS>
-__global__ void __launch_bounds__(32) wgrad_reduce_kernel(const float *part, int nctas, float *gw, int cin_true,
-                                                          int cout_true)
+template <int CIN, int COUT, int KS, int MODE>
+struct WgGeom {
+    static constexpr int P = KS / 2, C8 = CIN / 8, O8 = COUT / 8, TAPS = KS * KS;
+    static constexpr int NG = TAPS * CIN > 512 ? KS : 1;  // tap columns split over blockIdx.y
+    static constexpr int KXN = KS / NG;                   // tap columns per CTA
+    static constexpr int XH = MODE ? 17 : 16 + 2 * P, XW = MODE ? 9 : 8 + 2 * P;  // staged rows and columns
+    static constexpr int RP = C8 * XW * 16;                                       // one row, all chunks
+    static constexpr int XP = (XH * RP + 127) / 128 * 128;                        // x (MODE 1: one parity plane)
+    static constexpr int NXP = MODE ? 4 : 1;
+    static constexpr int DP = 16 * 8 * 16;                                        // one dz plane
+    static constexpr int STAGE = NXP * XP + O8 * DP;
+    static constexpr int NBUF = 4 * STAGE <= 150 * 1024 ? 4 : 2;
+    static constexpr int TMA_BYTES = NXP * XH * RP + O8 * DP;
+    static constexpr int PAD = (8 - O8) * DP;  // the 64 rows of A reach past the last stage
+    static constexpr int SMEM = 128 + NBUF * STAGE + PAD + (2 * NBUF + 1) * 8 + 16;
+    static constexpr int COLS = tmem_cols<KXN * KS * CIN>();
+    static constexpr int CTOT = TAPS * CIN + 8;  // columns of a partial: (kx, ky, channel), then the bias
+    // tap rows of one MMA: MODE 0 as many as N = 256 holds; MODE 1 rows 0 and 2, then row 1
+    static constexpr int KYN = KS == 1 ? 1 : MODE ? 2 : (3 * CIN <= 256 ? 3 : 2);
+};
+constexpr int kWgThreads = 128;
+
+// instruction descriptor, kind::f16: D FP32, A and B BF16, both MN-major, M = 64, N = n
+__host__ __device__ constexpr uint32_t umma_idesc_mn64(int n)
 {
-    constexpr int M = KS * KS * CIN, NB = 64;
-    for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < M * COUT; f += gridDim.x * blockDim.x) {
-        const int o = f % COUT, row = f / COUT, i = row % CIN, tap = row / CIN;
-        if (i >= cin_true || o >= cout_true) continue;
-        const float *p = part + f;
-        // the partials in CTA order; each batch's loads are issued (in order, as volatile loads)
-        // before any of its additions, so a thread has NB of them in flight
-        float s = 0.f;
-        int b = 0;
-        for (; b + NB <= nctas; b += NB) {
-            float v[NB];
+    return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(64 >> 4) << 24);
+}
+
+// The MMAs of one staged tile, tap columns [kx0, kx0 + KXN)
+template <int CIN, int COUT, int KS, int MODE>
+__device__ __forceinline__ void wgrad_mmas(uint32_t stage, uint32_t tmem, int kx0, bool first)
+{
+    using G = WgGeom<CIN, COUT, KS, MODE>;
+    // MN-major, no swizzle: LBO between K groups (8 pixels), SBO between groups of 8 channels
+    const uint64_t ad0 = umma_sdesc(stage + G::NXP * G::XP, 128, G::DP);
+    const uint64_t bd0 = umma_sdesc(stage, G::RP, G::XW * 16);
 #pragma unroll
-            for (int u = 0; u < NB; ++u)
-                asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v[u]) : "l"(p + (size_t)(b + u) * M * COUT));
+    for (int k = 0; k < G::KXN; ++k) {
+        const int kx = kx0 + k;
 #pragma unroll
-            for (int u = 0; u < NB; ++u) s += v[u];
+        for (int s = 0; s < KS; s += G::KYN) {  // slots s .. of the column (MODE 1: ky = 0, 2, 1)
+            constexpr int kyn = G::KYN;
+            const int ns = KS - s < kyn ? KS - s : kyn;
+            uint32_t off;
+            if (MODE) off = (uint32_t)((2 * (s == 0) + (kx != 1)) * G::XP + (s != 0) * G::RP + (kx != 0) * 16);
+            else off = (uint32_t)(s * G::RP + kx * 16);
+            const uint32_t idesc = umma_idesc_mn64(ns * CIN), d = tmem + (uint32_t)((k * KS + s) * CIN);
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks)
+                umma_bf16(d, ad0 + (uint64_t)((ks * 256) >> 4), bd0 + (uint64_t)((off + 2 * ks * G::RP) >> 4), idesc,
+                          (first && ks == 0) ? 0u : 1u);
         }
-        for (; b < nctas; ++b) s += p[(size_t)b * M * COUT];
-        gw[((size_t)o * cin_true + i) * (KS * KS) + tap] += s;
     }
 }
 
-template <int CIN, int COUT, int KS>
-struct WgGeom {
-    static constexpr int P = KS / 2, SH = 8 + 2 * P, SW = 8 + 2 * P, C8 = CIN / 8, O8 = COUT / 8;
-    static constexpr int M = KS * KS * CIN, MT = (M + 127) / 128;
-    static constexpr int XP = (SH * SW * 16 + 127) / 128 * 128;  // one staged x chunk plane
-    static constexpr int STAGE = C8 * XP + O8 * 1024;            // x planes, then dz planes [8][8][8]
-    static constexpr int ABYTES = MT * 16384, BBYTES = O8 * 1024;
-    static constexpr int SMEM = 128 + 2 * STAGE + ABYTES + BBYTES + 16;
-    static constexpr int COLS = tmem_cols<MT * COUT>();
-    static constexpr int NU = KS * KS * C8 * 8;  // A core matrices per tile (tap, chunk, pixel row)
-    static_assert(MT * COUT <= 512, "accumulators exceed tensor memory");
-};
-
-__device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3)
+template <int CIN, int COUT, int KS, int MODE>
+__global__ void __launch_bounds__(kWgThreads) wgrad_tc_kernel(const __grid_constant__ WgradArgs a)
 {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-                 : "r"(addr));
-}
-
-template <int CIN, int COUT, int KS>
-__global__ void __launch_bounds__(128) wgrad_tc_kernel(const WgradArgs a)
-{
-    using G = WgGeom<CIN, COUT, KS>;
-    constexpr int P = G::P, SW = G::SW, C8 = G::C8, O8 = G::O8, XP = G::XP, MT = G::MT;
-    static_assert(CIN % 16 == 0 && COUT % 16 == 0, "UMMA shape");
+    using G = WgGeom<CIN, COUT, KS, MODE>;
+    static_assert(CIN % 16 == 0 && COUT % 16 == 0 && COUT <= 64 && (MODE == 0 || KS == 3), "UMMA shape");
+    constexpr int NBUF = G::NBUF;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char *base = smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127);
-    unsigned char *stage0 = base;
-    unsigned char *opA = base + 2 * G::STAGE;
-    unsigned char *opB = opA + G::ABYTES;
-    uint64_t *done = reinterpret_cast<uint64_t *>(opB + G::BBYTES);
+    uint64_t *full = reinterpret_cast<uint64_t *>(base + NBUF * G::STAGE + G::PAD);
+    uint64_t *empty = full + NBUF, *done = empty + NBUF;
     __shared__ uint32_t s_tmem;
-    __shared__ int s_fail;
+    __shared__ int s_issued, s_consumed, s_fail;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int tiles_x = (a.W + 7) / 8, tiles_y = (a.H + 7) / 8;
-    const long long ntiles = (long long)a.N * tiles_x * tiles_y;
-    const long long t0 = (long long)blockIdx.x * a.tiles_per_cta;
-    const long long t1 = t0 + a.tiles_per_cta < ntiles ? t0 + a.tiles_per_cta : ntiles;
+    const int tiles_x = (a.W + 7) / 8, tiles_y = (a.H + 15) / 16;
+    const int per_img = tiles_x * tiles_y, ntiles = a.N * per_img;
+    const int mine = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&s_tmem)),
                      "r"(G::COLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
     }
     if (tid == 0) {
+        for (int i = 0; i < NBUF; ++i) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(full + i)));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;\n" ::"r"(smem_u32(empty + i)));  // MMAs, bias warp
+        }
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(done)));
         asm volatile("fence.mbarrier_init.release.cluster;\n");
-        s_fail = 0;
+        s_issued = s_consumed = s_fail = 0;
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n");
     const uint32_t tmem = s_tmem;
+    pdl_trigger();
+    pdl_wait();
 
-    auto stage = [&](long long t, unsigned char *sb) {
-        const int n = (int)(t / ((long long)tiles_x * tiles_y));
-        const int r = (int)(t % ((long long)tiles_x * tiles_y));
-        const int ty0 = (r / tiles_x) * 8, tx0 = (r % tiles_x) * 8;
-        for (int e = tid; e < C8 * G::SH * SW; e += 128) {
-            const int c8 = e / (G::SH * SW), pix = e % (G::SH * SW);
-            const int yy = ty0 - P + pix / SW, xx = tx0 - P + pix % SW;
-            const bool in = yy >= 0 && yy < a.H && xx >= 0 && xx < a.W;
-            const bf16 *src = in ? a.x + (((size_t)n * a.H + yy) * a.W + xx) * CIN + c8 * 8 : a.x;
-            cp_async16(sb + c8 * XP + pix * 16, src, in);
-        }
-        unsigned char *sd = sb + C8 * XP;
-        for (int e = tid; e < O8 * 64; e += 128) {
-            const int o8 = e / 64, pix = e % 64;
-            const int yy = ty0 + pix / 8, xx = tx0 + pix % 8;
-            const bool in = yy < a.H && xx < a.W;
-            const bf16 *src = in ? a.dz + (((size_t)n * a.H + yy) * a.W + xx) * COUT + o8 * 8 : a.dz;
-            cp_async16(sd + o8 * 1024 + pix * 16, src, in);
-        }
-    };
-
-    constexpr uint32_t idesc = umma_idesc(COUT);
-    int it = 0;
-    if (t0 < t1) stage(t0, stage0);
-    cp_async_commit();
-    for (long long t = t0; t < t1; ++t, ++it) {
-        unsigned char *sb = stage0 + (it & 1) * G::STAGE;
-        if (t + 1 < t1) stage(t + 1, stage0 + ((it + 1) & 1) * G::STAGE);
-        cp_async_commit();
-        cp_async_wait<1>();
-        // the MMAs of the previous tile must have read the operands before they are rebuilt
-        if (it > 0 && !mbar_wait_warp(smem_u32(done), (uint32_t)((it - 1) & 1))) {
-            if (lane == 0) s_fail = 1;
-        }
-        __syncthreads();
-        if (s_fail) break;
-        // A: unit q = (tap, chunk, pixel row ty); lanes 8j..8j+7 address unit q + j, row tx
-        const uint32_t xs = smem_u32(sb), as = smem_u32(opA);
-        for (int q = 4 * warp; q < G::NU; q += 16) {
-            const int u = q + (lane >> 3), tx = lane & 7;
-            const int ty = u % 8, c8 = (u / 8) % C8, tap = u / (8 * C8);
-            const int dy = tap / KS, dx = tap % KS;
-            uint32_t v[4];
-            ldsm_x4_trans(xs + c8 * XP + ((ty + dy) * SW + tx + dx) * 16, v[0], v[1], v[2], v[3]);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int uj = q + j, tyj = uj % 8, m0 = (uj / (8 * C8)) * CIN + ((uj / 8) % C8) * 8;
-                const uint32_t dst = as + (m0 / 128) * 16384 + (tyj * 16 + (m0 % 128) / 8) * 128 + lane * 4;
-                asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(dst), "r"(v[j]) : "memory");
+    if (warp == 1 && lane == 0) {  // producer
+        for (int j = 0; j < mine; ++j) {
+            const int st = j % NBUF;
+            if (j >= NBUF && !mbar_wait_thread(smem_u32(empty + st), (uint32_t)((j / NBUF - 1) & 1))) {
+                s_fail = 1;
+                break;
             }
-        }
-        // B: unit q = (channel group og, pixel row ty)
-        const uint32_t ds = xs + C8 * XP, bs = smem_u32(opB);
-        for (int q = 4 * warp; q < O8 * 8; q += 16) {
-            const int u = q + (lane >> 3), tx = lane & 7;
-            const int ty = u % 8, og = u / 8;
-            uint32_t v[4];
-            ldsm_x4_trans(ds + og * 1024 + (ty * 8 + tx) * 16, v[0], v[1], v[2], v[3]);
+            const int t = blockIdx.x + j * gridDim.x, n = t / per_img, r = t % per_img;
+            const int ty0 = (r / tiles_x) * 16, tx0 = (r % tiles_x) * 8;
+            const uint32_t bar = smem_u32(full + st), dst = smem_u32(base + st * G::STAGE);
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(G::TMA_BYTES) : "memory");
+            if (MODE) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int uj = q + j;
-                const uint32_t dst = bs + ((uj % 8) * O8 + uj / 8) * 128 + lane * 4;
-                asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(dst), "r"(v[j]) : "memory");
+                for (int pp = 0; pp < 4; ++pp) tma_load_5d(dst + pp * G::XP, &a.tx, 4 * (tx0 - 1), 0, ty0 - 1, pp, n, bar);
+            } else if (a.layout == kNHWC) {
+                tma_load_5d(dst, &a.tx, 0, tx0 - G::P, 0, ty0 - G::P, n, bar);
+            } else {
+                tma_load_4d(dst, &a.tx, 4 * (tx0 - G::P), 0, ty0 - G::P, n, bar);
             }
+            load_planes<G::O8, G::DP>(dst + G::NXP * G::XP, &a.tdz, a.layout, tx0, ty0, n, bar);
+            s_issued = j + 1;
         }
-        asm volatile("fence.proxy.async.shared::cta;\n");  // operands visible to the tensor core
-        __syncthreads();
-        if (tid == 0) {
+    } else if (warp == 2 && lane == 0) {  // MMA issuer
+        int j = 0;
+        for (; j < mine; ++j) {
+            const int st = j % NBUF;
+            if (!mbar_wait_thread(smem_u32(full + st), (uint32_t)((j / NBUF) & 1))) {
+                s_fail = 1;
+                break;
+            }
+            s_consumed = j + 1;
             asm volatile("tcgen05.fence::after_thread_sync;\n");
-            const uint64_t ad0 = umma_sdesc(as, 2048, 128), bd0 = umma_sdesc(bs, O8 * 128, 128);
+            wgrad_mmas<CIN, COUT, KS, MODE>(smem_u32(base + st * G::STAGE), tmem, G::NG > 1 ? (int)blockIdx.y : 0, j == 0);
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                smem_u32(empty + st)));
+        }
+        if (mine > 0 && j == mine)
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_u32(done)));
+    } else if (warp == 3) {  // bias gradient: LP lanes per 8-channel chunk of dz, every LP-th pixel each
+        constexpr int LP = 32 / G::O8;
+        const int o8 = lane / LP, l = lane % LP;
+        float acc[8] = {};
+        for (int j = 0; j < mine; ++j) {
+            const int st = j % NBUF;
+            if (!mbar_wait_warp(smem_u32(full + st), (uint32_t)((j / NBUF) & 1))) {
+                if (lane == 0) s_fail = 1;
+                break;
+            }
+            if (blockIdx.y == 0) {
+                const uint4 *dz = reinterpret_cast<const uint4 *>(base + st * G::STAGE + G::NXP * G::XP + o8 * G::DP) + l;
 #pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                const uint64_t bd = bd0 + (uint64_t)((2 * s * O8 * 128) >> 4);
+                for (int p = 0; p < 128 / LP; ++p) {
+                    const uint4 v = dz[p * LP];
+                    const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
 #pragma unroll
-                for (int mt = 0; mt < MT; ++mt) {
-                    const uint64_t ad = ad0 + (uint64_t)((mt * 16384 + 2 * s * 2048) >> 4);
-                    umma_bf16(tmem + (uint32_t)(mt * COUT), ad, bd, idesc, (it > 0 || s > 0) ? 1u : 0u);
+                    for (int i = 0; i < 4; ++i) {
+                        acc[2 * i] += __low2float(h[i]);
+                        acc[2 * i + 1] += __high2float(h[i]);
+                    }
                 }
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                smem_u32(done)));
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(empty + st)) : "memory");
+        }
+        if (blockIdx.y == 0) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+#pragma unroll
+                for (int o = LP / 2; o > 0; o >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+                if (l == 0) a.part[((size_t)blockIdx.x * COUT + o8 * 8 + i) * G::CTOT + G::TAPS * CIN] = acc[i];
+            }
         }
     }
-    cp_async_wait<0>();
-    bool ok = !s_fail;
-    if (ok && it > 0 && !mbar_wait_warp(smem_u32(done), (uint32_t)((it - 1) & 1))) {
-        ok = false;
+    __syncwarp();
+    __syncthreads();  // the issuing lanes are through
+    if (!s_fail && mine > 0 && !mbar_wait_warp(smem_u32(done), 0u)) {
         if (lane == 0) s_fail = 1;
     }
     __syncthreads();
     if (s_fail) {
         if (tid == 0 && a.status) atomicExch(a.status, FLNR_STATUS_TIMEOUT);
-    } else if (it > 0) {
+        if (tid == 32)  // let copies still in flight land before the CTA exits
+            for (int j = s_consumed; j < s_issued; ++j) mbar_wait_thread(smem_u32(full + j % NBUF), (uint32_t)((j / NBUF) & 1));
+    } else if (16 * warp < COUT) {
+        // M = 64: rows 16 w .. 16 w + 15 in lanes 0-15 of lane quarter w
         asm volatile("tcgen05.fence::after_thread_sync;\n");
-        const int r = 32 * warp + lane;
+        float *dst = a.part + ((size_t)blockIdx.x * COUT + 16 * warp + lane) * G::CTOT + blockIdx.y * (G::KXN * KS * CIN);
 #pragma unroll 1
-        for (int mt = 0; mt < MT; ++mt) {
-            const int m = mt * 128 + r;
+        for (int c = 0; c < G::KXN * KS * CIN; c += 16) {
+            float v[16] = {};
+            if (mine > 0) tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c, v);
+            asm volatile("tcgen05.wait::ld.sync.aligned;\n");
+            if (lane < 16) {
 #pragma unroll
-            for (int o0 = 0; o0 < COUT; o0 += 16) {
-                float v[16];
-                tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(mt * COUT + o0), v);
-                asm volatile("tcgen05.wait::ld.sync.aligned;\n");
-                if (m < G::M) {  // this CTA's partial row, summed in a fixed order by wgrad_reduce_kernel
-                    float4 *dst = reinterpret_cast<float4 *>(a.part + ((size_t)blockIdx.x * G::M + m) * COUT + o0);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) dst[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-                }
+                for (int j = 0; j < 4; ++j)
+                    *reinterpret_cast<float4 *>(dst + c + 4 * j) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             }
         }
     }
@@ -1314,12 +1462,71 @@ __global__ void __launch_bounds__(128) wgrad_tc_kernel(const WgradArgs a)
     }
 }
 
+// The layers' partials into the FP32 master gradients, one launch for all of them: element f of
+// a layer is (o, column) of its slices [slices][COUT][CTOT]; 32 consecutive elements per CTA
+// (coalesced), sixteen warps take slices w, w + 16, ... in turn and their sums are added in warp
+// order, so the result is the same every run.  Padding channels are skipped.
+struct RedLayer {
+    const float *part;
+    float *gw, *gb;
+    int slices, cout, cin, ks, s2, cin_true, cout_true, first_block;
+};
+struct RedArgs {
+    RedLayer l[kNL];
+    int n = 0, blocks = 0;
+};
+constexpr int kRedWarps = 16;
+
+__global__ void __launch_bounds__(32 * kRedWarps) wgrad_reduce_kernel(const __grid_constant__ RedArgs a)
+{
+    pdl_trigger();
+    pdl_wait();
+    int k = 0;
+    while (k + 1 < a.n && (int)blockIdx.x >= a.l[k + 1].first_block) ++k;
+    const RedLayer &l = a.l[k];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int taps = l.ks * l.ks, ctot = taps * l.cin + 8, total = l.cout * ctot;
+    const int f = (blockIdx.x - l.first_block) * 32 + lane;
+    __shared__ float s_sum[kRedWarps][32];
+    float s = 0.f;
+    if (f < total) {
+        const float *p = l.part + f;
+        constexpr int NB = 10;  // loads in flight: all of a warp's slices on 152 SMs
+        for (int j = w; j < l.slices; j += NB * kRedWarps) {
+            float v[NB];
+#pragma unroll
+            for (int u = 0; u < NB; ++u) {
+                const int jj = j + u * kRedWarps;
+                v[u] = jj < l.slices ? __ldg(p + (size_t)jj * total) : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < NB; ++u) s += v[u];
+        }
+    }
+    s_sum[w][lane] = s;
+    __syncthreads();
+    if (w != 0 || f >= total) return;
+#pragma unroll
+    for (int u = 1; u < kRedWarps; ++u) s += s_sum[u][lane];
+    const int o = f / ctot, c = f % ctot;
+    if (o >= l.cout_true) return;
+    if (c == taps * l.cin) {
+        l.gb[o] += s;
+    } else if (c < taps * l.cin) {
+        const int i = c % l.cin, slot = c / l.cin % l.ks, kx = c / (l.cin * l.ks);
+        const int ky = l.s2 ? (slot == 1 ? 2 : slot == 2 ? 1 : 0) : slot;
+        if (i < l.cin_true) l.gw[((size_t)o * l.cin_true + i) * taps + ky * l.ks + kx] += s;
+    }
+}
+
 // ---------------------------------------------------------------------------------------
 // Elementwise and layout kernels
-// planar fp32 [N][11][H][W] -> NHWC bf16 with 16 channels (11 used); the radiance channels
+// planar fp32 [N][11][H][W] -> bf16 planes with 16 channels (11 used); the radiance channels
 // enter the network as log(1 + max(Y, 0)), which keeps fireflies from dominating the features
 __global__ void pack_input_kernel(const float *in, bf16 *x, int N, int H, int W)
 {
+    pdl_trigger();
+    pdl_wait();
     const size_t hw = (size_t)H * W, total = (size_t)N * hw;
     for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < total; p += (size_t)gridDim.x * blockDim.x) {
         const size_t n = p / hw, o = p % hw;
@@ -1331,25 +1538,28 @@ __global__ void pack_input_kernel(const float *in, bf16 *x, int N, int H, int W)
             else if (c < 11) u = log1pf(fmaxf(in[(n * 11 + c) * hw + o], 0.f));  // radiance: log(1 + max(Y, 0))
             v[c] = __float2bfloat16(u);
         }
-        *reinterpret_cast<uint4 *>(x + p * 16) = *reinterpret_cast<uint4 *>(v);
-        *reinterpret_cast<uint4 *>(x + p * 16 + 8) = *reinterpret_cast<uint4 *>(v + 8);
+        *reinterpret_cast<uint4 *>(x + (2 * n * hw + o) * 8) = *reinterpret_cast<uint4 *>(v);
+        *reinterpret_cast<uint4 *>(x + ((2 * n + 1) * hw + o) * 8) = *reinterpret_cast<uint4 *>(v + 8);
     }
 }
 
-// gradient with respect to the network's planar input [N][11][H][W] from the gradient dx
-// [N][H][W][16] with respect to the packed input x: the guides pass through; a radiance
+// gradient with respect to the network's planar input [N][11][H][W] from the gradient dx (bf16
+// planes, 16 channels) with respect to the packed input x: the guides pass through; a radiance
 // channel was read as L = log(1 + max(Y, 0)), whose derivative is 1 / (1 + Y) = exp(-L) for
 // Y > 0 and 0 for Y < 0 (L is the stored bfloat16 value, so Y > 0 exactly when L > 0)
 __global__ void unpack_grad_kernel(const bf16 *dx, const bf16 *x, float *g, int N, int H, int W)
 {
+    pdl_trigger();
+    pdl_wait();
     const size_t hw = (size_t)H * W, total = (size_t)N * hw;
     for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < total; p += (size_t)gridDim.x * blockDim.x) {
         const size_t n = p / hw, o = p % hw;
 #pragma unroll
         for (int c = 0; c < 11; ++c) {
-            float d = __bfloat162float(dx[p * 16 + c]);
+            const size_t e = ((2 * n + c / 8) * hw + o) * 8 + c % 8;
+            float d = __bfloat162float(dx[e]);
             if (c >= 8) {
-                const float L = __bfloat162float(x[p * 16 + c]);
+                const float L = __bfloat162float(x[e]);
                 d = L > 0.f ? d * expf(-L) : 0.f;
             }
             g[(n * 11 + c) * hw + o] = d;
@@ -1357,72 +1567,44 @@ __global__ void unpack_grad_kernel(const bf16 *dx, const bf16 *x, float *g, int 
     }
 }
 
-// nearest 2x upsampling of lo [N][H/2][W/2][Ca] concatenated with skip [N][H][W][Cb] (the
-// input of a decoder level, materialised for its weight gradient)
+// nearest 2x upsampling of lo (Ca channels, H/2 x W/2) concatenated with skip (Cb channels,
+// H x W), all bf16 planes (the input of a decoder level, materialised for its weight gradient)
 __global__ void upcat_kernel(const bf16 *lo, const bf16 *skip, bf16 *y, int N, int H, int W, int Ca, int Cb)
 {
-    // one thread per (pixel, 8-channel group) of y [N][H][W][Ca + Cb]: 16-byte copies
-    const int C8 = (Ca + Cb) / 8, A8 = Ca / 8;
-    const long long total = (long long)N * H * W * C8;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
-        const int c8 = (int)(e % C8);
-        const long long p = e / C8;
+    pdl_trigger();
+    pdl_wait();
+    // one thread per pixel of a chunk plane of y: 16-byte copies
+    const int C8 = (Ca + Cb) / 8, A8 = Ca / 8, B8 = Cb / 8, hw = H * W;
+    const size_t total = (size_t)N * C8 * hw;
+    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
+        const int q = (int)(e / hw), p = (int)(e % hw), n = q / C8, c8 = q % C8;
         const uint4 *src;
-        if (c8 < A8) {
-            const int x = (int)(p % W);
-            const long long rowp = p / W;  // n * H + y
-            const int yy = (int)(rowp % H);
-            const long long n = rowp / H;
-            src = reinterpret_cast<const uint4 *>(lo + ((n * (H / 2) + yy / 2) * (W / 2) + x / 2) * Ca + c8 * 8);
-        } else {
-            src = reinterpret_cast<const uint4 *>(skip + p * Cb + (c8 - A8) * 8);
-        }
+        if (c8 < A8)
+            src = reinterpret_cast<const uint4 *>(lo) + (size_t)(n * A8 + c8) * (hw / 4) + (size_t)(p / W / 2) * (W / 2) + p % W / 2;
+        else
+            src = reinterpret_cast<const uint4 *>(skip) + (size_t)(n * B8 + c8 - A8) * hw + p;
         reinterpret_cast<uint4 *>(y)[e] = *src;
     }
 }
 
-// gradient of the sigmoid output head (nout planar outputs): dz[p][c] = g * s (1 - s) for
-// c < nout, 0 for the pads of the 16 channels
-__global__ void sigmoid_bwd_kernel(const float *g, const float *s, bf16 *dz, int N, int H, int W, int nout)
-{
-    const size_t hw = (size_t)H * W, total = (size_t)N * hw;
-    for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < total; p += (size_t)gridDim.x * blockDim.x) {
-        const size_t n = p / hw, o = p % hw;
-        alignas(16) bf16 v[16];
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-            float d = 0.f;
-            if (c < nout) {
-                const float sv = s[(n * nout + c) * hw + o];
-                d = g[(n * nout + c) * hw + o] * sv * (1.f - sv);
-            }
-            v[c] = __float2bfloat16(d);
-        }
-        *reinterpret_cast<uint4 *>(dz + p * 16) = *reinterpret_cast<uint4 *>(v);
-        *reinterpret_cast<uint4 *>(dz + p * 16 + 8) = *reinterpret_cast<uint4 *>(v + 8);
-    }
-}
-
-// backward of up ++ skip: g_lo[q][c] = mask(lo) * sum_{2x2} gy[p][c] (c < Ca);
-// g_skip[p][c] = gy[p][Ca + c] (unmasked, the caller masks where the skip is consumed)
+// backward of up ++ skip (bf16 planes): g_lo[q][c] = mask(lo) * sum_{2x2} gy[p][c] (c < Ca);
+// g_skip[p][c] = gy[p][Ca + c] in fp32 planes (unmasked, the caller masks where the skip is
+// consumed)
 __global__ void upcat_bwd_kernel(const bf16 *gy, const bf16 *lo, bf16 *g_lo, float *g_skip, int N, int H, int W,
                                  int Ca, int Cb)
 {
-    // eight channels of one pixel per thread (Ca and Cb are multiples of 8): 16-byte loads and
-    // stores, the index arithmetic once per eight values
-    const int C = Ca + Cb, Hl = H / 2, Wl = W / 2;
-    const size_t tl = (size_t)N * Hl * Wl * Ca / 8, ts = (size_t)N * H * W * Cb / 8;
-    for (size_t e8 = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e8 < tl + ts; e8 += (size_t)gridDim.x * blockDim.x) {
-        if (e8 < tl) {
-            const size_t e = 8 * e8;
-            const int c = (int)(e % Ca);
-            const size_t q = e / Ca;
-            const int xl = (int)(q % Wl), yl = (int)((q / Wl) % Hl), n = (int)(q / ((size_t)Wl * Hl));
-            const size_t b = (((size_t)n * H + 2 * yl) * W + 2 * xl) * C + c;
-            const uint4 r0 = *reinterpret_cast<const uint4 *>(gy + b), r1 = *reinterpret_cast<const uint4 *>(gy + b + C);
-            const uint4 r2 = *reinterpret_cast<const uint4 *>(gy + b + (size_t)W * C);
-            const uint4 r3 = *reinterpret_cast<const uint4 *>(gy + b + (size_t)W * C + C);
-            const uint4 l = *reinterpret_cast<const uint4 *>(lo + e);
+    pdl_trigger();
+    pdl_wait();
+    // eight channels of one pixel per thread: 16-byte loads and stores
+    const int A8 = Ca / 8, B8 = Cb / 8, C8 = A8 + B8, hw = H * W, hl = hw / 4, Wl = W / 2;
+    const size_t tl = (size_t)N * A8 * hl, ts = (size_t)N * B8 * hw;
+    const uint4 *g4 = reinterpret_cast<const uint4 *>(gy);
+    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < tl + ts; e += (size_t)gridDim.x * blockDim.x) {
+        if (e < tl) {
+            const int q = (int)(e / hl), pl = (int)(e % hl), n = q / A8, c8 = q % A8;
+            const size_t b = (size_t)(n * C8 + c8) * hw + (size_t)(2 * (pl / Wl)) * W + 2 * (pl % Wl);
+            const uint4 r0 = g4[b], r1 = g4[b + 1], r2 = g4[b + W], r3 = g4[b + W + 1];
+            const uint4 l = reinterpret_cast<const uint4 *>(lo)[e];
             const bf16 *g0 = reinterpret_cast<const bf16 *>(&r0), *g1 = reinterpret_cast<const bf16 *>(&r1);
             const bf16 *g2 = reinterpret_cast<const bf16 *>(&r2), *g3 = reinterpret_cast<const bf16 *>(&r3);
             const bf16 *lv = reinterpret_cast<const bf16 *>(&l);
@@ -1434,55 +1616,55 @@ __global__ void upcat_bwd_kernel(const bf16 *gy, const bf16 *lo, bf16 *g_lo, flo
                                   __bfloat162float(g3[i]);
                 ov[i] = __float2bfloat16(__bfloat162float(lv[i]) > 0.f ? sum : 0.f);
             }
-            *reinterpret_cast<uint4 *>(g_lo + e) = o;
+            reinterpret_cast<uint4 *>(g_lo)[e] = o;
         } else {
-            const size_t f = 8 * (e8 - tl);
-            const int c = (int)(f % Cb);
-            const uint4 r = *reinterpret_cast<const uint4 *>(gy + (f / Cb) * C + Ca + c);
+            const size_t f = e - tl;
+            const int q = (int)(f / hw), p = (int)(f % hw), n = q / B8, c8 = q % B8;
+            const uint4 r = g4[(size_t)(n * C8 + A8 + c8) * hw + p];
             const bf16 *rv = reinterpret_cast<const bf16 *>(&r);
             float4 v0, v1;
             v0.x = __bfloat162float(rv[0]); v0.y = __bfloat162float(rv[1]);
             v0.z = __bfloat162float(rv[2]); v0.w = __bfloat162float(rv[3]);
             v1.x = __bfloat162float(rv[4]); v1.y = __bfloat162float(rv[5]);
             v1.z = __bfloat162float(rv[6]); v1.w = __bfloat162float(rv[7]);
-            *reinterpret_cast<float4 *>(g_skip + f) = v0;
-            *reinterpret_cast<float4 *>(g_skip + f + 4) = v1;
+            *reinterpret_cast<float4 *>(g_skip + 8 * f) = v0;
+            *reinterpret_cast<float4 *>(g_skip + 8 * f + 4) = v1;
         }
     }
 }
 
-// Gradient with respect to the pre-activation of a layer whose ReLU output f [N][Ho][Wo][C]
-// feeds the next encoder convolution (gradient g_path, bf16) and, when g_skip is given, a
-// decoder skip (fp32): dz = mask(f) * (g_skip + g_path); no mask when f is NULL.  S = 2 (the
-// layer strides by 2): dz is written zero-upsampled onto the layer's input grid
-// [N][2Ho][2Wo][C], nonzero only at even rows and columns, so that the stride-1 input- and
-// weight-gradient kernels at the input's size give the stride-2 layer's gradients.
+// Gradient with respect to the pre-activation of a layer whose ReLU output f (C channels,
+// Ho x Wo) feeds the next encoder convolution (gradient g_path, bf16 planes) and, when g_skip is
+// given, a decoder skip (fp32 planes): dz = mask(f) * (g_skip + g_path); no mask when f is NULL.
+// S = 2 (the layer strides by 2): dz is written zero-upsampled onto the layer's input grid
+// 2Ho x 2Wo, nonzero only at even rows and columns, so that the stride-1 input-gradient kernel
+// gives the stride-2 layer's gradient, and, when dlo is given, at its own size too (for the
+// weight gradient).
 template <int S>
-__global__ void join_bwd_kernel(const float *g_skip, const bf16 *g_path, const bf16 *f, bf16 *dz, int N, int Ho, int Wo,
-                                int C)
+__global__ void join_bwd_kernel(const float *g_skip, const bf16 *g_path, const bf16 *f, bf16 *dz, bf16 *dlo, int N,
+                                int Ho, int Wo, int C)
 {
-    // eight channels of one pixel per thread (C a multiple of 8): 16-byte loads and stores
-    const int H = S * Ho, W = S * Wo;
-    const size_t total8 = (size_t)N * H * W * C / 8;
-    for (size_t e8 = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e8 < total8; e8 += (size_t)gridDim.x * blockDim.x) {
-        const size_t e = 8 * e8;
-        const int c = (int)(e % C);
-        const size_t p = e / C;
-        const int x = (int)(p % W), y = (int)((p / W) % H), n = (int)(p / ((size_t)W * H));
+    pdl_trigger();
+    pdl_wait();
+    // eight channels of one pixel per thread: 16-byte loads and stores
+    const int hw = S * Ho * S * Wo, W = S * Wo;
+    const size_t total = (size_t)N * (C / 8) * hw;
+    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
+        const int k = (int)(e / hw), p = (int)(e % hw), x = p % W, y = p / W;
         uint4 o = make_uint4(0u, 0u, 0u, 0u);  // bfloat16 +0
         if (S == 1 || ((x | y) & 1) == 0) {
-            const size_t q = (((size_t)n * Ho + y / S) * Wo + x / S) * C + c;
-            const uint4 gp = *reinterpret_cast<const uint4 *>(g_path + q);
+            const size_t q = (size_t)k * Ho * Wo + (size_t)(y / S) * Wo + x / S;
+            const uint4 gp = reinterpret_cast<const uint4 *>(g_path)[q];
             const bf16 *gv = reinterpret_cast<const bf16 *>(&gp);
             float sk[8];
             if (g_skip) {
-                const float4 s0 = *reinterpret_cast<const float4 *>(g_skip + q);
-                const float4 s1 = *reinterpret_cast<const float4 *>(g_skip + q + 4);
+                const float4 s0 = *reinterpret_cast<const float4 *>(g_skip + 8 * q);
+                const float4 s1 = *reinterpret_cast<const float4 *>(g_skip + 8 * q + 4);
                 sk[0] = s0.x; sk[1] = s0.y; sk[2] = s0.z; sk[3] = s0.w;
                 sk[4] = s1.x; sk[5] = s1.y; sk[6] = s1.z; sk[7] = s1.w;
             }
             uint4 fm = make_uint4(0u, 0u, 0u, 0u);
-            if (f) fm = *reinterpret_cast<const uint4 *>(f + q);
+            if (f) fm = reinterpret_cast<const uint4 *>(f)[q];
             const bf16 *fv = reinterpret_cast<const bf16 *>(&fm);
             bf16 *ov = reinterpret_cast<bf16 *>(&o);
 #pragma unroll
@@ -1491,70 +1673,46 @@ __global__ void join_bwd_kernel(const float *g_skip, const bf16 *g_path, const b
                 if (f && !(__bfloat162float(fv[i]) > 0.f)) v = 0.f;
                 ov[i] = __float2bfloat16(v);
             }
+            if (S == 2 && dlo) reinterpret_cast<uint4 *>(dlo)[q] = o;
         }
-        *reinterpret_cast<uint4 *>(dz + e) = o;
+        reinterpret_cast<uint4 *>(dz)[e] = o;
     }
 }
 
-// Bias gradients gb[c] += sum over the pixels of dz[p][c], without atomics and in a fixed
-// order, in two passes: thread (t, c) of bias_part_kernel sums dz[p][c] over the pixels
-// p = t, t + 256, t + 512, ... in turn (consecutive threads take consecutive channels, so a
-// warp reads consecutive values; one warp per CTA, so the 256 C threads spread over 8 C SMs),
-// and bias_tree_kernel, one CTA per channel, adds the 256 partial sums by halving.  These are
-// the partial sums and the tree of one 256-thread CTA per channel walking the pixels, only
-// spread so that the loads are coalesced and many are in flight.
-__device__ __forceinline__ unsigned short ld_b16(const bf16 *p)
+// zero-upsampling of an NHWC gradient [N][Ho][Wo][C] onto [N][2Ho][2Wo][C] (flnr_layer)
+__global__ void spread_nhwc_kernel(const bf16 *g, bf16 *dz, int N, int Ho, int Wo, int C)
 {
-    unsigned short v;
-    asm volatile("ld.global.nc.b16 %0, [%1];" : "=h"(v) : "l"(p));
-    return v;
-}
-
-__global__ void __launch_bounds__(32) bias_part_kernel(const bf16 *dz, float *part, long long P, int C)
-{
-    constexpr int NB = 128;  // loads issued ahead of their additions
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= 256 * C) return;
-    const int t = g / C, c = g % C;
-    // the pixels in turn; each batch's loads are issued (in order, as volatile loads) before
-    // any of its additions, so a thread has NB of them in flight
-    float s = 0.f;
-    long long p = t;
-    for (; p + (NB - 1) * 256LL < P; p += NB * 256LL) {
-        unsigned short v[NB];
-#pragma unroll
-        for (int u = 0; u < NB; ++u) v[u] = ld_b16(dz + (p + (long long)u * 256) * C + c);
-#pragma unroll
-        for (int u = 0; u < NB; ++u) s += __bfloat162float(__ushort_as_bfloat16(v[u]));
+    pdl_trigger();
+    pdl_wait();
+    const int C8 = C / 8, W = 2 * Wo, H = 2 * Ho;
+    const size_t total = (size_t)N * H * W * C8;
+    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
+        const size_t p = e / C8;
+        const int c8 = (int)(e % C8), x = (int)(p % W), y = (int)(p / W % H);
+        const size_t n = p / ((size_t)W * H);
+        uint4 o = make_uint4(0u, 0u, 0u, 0u);
+        if (((x | y) & 1) == 0) o = reinterpret_cast<const uint4 *>(g)[((n * Ho + y / 2) * Wo + x / 2) * C8 + c8];
+        reinterpret_cast<uint4 *>(dz)[e] = o;
     }
-    for (; p < P; p += 256) s += __bfloat162float(dz[p * C + c]);
-    part[(size_t)t * C + c] = s;
 }
 
-__global__ void __launch_bounds__(256) bias_tree_kernel(const float *part, float *gb, int C)
+// Every layer's master fp32 [Cout][Cin][k][k] -> forward bf16 [tap][CoutP][CinP] and dgrad bf16
+// [tap'][CinP][CoutP] with tap' = taps - 1 - tap (rotated by 180 degrees), zero pads; blockIdx.y
+// is the layer (one launch for the twelve: 21 us of twelve launches per training step before).
+struct WeightsArgs {
+    const float *w[kNL];
+    bf16 *wf[kNL], *wd[kNL];
+    int cin[kNL], cout[kNL], k[kNL];
+};
+__global__ void weights_kernel(const __grid_constant__ WeightsArgs a)
 {
-    __shared__ float red[256];
-    const int c = blockIdx.x, t = threadIdx.x;
-    red[t] = part[(size_t)t * C + c];
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (t < o) red[t] += red[t + o];
-        __syncthreads();
-    }
-    if (t == 0) gb[c] += red[0];
-}
-
-// master fp32 [Cout][Cin][k][k] -> forward bf16 [tap][CoutP][CinP] and dgrad bf16
-// [tap'][CinP][CoutP] with tap' = taps - 1 - tap (rotated by 180 degrees), zero pads
-__global__ void weights_kernel(const float *w, bf16 *wf, bf16 *wd, int cin, int cout, int cinp, int coutp, int k)
-{
-    const int taps = k * k;
-    const int total = taps * coutp * cinp;
+    const int l = blockIdx.y, cin = a.cin[l], cout = a.cout[l], cinp = pad16(cin), coutp = pad16(cout);
+    const int taps = a.k[l] * a.k[l], total = taps * coutp * cinp;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
         const int i = e % cinp, o = (e / cinp) % coutp, tap = e / (cinp * coutp);
-        const float v = (i < cin && o < cout) ? w[((size_t)o * cin + i) * taps + tap] : 0.f;
-        wf[e] = __float2bfloat16(v);
-        wd[((size_t)(taps - 1 - tap) * cinp + i) * coutp + o] = __float2bfloat16(v);
+        const float v = (i < cin && o < cout) ? a.w[l][((size_t)o * cin + i) * taps + tap] : 0.f;
+        a.wf[l][e] = __float2bfloat16(v);
+        a.wd[l][((size_t)(taps - 1 - tap) * cinp + i) * coutp + o] = __float2bfloat16(v);
     }
 }
 
@@ -1664,260 +1822,313 @@ cudaError_t make_tmap_parity(CUtensorMap *m, const void *base, int C, int W, int
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// Launch of the warp-specialised convolution.  The occupancy API reports one CTA per SM for
-// kernels that allocate tensor memory, so the resident count is computed here from the
-// kernel's registers, shared memory and threads, and capped at 512 / (TMEM columns per CTA);
-// where threads alone would allow more CTAs than TMEM can hold, the shared-memory request is
-// raised so that no more can be resident (an allocation never has to wait for another CTA).
-template <int CIN, int COUT, int KS, int ACT, int OUTM, bool MASK = false>
-cudaError_t conv_ws_launch(const ConvArgs &a, cudaStream_t st)
+// 4-D map of planes of 16-byte pixels [N][P][H][W] (32-bit elements, four per pixel): box bw
+// columns x bh rows of one plane, zero fill outside
+cudaError_t make_tmap_planes(CUtensorMap *m, const void *base, int P, int W, int H, int N, int bw, int bh)
 {
-    using G = WsGeom<CIN, COUT, KS>;
-    constexpr int kSmemPerSm = 228 * 1024, kReservedPerCta = 1024, kThreadsPerSm = 2048;
-    constexpr int tmem_cap = 512 / G::COLS;
-    constexpr int min_smem = tmem_cap < kThreadsPerSm / kWsThreads ? kSmemPerSm / tmem_cap - kReservedPerCta - 256 : 0;
-    constexpr size_t smem = (size_t)(G::SMEM > min_smem ? G::SMEM : min_smem);
-    static_assert(smem <= 227 * 1024, "warp-specialised conv tile does not fit in shared memory");
-    auto kern = conv_ws_kernel<CIN, COUT, KS, ACT, OUTM, MASK>;
-    static int per_sm = 0, n_sm = 0;
-    if (per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        cudaFuncAttributes fa;
-        if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
-        int dev = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        // registers are split over the SM's four sub-partitions: warps per sub-partition first
-        const int regs_per_warp = (fa.numRegs * 32 + 255) / 256 * 256;
-        const int by_regs = (4 * (16384 / regs_per_warp)) / (kWsThreads / 32);
-        const int by_smem = kSmemPerSm / ((int)smem + (int)fa.sharedSizeBytes + kReservedPerCta);
-        int r = kThreadsPerSm / kWsThreads;
-        r = r < by_regs ? r : by_regs;
-        r = r < by_smem ? r : by_smem;
-        r = r < tmem_cap ? r : tmem_cap;
-        if (r < 1) return cudaErrorInvalidConfiguration;
-        per_sm = r;
+    PFN_cuTensorMapEncodeTiled_v12000 fn = tmap_encoder();
+    if (!fn) return cudaErrorNotSupported;
+    const cuuint64_t row = (cuuint64_t)W * 16;
+    const cuuint64_t dims[4] = {(cuuint64_t)4 * W, (cuuint64_t)H, (cuuint64_t)P, (cuuint64_t)N};
+    const cuuint64_t strides[3] = {row, row * H, row * H * P};
+    const cuuint32_t box[4] = {(cuuint32_t)(4 * bw), (cuuint32_t)bh, 1, 1};
+    const cuuint32_t es[4] = {1, 1, 1, 1};
+    const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, const_cast<void *>(base), dims, strides, box, es,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+// 5-D map of a kPlanes tensor (H, W even) that stages one parity plane per box: dims (16 values
+// of a column pair, W/2 column pairs, 2 row parities, H/2 row pairs, C/8 * N chunk planes); box
+// (8, bw, 1, bh, 1).  The start value 8 b selects column parity b.
+cudaError_t make_tmap_pairs(CUtensorMap *m, const void *base, int C, int W, int H, int N, int bw, int bh)
+{
+    PFN_cuTensorMapEncodeTiled_v12000 fn = tmap_encoder();
+    if (!fn) return cudaErrorNotSupported;
+    const cuuint64_t row = (cuuint64_t)W * 16;
+    const cuuint64_t dims[5] = {16, (cuuint64_t)W / 2, 2, (cuuint64_t)H / 2, (cuuint64_t)(C / 8) * N};
+    const cuuint64_t strides[4] = {32, row, 2 * row, row * H};
+    const cuuint32_t box[5] = {8, (cuuint32_t)bw, 1, (cuuint32_t)bh, 1};
+    const cuuint32_t es[5] = {1, 1, 1, 1, 1};
+    const CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(base), dims, strides, box, es,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+// Map of x for the weight gradients, boxes in the order [row][chunk][col][8]: a kNHWC or kPlanes
+// tensor (box bw columns x all chunks x bh rows), or one parity plane of a kParity tensor
+// (W, H: the plane's size).
+cudaError_t make_tmap_rows(CUtensorMap *m, int layout, const void *base, int C, int W, int H, int N, int bw, int bh)
+{
+    PFN_cuTensorMapEncodeTiled_v12000 fn = tmap_encoder();
+    if (!fn) return cudaErrorNotSupported;
+    const cuuint64_t w = W, h = H, n = N, c8 = C / 8, row = w * 16;
+    const cuuint32_t es[5] = {1, 1, 1, 1, 1}, b4 = 4 * bw, bb = bw, hh = bh, cc = C / 8;
+    CUresult r;
+    if (layout == kNHWC) {
+        const cuuint64_t dims[5] = {8, w, c8, h, n}, st[4] = {c8 * 16, 16, c8 * row, c8 * row * h};
+        const cuuint32_t box[5] = {8, bb, cc, hh, 1};
+        r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(base), dims, st, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    } else if (layout == kPlanes) {
+        const cuuint64_t dims[4] = {4 * w, c8, h, n}, st[3] = {row * h, row, row * h * c8};
+        const cuuint32_t box[4] = {b4, cc, hh, 1};
+        r = fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, const_cast<void *>(base), dims, st, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    } else {
+        const cuuint64_t dims[5] = {4 * w, c8, h, 4, n}, st[4] = {4 * row * h, row, row * h, 4 * row * h * c8};
+        const cuuint32_t box[5] = {b4, cc, hh, 1, 1};
+        r = fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT32, 5, const_cast<void *>(base), dims, st, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     }
-    const long long ntiles = (long long)a.N * ((a.H + G::TH - 1) / G::TH) * ((a.W + G::TW - 1) / G::TW);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+// the map of a tensor in layout kNHWC or kPlanes, for load_planes
+cudaError_t make_tmap_tile(CUtensorMap *m, int layout, const void *base, int C, int W, int H, int N, int bw, int bh)
+{
+    return layout == kNHWC ? make_tmap(m, base, C, W, H, N, bw, bh) : make_tmap_planes(m, base, C / 8, W, H, N, bw, bh);
+}
+
+// Resident CTAs per SM of a kernel that allocates tensor memory.  The occupancy API reports one
+// CTA per SM for such kernels, so the count is computed here from the kernel's registers,
+// shared memory and threads, and capped at 512 / (tensor-memory columns per CTA); where threads
+// alone would allow more CTAs than tensor memory can hold, the shared-memory request is raised
+// (tc_smem) so that no more can be resident (an allocation never has to wait for another CTA).
+constexpr int kSmemPerSm = 228 * 1024, kReservedPerCta = 1024, kThreadsPerSm = 2048;
+constexpr size_t tc_smem(int smem, int cols, int threads)
+{
+    const int cap = 512 / cols;
+    const int least = cap < kThreadsPerSm / threads ? kSmemPerSm / cap - kReservedPerCta - 256 : 0;
+    return (size_t)(smem > least ? smem : least);
+}
+struct Resident {
+    int per_sm = 0, n_sm = 0;
+};
+template <class K>
+cudaError_t resident(K kern, int threads, size_t smem, int cols, Resident &out)
+{
+    if (out.per_sm > 0) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+    cudaFuncAttributes fa;
+    if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
+    int dev = 0, n_sm = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    // registers are split over the SM's four sub-partitions: warps per sub-partition first
+    const int regs_per_warp = (fa.numRegs * 32 + 255) / 256 * 256;
+    const int by_regs = (4 * (16384 / regs_per_warp)) / (threads / 32);
+    const int by_smem = kSmemPerSm / ((int)smem + (int)fa.sharedSizeBytes + kReservedPerCta);
+    int r = kThreadsPerSm / threads;
+    r = r < by_regs ? r : by_regs;
+    r = r < by_smem ? r : by_smem;
+    r = r < 512 / cols ? r : 512 / cols;
+    if (r < 1) return cudaErrorInvalidConfiguration;
+    out.n_sm = n_sm;
+    out.per_sm = r;
+    return cudaSuccess;
+}
+
+// Stages of a map of N images.  NT tiles per stage share a halo, a hand-over of the barriers and
+// eight epilogue warps; they are taken as soon as half the SMs get a stage (a 1920x1080 forward
+// pass takes 472 us with several tiles per stage and 516 us with one, forward and backward over
+// 16 x 128^2 572 and 621 us); smaller maps would leave the chip idle.
+long long stages(int N, int H, int W, int tw) { return (long long)N * ((H + 15) / 16) * ((W + tw - 1) / tw); }
+
+// Launch of the warp-specialised convolution with NT tiles per stage; when only asked, *fits
+// reports whether that many per stage is the better choice.
+template <int CIN, int COUT, int KS, int ACT, int OUTM, bool MASK, int NT>
+cudaError_t conv_ws_launch_nt(const ConvArgs &a, bool ask, bool *fits, cudaStream_t st)
+{
+    using G = WsGeom<CIN, COUT, KS, NT>;
+    constexpr size_t smem = tc_smem(G::SMEM, G::COLS, G::THREADS);
+    static_assert(smem <= 227 * 1024, "warp-specialised conv tile does not fit in shared memory");
+    auto kern = conv_ws_kernel<CIN, COUT, KS, ACT, OUTM, MASK, NT>;
+    static Resident res;
+    cudaError_t e = resident(kern, G::THREADS, smem, G::COLS, res);
+    if (e != cudaSuccess) return e;
+    const long long ntiles = stages(a.N, a.H, a.W, G::TW), cap = (long long)res.per_sm * res.n_sm;
+    if (ask) {
+        *fits = 2 * ntiles >= res.n_sm;
+        return cudaSuccess;
+    }
     if (ntiles <= 0) return cudaSuccess;
     TcArgs ta;
     std::memset(&ta, 0, sizeof(ta));
     ta.c = a;
-    cudaError_t e = make_tmap(&ta.tm, a.x, CIN, a.W, a.H, a.N, G::SW, G::SH);
+    if ((e = make_tmap_tile(&ta.tm, a.lx, a.x, CIN, a.W, a.H, a.N, G::SW, G::SH)) != cudaSuccess) return e;
+    return launch_pdl(kern, (int)(ntiles < cap ? ntiles : cap), G::THREADS, smem, st, ta);
+}
+template <int CIN, int COUT, int KS, int ACT, int OUTM, bool MASK>
+cudaError_t conv_ws_launch(const ConvArgs &a, cudaStream_t st)
+{
+    constexpr int NT = CIN <= 32 && COUT <= 32 ? 4 : 2;
+    bool wide = false;
+    cudaError_t e = conv_ws_launch_nt<CIN, COUT, KS, ACT, OUTM, MASK, NT>(a, true, &wide, st);
     if (e != cudaSuccess) return e;
-    const long long cap = (long long)per_sm * n_sm;
-    kern<<<(int)(ntiles < cap ? ntiles : cap), kWsThreads, smem, st>>>(ta);
-    return cudaGetLastError();
+    if (wide) return conv_ws_launch_nt<CIN, COUT, KS, ACT, OUTM, MASK, NT>(a, false, nullptr, st);
+    return conv_ws_launch_nt<CIN, COUT, KS, ACT, OUTM, MASK, 1>(a, false, nullptr, st);
 }
 
 // Input gradient of a layer on the tensor cores: the stride-1 convolution of dz with the
 // layer's weights rotated by 180 degrees and transposed ([tap][CinP][CoutP]), no bias, no
-// activation, times (mask > 0) when MASK (the ReLU of the layer input).  a: x = dz
-// [N][H][W][CIN], w, mask [N][H][W][COUT], y [N][H][W][ystride].
+// activation, times (mask > 0) when MASK (the ReLU of the layer input, in layout lm).
 template <int CIN, int COUT, int KS, bool MASK>
-cudaError_t dgrad_launch(ConvArgs a, int *status, cudaStream_t st)
+cudaError_t dgrad_launch(const bf16 *dz, const bf16 *wd, const bf16 *mask, bf16 *dx, int N, int H, int W, int *status,
+                         cudaStream_t st, int lm = kPlanes)
 {
-    a.bias = nullptr;
-    a.nbias = 0;
+    ConvArgs a{};
+    a.x = dz;
+    a.w = wd;
+    a.mask = mask;
+    a.y = dx;
+    a.N = N;
+    a.H = H;
+    a.W = W;
+    a.lx = a.ly = kPlanes;
+    a.lm = lm;
     a.status = status;
     return conv_ws_launch<CIN, COUT, KS, 0, 0, MASK>(a, st);
 }
 
-// Launch of the fused KS x KS + 1x1 pair (c: first layer, c2: the 1x1 layer); residency
-// computed as for conv_ws_launch.
-template <int CIN, int COUT, int KS, int COUT2, int ACT2, int OUTM2>
-cudaError_t conv_tail_launch(const ConvArgs &c, const ConvArgs &c2, cudaStream_t st)
+// Launch of the fused KS x KS + 1x1 pair (c: first layer, c2: the 1x1 layer); NT as for
+// conv_ws_launch.
+template <int CIN, int COUT, int KS, int COUT2, int ACT2, int OUTM2, int NT>
+cudaError_t conv_tail_launch_nt(const ConvArgs &c, const ConvArgs &c2, bf16 *w2_kept, float *b2_kept, bool ask, bool *fits,
+                                cudaStream_t st)
 {
-    using T = TailGeom<CIN, COUT, KS, COUT2>;
+    using T = TailGeom<CIN, COUT, KS, COUT2, NT>;
     using G = typename T::G1;
-    constexpr int kSmemPerSm = 228 * 1024, kReservedPerCta = 1024, kThreadsPerSm = 2048;
-    constexpr int tmem_cap = 512 / T::COLS;
-    constexpr int min_smem = tmem_cap < kThreadsPerSm / kWsThreads ? kSmemPerSm / tmem_cap - kReservedPerCta - 256 : 0;
-    constexpr size_t smem = (size_t)(T::SMEM > min_smem ? T::SMEM : min_smem);
+    constexpr size_t smem = tc_smem(T::SMEM, T::COLS, G::THREADS);
     static_assert(smem <= 227 * 1024, "fused conv stage does not fit in shared memory");
-    auto kern = conv_tail_kernel<CIN, COUT, KS, COUT2, ACT2, OUTM2>;
-    static int per_sm = 0, n_sm = 0;
-    if (per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        cudaFuncAttributes fa;
-        if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
-        int dev = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        const int regs_per_warp = (fa.numRegs * 32 + 255) / 256 * 256;
-        const int by_regs = (4 * (16384 / regs_per_warp)) / (kWsThreads / 32);
-        const int by_smem = kSmemPerSm / ((int)smem + (int)fa.sharedSizeBytes + kReservedPerCta);
-        int r = kThreadsPerSm / kWsThreads;
-        r = r < by_regs ? r : by_regs;
-        r = r < by_smem ? r : by_smem;
-        r = r < tmem_cap ? r : tmem_cap;
-        if (r < 1) return cudaErrorInvalidConfiguration;
-        per_sm = r;
+    auto kern = conv_tail_kernel<CIN, COUT, KS, COUT2, ACT2, OUTM2, NT>;
+    static Resident res;
+    cudaError_t e = resident(kern, G::THREADS, smem, T::COLS, res);
+    if (e != cudaSuccess) return e;
+    const long long ntiles = stages(c.N, c.H, c.W, G::TW), cap = (long long)res.per_sm * res.n_sm;
+    if (ask) {
+        *fits = 2 * ntiles >= res.n_sm;
+        return cudaSuccess;
     }
-    const long long ntiles = (long long)c.N * ((c.H + G::TH - 1) / G::TH) * ((c.W + G::TW - 1) / G::TW);
     if (ntiles <= 0) return cudaSuccess;
     TailArgs ta;
     std::memset(&ta, 0, sizeof(ta));
     ta.c = c;
     ta.c2 = c2;
-    cudaError_t e = make_tmap(&ta.tm, c.x, CIN, c.W, c.H, c.N, G::SW, G::SH);
+    ta.w2_kept = w2_kept;
+    ta.b2_kept = b2_kept;
+    if ((e = make_tmap_tile(&ta.tm, c.lx, c.x, CIN, c.W, c.H, c.N, G::SW, G::SH)) != cudaSuccess) return e;
+    return launch_pdl(kern, (int)(ntiles < cap ? ntiles : cap), G::THREADS, smem, st, ta);
+}
+template <int CIN, int COUT, int KS, int COUT2, int ACT2, int OUTM2>
+cudaError_t conv_tail_launch(const ConvArgs &c, const ConvArgs &c2, cudaStream_t st, bf16 *w2_kept = nullptr,
+                             float *b2_kept = nullptr)
+{
+    bool wide = false;
+    cudaError_t e = conv_tail_launch_nt<CIN, COUT, KS, COUT2, ACT2, OUTM2, 4>(c, c2, w2_kept, b2_kept, true, &wide, st);
     if (e != cudaSuccess) return e;
-    const long long cap = (long long)per_sm * n_sm;
-    kern<<<(int)(ntiles < cap ? ntiles : cap), kWsThreads, smem, st>>>(ta);
-    return cudaGetLastError();
+    if (wide) return conv_tail_launch_nt<CIN, COUT, KS, COUT2, ACT2, OUTM2, 4>(c, c2, w2_kept, b2_kept, false, nullptr, st);
+    return conv_tail_launch_nt<CIN, COUT, KS, COUT2, ACT2, OUTM2, 1>(c, c2, w2_kept, b2_kept, false, nullptr, st);
 }
 
-// Launch of the parity-class decoder convolution (a.x = lo, a.x2 = skip; H, W even);
-// residency computed as for conv_ws_launch.
+// Launch of the parity-class decoder convolution (a.x = lo, a.x2 = skip, both in layout a.lx;
+// H, W even).
 template <int CA, int CB, int COUT, int NBUF>
 cudaError_t conv_up_launch(const ConvArgs &a, cudaStream_t st)
 {
     using G = UpGeom<CA, CB, COUT, NBUF>;
-    constexpr int kSmemPerSm = 228 * 1024, kReservedPerCta = 1024, kThreadsPerSm = 2048;
-    constexpr int tmem_cap = 512 / G::COLS;
-    constexpr int min_smem = tmem_cap < kThreadsPerSm / kWsThreads ? kSmemPerSm / tmem_cap - kReservedPerCta - 256 : 0;
-    constexpr size_t smem = (size_t)(G::SMEM > min_smem ? G::SMEM : min_smem);
+    constexpr size_t smem = tc_smem(G::SMEM, G::COLS, kWsThreads);
     static_assert(smem <= 227 * 1024, "decoder conv stage does not fit in shared memory");
     auto kern = conv_up_kernel<CA, CB, COUT, NBUF>;
-    static int per_sm = 0, n_sm = 0;
-    if (per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        cudaFuncAttributes fa;
-        if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
-        int dev = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        const int regs_per_warp = (fa.numRegs * 32 + 255) / 256 * 256;
-        const int by_regs = (4 * (16384 / regs_per_warp)) / (kWsThreads / 32);
-        const int by_smem = kSmemPerSm / ((int)smem + (int)fa.sharedSizeBytes + kReservedPerCta);
-        int r = kThreadsPerSm / kWsThreads;
-        r = r < by_regs ? r : by_regs;
-        r = r < by_smem ? r : by_smem;
-        r = r < tmem_cap ? r : tmem_cap;
-        if (r < 1) return cudaErrorInvalidConfiguration;
-        per_sm = r;
-    }
+    static Resident res;
+    cudaError_t e = resident(kern, kWsThreads, smem, G::COLS, res);
+    if (e != cudaSuccess) return e;
     if ((a.H | a.W) & 1) return cudaErrorInvalidValue;
-    const long long ntiles = (long long)a.N * ((a.H / 2 + 15) / 16) * ((a.W / 2 + 7) / 8);
+    const long long ntiles = stages(a.N, a.H / 2, a.W / 2, 8), cap = (long long)res.per_sm * res.n_sm;
     if (ntiles <= 0) return cudaSuccess;
     UpArgs ua;
     std::memset(&ua, 0, sizeof(ua));
     ua.c = a;
-    cudaError_t e = make_tmap(&ua.tlo, a.x, CA, a.W / 2, a.H / 2, a.N, G::SW, G::SH);
+    if ((e = make_tmap_tile(&ua.tlo, a.lx, a.x, CA, a.W / 2, a.H / 2, a.N, G::SW, G::SH)) != cudaSuccess) return e;
+    e = a.lx == kNHWC ? make_tmap_parity(&ua.tskip, a.x2, CB, a.W, a.H, a.N, G::SW, G::SH)
+                      : make_tmap_pairs(&ua.tskip, a.x2, CB, a.W, a.H, a.N, G::SW, G::SH);
     if (e != cudaSuccess) return e;
-    if ((e = make_tmap_parity(&ua.tskip, a.x2, CB, a.W, a.H, a.N, G::SW, G::SH)) != cudaSuccess) return e;
-    const long long cap = (long long)per_sm * n_sm;
-    kern<<<(int)(ntiles < cap ? ntiles : cap), kWsThreads, smem, st>>>(ua);
-    return cudaGetLastError();
+    return launch_pdl(kern, (int)(ntiles < cap ? ntiles : cap), kWsThreads, smem, st, ua);
 }
 
 // Launch of the stride-2 convolution (a.H, a.W: the input's size, both even; output at half
-// size); residency computed as for conv_ws_launch.
+// size).
 template <int CIN, int COUT, int NBUF>
 cudaError_t conv_s2_launch(const ConvArgs &a, cudaStream_t st)
 {
     using G = S2Geom<CIN, COUT, NBUF>;
-    constexpr int kSmemPerSm = 228 * 1024, kReservedPerCta = 1024, kThreadsPerSm = 2048;
-    constexpr int tmem_cap = 512 / G::COLS;
-    constexpr int min_smem = tmem_cap < kThreadsPerSm / kWsThreads ? kSmemPerSm / tmem_cap - kReservedPerCta - 256 : 0;
-    constexpr size_t smem = (size_t)(G::SMEM > min_smem ? G::SMEM : min_smem);
+    constexpr size_t smem = tc_smem(G::SMEM, G::COLS, kWsThreads);
     static_assert(smem <= 227 * 1024, "stride-2 conv stage does not fit in shared memory");
     auto kern = conv_s2_kernel<CIN, COUT, NBUF>;
-    static int per_sm = 0, n_sm = 0;
-    if (per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        cudaFuncAttributes fa;
-        if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
-        int dev = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        const int regs_per_warp = (fa.numRegs * 32 + 255) / 256 * 256;
-        const int by_regs = (4 * (16384 / regs_per_warp)) / (kWsThreads / 32);
-        const int by_smem = kSmemPerSm / ((int)smem + (int)fa.sharedSizeBytes + kReservedPerCta);
-        int r = kThreadsPerSm / kWsThreads;
-        r = r < by_regs ? r : by_regs;
-        r = r < by_smem ? r : by_smem;
-        r = r < tmem_cap ? r : tmem_cap;
-        if (r < 1) return cudaErrorInvalidConfiguration;
-        per_sm = r;
-    }
+    static Resident res;
+    cudaError_t e = resident(kern, kWsThreads, smem, G::COLS, res);
+    if (e != cudaSuccess) return e;
     if ((a.H | a.W) & 1) return cudaErrorInvalidValue;
-    const long long ntiles = (long long)a.N * ((a.H / 2 + G::TH - 1) / G::TH) * ((a.W / 2 + G::TW - 1) / G::TW);
+    const long long ntiles = stages(a.N, a.H / 2, a.W / 2, G::TW), cap = (long long)res.per_sm * res.n_sm;
     if (ntiles <= 0) return cudaSuccess;
     S2Args sa;
     std::memset(&sa, 0, sizeof(sa));
     sa.c = a;
-    cudaError_t e = make_tmap_parity(&sa.te, a.x, CIN, a.W, a.H, a.N, G::WE, G::SH);
-    if (e != cudaSuccess) return e;
-    if ((e = make_tmap_parity(&sa.to, a.x, CIN, a.W, a.H, a.N, G::WO, G::SH)) != cudaSuccess) return e;
-    const long long cap = (long long)per_sm * n_sm;
-    kern<<<(int)(ntiles < cap ? ntiles : cap), kWsThreads, smem, st>>>(sa);
-    return cudaGetLastError();
+    if (a.lx == kNHWC) {
+        if ((e = make_tmap_parity(&sa.te, a.x, CIN, a.W, a.H, a.N, G::WE, G::SH)) != cudaSuccess) return e;
+        if ((e = make_tmap_parity(&sa.to, a.x, CIN, a.W, a.H, a.N, G::WO, G::SH)) != cudaSuccess) return e;
+    } else {
+        if ((e = make_tmap_planes(&sa.te, a.x, CIN / 2, a.W / 2, a.H / 2, a.N, G::WE, G::SH)) != cudaSuccess) return e;
+        if ((e = make_tmap_planes(&sa.to, a.x, CIN / 2, a.W / 2, a.H / 2, a.N, G::WO, G::SH)) != cudaSuccess) return e;
+    }
+    return launch_pdl(kern, (int)(ntiles < cap ? ntiles : cap), kWsThreads, smem, st, sa);
 }
 
-// Launch of the tensor-core weight gradient: one CTA per resident slot, each over a
-// contiguous range of 8 x 8 pixel tiles.  Residency as for conv_ws_launch: the shared-memory
-// request is raised where needed so that no more CTAs than tensor memory can hold share an SM.
-template <int CIN, int COUT, int KS>
-cudaError_t wgrad_launch(const bf16 *x, const bf16 *dz, float *gw, int N, int H, int W, int cin_true, int cout_true,
-                         float *part, size_t part_floats, int *status, cudaStream_t st)
+// Where a layer's gradients go: its partials (n_sm slices), master weight and bias gradients
+struct WgradDest {
+    float *part, *gw, *gb;
+    int cin_true, cout_true;
+};
+
+// Launch of a layer's weight and bias gradient over dz [N][H][W] (MODE 1: x is the kParity input
+// of twice that size): one CTA per SM (and tap group), and the layer's entry for the reduction.
+template <int CIN, int COUT, int KS, int MODE>
+cudaError_t wgrad_launch(const bf16 *x, const bf16 *dz, int layout, int N, int H, int W, const WgradDest &d, RedArgs &ra,
+                         int n_sm, int *status, cudaStream_t st)
 {
-    using G = WgGeom<CIN, COUT, KS>;
-    constexpr int kSmemPerSm = 228 * 1024, kReservedPerCta = 1024, kThreads = 128, kThreadsPerSm = 2048;
-    constexpr int tmem_cap = 512 / G::COLS;
-    constexpr int min_smem = tmem_cap < kThreadsPerSm / kThreads ? kSmemPerSm / tmem_cap - kReservedPerCta - 256 : 0;
-    constexpr size_t smem = (size_t)(G::SMEM > min_smem ? G::SMEM : min_smem);
+    using G = WgGeom<CIN, COUT, KS, MODE>;
+    constexpr size_t smem = tc_smem(G::SMEM, G::COLS, kWgThreads);
     static_assert(smem <= 227 * 1024, "weight-gradient tile does not fit in shared memory");
-    auto kern = wgrad_tc_kernel<CIN, COUT, KS>;
-    static int per_sm = 0, n_sm = 0;
-    if (per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        cudaFuncAttributes fa;
-        if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
-        int dev = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        const int regs_per_warp = (fa.numRegs * 32 + 255) / 256 * 256;
-        const int by_regs = (4 * (16384 / regs_per_warp)) / (kThreads / 32);
-        const int by_smem = kSmemPerSm / ((int)smem + (int)fa.sharedSizeBytes + kReservedPerCta);
-        int r = kThreadsPerSm / kThreads;
-        r = r < by_regs ? r : by_regs;
-        r = r < by_smem ? r : by_smem;
-        r = r < tmem_cap ? r : tmem_cap;
-        if (r < 1) return cudaErrorInvalidConfiguration;
-        per_sm = r;
-    }
-    const long long ntiles = (long long)N * ((H + 7) / 8) * ((W + 7) / 8);
-    if (ntiles <= 0) return cudaSuccess;
-    long long slots = (long long)per_sm * n_sm;
-    const long long fit = (long long)(part_floats / ((size_t)G::M * COUT));  // partial slots the buffer holds
-    if (slots > fit) slots = fit;
-    if (slots < 1) return cudaErrorInvalidValue;
-    const long long ctas = ntiles < slots ? ntiles : slots;
-    WgradArgs a{x, dz, gw, part, N, H, W, cin_true, cout_true, (int)((ntiles + ctas - 1) / ctas), status};
-    const long long grid = (ntiles + a.tiles_per_cta - 1) / a.tiles_per_cta;
-    kern<<<(int)grid, kThreads, smem, st>>>(a);
-    cudaError_t e = cudaGetLastError();
+    auto kern = wgrad_tc_kernel<CIN, COUT, KS, MODE>;
+    static Resident res;
+    cudaError_t e = resident(kern, kWgThreads, smem, G::COLS, res);
     if (e != cudaSuccess) return e;
-    // one warp per CTA: the M COUT chains of additions spread over as many SMs as they fill
-    wgrad_reduce_kernel<CIN, COUT, KS><<<(KS * KS * CIN * COUT + 31) / 32, 32, 0, st>>>(part, (int)grid, gw, cin_true,
-                                                                                       cout_true);
-    return cudaGetLastError();
+    const long long ntiles = stages(N, H, W, 8);
+    const int slots = n_sm / G::NG > 0 ? n_sm / G::NG : 1;
+    const int slices = (int)(ntiles < slots ? ntiles : slots);
+    WgradArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.part = d.part;
+    a.N = N;
+    a.H = H;
+    a.W = W;
+    a.layout = layout;
+    a.status = status;
+    if ((e = make_tmap_rows(&a.tx, MODE ? kParity : layout, x, CIN, W, H, N, G::XW, G::XH)) != cudaSuccess) return e;
+    if ((e = make_tmap_tile(&a.tdz, layout, dz, COUT, W, H, N, 8, 16)) != cudaSuccess) return e;
+    ra.l[ra.n++] = RedLayer{d.part, d.gw, d.gb, slices, COUT, CIN, KS, MODE, d.cin_true, d.cout_true, ra.blocks};
+    ra.blocks += (COUT * G::CTOT + 31) / 32;
+    return launch_pdl(kern, dim3(slices, G::NG), kWgThreads, smem, st, a);
+}
+
+cudaError_t wgrad_reduce(const RedArgs &ra, cudaStream_t st)
+{
+    return launch_pdl(wgrad_reduce_kernel, ra.blocks, 32 * kRedWarps, 0, st, ra);
 }
 
 }  // namespace
@@ -1937,11 +2148,12 @@ struct flnr_net {
     std::vector<void *> bufs;
     // activations (bf16 NHWC) and gradients
     __nv_bfloat16 *x0, *a0, *f0, *a1, *f1, *a2, *f2, *c1, *a3, *d1, *c0, *a4, *d0, *a5;
-    __nv_bfloat16 *gA, *gB, *gC, *gLo;  // gradient scratch (largest: 48 channels at full res)
+    __nv_bfloat16 *gA, *gB, *gC, *gLo, *gLo2;  // gradient scratch (largest: 48 channels at full res)
     float *gskip0, *gskip1;             // skip gradients (fp32)
-    float *wpart = nullptr;             // per-CTA partial weight gradients (fixed-order reduction)
-    size_t wpart_floats = 0;
-    float *out = nullptr;               // last forward output, planar fp32 [N][8][H][W]
+    float *wpart = nullptr;             // partial weight and bias gradients of every layer
+    size_t wpart_off[flnr::kNL] = {};   // (fixed-order reduction), layer l's from wpart_off[l] on
+    __nv_bfloat16 *head_w = nullptr;    // the head's weights and biases of the last forward pass
+    float *head_b = nullptr;
     int *status = nullptr;              // device status word of the tensor-core kernels
     int N = 0, H = 0, W = 0;            // shape of the last forward
     bool weights_fresh = false;
@@ -1967,15 +2179,25 @@ flnr::LayerDef layer_def(int nout, int l)
     return d;
 }
 
+flnr::WgradDest wgrad_dest(flnr_net *n, int l)
+{
+    const auto d = layer_def(n->nout, l);
+    return {n->wpart + n->wpart_off[l], n->g + n->poff[l][0], n->g + n->poff[l][1], d.cin, d.cout};
+}
+
 cudaError_t refresh_weights(flnr_net *n, cudaStream_t st)
 {
+    flnr::WeightsArgs wa;
     for (int l = 0; l < flnr::kNL; ++l) {
         const auto d = layer_def(n->nout, l);
-        const int cinp = flnr::pad16(d.cin), coutp = flnr::pad16(d.cout);
-        const int total = d.k * d.k * cinp * coutp;
-        flnr::weights_kernel<<<(total + 255) / 256, 256, 0, st>>>(n->w + n->poff[l][0], n->wf[l], n->wd[l], d.cin,
-                                                                   d.cout, cinp, coutp, d.k);
+        wa.w[l] = n->w + n->poff[l][0];
+        wa.wf[l] = n->wf[l];
+        wa.wd[l] = n->wd[l];
+        wa.cin[l] = d.cin;
+        wa.cout[l] = d.cout;
+        wa.k[l] = d.k;
     }
+    flnr::weights_kernel<<<dim3(64, flnr::kNL), 256, 0, st>>>(wa);
     n->weights_fresh = true;
     return cudaGetLastError();
 }
@@ -2029,11 +2251,18 @@ int flnr_create(int max_pixels, int outputs, flnr_net **out)
     st |= nalloc(n, &n->a3, P2 * 32) | nalloc(n, &n->d1, P2 * 32) | nalloc(n, &n->c0, P * 48);
     st |= nalloc(n, &n->a4, P * 16) | nalloc(n, &n->d0, P * 16) | nalloc(n, &n->a5, P * 16);
     st |= nalloc(n, &n->gA, P * 48) | nalloc(n, &n->gB, P * 48) | nalloc(n, &n->gC, P * 48) | nalloc(n, &n->gLo, P * 16);
-    st |= nalloc(n, &n->gskip0, P * 16) | nalloc(n, &n->gskip1, P2 * 32) | nalloc(n, &n->out, P * 16);
+    st |= nalloc(n, &n->gLo2, P2 * 32);
+    st |= nalloc(n, &n->gskip0, P * 16) | nalloc(n, &n->gskip1, P2 * 32);
+    st |= nalloc(n, &n->head_w, 16 * 16) | nalloc(n, &n->head_b, 16);
     st |= nalloc(n, &n->status, 1);
-    // partial weight gradients: two CTAs per SM of the largest layer (e2b, 9 * 64 x 64)
-    n->wpart_floats = 2 * (size_t)n->n_sm * 9 * 64 * 64;
-    st |= nalloc(n, &n->wpart, n->wpart_floats);
+    // partial gradients: one slice per SM of each layer's [Cout][k k Cin + 8] sums
+    size_t wp = 0;
+    for (int l = 0; l < flnr::kNL; ++l) {
+        const auto &d = flnr::kLayers[l];
+        n->wpart_off[l] = wp;
+        wp += (size_t)n->n_sm * flnr::pad16(d.cout) * (d.k * d.k * flnr::pad16(d.cin) + 8);
+    }
+    st |= nalloc(n, &n->wpart, wp);
     if (st != FLR_OK) {
         flnr_destroy(n);
         return FLR_ERR_NOMEM;
@@ -2124,38 +2353,40 @@ int flnr_guide_forward(flnr_net *n, const float *in, float *guide_out, int N, in
     const size_t P = (size_t)N * H * W;
     const int H2 = H / 2, W2 = W / 2;
     auto bias = [&](int l) { return n->w + n->poff[l][1]; };
-    pack_input_kernel<<<egrid(P), 256, 0, st>>>(in, n->x0, N, H, W);
-    FLNR_TRY(cudaGetLastError());
+    FLNR_TRY(launch_pdl(pack_input_kernel, egrid(P), 256, 0, st, in, n->x0, N, H, W));
     const ConvArgs z{};
-    auto conv = [&](const __nv_bfloat16 *x, int l, __nv_bfloat16 *y, int h, int w) {
+    auto conv = [&](const __nv_bfloat16 *x, int l, __nv_bfloat16 *y, int h, int w, int ly = kPlanes) {
         ConvArgs c = z;
         c.x = x; c.w = n->wf[l]; c.bias = bias(l); c.y = y; c.N = N; c.H = h; c.W = w;
-        c.ystride = pad16(kLayers[l].cout); c.nbias = layer_def(n->nout, l).cout; c.status = n->status;
+        c.lx = kPlanes; c.ly = ly; c.nbias = layer_def(n->nout, l).cout; c.status = n->status;
         return c;
     };
     ConvArgs c;
     // in0 and in1 in one pass (a0, which the backward pass reads, is still stored)
     FLNR_TRY((conv_tail_launch<16, 16, 3, 16, 1, 0>(conv(n->x0, 0, n->a0, H, W), conv(n->a0, 1, n->f0, H, W), st)));
     // encoder blocks: a 3x3 convolution, then a stride-2 one (sizes passed: the input's)
-    FLNR_TRY((conv_ws_launch<16, 32, 3, 1, 0>(conv(n->f0, 2, n->a1, H, W), st)));
-    FLNR_TRY((conv_s2_launch<32, 32, 2>(conv(n->a1, 3, n->f1, H, W), st)));
-    FLNR_TRY((conv_ws_launch<32, 64, 3, 1, 0>(conv(n->f1, 4, n->a2, H2, W2), st)));
-    FLNR_TRY((conv_s2_launch<64, 64, 2>(conv(n->a2, 5, n->f2, H2, W2), st)));
+    FLNR_TRY((conv_ws_launch<16, 32, 3, 1, 0, false>(conv(n->f0, 2, n->a1, H, W, kParity), st)));
+    c = conv(n->a1, 3, n->f1, H, W);
+    c.lx = kParity;
+    FLNR_TRY((conv_s2_launch<32, 32, 2>(c, st)));
+    FLNR_TRY((conv_ws_launch<32, 64, 3, 1, 0, false>(conv(n->f1, 4, n->a2, H2, W2, kParity), st)));
+    c = conv(n->a2, 5, n->f2, H2, W2);
+    c.lx = kParity;
+    FLNR_TRY((conv_s2_launch<64, 64, 2>(c, st)));
     c = conv(n->f2, 6, n->a3, H2, W2);  // input up(f2) ++ f1, formed while staging
     c.x2 = n->f1;
     FLNR_TRY((conv_up_launch<64, 32, 32, 2>(c, st)));
-    FLNR_TRY((conv_ws_launch<32, 32, 3, 1, 0>(conv(n->a3, 7, n->d1, H2, W2), st)));
+    FLNR_TRY((conv_ws_launch<32, 32, 3, 1, 0, false>(conv(n->a3, 7, n->d1, H2, W2), st)));
     c = conv(n->d1, 8, n->a4, H, W);  // input up(d1) ++ f0
     c.x2 = n->f0;
     FLNR_TRY((conv_up_launch<32, 16, 16, 2>(c, st)));
-    FLNR_TRY((conv_ws_launch<16, 16, 3, 1, 0>(conv(n->a4, 9, n->d0, H, W), st)));
-    float *yf = guide_out ? guide_out : n->out;
+    FLNR_TRY((conv_ws_launch<16, 16, 3, 1, 0, false>(conv(n->a4, 9, n->d0, H, W), st)));
     c = conv(n->a5, 11, nullptr, H, W);
-    c.yf = yf;
-    // o0 and the head o1 (sigmoid into planar FP32) in one pass; a5 is still stored
-    FLNR_TRY((conv_tail_launch<16, 16, 3, 16, 2, 1>(conv(n->d0, 10, n->a5, H, W), c, st)));
-    if (guide_out)
-        FLNR_TRY(cudaMemcpyAsync(n->out, guide_out, P * n->nout * sizeof(float), cudaMemcpyDeviceToDevice, st));
+    c.yf = guide_out;
+    // o0 and the head o1 (sigmoid into planar FP32) in one pass; a5 is still stored, and the
+    // backward pass forms the guides again from it (a copy of the guides cost 133 MB of traffic,
+    // 21 us, per 1920x1080 frame)
+    FLNR_TRY((conv_tail_launch<16, 16, 3, 16, 2, 1>(conv(n->d0, 10, n->a5, H, W), c, st, n->head_w, n->head_b)));
     return FLR_OK;
 }
 
@@ -2166,74 +2397,62 @@ int flnr_guide_backward(flnr_net *n, const float *grad_out, float *grad_in, void
     cudaStream_t st = (cudaStream_t)stream;
     const int N = n->N, H = n->H, W = n->W, H2 = H / 2, W2 = W / 2, H4 = H / 4, W4 = W / 4;
     const size_t P = (size_t)N * H * W;
-    auto gw = [&](int l) { return n->g + n->poff[l][0]; };
-    auto gb = [&](int l) { return n->g + n->poff[l][1]; };
-    auto bgrad = [&](const __nv_bfloat16 *dz, long long pix, int C, int ctrue, int l) {
-        bias_part_kernel<<<8 * C, 32, 0, st>>>(dz, n->wpart, pix, C);  // 256 C threads; wpart is free between layers
-        bias_tree_kernel<<<ctrue, 256, 0, st>>>(n->wpart, gb(l), C);
-    };
-    // output head: sigmoid, o1 (1x1, 16 -> 8 padded to 16), o0
-    sigmoid_bwd_kernel<<<egrid(P), 256, 0, st>>>(grad_out, n->out, n->gA, N, H, W, n->nout);
-    FLNR_TRY((wgrad_launch<16, 16, 1>(n->a5, n->gA, gw(11), N, H, W, 16, n->nout, n->wpart, n->wpart_floats, n->status, st)));
-    bgrad(n->gA, (long long)P, 16, n->nout, 11);
-    FLNR_TRY((dgrad_launch<16, 16, 1, true>({n->gA, n->wd[11], n->a5, nullptr, n->gB, nullptr, N, H, W, 16}, n->status, st)));
-    FLNR_TRY((wgrad_launch<16, 16, 3>(n->d0, n->gB, gw(10), N, H, W, 16, 16, n->wpart, n->wpart_floats, n->status, st)));
-    bgrad(n->gB, (long long)P, 16, 16, 10);
-    FLNR_TRY((dgrad_launch<16, 16, 3, true>({n->gB, n->wd[10], n->d0, nullptr, n->gA, nullptr, N, H, W, 16}, n->status, st)));
+    // every layer's weight and bias gradient goes to its partials; one reduction at the end
+    RedArgs ra;
+#define FLNR_WGRAD(ci, co, ks, mode, l, x, dz, h, w) \
+    FLNR_TRY((wgrad_launch<ci, co, ks, mode>(x, dz, kPlanes, N, h, w, wgrad_dest(n, l), ra, n->n_sm, n->status, st)))
+    // output head: sigmoid of o1 (1x1, 16 -> 8 padded to 16; the forward pass's products and
+    // weights again) and its gradient, then o1 and o0
+    ConvArgs hc{};
+    hc.x = n->a5; hc.w = n->head_w; hc.bias = n->head_b; hc.y = n->gA; hc.g = grad_out; hc.N = N; hc.H = H; hc.W = W;
+    hc.lx = hc.ly = kPlanes; hc.nbias = n->nout; hc.status = n->status;
+    FLNR_TRY((conv_ws_launch<16, 16, 1, 2, 2, false>(hc, st)));
+    FLNR_WGRAD(16, 16, 1, 0, 11, n->a5, n->gA, H, W);
+    FLNR_TRY((dgrad_launch<16, 16, 1, true>(n->gA, n->wd[11], n->a5, n->gB, N, H, W, n->status, st)));
+    FLNR_WGRAD(16, 16, 3, 0, 10, n->d0, n->gB, H, W);
+    FLNR_TRY((dgrad_launch<16, 16, 3, true>(n->gB, n->wd[10], n->d0, n->gA, N, H, W, n->status, st)));
     // decoder level 0
-    FLNR_TRY((wgrad_launch<16, 16, 3>(n->a4, n->gA, gw(9), N, H, W, 16, 16, n->wpart, n->wpart_floats, n->status, st)));
-    bgrad(n->gA, (long long)P, 16, 16, 9);
-    FLNR_TRY((dgrad_launch<16, 16, 3, true>({n->gA, n->wd[9], n->a4, nullptr, n->gB, nullptr, N, H, W, 16}, n->status, st)));
-    upcat_kernel<<<egrid(P * 6), 256, 0, st>>>(n->d1, n->f0, n->c0, N, H, W, 32, 16);  // d0a's input
-    FLNR_TRY(cudaGetLastError());
-    FLNR_TRY((wgrad_launch<48, 16, 3>(n->c0, n->gB, gw(8), N, H, W, 48, 16, n->wpart, n->wpart_floats, n->status, st)));
-    bgrad(n->gB, (long long)P, 16, 16, 8);
-    FLNR_TRY((dgrad_launch<16, 48, 3, false>({n->gB, n->wd[8], nullptr, nullptr, n->gC, nullptr, N, H, W, 48}, n->status, st)));
-    upcat_bwd_kernel<<<egrid(P * 48 / 8), 256, 0, st>>>(n->gC, n->d1, n->gLo, n->gskip0, N, H, W, 32, 16);  // gLo = dz(d1b)
+    FLNR_WGRAD(16, 16, 3, 0, 9, n->a4, n->gA, H, W);
+    FLNR_TRY((dgrad_launch<16, 16, 3, true>(n->gA, n->wd[9], n->a4, n->gB, N, H, W, n->status, st)));
+    FLNR_TRY(launch_pdl(upcat_kernel, egrid(P * 6), 256, 0, st, n->d1, n->f0, n->c0, N, H, W, 32, 16));  // d0a's input
+    FLNR_WGRAD(48, 16, 3, 0, 8, n->c0, n->gB, H, W);
+    FLNR_TRY((dgrad_launch<16, 48, 3, false>(n->gB, n->wd[8], nullptr, n->gC, N, H, W, n->status, st)));
+    FLNR_TRY(launch_pdl(upcat_bwd_kernel, egrid(P * 48 / 8), 256, 0, st, n->gC, n->d1, n->gLo, n->gskip0, N, H, W, 32, 16));  // gLo = dz(d1b)
     // decoder level 1 (H/2)
     const size_t P2 = P / 4;
-    FLNR_TRY((wgrad_launch<32, 32, 3>(n->a3, n->gLo, gw(7), N, H2, W2, 32, 32, n->wpart, n->wpart_floats, n->status, st)));
-    bgrad(n->gLo, (long long)P2, 32, 32, 7);
-    FLNR_TRY((dgrad_launch<32, 32, 3, true>({n->gLo, n->wd[7], n->a3, nullptr, n->gA, nullptr, N, H2, W2, 32}, n->status, st)));
-    upcat_kernel<<<egrid(P2 * 12), 256, 0, st>>>(n->f2, n->f1, n->c1, N, H2, W2, 64, 32);  // d1a's input
-    FLNR_TRY(cudaGetLastError());
-    FLNR_TRY((wgrad_launch<96, 32, 3>(n->c1, n->gA, gw(6), N, H2, W2, 96, 32, n->wpart, n->wpart_floats, n->status, st)));
-    bgrad(n->gA, (long long)P2, 32, 32, 6);
-    FLNR_TRY((dgrad_launch<32, 96, 3, false>({n->gA, n->wd[6], nullptr, nullptr, n->gC, nullptr, N, H2, W2, 96}, n->status, st)));
-    upcat_bwd_kernel<<<egrid(P2 * 96 / 8), 256, 0, st>>>(n->gC, n->f2, n->gLo, n->gskip1, N, H2, W2, 64, 32);  // gLo = dz(e2b)
-    // encoder level 2: e2b (stride 2, H/2 -> H/4), then e2a (H/2).  A stride-2 layer's
-    // gradients are those of the stride-1 kernels at its input's size on dz zero-upsampled
-    // onto that grid.
-    const size_t P4 = P / 16;
-    bgrad(n->gLo, (long long)P4, 64, 64, 5);
-    join_bwd_kernel<2><<<egrid(P2 * 64 / 8), 256, 0, st>>>(nullptr, n->gLo, nullptr, n->gB, N, H4, W4, 64);
-    FLNR_TRY(cudaGetLastError());
-    FLNR_TRY((wgrad_launch<64, 64, 3>(n->a2, n->gB, gw(5), N, H2, W2, 64, 64, n->wpart, n->wpart_floats, n->status, st)));
-    FLNR_TRY((dgrad_launch<64, 64, 3, true>({n->gB, n->wd[5], n->a2, nullptr, n->gA, nullptr, N, H2, W2, 64}, n->status, st)));
-    FLNR_TRY((wgrad_launch<32, 64, 3>(n->f1, n->gA, gw(4), N, H2, W2, 32, 64, n->wpart, n->wpart_floats, n->status, st)));
-    bgrad(n->gA, (long long)P2, 64, 64, 4);
-    FLNR_TRY((dgrad_launch<64, 32, 3, false>({n->gA, n->wd[4], nullptr, nullptr, n->gB, nullptr, N, H2, W2, 32}, n->status, st)));
+    FLNR_WGRAD(32, 32, 3, 0, 7, n->a3, n->gLo, H2, W2);
+    FLNR_TRY((dgrad_launch<32, 32, 3, true>(n->gLo, n->wd[7], n->a3, n->gA, N, H2, W2, n->status, st)));
+    FLNR_TRY(launch_pdl(upcat_kernel, egrid(P2 * 12), 256, 0, st, n->f2, n->f1, n->c1, N, H2, W2, 64, 32));  // d1a's input
+    FLNR_WGRAD(96, 32, 3, 0, 6, n->c1, n->gA, H2, W2);
+    FLNR_TRY((dgrad_launch<32, 96, 3, false>(n->gA, n->wd[6], nullptr, n->gC, N, H2, W2, n->status, st)));
+    FLNR_TRY(launch_pdl(upcat_bwd_kernel, egrid(P2 * 96 / 8), 256, 0, st, n->gC, n->f2, n->gLo, n->gskip1, N, H2, W2, 64, 32));  // gLo = dz(e2b)
+    // encoder level 2: e2b (stride 2, H/2 -> H/4), then e2a (H/2).  A stride-2 layer's input
+    // gradient is that of the stride-1 kernel at its input's size on dz zero-upsampled onto
+    // that grid; its weight gradient takes dz as it is.
+    FLNR_WGRAD(64, 64, 3, 1, 5, n->a2, n->gLo, H4, W4);
+    FLNR_TRY(launch_pdl(join_bwd_kernel<2>, egrid(P2 * 64 / 8), 256, 0, st, nullptr, n->gLo, nullptr, n->gB, nullptr, N, H4, W4, 64));
+    FLNR_TRY((dgrad_launch<64, 64, 3, true>(n->gB, n->wd[5], n->a2, n->gA, N, H2, W2, n->status, st, kParity)));
+    FLNR_WGRAD(32, 64, 3, 0, 4, n->f1, n->gA, H2, W2);
+    FLNR_TRY((dgrad_launch<64, 32, 3, false>(n->gA, n->wd[4], nullptr, n->gB, N, H2, W2, n->status, st)));
     // encoder level 1: e1b (stride 2, H -> H/2; f1 also feeds the d1a skip), then e1a (H)
-    join_bwd_kernel<2><<<egrid(P * 32 / 8), 256, 0, st>>>(n->gskip1, n->gB, n->f1, n->gC, N, H2, W2, 32);
-    FLNR_TRY(cudaGetLastError());
-    FLNR_TRY((wgrad_launch<32, 32, 3>(n->a1, n->gC, gw(3), N, H, W, 32, 32, n->wpart, n->wpart_floats, n->status, st)));
-    bgrad(n->gC, (long long)P, 32, 32, 3);
-    FLNR_TRY((dgrad_launch<32, 32, 3, true>({n->gC, n->wd[3], n->a1, nullptr, n->gA, nullptr, N, H, W, 32}, n->status, st)));
-    FLNR_TRY((wgrad_launch<16, 32, 3>(n->f0, n->gA, gw(2), N, H, W, 16, 32, n->wpart, n->wpart_floats, n->status, st)));
-    bgrad(n->gA, (long long)P, 32, 32, 2);
-    FLNR_TRY((dgrad_launch<32, 16, 3, false>({n->gA, n->wd[2], nullptr, nullptr, n->gB, nullptr, N, H, W, 16}, n->status, st)));
-    join_bwd_kernel<1><<<egrid(P * 16 / 8), 256, 0, st>>>(n->gskip0, n->gB, n->f0, n->gLo, N, H, W, 16);  // dz(in1)
+    FLNR_TRY(launch_pdl(join_bwd_kernel<2>, egrid(P * 32 / 8), 256, 0, st, n->gskip1, n->gB, n->f1, n->gC, n->gLo2, N, H2, W2, 32));
+    FLNR_WGRAD(32, 32, 3, 1, 3, n->a1, n->gLo2, H2, W2);
+    FLNR_TRY((dgrad_launch<32, 32, 3, true>(n->gC, n->wd[3], n->a1, n->gA, N, H, W, n->status, st, kParity)));
+    FLNR_WGRAD(16, 32, 3, 0, 2, n->f0, n->gA, H, W);
+    FLNR_TRY((dgrad_launch<32, 16, 3, false>(n->gA, n->wd[2], nullptr, n->gB, N, H, W, n->status, st)));
+    FLNR_TRY(launch_pdl(join_bwd_kernel<1>, egrid(P * 16 / 8), 256, 0, st, n->gskip0, n->gB, n->f0, n->gLo, nullptr, N, H, W, 16));  // dz(in1)
     // input projection (H)
-    FLNR_TRY((wgrad_launch<16, 16, 1>(n->a0, n->gLo, gw(1), N, H, W, 16, 16, n->wpart, n->wpart_floats, n->status, st)));
-    bgrad(n->gLo, (long long)P, 16, 16, 1);
-    FLNR_TRY((dgrad_launch<16, 16, 1, true>({n->gLo, n->wd[1], n->a0, nullptr, n->gA, nullptr, N, H, W, 16}, n->status, st)));
-    FLNR_TRY((wgrad_launch<16, 16, 3>(n->x0, n->gA, gw(0), N, H, W, 11, 16, n->wpart, n->wpart_floats, n->status, st)));
-    bgrad(n->gA, (long long)P, 16, 16, 0);
+    FLNR_WGRAD(16, 16, 1, 0, 1, n->a0, n->gLo, H, W);
+    FLNR_TRY((dgrad_launch<16, 16, 1, true>(n->gLo, n->wd[1], n->a0, n->gA, N, H, W, n->status, st)));
+    FLNR_WGRAD(16, 16, 3, 0, 0, n->x0, n->gA, H, W);
+#undef FLNR_WGRAD
     if (grad_in) {  // through in0 to the packed input, then through the input transform
-        FLNR_TRY((dgrad_launch<16, 16, 3, false>({n->gA, n->wd[0], nullptr, nullptr, n->gB, nullptr, N, H, W, 16}, n->status, st)));
-        unpack_grad_kernel<<<egrid(P), 256, 0, st>>>(n->gB, n->x0, grad_in, N, H, W);
+        FLNR_TRY((dgrad_launch<16, 16, 3, false>(n->gA, n->wd[0], nullptr, n->gB, N, H, W, n->status, st)));
+        FLNR_TRY(launch_pdl(unpack_grad_kernel, egrid(P), 256, 0, st, n->gB, n->x0, grad_in, N, H, W));
     }
-    return cudaGetLastError() == cudaSuccess ? FLR_OK : FLR_ERR_CUDA;
+    FLNR_TRY(cudaGetLastError());
+    FLNR_TRY(wgrad_reduce(ra, st));
+    return FLR_OK;
 }
 
 }  // extern "C"
@@ -2259,12 +2478,11 @@ int layer_ops(flnr_net *n, int l, int op, const void *a, const void *b, const vo
         c.N = N;
         c.H = H;
         c.W = W;
-        c.ystride = CO;
-        c.nbias = d.cout;
+        c.nbias = d.cout;  // lx, ly: NHWC
         c.status = n->status;
         if constexpr (HEAD) {
             c.yf = (float *)out;
-            FLNR_TRY((conv_ws_launch<CI, CO, KS, 2, 1>(c, st)));
+            FLNR_TRY((conv_ws_launch<CI, CO, KS, 2, 1, false>(c, st)));
         } else {
             c.y = (bf *)out;
             if constexpr (CA > 0) {
@@ -2279,7 +2497,7 @@ int layer_ops(flnr_net *n, int l, int op, const void *a, const void *b, const vo
                 if ((H | W) & 1) return FLR_ERR_ARG;
                 FLNR_TRY((conv_s2_launch<CI, CO, 2>(c, st)));
             } else {
-                FLNR_TRY((conv_ws_launch<CI, CO, KS, 1, 0>(c, st)));
+                FLNR_TRY((conv_ws_launch<CI, CO, KS, 1, 0, false>(c, st)));
             }
         }
         return FLR_OK;
@@ -2288,20 +2506,25 @@ int layer_ops(flnr_net *n, int l, int op, const void *a, const void *b, const vo
     if constexpr (S2) {  // dz [N][H/2][W/2][CO], zero-upsampled onto the input grid in scratch
         if ((H | W) & 1) return FLR_ERR_ARG;
         if (P * CO > (long long)n->max_pix * 48) return FLR_ERR_UNSUPPORTED;
-        join_bwd_kernel<2><<<egrid((size_t)P * CO / 8), 256, 0, st>>>(nullptr, dz, nullptr, n->gC, N, H / 2, W / 2, CO);
-        FLNR_TRY(cudaGetLastError());
+        FLNR_TRY(launch_pdl(spread_nhwc_kernel, egrid((size_t)P * CO / 8), 256, 0, st, dz, n->gC, N, H / 2, W / 2, CO));
         dz = n->gC;
     }
     if (op == FLNR_OP_DGRAD) {
-        if (mask)
-            FLNR_TRY((dgrad_launch<CO, CI, KS, true>({dz, n->wd[l], (const bf *)mask, nullptr, (bf *)out, nullptr, N, H, W, CI}, n->status, st)));
-        else
-            FLNR_TRY((dgrad_launch<CO, CI, KS, false>({dz, n->wd[l], nullptr, nullptr, (bf *)out, nullptr, N, H, W, CI}, n->status, st)));
+        ConvArgs c{};  // NHWC
+        c.x = dz;
+        c.w = n->wd[l];
+        c.mask = (const bf *)mask;
+        c.y = (bf *)out;
+        c.N = N;
+        c.H = H;
+        c.W = W;
+        c.status = n->status;
+        if (mask) FLNR_TRY((conv_ws_launch<CO, CI, KS, 0, 0, true>(c, st)));
+        else FLNR_TRY((conv_ws_launch<CO, CI, KS, 0, 0, false>(c, st)));
     } else {
-        FLNR_TRY((wgrad_launch<CI, CO, KS>((const bf *)a, dz, n->g + n->poff[l][0], N, H, W, d.cin, d.cout, n->wpart, n->wpart_floats, n->status, st)));
-        bias_part_kernel<<<8 * CO, 32, 0, st>>>(dz, n->wpart, P, CO);
-        bias_tree_kernel<<<d.cout, 256, 0, st>>>(n->wpart, n->g + n->poff[l][1], CO);
-        FLNR_TRY(cudaGetLastError());
+        RedArgs ra;
+        FLNR_TRY((wgrad_launch<CI, CO, KS, 0>((const bf *)a, dz, kNHWC, N, H, W, wgrad_dest(n, l), ra, n->n_sm, n->status, st)));
+        FLNR_TRY(wgrad_reduce(ra, st));
     }
     return FLR_OK;
 }
