@@ -118,3 +118,20 @@ def test_generic_kernel_shared_memory_is_only_raised(flr):
     assert rel_err(out.cpu().numpy(), oracle.flr_forward(g, y, 12, 1e-3, coef_radius=3)) <= TOL
     big.close()
     small.close()
+
+
+@pytest.mark.parametrize("H,W,r,rc", [(1, 4, 8, 8), (2, 4, 5, 5), (65, 92, 8, 0), (33, 88, 5, 5), (43, 164, 8, 8)])
+def test_partly_flagged_batches_and_pairs(flr, H, W, r, rc):
+    """Batches of two rows and pixel pairs of which one, both or none is flagged (the threshold is
+    the median pivot ratio's order, so about half the pixels are), a last batch of one row, strips
+    wider than the image: the packed solve, the list in (row, column) order and the FP64 shares.
+    Bar: the parity metric's, as for every uniform frame."""
+    g, y = synth.random_frame(H * 11 + W, H, W, 8)
+    ref = oracle.flr_forward(g, y, r, 1e-3, coef_radius=rc)
+    flagged = []
+    for pivot in (0.5, 0.8):
+        got, st = run(flr, g, y, r, rc, pivot_ratio=pivot)
+        assert np.all(np.isfinite(got)) and st["resolved"] == st["flagged"]
+        assert rel_err(got, ref) <= TOL
+        flagged.append(st["flagged"])
+    assert flagged[0] <= flagged[1] <= H * W
