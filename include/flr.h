@@ -334,19 +334,19 @@ int flr_denoise_batch(flr_handle *h, int n, const flr_frame *frames, void *strea
 
 /*
  * Batched fast FLR / joint denoising and upsampling (Sec. 3.2, 3.2.1) of n <= FLR_MAX_BATCH
- * frames of mixed sizes in ONE persistent cooperative kernel launch: every stage of every
- * frame is a work item of the same kernel, with a grid barrier between the four stages.
+ * frames of mixed sizes: each of the four stages is one launch over the work items of all
+ * frames (the last one two if only some frames' rows start on 16-byte boundaries).
  * The frame table is passed by value in the kernel parameters, so the call can be captured
  * in a CUDA graph once flr_fast_reserve_batch has allocated the workspace for these sizes
  * (after that the call allocates nothing).  Supported for q in {1, 4, 8} and every factor.
- * Each barrier wait is bounded (2 s): if it runs out, the kernel records FLR_BATCH_TIMEOUT
+ * Each device wait is bounded (1 s): if it runs out, the kernel records FLR_BATCH_TIMEOUT
  * and finishes without hanging; flr_fast_batch_status reports it.
  * Errors: FLR_ERR_ARG, FLR_ERR_ALIGN, FLR_ERR_UNSUPPORTED, FLR_ERR_NOMEM, FLR_ERR_CUDA.
  */
 int flr_fast_reserve_batch(flr_fast_handle *h, int n, const flr_frame *frames);
 int flr_fast_denoise_batch(flr_fast_handle *h, int n, const flr_frame *frames, void *stream);
 
-/* Waits for the last batch and returns FLR_OK, or FLR_ERR_TIMEOUT if a barrier ran out. */
+/* Waits for the last batch and returns FLR_OK, or FLR_ERR_TIMEOUT if a wait ran out. */
 int flr_fast_batch_status(flr_fast_handle *h);
 
 /*

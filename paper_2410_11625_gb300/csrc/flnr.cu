@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "flr.h"
+#include "pdl.cuh"
 
 namespace flnr {
 namespace {
@@ -49,32 +50,11 @@ constexpr LayerDef kLayers[kNL] = {
 __host__ __device__ constexpr int pad16(int c) { return (c + 15) / 16 * 16; }
 
 // ---------------------------------------------------------------------------------------
-// Programmatic dependent launch.  The network is a chain of short kernels, each reading what the
-// one before wrote, and at 16 x 128^2 a training pass lost 120 us of 690 between them.  A kernel
-// launched with launch_pdl may start when every CTA of its predecessor has called pdl_trigger (or
-// exited); it must call pdl_wait, which returns when the predecessor has finished and its writes
-// are visible, before it touches global memory.  Only the set-up of barriers and tensor memory
-// runs ahead.  A kernel that allocates tensor memory triggers after its allocation: its
+// Every launch is a programmatic dependent one (pdl.cuh).  The network is a chain of short
+// kernels, each reading what the one before wrote, and at 16 x 128^2 a training pass lost 120 us
+// of 690 between them.  A kernel that allocates tensor memory triggers after its allocation: its
 // successor's CTAs, which may be resident beside it and hold columns while they wait, then cannot
 // keep it from allocating.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-
-template <class... P, class... A>
-cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A &&...args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
-}
 
 // ---------------------------------------------------------------------------------------
 // Asynchronous 16-byte global -> shared copies (zero fill when !valid).
@@ -407,8 +387,8 @@ __global__ void __launch_bounds__(WsGeom<CIN, COUT, KS, NT>::THREADS) conv_ws_ke
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
     __syncthreads();  // tensor memory allocated
-    pdl_trigger();
-    pdl_wait();
+    pdl::trigger();
+    pdl::wait();
     for (int i = tid; i < KS * KS * COUT * C8; i += G::THREADS) {
         const int c8 = i % C8, row = i / C8, tap = row / COUT, co = row % COUT;
         cp_async16(sw + ((tap * C8 + c8) * COUT + co) * 16, a.w + (size_t)row * CIN + c8 * 8, true);
@@ -604,8 +584,8 @@ __global__ void __launch_bounds__(WsGeom<CIN, COUT, KS, NT>::THREADS) conv_tail_
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
     __syncthreads();  // tensor memory allocated
-    pdl_trigger();
-    pdl_wait();
+    pdl::trigger();
+    pdl::wait();
     for (int i = tid; i < KS * KS * COUT * C8; i += G::THREADS) {
         const int c8 = i % C8, row = i / C8, tap = row / COUT, co = row % COUT;
         cp_async16(sw + ((tap * C8 + c8) * COUT + co) * 16, a.w + (size_t)row * CIN + c8 * 8, true);
@@ -889,8 +869,8 @@ __global__ void __launch_bounds__(kWsThreads) conv_up_kernel(const __grid_consta
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
     __syncthreads();  // tensor memory allocated
-    pdl_trigger();
-    pdl_wait();
+    pdl::trigger();
+    pdl::wait();
     // weights: global [tap][COUT][CA + CB] -> shared [tap][c8][COUT][8] (lo chunks first)
     for (int i = tid; i < 9 * COUT * C8; i += kWsThreads) {
         const int c8 = i % C8, row = i / C8, tap = row / COUT, co = row % COUT;
@@ -1105,8 +1085,8 @@ __global__ void __launch_bounds__(kWsThreads) conv_s2_kernel(const __grid_consta
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
     __syncthreads();  // tensor memory allocated
-    pdl_trigger();
-    pdl_wait();
+    pdl::trigger();
+    pdl::wait();
     for (int i = tid; i < 9 * COUT * C8; i += kWsThreads) {
         const int c8 = i % C8, row = i / C8, tap = row / COUT, co = row % COUT;
         cp_async16(sw + ((tap * C8 + c8) * COUT + co) * 16, a.w + (size_t)row * CIN + c8 * 8, true);
@@ -1352,8 +1332,8 @@ __global__ void __launch_bounds__(kWgThreads) wgrad_tc_kernel(const __grid_const
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n");
     const uint32_t tmem = s_tmem;
-    pdl_trigger();
-    pdl_wait();
+    pdl::trigger();
+    pdl::wait();
 
     if (warp == 1 && lane == 0) {  // producer
         for (int j = 0; j < mine; ++j) {
@@ -1479,8 +1459,8 @@ constexpr int kRedWarps = 16;
 
 __global__ void __launch_bounds__(32 * kRedWarps) wgrad_reduce_kernel(const __grid_constant__ RedArgs a)
 {
-    pdl_trigger();
-    pdl_wait();
+    pdl::trigger();
+    pdl::wait();
     int k = 0;
     while (k + 1 < a.n && (int)blockIdx.x >= a.l[k + 1].first_block) ++k;
     const RedLayer &l = a.l[k];
@@ -1525,8 +1505,8 @@ __global__ void __launch_bounds__(32 * kRedWarps) wgrad_reduce_kernel(const __gr
 // enter the network as log(1 + max(Y, 0)), which keeps fireflies from dominating the features
 __global__ void pack_input_kernel(const float *in, bf16 *x, int N, int H, int W)
 {
-    pdl_trigger();
-    pdl_wait();
+    pdl::trigger();
+    pdl::wait();
     const size_t hw = (size_t)H * W, total = (size_t)N * hw;
     for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < total; p += (size_t)gridDim.x * blockDim.x) {
         const size_t n = p / hw, o = p % hw;
@@ -1549,8 +1529,8 @@ __global__ void pack_input_kernel(const float *in, bf16 *x, int N, int H, int W)
 // Y > 0 and 0 for Y < 0 (L is the stored bfloat16 value, so Y > 0 exactly when L > 0)
 __global__ void unpack_grad_kernel(const bf16 *dx, const bf16 *x, float *g, int N, int H, int W)
 {
-    pdl_trigger();
-    pdl_wait();
+    pdl::trigger();
+    pdl::wait();
     const size_t hw = (size_t)H * W, total = (size_t)N * hw;
     for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < total; p += (size_t)gridDim.x * blockDim.x) {
         const size_t n = p / hw, o = p % hw;
@@ -1571,8 +1551,8 @@ __global__ void unpack_grad_kernel(const bf16 *dx, const bf16 *x, float *g, int 
 // H x W), all bf16 planes (the input of a decoder level, materialised for its weight gradient)
 __global__ void upcat_kernel(const bf16 *lo, const bf16 *skip, bf16 *y, int N, int H, int W, int Ca, int Cb)
 {
-    pdl_trigger();
-    pdl_wait();
+    pdl::trigger();
+    pdl::wait();
     // one thread per pixel of a chunk plane of y: 16-byte copies
     const int C8 = (Ca + Cb) / 8, A8 = Ca / 8, B8 = Cb / 8, hw = H * W;
     const size_t total = (size_t)N * C8 * hw;
@@ -1593,8 +1573,8 @@ __global__ void upcat_kernel(const bf16 *lo, const bf16 *skip, bf16 *y, int N, i
 __global__ void upcat_bwd_kernel(const bf16 *gy, const bf16 *lo, bf16 *g_lo, float *g_skip, int N, int H, int W,
                                  int Ca, int Cb)
 {
-    pdl_trigger();
-    pdl_wait();
+    pdl::trigger();
+    pdl::wait();
     // eight channels of one pixel per thread: 16-byte loads and stores
     const int A8 = Ca / 8, B8 = Cb / 8, C8 = A8 + B8, hw = H * W, hl = hw / 4, Wl = W / 2;
     const size_t tl = (size_t)N * A8 * hl, ts = (size_t)N * B8 * hw;
@@ -1644,8 +1624,8 @@ template <int S>
 __global__ void join_bwd_kernel(const float *g_skip, const bf16 *g_path, const bf16 *f, bf16 *dz, bf16 *dlo, int N,
                                 int Ho, int Wo, int C)
 {
-    pdl_trigger();
-    pdl_wait();
+    pdl::trigger();
+    pdl::wait();
     // eight channels of one pixel per thread: 16-byte loads and stores
     const int hw = S * Ho * S * Wo, W = S * Wo;
     const size_t total = (size_t)N * (C / 8) * hw;
@@ -1682,8 +1662,8 @@ __global__ void join_bwd_kernel(const float *g_skip, const bf16 *g_path, const b
 // zero-upsampling of an NHWC gradient [N][Ho][Wo][C] onto [N][2Ho][2Wo][C] (flnr_layer)
 __global__ void spread_nhwc_kernel(const bf16 *g, bf16 *dz, int N, int Ho, int Wo, int C)
 {
-    pdl_trigger();
-    pdl_wait();
+    pdl::trigger();
+    pdl::wait();
     const int C8 = C / 8, W = 2 * Wo, H = 2 * Ho;
     const size_t total = (size_t)N * H * W * C8;
     for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
@@ -1962,7 +1942,7 @@ cudaError_t conv_ws_launch_nt(const ConvArgs &a, bool ask, bool *fits, cudaStrea
     std::memset(&ta, 0, sizeof(ta));
     ta.c = a;
     if ((e = make_tmap_tile(&ta.tm, a.lx, a.x, CIN, a.W, a.H, a.N, G::SW, G::SH)) != cudaSuccess) return e;
-    return launch_pdl(kern, (int)(ntiles < cap ? ntiles : cap), G::THREADS, smem, st, ta);
+    return pdl::launch(kern, (int)(ntiles < cap ? ntiles : cap), G::THREADS, smem, st, ta);
 }
 template <int CIN, int COUT, int KS, int ACT, int OUTM, bool MASK>
 cudaError_t conv_ws_launch(const ConvArgs &a, cudaStream_t st)
@@ -2023,7 +2003,7 @@ cudaError_t conv_tail_launch_nt(const ConvArgs &c, const ConvArgs &c2, bf16 *w2_
     ta.w2_kept = w2_kept;
     ta.b2_kept = b2_kept;
     if ((e = make_tmap_tile(&ta.tm, c.lx, c.x, CIN, c.W, c.H, c.N, G::SW, G::SH)) != cudaSuccess) return e;
-    return launch_pdl(kern, (int)(ntiles < cap ? ntiles : cap), G::THREADS, smem, st, ta);
+    return pdl::launch(kern, (int)(ntiles < cap ? ntiles : cap), G::THREADS, smem, st, ta);
 }
 template <int CIN, int COUT, int KS, int COUT2, int ACT2, int OUTM2>
 cudaError_t conv_tail_launch(const ConvArgs &c, const ConvArgs &c2, cudaStream_t st, bf16 *w2_kept = nullptr,
@@ -2058,7 +2038,7 @@ cudaError_t conv_up_launch(const ConvArgs &a, cudaStream_t st)
     e = a.lx == kNHWC ? make_tmap_parity(&ua.tskip, a.x2, CB, a.W, a.H, a.N, G::SW, G::SH)
                       : make_tmap_pairs(&ua.tskip, a.x2, CB, a.W, a.H, a.N, G::SW, G::SH);
     if (e != cudaSuccess) return e;
-    return launch_pdl(kern, (int)(ntiles < cap ? ntiles : cap), kWsThreads, smem, st, ua);
+    return pdl::launch(kern, (int)(ntiles < cap ? ntiles : cap), kWsThreads, smem, st, ua);
 }
 
 // Launch of the stride-2 convolution (a.H, a.W: the input's size, both even; output at half
@@ -2086,7 +2066,7 @@ cudaError_t conv_s2_launch(const ConvArgs &a, cudaStream_t st)
         if ((e = make_tmap_planes(&sa.te, a.x, CIN / 2, a.W / 2, a.H / 2, a.N, G::WE, G::SH)) != cudaSuccess) return e;
         if ((e = make_tmap_planes(&sa.to, a.x, CIN / 2, a.W / 2, a.H / 2, a.N, G::WO, G::SH)) != cudaSuccess) return e;
     }
-    return launch_pdl(kern, (int)(ntiles < cap ? ntiles : cap), kWsThreads, smem, st, sa);
+    return pdl::launch(kern, (int)(ntiles < cap ? ntiles : cap), kWsThreads, smem, st, sa);
 }
 
 // Where a layer's gradients go: its partials (n_sm slices), master weight and bias gradients
@@ -2123,12 +2103,12 @@ cudaError_t wgrad_launch(const bf16 *x, const bf16 *dz, int layout, int N, int H
     if ((e = make_tmap_tile(&a.tdz, layout, dz, COUT, W, H, N, 8, 16)) != cudaSuccess) return e;
     ra.l[ra.n++] = RedLayer{d.part, d.gw, d.gb, slices, COUT, CIN, KS, MODE, d.cin_true, d.cout_true, ra.blocks};
     ra.blocks += (COUT * G::CTOT + 31) / 32;
-    return launch_pdl(kern, dim3(slices, G::NG), kWgThreads, smem, st, a);
+    return pdl::launch(kern, dim3(slices, G::NG), kWgThreads, smem, st, a);
 }
 
 cudaError_t wgrad_reduce(const RedArgs &ra, cudaStream_t st)
 {
-    return launch_pdl(wgrad_reduce_kernel, ra.blocks, 32 * kRedWarps, 0, st, ra);
+    return pdl::launch(wgrad_reduce_kernel, ra.blocks, 32 * kRedWarps, 0, st, ra);
 }
 
 }  // namespace
@@ -2353,7 +2333,7 @@ int flnr_guide_forward(flnr_net *n, const float *in, float *guide_out, int N, in
     const size_t P = (size_t)N * H * W;
     const int H2 = H / 2, W2 = W / 2;
     auto bias = [&](int l) { return n->w + n->poff[l][1]; };
-    FLNR_TRY(launch_pdl(pack_input_kernel, egrid(P), 256, 0, st, in, n->x0, N, H, W));
+    FLNR_TRY(pdl::launch(pack_input_kernel, egrid(P), 256, 0, st, in, n->x0, N, H, W));
     const ConvArgs z{};
     auto conv = [&](const __nv_bfloat16 *x, int l, __nv_bfloat16 *y, int h, int w, int ly = kPlanes) {
         ConvArgs c = z;
@@ -2414,33 +2394,33 @@ int flnr_guide_backward(flnr_net *n, const float *grad_out, float *grad_in, void
     // decoder level 0
     FLNR_WGRAD(16, 16, 3, 0, 9, n->a4, n->gA, H, W);
     FLNR_TRY((dgrad_launch<16, 16, 3, true>(n->gA, n->wd[9], n->a4, n->gB, N, H, W, n->status, st)));
-    FLNR_TRY(launch_pdl(upcat_kernel, egrid(P * 6), 256, 0, st, n->d1, n->f0, n->c0, N, H, W, 32, 16));  // d0a's input
+    FLNR_TRY(pdl::launch(upcat_kernel, egrid(P * 6), 256, 0, st, n->d1, n->f0, n->c0, N, H, W, 32, 16));  // d0a's input
     FLNR_WGRAD(48, 16, 3, 0, 8, n->c0, n->gB, H, W);
     FLNR_TRY((dgrad_launch<16, 48, 3, false>(n->gB, n->wd[8], nullptr, n->gC, N, H, W, n->status, st)));
-    FLNR_TRY(launch_pdl(upcat_bwd_kernel, egrid(P * 48 / 8), 256, 0, st, n->gC, n->d1, n->gLo, n->gskip0, N, H, W, 32, 16));  // gLo = dz(d1b)
+    FLNR_TRY(pdl::launch(upcat_bwd_kernel, egrid(P * 48 / 8), 256, 0, st, n->gC, n->d1, n->gLo, n->gskip0, N, H, W, 32, 16));  // gLo = dz(d1b)
     // decoder level 1 (H/2)
     const size_t P2 = P / 4;
     FLNR_WGRAD(32, 32, 3, 0, 7, n->a3, n->gLo, H2, W2);
     FLNR_TRY((dgrad_launch<32, 32, 3, true>(n->gLo, n->wd[7], n->a3, n->gA, N, H2, W2, n->status, st)));
-    FLNR_TRY(launch_pdl(upcat_kernel, egrid(P2 * 12), 256, 0, st, n->f2, n->f1, n->c1, N, H2, W2, 64, 32));  // d1a's input
+    FLNR_TRY(pdl::launch(upcat_kernel, egrid(P2 * 12), 256, 0, st, n->f2, n->f1, n->c1, N, H2, W2, 64, 32));  // d1a's input
     FLNR_WGRAD(96, 32, 3, 0, 6, n->c1, n->gA, H2, W2);
     FLNR_TRY((dgrad_launch<32, 96, 3, false>(n->gA, n->wd[6], nullptr, n->gC, N, H2, W2, n->status, st)));
-    FLNR_TRY(launch_pdl(upcat_bwd_kernel, egrid(P2 * 96 / 8), 256, 0, st, n->gC, n->f2, n->gLo, n->gskip1, N, H2, W2, 64, 32));  // gLo = dz(e2b)
+    FLNR_TRY(pdl::launch(upcat_bwd_kernel, egrid(P2 * 96 / 8), 256, 0, st, n->gC, n->f2, n->gLo, n->gskip1, N, H2, W2, 64, 32));  // gLo = dz(e2b)
     // encoder level 2: e2b (stride 2, H/2 -> H/4), then e2a (H/2).  A stride-2 layer's input
     // gradient is that of the stride-1 kernel at its input's size on dz zero-upsampled onto
     // that grid; its weight gradient takes dz as it is.
     FLNR_WGRAD(64, 64, 3, 1, 5, n->a2, n->gLo, H4, W4);
-    FLNR_TRY(launch_pdl(join_bwd_kernel<2>, egrid(P2 * 64 / 8), 256, 0, st, nullptr, n->gLo, nullptr, n->gB, nullptr, N, H4, W4, 64));
+    FLNR_TRY(pdl::launch(join_bwd_kernel<2>, egrid(P2 * 64 / 8), 256, 0, st, nullptr, n->gLo, nullptr, n->gB, nullptr, N, H4, W4, 64));
     FLNR_TRY((dgrad_launch<64, 64, 3, true>(n->gB, n->wd[5], n->a2, n->gA, N, H2, W2, n->status, st, kParity)));
     FLNR_WGRAD(32, 64, 3, 0, 4, n->f1, n->gA, H2, W2);
     FLNR_TRY((dgrad_launch<64, 32, 3, false>(n->gA, n->wd[4], nullptr, n->gB, N, H2, W2, n->status, st)));
     // encoder level 1: e1b (stride 2, H -> H/2; f1 also feeds the d1a skip), then e1a (H)
-    FLNR_TRY(launch_pdl(join_bwd_kernel<2>, egrid(P * 32 / 8), 256, 0, st, n->gskip1, n->gB, n->f1, n->gC, n->gLo2, N, H2, W2, 32));
+    FLNR_TRY(pdl::launch(join_bwd_kernel<2>, egrid(P * 32 / 8), 256, 0, st, n->gskip1, n->gB, n->f1, n->gC, n->gLo2, N, H2, W2, 32));
     FLNR_WGRAD(32, 32, 3, 1, 3, n->a1, n->gLo2, H2, W2);
     FLNR_TRY((dgrad_launch<32, 32, 3, true>(n->gC, n->wd[3], n->a1, n->gA, N, H, W, n->status, st, kParity)));
     FLNR_WGRAD(16, 32, 3, 0, 2, n->f0, n->gA, H, W);
     FLNR_TRY((dgrad_launch<32, 16, 3, false>(n->gA, n->wd[2], nullptr, n->gB, N, H, W, n->status, st)));
-    FLNR_TRY(launch_pdl(join_bwd_kernel<1>, egrid(P * 16 / 8), 256, 0, st, n->gskip0, n->gB, n->f0, n->gLo, nullptr, N, H, W, 16));  // dz(in1)
+    FLNR_TRY(pdl::launch(join_bwd_kernel<1>, egrid(P * 16 / 8), 256, 0, st, n->gskip0, n->gB, n->f0, n->gLo, nullptr, N, H, W, 16));  // dz(in1)
     // input projection (H)
     FLNR_WGRAD(16, 16, 1, 0, 1, n->a0, n->gLo, H, W);
     FLNR_TRY((dgrad_launch<16, 16, 1, true>(n->gLo, n->wd[1], n->a0, n->gA, N, H, W, n->status, st)));
@@ -2448,7 +2428,7 @@ int flnr_guide_backward(flnr_net *n, const float *grad_out, float *grad_in, void
 #undef FLNR_WGRAD
     if (grad_in) {  // through in0 to the packed input, then through the input transform
         FLNR_TRY((dgrad_launch<16, 16, 3, false>(n->gA, n->wd[0], nullptr, n->gB, N, H, W, n->status, st)));
-        FLNR_TRY(launch_pdl(unpack_grad_kernel, egrid(P), 256, 0, st, n->gB, n->x0, grad_in, N, H, W));
+        FLNR_TRY(pdl::launch(unpack_grad_kernel, egrid(P), 256, 0, st, n->gB, n->x0, grad_in, N, H, W));
     }
     FLNR_TRY(cudaGetLastError());
     FLNR_TRY(wgrad_reduce(ra, st));
@@ -2506,7 +2486,7 @@ int layer_ops(flnr_net *n, int l, int op, const void *a, const void *b, const vo
     if constexpr (S2) {  // dz [N][H/2][W/2][CO], zero-upsampled onto the input grid in scratch
         if ((H | W) & 1) return FLR_ERR_ARG;
         if (P * CO > (long long)n->max_pix * 48) return FLR_ERR_UNSUPPORTED;
-        FLNR_TRY(launch_pdl(spread_nhwc_kernel, egrid((size_t)P * CO / 8), 256, 0, st, dz, n->gC, N, H / 2, W / 2, CO));
+        FLNR_TRY(pdl::launch(spread_nhwc_kernel, egrid((size_t)P * CO / 8), 256, 0, st, dz, n->gC, N, H / 2, W / 2, CO));
         dz = n->gC;
     }
     if (op == FLNR_OP_DGRAD) {

@@ -1,12 +1,12 @@
 // flr_fast.cu -- the paper's fast FLR (Sec. 3.2) and its joint denoising and upsampling
 // (Sec. 3.2.1) on sm_103a, behind the flr_fast_* entry points of include/flr.h.
 //
-// The paper's four steps, as four kernels:
+// The paper's four steps, as four kernels over all the frames of a call:
 //   1. block_moments: outer products of the shifted inputs summed over F x F blocks of the
 //      input grid (the strided box filter);  one thread per pair of input columns walks the
-//      F rows of its block row, then a shuffle tree over the F / 2 lanes of a block reduces
-//      them;
-//   2. blur_h:  horizontal Gaussian over the block grid (one thread per channel and block);
+//      F rows of its block row, fed by its own ring of asynchronous copies, then the F / 2 lanes
+//      of a block fold their sums;
+//   2. blur_h:  horizontal Gaussian over the block grid (one thread per block);
 //   3. blur_v_solve: vertical Gaussian, then the centred ridge model of every block in
 //      registers (the window sums staged per thread in shared memory); a block whose
 //      Cholesky pivot ratio falls to tau or below is re-solved in FP64 from the same sums;
@@ -15,6 +15,8 @@
 // Only step 1 and step 4 touch full-resolution data: the input is read once (44 B per
 // input pixel for Q = 8), the map guide once and the output written once (32 + 12 B per
 // output pixel); everything in between lives in (F^2)-times smaller planes that stay in L2.
+// At 1920x1080, F = 8, without overlap: 21 + 9 + 10 + 14 us (26.5 + 9 + 11.6 + 19 before the ring,
+// the block-major models and the packed apply), 57 us in all (77); the bytes alone take 17 us.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -23,10 +25,10 @@
 #include <cstring>
 #include <new>
 #include <utility>
-#include <vector>
 
 #include "flr.h"
 #include "flr_fast_stages.cuh"
+#include "pdl.cuh"
 #include "tma.cuh"
 
 namespace flr {
@@ -35,31 +37,79 @@ namespace {
 using fast::FastArgs;
 using fast::kMaxTaps;
 
-template <int Q, int F>
-__global__ void __launch_bounds__(256, 2) block_moments_kernel(const FastArgs a)
+// The blurs are bound by the latency of their loads, 82 per tap: two CTAs of 128 threads per SM
+// with up to 255 registers let the compiler keep more of them in flight than it does by itself
+// (146 registers): 63.7 -> 57.4 us for the whole frame at 1920x1080.  CTAs of 64 threads: 74.9 us.
+constexpr int kBlurThreads = 128;
+
+// The frames of one call: one (N = 1), or up to FLR_MAX_BATCH of mixed sizes (N = FLR_MAX_BATCH).
+// Stage s of frame i covers CTAs (stages 1 to 3) or work items (stage 4) off[s][i] .. off[s][i + 1].
+// A batch is the four stages over all its frames, not four launches per frame: 8 frames fill the
+// chip's last wave of each stage once instead of eight times.  (One persistent kernel over the
+// stages with grid barriers between them, the form before this, ran every stage at the occupancy
+// of the most demanding one, 8 warps per SM: 488 us for 3 frames each of 1280x720 and 1920x1080
+// and 2 of 2560x1440 outputs.)
+template <int N>
+struct FrameTable {
+    FastArgs f[N];
+    int n;
+    unsigned off[4][N + 1];
+    unsigned long long *count;  // zeroed by stage 1, counted by stage 3
+    int *status;                // zeroed by stage 1 if not NULL (the batch's status word)
+};
+
+template <int N>
+__device__ __forceinline__ int frame_of(const FrameTable<N> &t, int stage, unsigned item)
 {
-    fast::stage_moments<Q, F>(a, blockIdx.y, blockIdx.x);
+    int f = 0;
+    if (N > 1)
+        while (f + 1 < t.n && item >= t.off[stage][f + 1]) ++f;
+    return f;
 }
 
-template <int Q>
-__global__ void __launch_bounds__(128) blur_h_kernel(const FastArgs a)
+template <int Q, int F, int N>
+__global__ void __launch_bounds__(fast::kMomThreads, 512 / fast::kMomThreads) block_moments_kernel(const __grid_constant__ FrameTable<N> t)
 {
-    fast::stage_blur_h<Q>(a, (size_t)blockIdx.x * blockDim.x + threadIdx.x);
+    extern __shared__ __align__(16) float ring[];
+    pdl::trigger();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *t.count = 0ull;
+        if (t.status) *t.status = 0;
+    }
+    const int f = frame_of(t, 0, blockIdx.x);
+    const FastArgs &a = t.f[f];
+    const int item = (int)(blockIdx.x - t.off[0][f]), chunks = fast::moment_chunks(a.Wi);
+    fast::stage_moments<Q, F>(a, item / chunks, item % chunks, ring);
 }
 
-template <int Q>
-__global__ void __launch_bounds__(128) blur_v_solve_kernel(const FastArgs a)
+template <int Q, int N>
+__global__ void __launch_bounds__(kBlurThreads, 2) blur_h_kernel(const __grid_constant__ FrameTable<N> t)
 {
-    extern __shared__ float sS[];  // [NCH][blockDim.x]
-    fast::stage_blur_v_solve<Q>(a, (size_t)blockIdx.x * blockDim.x + threadIdx.x, sS + threadIdx.x, blockDim.x);
+    pdl::trigger();
+    const int f = frame_of(t, 1, blockIdx.x);
+    pdl::wait();
+    fast::stage_blur_h<Q>(t.f[f], (size_t)(blockIdx.x - t.off[1][f]) * kBlurThreads + threadIdx.x);
 }
 
-template <int Q>
-__global__ void __launch_bounds__(256) fast_apply_kernel(const FastArgs a)
+template <int Q, int N>
+__global__ void __launch_bounds__(kBlurThreads, 2) blur_v_solve_kernel(const __grid_constant__ FrameTable<N> t)
 {
-    const size_t runs = (size_t)a.Ho * (a.Wo / (a.F * a.s) + 2);
-    for (size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x; t < runs; t += (size_t)gridDim.x * blockDim.x)
-        fast::stage_apply<Q>(a, t);
+    extern __shared__ float sS[];  // [NCH][kBlurThreads]
+    pdl::trigger();
+    const int f = frame_of(t, 2, blockIdx.x);
+    pdl::wait();
+    fast::stage_blur_v_solve<Q>(t.f[f], (size_t)(blockIdx.x - t.off[2][f]) * kBlurThreads + threadIdx.x, sS + threadIdx.x,
+                                kBlurThreads);
+}
+
+template <int Q, int N>
+__global__ void __launch_bounds__(256) fast_apply_kernel(const __grid_constant__ FrameTable<N> t)
+{
+    pdl::wait();
+    for (unsigned item = blockIdx.x; item < t.off[3][t.n]; item += gridDim.x) {
+        const int f = frame_of(t, 3, item);
+        fast::stage_apply<Q>(t.f[f], (size_t)(item - t.off[3][f]) * 256 + threadIdx.x);
+    }
 }
 
 // ---- parameter gradients (sigma and the regularisation terms) ---------------------------
@@ -111,9 +161,10 @@ __global__ void __launch_bounds__(256) dot_final_kernel(const double *part, doub
 constexpr int kFW = 128;
 constexpr unsigned long long kFastTimeoutNs = 1000000000ull;
 
+template <int N>
 struct alignas(128) FastKArgs {
-    CUtensorMap t0;  // map-guide planes [Q][Ho][Wo], box (kFW, P, Q)
-    FastArgs a;
+    CUtensorMap t0[N];  // map-guide planes [Q][Ho][Wo], box (kFW, P, Q)
+    FrameTable<N> t;
 };
 
 __device__ __forceinline__ float *align128(float *p)
@@ -125,21 +176,22 @@ __device__ __forceinline__ float *align128(float *p)
 // rows [P i - P/2, P i + P/2), which all interpolate between the same two block rows; the
 // item loads those rows of the Q map-guide planes.  Thread t owns output column kFW cx + t:
 // it interpolates its corner models horizontally once per item (top and bottom block row),
-// then for each row vertically, and applies them.  The coordinates are the exact rational
-// ones of fast::stage_apply.
-template <int Q>
-__global__ void __launch_bounds__(kFW, 3) apply_tma_kernel(const __grid_constant__ FastKArgs k)
+// while the item's rows are still on their way, then for each row vertically, and applies them,
+// two guides per instruction (packed FP32).  The coordinates are the exact rational ones of
+// fast::stage_apply.  PC: P known at compile time (the weights' divisions become products), or 0.
+template <int Q, int N, int PC>
+__global__ void __launch_bounds__(kFW, 3) apply_tma_kernel(const __grid_constant__ FastKArgs<N> k)
 {
-    constexpr int NC = 3 * (Q + 1), PMAX = 8, STAGE = Q * PMAX * kFW;
-    const FastArgs &a = k.a;
+    using M = fast::Model<Q>;
+    constexpr int PMAX = 8, STAGE = Q * PMAX * kFW, CS = M::CS, QE = M::QE;
     extern __shared__ __align__(16) float smem[];
     float *base = align128(smem);
     uint64_t *bar = reinterpret_cast<uint64_t *>(base + 2 * STAGE);
     __shared__ int s_abort;
     const int tid = threadIdx.x, lane = tid & 31;
-    const int P = a.F * a.s, den = 2 * P;
-    const int ncx = (a.Wo + kFW - 1) / kFW, nitems = (a.Hb + 1) * ncx;
-    const size_t oplane = (size_t)a.Ho * a.Wo, bplane = (size_t)a.Hb * a.Wb;
+    const unsigned nitems = k.t.off[3][k.t.n];
+    const int P = PC ? PC : k.t.f[0].F * k.t.f[0].s, den = 2 * P;  // the handle's: the same for every frame
+    int *status = k.t.f[0].status;
     if (tid == 0) {
         s_abort = 0;
         tma::mbar_init(bar, 1);
@@ -147,72 +199,94 @@ __global__ void __launch_bounds__(kFW, 3) apply_tma_kernel(const __grid_constant
         tma::mbar_init_fence();
     }
     __syncthreads();
-    auto issue = [&](int item, int st) {
-        const int ci = item / ncx, cx = item % ncx;
+    auto issue = [&](unsigned item, int st) {
+        const int f = frame_of(k.t, 3, item);
+        const int local = (int)(item - k.t.off[3][f]), ncx = (k.t.f[f].Wo + kFW - 1) / kFW;
+        const int ci = local / ncx, cx = local % ncx;
         tma::mbar_expect_tx(bar + st, (unsigned)(Q * P * kFW * 4));
-        tma::load_3d_hint(base + st * STAGE, &k.t0, cx * kFW, P * ci - P / 2, 0, bar + st, fast::l2_policy_stream());
+        tma::load_3d_hint(base + st * STAGE, &k.t0[f], cx * kFW, P * ci - P / 2, 0, bar + st, fast::l2_policy_stream());
     };
-    if (tid == 0 && (int)blockIdx.x < nitems) issue(blockIdx.x, 0);
-    float sh[Q + 3];
-#pragma unroll
-    for (int q = 0; q < Q + 3; ++q) sh[q] = a.shift[q];
+    // the map guide is the caller's, complete before stage 1 began: its first rows come ahead of
+    // the block models
+    if (tid == 0 && blockIdx.x < nitems) issue(blockIdx.x, 0);
+    pdl::wait();
     int it = 0;
-    for (int item = blockIdx.x; item < nitems; item += gridDim.x, ++it) {
+    for (unsigned item = blockIdx.x; item < nitems; item += gridDim.x, ++it) {
         const int st = it & 1;
-        if (tid == 0 && item + (int)gridDim.x < nitems) {
+        const int f = frame_of(k.t, 3, item);
+        const FastArgs &a = k.t.f[f];
+        const int ncx = (a.Wo + kFW - 1) / kFW, local = (int)(item - k.t.off[3][f]);
+        if (tid == 0 && item + gridDim.x < nitems) {
             asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
             issue(item + gridDim.x, st ^ 1);
         }
-        if (!tma::wait_warp(bar + st, (uint32_t)((it >> 1) & 1), kFastTimeoutNs) && lane == 0) {
-            s_abort = 1;
-            if (a.status) atomicExch(a.status, 1);
-        }
-        __syncthreads();
-        if (s_abort) break;
-        const float *T = base + st * STAGE;  // [Q][P][kFW]
-        const int ci = item / ncx, cx = item % ncx;
-        const int x = cx * kFW + tid;
+        const int ci = local / ncx, cx = local % ncx;
+        const int x = min(cx * kFW + tid, a.Wo - 1);
         const int ya = P * ci - P / 2;       // first output row of the cell (may be < 0)
-        if (x < a.Wo) {
-            // block rows of the cell (the same for all its rows)
-            const int yfirst = max(ya, 0);
-            const int ny0 = min(max(2 * yfirst + 1 - P, 0), (a.Hb - 1) * den);
-            const int i0 = min(ny0 / den, max(a.Hb - 2, 0)), i1 = min(i0 + 1, a.Hb - 1);
+        // block rows of the cell (the same for all its rows)
+        const int ny0 = min(max(2 * max(ya, 0) + 1 - P, 0), (a.Hb - 1) * den);
+        const int i0 = min(ny0 / den, max(a.Hb - 2, 0)), i1 = min(i0 + 1, a.Hb - 1);
+        float2 top[CS / 2], dtb[CS / 2];  // horizontally interpolated top row, bottom minus top
+        {
             // block columns and weight of this column
             const int r = (x + P / 2) / P;
             const int jl = min(max(r - 1, 0), a.Wb - 1), jr = min(max(r, 0), a.Wb - 1);
             const int nx = min(max(2 * x + 1 - P, 0), (a.Wb - 1) * den);
             const float fx = fminf(fmaxf((float)(nx - (r - 1) * den) / (float)den, 0.f), 1.f);
-            float top[NC], dtb[NC];  // horizontally interpolated top row, bottom minus top
-            {
-                const size_t t0 = (size_t)i0 * a.Wb, t1 = (size_t)i1 * a.Wb;
+            const float4 *l0 = reinterpret_cast<const float4 *>(a.coef + ((size_t)i0 * a.Wb + jl) * CS);
+            const float4 *l1 = reinterpret_cast<const float4 *>(a.coef + ((size_t)i1 * a.Wb + jl) * CS);
+            const int step = (jr - jl) * (CS / 4);
+            const float2 fx2 = make_float2(fx, fx), minus = make_float2(-1.f, -1.f);
 #pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    const float *pc = a.coef + c * bplane;
-                    const float l0 = __ldg(pc + t0 + jl), l1 = __ldg(pc + t1 + jl);
-                    const float d0 = __ldg(pc + t0 + jr) - l0, d1 = __ldg(pc + t1 + jr) - l1;
-                    top[c] = fmaf(fx, d0, l0);
-                    dtb[c] = fmaf(fx, d1, l1) - top[c];
+            for (int c = 0; c < CS / 4; ++c) {
+                const float4 tl = __ldg(l0 + c), tr = __ldg(l0 + step + c), bl = __ldg(l1 + c), br = __ldg(l1 + step + c);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float2 t0 = h ? make_float2(tl.z, tl.w) : make_float2(tl.x, tl.y);
+                    const float2 t1 = h ? make_float2(tr.z, tr.w) : make_float2(tr.x, tr.y);
+                    const float2 b0 = h ? make_float2(bl.z, bl.w) : make_float2(bl.x, bl.y);
+                    const float2 b1 = h ? make_float2(br.z, br.w) : make_float2(br.x, br.y);
+                    const float2 tp = __ffma2_rn(fx2, __ffma2_rn(t0, minus, t1), t0);
+                    top[2 * c + h] = tp;
+                    dtb[2 * c + h] = __ffma2_rn(tp, minus, __ffma2_rn(fx2, __ffma2_rn(b0, minus, b1), b0));
                 }
             }
-            for (int t = 0; t < P; ++t) {
-                const int yo = ya + t;
-                if (yo < 0 || yo >= a.Ho) continue;
-                const int ny = min(max(2 * yo + 1 - P, 0), (a.Hb - 1) * den);
-                const float fy = (float)(ny - i0 * den) / (float)den;
-                float z[Q];
+        }
+        float2 nsh[QE / 2];  // minus the frame reference, in pairs
 #pragma unroll
-                for (int i = 0; i < Q; ++i) z[i] = T[(i * P + t) * kFW + tid] - sh[i];
-                const size_t off = (size_t)yo * a.Wo + x;
+        for (int i = 0; i < QE; i += 2) nsh[i / 2] = make_float2(-a.shift[i], i + 1 < Q ? -a.shift[i + 1] : 0.f);
+        const float shr[3] = {a.shift[Q], a.shift[Q + 1], a.shift[Q + 2]};
+        if (!tma::wait_warp(bar + st, (uint32_t)((it >> 1) & 1), kFastTimeoutNs) && lane == 0) {
+            s_abort = 1;
+            if (status) atomicExch(status, 1);
+        }
+        __syncthreads();
+        if (s_abort) break;
+        const float *T = base + st * STAGE + tid;  // [Q][P][kFW]
+        if (cx * kFW + tid < a.Wo) {
+            const size_t oplane = (size_t)a.Ho * a.Wo;
+            const int t0 = max(-ya, 0), t1 = min(P, a.Ho - ya);
+            float *out = a.out + (size_t)(ya + t0) * a.Wo + x;
+#pragma unroll 2
+            for (int t = t0; t < t1; ++t, out += a.Wo) {
+                const int ny = min(max(2 * (ya + t) + 1 - P, 0), (a.Hb - 1) * den);
+                const float fy = (float)(ny - i0 * den) / (float)den;
+                const float2 fy2 = make_float2(fy, fy), one = make_float2(1.f, 1.f);
+                float2 z[QE / 2], o2[3];
+#pragma unroll
+                for (int i = 0; i < QE; i += 2)
+                    z[i / 2] = __ffma2_rn(make_float2(T[(i * P + t) * kFW], i + 1 < Q ? T[((i + 1) * P + t) * kFW] : 0.f),
+                                          one, nsh[i / 2]);
+                float bias[3] = {fmaf(fy, dtb[0].x, top[0].x), fmaf(fy, dtb[0].y, top[0].y), fmaf(fy, dtb[1].x, top[1].x)};
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    float o = fmaf(fy, dtb[c], top[c]);
+                    o2[c] = make_float2(0.f, 0.f);
 #pragma unroll
-                    for (int i = 0; i < Q; ++i) {
-                        const int kk = 3 * (i + 1) + c;
-                        o = fmaf(fmaf(fy, dtb[kk], top[kk]), z[i], o);
+                    for (int i = 0; i < QE; i += 2) {
+                        const int m = M::at(c, i) / 2;
+                        o2[c] = __ffma2_rn(__ffma2_rn(fy2, dtb[m], top[m]), z[i / 2], o2[c]);
                     }
-                    __stcs(a.out + c * oplane + off, o + sh[Q + c]);  // streamed: not kept in L2
+                    __stcs(out + c * oplane, (bias[c] + (o2[c].x + o2[c].y)) + shr[c]);  // streamed: not kept in L2
                 }
             }
         }
@@ -237,59 +311,110 @@ int fast_n_sm()
     return n;
 }
 
-template <int Q, int F>
-cudaError_t launch_moments(const FastArgs &a, cudaStream_t st)
+// Table of the frames f[0..n) with the CTAs of stages 1 to 3; stage 4's items are its launch's.
+template <int N>
+void fill_table(FrameTable<N> &t, int n, const FastArgs *f, unsigned long long *count, int *status)
 {
-    dim3 g1(fast::moment_chunks(a.Wi), a.Hb);
-    block_moments_kernel<Q, F><<<g1, 256, 0, st>>>(a);
-    return cudaGetLastError();
-}
-
-template <int Q>
-cudaError_t launch_apply_fast(const FastArgs &a, cudaStream_t st)
-{
-    const int P = a.F * a.s;
-    const bool aligned = (a.Wo & 3) == 0 && ((uintptr_t)a.map_guide & 15) == 0 && P <= 8;
-    if (aligned) {
-        FastKArgs k;
-        std::memset(&k, 0, sizeof(k));
-        k.a = a;
-        if (tma::encode_planes_f32(&k.t0, a.map_guide, a.Wo, a.Ho, Q, kFW, P, Q) == cudaSuccess) {
-            const size_t smem = apply_tma_smem<Q>();
-            cudaError_t e = cudaFuncSetAttribute(apply_tma_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            // three CTAs per SM need the whole unified L1 / shared array as shared memory
-            e = cudaFuncSetAttribute(apply_tma_kernel<Q>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxShared);
-            if (e != cudaSuccess) return e;
-            const int nitems = (a.Hb + 1) * ((a.Wo + kFW - 1) / kFW);
-            const int grid = nitems < 3 * fast_n_sm() ? nitems : 3 * fast_n_sm();  // three CTAs per SM
-            apply_tma_kernel<Q><<<grid, kFW, smem, st>>>(k);
-            return cudaGetLastError();
-        }
+    t.n = n;
+    t.count = count;
+    t.status = status;
+    for (int s = 0; s < 4; ++s) t.off[s][0] = 0;
+    for (int i = 0; i < n; ++i) {
+        t.f[i] = f[i];
+        const size_t nb = (size_t)f[i].Hb * f[i].Wb;
+        t.off[0][i + 1] = t.off[0][i] + (unsigned)f[i].Hb * fast::moment_chunks(f[i].Wi);
+        t.off[1][i + 1] = t.off[1][i] + (unsigned)((nb + kBlurThreads - 1) / kBlurThreads);
+        t.off[2][i + 1] = t.off[1][i + 1];
+        t.off[3][i + 1] = t.off[3][i];
     }
-    const size_t runs = (size_t)a.Ho * (a.Wo / (a.F * a.s) + 2);
-    fast_apply_kernel<Q><<<(unsigned)((runs + 255) / 256 < 16384 ? (runs + 255) / 256 : 16384), 256, 0, st>>>(a);
+}
+
+template <int Q, int F, int N>
+cudaError_t launch_moments(const FrameTable<N> &t, cudaStream_t st)
+{
+    constexpr size_t smem = fast::moments_smem<Q>();
+    const cudaError_t e = cudaFuncSetAttribute(block_moments_kernel<Q, F, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    block_moments_kernel<Q, F, N><<<t.off[0][t.n], fast::kMomThreads, smem, st>>>(t);
     return cudaGetLastError();
 }
 
-template <int Q>
-cudaError_t launch_fast_q(const FastArgs &a, cudaStream_t st)
+template <int Q, int N>
+cudaError_t launch_moments_f(const FrameTable<N> &t, cudaStream_t st)
 {
-    cudaError_t e;
-    switch (a.F) {
-    case 2: e = launch_moments<Q, 2>(a, st); break;
-    case 4: e = launch_moments<Q, 4>(a, st); break;
-    case 8: e = launch_moments<Q, 8>(a, st); break;
+    switch (t.f[0].F) {
+    case 2: return launch_moments<Q, 2>(t, st);
+    case 4: return launch_moments<Q, 4>(t, st);
+    case 8: return launch_moments<Q, 8>(t, st);
     default: return cudaErrorInvalidValue;
     }
+}
+
+// One thread per output-row run, any row alignment and any P: the frames of t, whose stage-4
+// items are counted here.
+template <int Q, int N>
+cudaError_t launch_apply_runs(FrameTable<N> &t, cudaStream_t st)
+{
+    for (int i = 0; i < t.n; ++i) {
+        const size_t runs = (size_t)t.f[i].Ho * (t.f[i].Wo / (t.f[i].F * t.f[i].s) + 2);
+        t.off[3][i + 1] = t.off[3][i] + (unsigned)((runs + 255) / 256);
+    }
+    const unsigned ctas = t.off[3][t.n];
+    return pdl::launch(fast_apply_kernel<Q, N>, dim3(ctas < 16384 ? ctas : 16384), 256, 0, st, t);
+}
+
+// Stage 4.  Frames whose rows start on 16-byte boundaries, with P <= 8, take the TMA kernel; the
+// others (and frames whose tensor map is refused) the one above.
+template <int Q, int N>
+cudaError_t launch_apply_fast(const FrameTable<N> &all, cudaStream_t st)
+{
+    FastKArgs<N> k;
+    FrameTable<N> rest;
+    FastArgs tma_f[N], run_f[N];
+    int nt = 0, nr = 0;
+    std::memset(&k, 0, sizeof(k));
+    for (int i = 0; i < all.n; ++i) {
+        const FastArgs &a = all.f[i];
+        const int P = a.F * a.s;
+        const bool aligned = (a.Wo & 3) == 0 && ((uintptr_t)a.map_guide & 15) == 0 && P <= 8;
+        if (aligned && tma::encode_planes_f32(&k.t0[nt], a.map_guide, a.Wo, a.Ho, Q, kFW, P, Q) == cudaSuccess)
+            tma_f[nt++] = a;
+        else
+            run_f[nr++] = a;
+    }
+    if (nt > 0) {
+        fill_table(k.t, nt, tma_f, all.count, all.status);
+        for (int i = 0; i < nt; ++i)
+            k.t.off[3][i + 1] = k.t.off[3][i] + (unsigned)((tma_f[i].Hb + 1) * ((tma_f[i].Wo + kFW - 1) / kFW));
+        const size_t smem = apply_tma_smem<Q>();
+        auto kern = tma_f[0].F * tma_f[0].s == 8 ? apply_tma_kernel<Q, N, 8> : apply_tma_kernel<Q, N, 0>;
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        // three CTAs per SM need the whole unified L1 / shared array as shared memory
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+        if (e != cudaSuccess) return e;
+        const unsigned nitems = k.t.off[3][nt], most = 3 * (unsigned)fast_n_sm();  // three CTAs per SM
+        e = pdl::launch(kern, dim3(nitems < most ? nitems : most), kFW, smem, st, k);
+        if (e != cudaSuccess || nr == 0) return e;
+    }
+    fill_table(rest, nr, run_f, all.count, all.status);
+    return launch_apply_runs<Q>(rest, st);
+}
+
+// The four stages over n frames: each launch may start while its predecessor drains (pdl.cuh),
+// which hides three launch gaps of about 2.5 us each.
+template <int Q, int N>
+cudaError_t launch_fast_q(int n, const FastArgs *f, unsigned long long *count, int *status, cudaStream_t st)
+{
+    FrameTable<N> t;
+    fill_table(t, n, f, count, status);
+    cudaError_t e = launch_moments_f<Q>(t, st);
     if (e != cudaSuccess) return e;
-    const size_t nb = (size_t)a.Hb * a.Wb;
-    blur_h_kernel<Q><<<(unsigned)((nb + 127) / 128), 128, 0, st>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    blur_v_solve_kernel<Q><<<(unsigned)((nb + 127) / 128), 128, sizeof(float) * Chan<Q>::NCH * 128, st>>>(a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    return launch_apply_fast<Q>(a, st);
+    if ((e = pdl::launch(blur_h_kernel<Q, N>, dim3(t.off[1][n]), kBlurThreads, 0, st, t)) != cudaSuccess) return e;
+    e = pdl::launch(blur_v_solve_kernel<Q, N>, dim3(t.off[2][n]), kBlurThreads,
+                    sizeof(float) * Chan<Q>::NCH * kBlurThreads, st, t);
+    if (e != cudaSuccess) return e;
+    return launch_apply_fast<Q>(t, st);
 }
 
 // Parameter gradients of one frame: the forward's moments and horizontal blur, the
@@ -298,24 +423,20 @@ cudaError_t launch_fast_q(const FastArgs &a, cudaStream_t st)
 // the dot product with grad_out into grad[t].  dout: [3][Ho][Wo] scratch; part: kDotBlocks
 // doubles.
 template <int Q>
-cudaError_t launch_param_grad_q(const FastArgs &a, float *tshift, const float *grad_out, float *dout,
-                                double *part, double *grad, cudaStream_t st)
+cudaError_t launch_param_grad_q(const FastArgs &a, unsigned long long *count, float *tshift, const float *grad_out,
+                                float *dout, double *part, double *grad, cudaStream_t st)
 {
-    cudaError_t e;
-    switch (a.F) {
-    case 2: e = launch_moments<Q, 2>(a, st); break;
-    case 4: e = launch_moments<Q, 4>(a, st); break;
-    case 8: e = launch_moments<Q, 8>(a, st); break;
-    default: return cudaErrorInvalidValue;
-    }
+    FrameTable<1> t;
+    fill_table(t, 1, &a, count, (int *)nullptr);
+    cudaError_t e = launch_moments_f<Q>(t, st);
     if (e != cudaSuccess) return e;
     const size_t nb = (size_t)a.Hb * a.Wb;
     const unsigned gb = (unsigned)((nb + 127) / 128);
-    blur_h_kernel<Q><<<gb, 128, 0, st>>>(a);
-    FastArgs ad = a;  // the horizontal blur with w' = dw/dsigma into tmp2
-    ad.tmp = a.tmp2;
-    std::memcpy(ad.w, a.wd, sizeof(ad.w));
-    blur_h_kernel<Q><<<gb, 128, 0, st>>>(ad);
+    if ((e = pdl::launch(blur_h_kernel<Q, 1>, dim3(t.off[1][1]), kBlurThreads, 0, st, t)) != cudaSuccess) return e;
+    FrameTable<1> td = t;  // the horizontal blur with w' = dw/dsigma into tmp2
+    td.f[0].tmp = a.tmp2;
+    std::memcpy(td.f[0].w, a.wd, sizeof(a.wd));
+    if ((e = pdl::launch(blur_h_kernel<Q, 1>, dim3(t.off[1][1]), kBlurThreads, 0, st, td)) != cudaSuccess) return e;
     const size_t smem = sizeof(float) * 2 * Chan<Q>::NCH * 128;
     static bool attr_set = false;
     if (!attr_set) {
@@ -330,48 +451,59 @@ cudaError_t launch_param_grad_q(const FastArgs &a, float *tshift, const float *g
     // output carries no constant
     if ((e = cudaMemcpyAsync(tshift, a.shift, sizeof(float) * Q, cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(tshift + Q, 0, sizeof(float) * 3, st)) != cudaSuccess) return e;
-    const size_t runs = (size_t)a.Ho * (a.Wo / (a.F * a.s) + 2);
     const size_t npx = 3 * (size_t)a.Ho * a.Wo;
-    for (int t = 0; t < 3; ++t) {
-        FastArgs at = a;
-        at.coef = a.dcoef + (size_t)t * 3 * (Q + 1) * nb;
-        at.shift = tshift;
-        at.out = dout;
-        fast_apply_kernel<Q><<<(unsigned)((runs + 255) / 256 < 16384 ? (runs + 255) / 256 : 16384), 256, 0, st>>>(at);
+    for (int p = 0; p < 3; ++p) {
+        FrameTable<1> tp = t;
+        tp.f[0].coef = a.dcoef + (size_t)p * nb * fast::Model<Q>::CS;
+        tp.f[0].shift = tshift;
+        tp.f[0].out = dout;
+        if ((e = launch_apply_runs<Q>(tp, st)) != cudaSuccess) return e;
         dot_partial_kernel<<<kDotBlocks, 256, 0, st>>>(dout, grad_out, npx, part);
-        dot_final_kernel<<<1, kDotBlocks, 0, st>>>(part, grad + t);
+        dot_final_kernel<<<1, kDotBlocks, 0, st>>>(part, grad + p);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
-cudaError_t launch_param_grad(int q, const FastArgs &a, float *tshift, const float *grad_out, float *dout,
-                              double *part, double *grad, cudaStream_t st)
+cudaError_t launch_param_grad(int q, const FastArgs &a, unsigned long long *count, float *tshift, const float *grad_out,
+                              float *dout, double *part, double *grad, cudaStream_t st)
 {
     switch (q) {
-    case 1: return launch_param_grad_q<1>(a, tshift, grad_out, dout, part, grad, st);
-    case 2: return launch_param_grad_q<2>(a, tshift, grad_out, dout, part, grad, st);
-    case 3: return launch_param_grad_q<3>(a, tshift, grad_out, dout, part, grad, st);
-    case 4: return launch_param_grad_q<4>(a, tshift, grad_out, dout, part, grad, st);
-    case 5: return launch_param_grad_q<5>(a, tshift, grad_out, dout, part, grad, st);
-    case 6: return launch_param_grad_q<6>(a, tshift, grad_out, dout, part, grad, st);
-    case 7: return launch_param_grad_q<7>(a, tshift, grad_out, dout, part, grad, st);
-    case 8: return launch_param_grad_q<8>(a, tshift, grad_out, dout, part, grad, st);
+    case 1: return launch_param_grad_q<1>(a, count, tshift, grad_out, dout, part, grad, st);
+    case 2: return launch_param_grad_q<2>(a, count, tshift, grad_out, dout, part, grad, st);
+    case 3: return launch_param_grad_q<3>(a, count, tshift, grad_out, dout, part, grad, st);
+    case 4: return launch_param_grad_q<4>(a, count, tshift, grad_out, dout, part, grad, st);
+    case 5: return launch_param_grad_q<5>(a, count, tshift, grad_out, dout, part, grad, st);
+    case 6: return launch_param_grad_q<6>(a, count, tshift, grad_out, dout, part, grad, st);
+    case 7: return launch_param_grad_q<7>(a, count, tshift, grad_out, dout, part, grad, st);
+    case 8: return launch_param_grad_q<8>(a, count, tshift, grad_out, dout, part, grad, st);
     default: return cudaErrorInvalidValue;
     }
 }
 
-cudaError_t launch_fast(int q, const FastArgs &a, cudaStream_t st)
+cudaError_t launch_fast(int q, const FastArgs &a, unsigned long long *count, cudaStream_t st)
 {
     switch (q) {
-    case 1: return launch_fast_q<1>(a, st);
-    case 2: return launch_fast_q<2>(a, st);
-    case 3: return launch_fast_q<3>(a, st);
-    case 4: return launch_fast_q<4>(a, st);
-    case 5: return launch_fast_q<5>(a, st);
-    case 6: return launch_fast_q<6>(a, st);
-    case 7: return launch_fast_q<7>(a, st);
-    case 8: return launch_fast_q<8>(a, st);
+    case 1: return launch_fast_q<1, 1>(1, &a, count, nullptr, st);
+    case 2: return launch_fast_q<2, 1>(1, &a, count, nullptr, st);
+    case 3: return launch_fast_q<3, 1>(1, &a, count, nullptr, st);
+    case 4: return launch_fast_q<4, 1>(1, &a, count, nullptr, st);
+    case 5: return launch_fast_q<5, 1>(1, &a, count, nullptr, st);
+    case 6: return launch_fast_q<6, 1>(1, &a, count, nullptr, st);
+    case 7: return launch_fast_q<7, 1>(1, &a, count, nullptr, st);
+    case 8: return launch_fast_q<8, 1>(1, &a, count, nullptr, st);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+bool batch_supported(int q, int F) { return (q == 1 || q == 4 || q == 8) && (F == 2 || F == 4 || F == 8); }
+
+cudaError_t launch_fast_batch(int q, int n, const FastArgs *f, unsigned long long *count, int *status, cudaStream_t st)
+{
+    switch (q) {
+    case 1: return launch_fast_q<1, FLR_MAX_BATCH>(n, f, count, status, st);
+    case 4: return launch_fast_q<4, FLR_MAX_BATCH>(n, f, count, status, st);
+    case 8: return launch_fast_q<8, FLR_MAX_BATCH>(n, f, count, status, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -422,15 +554,23 @@ struct flr_fast_handle {
     float *gws = nullptr;
     size_t gws_floats = 0;
     double *gpart = nullptr;
-    // batch path: per-frame workspace, barrier words, status word
+    // batch path: per-frame workspace, status word
     float *bws = nullptr;
     size_t bws_floats = 0;
-    unsigned *bar = nullptr;  // [0] count, [1] generation, [2] status
+    int *bstatus = nullptr;
 };
 
 namespace {
 
-size_t block_floats(int q) { return 2 * (size_t)(q + 3 + q * (q + 1) / 2 + 3 * q) + (size_t)(q + 3) + 1 + 3 * (size_t)(q + 1); }
+int n_channels(int q) { return q + 3 + q * (q + 1) / 2 + 3 * q; }
+
+// Workspace of a frame of nb blocks: block sums and references, blurred sums and count, models
+// (16-byte aligned: up to 3 floats more)
+size_t frame_floats(int q, size_t nb)
+{
+    return nb * (2 * (size_t)n_channels(q) + (size_t)(q + 3) + 1 + flr::fast::model_floats(q)) + 4;
+}
+float *align16(float *p) { return (float *)(((uintptr_t)p + 15) & ~(uintptr_t)15); }
 
 // Fill one frame's arguments; ws points at its per-block workspace.
 void frame_args(const flr_fast_handle *h, const flr_frame &fr, float *ws, flr::fast::FastArgs &a)
@@ -438,14 +578,14 @@ void frame_args(const flr_fast_handle *h, const flr_frame &fr, float *ws, flr::f
     const int q = h->p.q, F = h->p.factor, s = h->p.scale;
     const int Hb = (fr.H + F - 1) / F, Wb = (fr.W + F - 1) / F;
     const size_t nb = (size_t)Hb * Wb;
-    const int nch = q + 3 + q * (q + 1) / 2 + 3 * q;
+    const int nch = n_channels(q);
     a.guide = fr.guide;
     a.rad = fr.radiance;
     a.map_guide = fr.map_guide ? fr.map_guide : fr.guide;
     a.out = fr.out;
     a.blk = ws;
     a.tmp = ws + nb * (nch + q + 3);
-    a.coef = a.tmp + nb * (nch + 1);
+    a.coef = align16(a.tmp + nb * (nch + 1));
     a.shift = h->shift;  // replaced per frame by the caller
     a.flag_count = h->count;
     a.Hi = fr.H;
@@ -477,7 +617,7 @@ int check_frames(const flr_fast_handle *h, int n, const flr_frame *frames, size_
         if (((uintptr_t)f.guide | (uintptr_t)f.radiance | (uintptr_t)f.out | (uintptr_t)f.map_guide) & 15u)
             return FLR_ERR_ALIGN;
         const size_t nb = (size_t)((f.H + h->p.factor - 1) / h->p.factor) * ((f.W + h->p.factor - 1) / h->p.factor);
-        total += nb * block_floats(h->p.q) + 64;  // + room for the frame's reference shift
+        total += frame_floats(h->p.q, nb) + 64;  // + room for the frame's reference shift
     }
     *floats = total;
     return FLR_OK;
@@ -524,7 +664,7 @@ int flr_fast_destroy(flr_fast_handle *h)
     cudaFree(h->gws);
     cudaFree(h->gpart);
     cudaFree(h->bws);
-    cudaFree(h->bar);
+    cudaFree(h->bstatus);
     cudaFree(h->shift);
     cudaFree(h->count);
     cudaFree(h->status);
@@ -542,12 +682,12 @@ int flr_fast_denoise(flr_fast_handle *h, const float *guide, const float *map_gu
     if (((uintptr_t)guide | (uintptr_t)radiance | (uintptr_t)out | (uintptr_t)map_guide) & 15u) return FLR_ERR_ALIGN;
     const int Hb = (Hi + F - 1) / F, Wb = (Wi + F - 1) / F;
     const size_t nb = (size_t)Hb * Wb;
-    const int nch = q + 3 + q * (q + 1) / 2 + 3 * q;
+    const int nch = n_channels(q);
     if (h->ws_blocks < nb || !h->ws) {
         cudaFree(h->ws);
         h->ws = nullptr;
         h->ws_blocks = 0;
-        if (cudaMalloc(&h->ws, nb * sizeof(float) * (2 * (size_t)nch + (size_t)(q + 3) + 1 + 3 * (size_t)(q + 1))) != cudaSuccess)
+        if (cudaMalloc(&h->ws, sizeof(float) * frame_floats(q, nb)) != cudaSuccess)
             return FLR_ERR_NOMEM;
         h->ws_blocks = nb;
     }
@@ -558,7 +698,7 @@ int flr_fast_denoise(flr_fast_handle *h, const float *guide, const float *map_gu
     a.out = out;
     a.blk = h->ws;
     a.tmp = h->ws + nb * (nch + q + 3);
-    a.coef = a.tmp + nb * (nch + 1);
+    a.coef = align16(a.tmp + nb * (nch + 1));
     a.shift = h->shift;
     a.flag_count = h->count;
     a.Hi = Hi;
@@ -578,8 +718,7 @@ int flr_fast_denoise(flr_fast_handle *h, const float *guide, const float *map_gu
     std::memcpy(a.w, h->w, sizeof(a.w));
     cudaStream_t st = (cudaStream_t)stream;
     h->last_stream = st;
-    cudaError_t e = cudaMemsetAsync(h->count, 0, sizeof(unsigned long long), st);
-    if (e == cudaSuccess) e = flr::launch_fast(q, a, st);
+    const cudaError_t e = flr::launch_fast(q, a, h->count, st);
     if (e != cudaSuccess) {
         std::snprintf(flr::g_fast_err, sizeof(flr::g_fast_err), "%s", cudaGetErrorString(e));
         return FLR_ERR_CUDA;
@@ -592,7 +731,7 @@ int flr_fast_reserve_batch(flr_fast_handle *h, int n, const flr_frame *frames)
     size_t floats = 0;
     int st = check_frames(h, n, frames, &floats);
     if (st != FLR_OK) return st;
-    if (!h->bar && cudaMalloc(&h->bar, 4 * sizeof(unsigned)) != cudaSuccess) return FLR_ERR_NOMEM;
+    if (!h->bstatus && cudaMalloc(&h->bstatus, sizeof(int)) != cudaSuccess) return FLR_ERR_NOMEM;
     if (h->bws_floats < floats || !h->bws) {
         cudaFree(h->bws);
         h->bws = nullptr;
@@ -608,7 +747,7 @@ int flr_fast_denoise_batch(flr_fast_handle *h, int n, const flr_frame *frames, v
     size_t floats = 0;
     int st = check_frames(h, n, frames, &floats);
     if (st != FLR_OK) return st;
-    if (h->bws_floats < floats || !h->bar) {
+    if (h->bws_floats < floats || !h->bstatus) {
         st = flr_fast_reserve_batch(h, n, frames);
         if (st != FLR_OK) return st;
     }
@@ -617,16 +756,13 @@ int flr_fast_denoise_batch(flr_fast_handle *h, int n, const flr_frame *frames, v
     for (int i = 0; i < n; ++i) {
         frame_args(h, frames[i], ws + 64, fa[i]);
         fa[i].shift = ws;  // this frame's reference shift
+        fa[i].status = h->bstatus;
         const size_t nb = (size_t)fa[i].Hb * fa[i].Wb;
-        ws += nb * block_floats(h->p.q) + 64;
+        ws += frame_floats(h->p.q, nb) + 64;
     }
-    std::vector<unsigned char> args(flr::batch_args_size());
-    flr::fill_batch_args(args.data(), n, fa, h->bar, h->bar + 1, (int *)(h->bar + 2));
     cudaStream_t s = (cudaStream_t)stream;
     h->last_stream = s;
-    cudaError_t e = cudaMemsetAsync(h->count, 0, sizeof(unsigned long long), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->bar, 0, 3 * sizeof(unsigned), s);
-    if (e == cudaSuccess) e = flr::launch_batch(h->p.q, h->p.factor, args.data(), s);
+    const cudaError_t e = flr::launch_fast_batch(h->p.q, n, fa, h->count, h->bstatus, s);
     if (e != cudaSuccess) {
         std::snprintf(flr::g_fast_err, sizeof(flr::g_fast_err), "%s", cudaGetErrorString(e));
         return FLR_ERR_CUDA;
@@ -636,10 +772,10 @@ int flr_fast_denoise_batch(flr_fast_handle *h, int n, const flr_frame *frames, v
 
 int flr_fast_batch_status(flr_fast_handle *h)
 {
-    if (!h || !h->bar) return FLR_ERR_ARG;
+    if (!h || !h->bstatus) return FLR_ERR_ARG;
     int status = 0;
     if (cudaStreamSynchronize(h->last_stream) != cudaSuccess ||
-        cudaMemcpy(&status, h->bar + 2, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+        cudaMemcpy(&status, h->bstatus, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
         return FLR_ERR_CUDA;
     return status == 0 ? FLR_OK : FLR_ERR_TIMEOUT;
 }
@@ -685,17 +821,17 @@ int flr_fast_param_grad(flr_fast_handle *h, const float *guide, const float *map
         return FLR_ERR_ALIGN;
     const int Hb = (Hi + F - 1) / F, Wb = (Wi + F - 1) / F;
     const size_t nb = (size_t)Hb * Wb, npx = (size_t)Hi * s * Wi * s;
-    const int nch = q + 3 + q * (q + 1) / 2 + 3 * q;
+    const int nch = n_channels(q);
     if (h->ws_blocks < nb || !h->ws) {
         cudaFree(h->ws);
         h->ws = nullptr;
         h->ws_blocks = 0;
-        if (cudaMalloc(&h->ws, nb * sizeof(float) * (2 * (size_t)nch + (size_t)(q + 3) + 1 + 3 * (size_t)(q + 1))) != cudaSuccess)
+        if (cudaMalloc(&h->ws, sizeof(float) * frame_floats(q, nb)) != cudaSuccess)
             return FLR_ERR_NOMEM;
         h->ws_blocks = nb;
     }
     // gradient workspace: tmp2, dcoef, tshift (32 floats), dout
-    const size_t off_dc = (size_t)(nch + 1) * nb, off_ts = off_dc + 9 * (size_t)(q + 1) * nb;
+    const size_t off_dc = ((size_t)(nch + 1) * nb + 3) & ~(size_t)3, off_ts = off_dc + 3 * (size_t)flr::fast::model_floats(q) * nb;
     const size_t off_out = (off_ts + 32 + 3) & ~(size_t)3, need = off_out + 3 * npx;
     if (h->gws_floats < need || !h->gws) {
         cudaFree(h->gws);
@@ -713,7 +849,7 @@ int flr_fast_param_grad(flr_fast_handle *h, const float *guide, const float *map
     a.out = nullptr;
     a.blk = h->ws;
     a.tmp = h->ws + nb * (nch + q + 3);
-    a.coef = a.tmp + nb * (nch + 1);
+    a.coef = align16(a.tmp + nb * (nch + 1));
     a.tmp2 = h->gws;
     a.dcoef = h->gws + off_dc;
     a.shift = h->shift;
@@ -736,9 +872,8 @@ int flr_fast_param_grad(flr_fast_handle *h, const float *guide, const float *map
     std::memcpy(a.wd, h->wd, sizeof(a.wd));
     cudaStream_t st = (cudaStream_t)stream;
     h->last_stream = st;
-    cudaError_t e = cudaMemsetAsync(h->count, 0, sizeof(unsigned long long), st);
-    if (e == cudaSuccess)
-        e = flr::launch_param_grad(q, a, h->gws + off_ts, grad_out, h->gws + off_out, h->gpart, grad, st);
+    const cudaError_t e =
+        flr::launch_param_grad(q, a, h->count, h->gws + off_ts, grad_out, h->gws + off_out, h->gpart, grad, st);
     if (e != cudaSuccess) {
         std::snprintf(flr::g_fast_err, sizeof(flr::g_fast_err), "%s", cudaGetErrorString(e));
         return FLR_ERR_CUDA;

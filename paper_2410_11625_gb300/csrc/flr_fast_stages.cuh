@@ -1,6 +1,5 @@
 // flr_fast_stages.cuh -- the four stages of the paper's fast FLR (Sec. 3.2, 3.2.1) as device
-// functions, shared by the one-kernel-per-stage path (flr_fast.cu) and the persistent
-// batched kernel (flr_batch.cu).
+// functions (flr_fast.cu has the kernels).
 #pragma once
 
 #include <utility>
@@ -45,24 +44,34 @@ __device__ __forceinline__ uint64_t l2_policy_stream()
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;\n" : "=l"(p));
     return p;
 }
-// 8-byte read-only load with an L2 eviction policy
-__device__ __forceinline__ float2 ld_f2_hint(const float *p, uint64_t pol)
+// Asynchronous 8- and 4-byte copies into shared memory, with an L2 eviction policy
+__device__ __forceinline__ void copy8_hint(uint32_t dst, const float *src, uint64_t pol)
 {
-    float2 v;
-    asm volatile("ld.global.nc.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;\n"
-                 : "=f"(v.x), "=f"(v.y)
-                 : "l"(p), "l"(pol));
-    return v;
+    asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], 8, %2;\n" ::"r"(dst), "l"(src), "l"(pol) : "memory");
 }
+__device__ __forceinline__ void copy4_hint(uint32_t dst, const float *src, uint64_t pol)
+{
+    asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], 4, %2;\n" ::"r"(dst), "l"(src), "l"(pol) : "memory");
+}
+
+// A block's model in memory: 16-byte aligned [biases of the 3 colours, 0][colour][QE], QE guide
+// coefficients rounded up to an even count (the last one 0 for odd Q), so that the apply reads a
+// corner with vector loads and works on pairs of guides.
+template <int Q>
+struct Model {
+    static constexpr int QE = (Q + 1) / 2 * 2, CS = (4 + 3 * QE + 3) / 4 * 4;
+    __host__ __device__ static constexpr int at(int c, int i) { return 4 + c * QE + i; }
+};
+__host__ __device__ constexpr int model_floats(int q) { return (4 + 3 * ((q + 1) / 2 * 2) + 3) / 4 * 4; }
 
 struct FastArgs {
     const float *guide, *rad, *map_guide;  // model inputs [q|3][Hi][Wi], map guide [q][Ho][Wo]
     float *out;                            // [3][Ho][Wo]
     float *blk;   // [NCH + Q+3][Hb][Wb]: block sums relative to the block's reference, then that reference
     float *tmp;   // [NCH + 1][Hb][Wb]: horizontally blurred sums (same reference), weighted count
-    float *coef;  // [(Q+1)*3][Hb][Wb]: block models relative to the frame reference
+    float *coef;  // [Hb][Wb] block models (struct Model) relative to the frame reference
     float *tmp2;  // parameter gradients: [NCH + 1][Hb][Wb] horizontal blur with the weights' sigma-derivative
-    float *dcoef; // parameter gradients: [3][(Q+1)*3][Hb][Wb] model tangents (sigma, eps, eps_mul)
+    float *dcoef; // parameter gradients: [3][Hb][Wb] model tangents (sigma, eps, eps_mul)
     float *shift;                          // frame reference shift, Q + 3 floats
     unsigned long long *flag_count;
     int Hi, Wi, Ho, Wo, Hb, Wb, F, s, taps;
@@ -74,17 +83,93 @@ struct FastArgs {
     int *status = nullptr;                 // set to 1 if a bounded device wait ran out (may be NULL)
 };
 
+// Sums over the LPB lanes of a block, O = 1, 2, .. LPB / 2 apart, by halving: in each step a lane
+// sends the half of its channels that its partner keeps, so NCH channels take about NCH shuffles
+// instead of NCH log2(LPB), and every lane stores its own share of the channels.  The sums are
+// those of a butterfly, bit for bit.  cnt of a's N channels, from ch0 on, exist.
+template <int N, int O, int LPB>
+__device__ __forceinline__ void fold_store(const float (&a)[N], int lane, int ch0, int cnt, float *dst, size_t bplane)
+{
+    if constexpr (O == LPB) {
+        float *p = dst + ch0 * bplane;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            if (i < cnt) *p = a[i];
+            p += bplane;
+        }
+    } else {
+        constexpr int H = (N + 1) / 2;
+        const bool up = (lane & O) != 0;
+        float b[H];
+#pragma unroll
+        for (int i = 0; i < H; ++i) {
+            const float hi = i + H < N ? a[i + H < N ? i + H : 0] : 0.f;
+            b[i] = (up ? hi : a[i]) + __shfl_xor_sync(0xffffffffu, up ? a[i] : hi, O);
+        }
+        fold_store<H, 2 * O, LPB>(b, lane, up ? ch0 + H : ch0, up ? cnt - H : (cnt < H ? cnt : H), dst, bplane);
+    }
+}
+
 // 1. block moments.  Block (i, j) covers input rows [iF, iF+F) and columns [jF, jF+F).
-// Work item (by, cx): block row by, input columns [512 cx, 512 cx + 512); 256 threads, each
-// summing two adjacent columns over the F rows (one 8-byte load per plane and row when the
-// rows are 8-byte aligned), then a shuffle tree over the F / 2 lanes of a block.
+// Work item (by, cx): block row by, input columns [256 cx, 256 cx + 256); 128 threads, each
+// summing two adjacent columns over the F rows, then fold_store over the F / 2 lanes of a block.
+// The rows come through a ring of kMomStages asynchronous copies that each thread keeps for
+// itself, without any barrier: a warp's 71 accumulators leave room for 16 warps per SM, too few to
+// cover DRAM latency with loads into registers, where a row waits out its load (long_scoreboard
+// 4.6 of 8.7 stall cycles per issue; 26.5 us at 1920x1080 against 21 us so).  One row's products are
+// the loop body: the rows unrolled are 20 KB of instructions that every warp fetches once.
+// Measured besides: the two columns' products as packed pairs (142 accumulators, 8 warps per SM)
+// 22 us; persistent CTAs whose ring runs on from item to item 33 us; 4 stages 21 us (but 74 against
+// 72 us for the whole 1280x720 -> 2560x1440 frame); 256 threads 22 us.
+constexpr int kMomThreads = 128, kMomStages = 2;
+template <int Q>
+constexpr size_t moments_smem()
+{
+    return sizeof(float) * kMomStages * (Q + 3) * 2 * kMomThreads;
+}
+
 template <int Q, int F>
-__device__ __forceinline__ void stage_moments(const FastArgs &a, int by, int cx)
+__device__ __forceinline__ void stage_moments(const FastArgs &a, int by, int cx, float *ring)
 {
     using C = Chan<Q>;
     constexpr int NS = Q + 3, LPB = F / 2;  // lanes per block
+    constexpr int D = F < kMomStages ? F : kMomStages;
     static_assert(F >= 2 && 32 % F == 0, "block width");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int x = cx * 2 * kMomThreads + 2 * tid;  // this thread's columns x, x + 1
+    const size_t plane = (size_t)a.Hi * a.Wi;
+    const int y0 = by * F, rows = min(F, a.Hi - y0);
+    // with an even width, x + 1 < Wi and the 8-byte copies are aligned (x even, planes 16-byte
+    // aligned)
+    const bool in = x < a.Wi, vec = (a.Wi & 1) == 0, two = x + 1 < a.Wi;
+    const uint64_t pol_keep = l2_policy_keep(), pol_stream = l2_policy_stream();
+    float2 *mine = reinterpret_cast<float2 *>(ring) + tid;  // [stage][slot][thread]
+    auto issue = [&](int row) {
+        if (row < rows && in) {
+            uint32_t dst = (uint32_t)__cvta_generic_to_shared(mine + (row % D) * NS * kMomThreads);
+            const float *pg = a.guide + (size_t)(y0 + row) * a.Wi + x, *pr = a.rad + (size_t)(y0 + row) * a.Wi + x;
+            if (vec) {
+#pragma unroll
+                for (int k = 0; k < Q; ++k, dst += 8 * kMomThreads, pg += plane) copy8_hint(dst, pg, pol_keep);
+#pragma unroll
+                for (int c = 0; c < 3; ++c, dst += 8 * kMomThreads, pr += plane) copy8_hint(dst, pr, pol_stream);
+            } else {
+#pragma unroll
+                for (int k = 0; k < Q; ++k, dst += 8 * kMomThreads, pg += plane) {
+                    copy4_hint(dst, pg, pol_keep);
+                    if (two) copy4_hint(dst + 4, pg + 1, pol_keep);
+                }
+#pragma unroll
+                for (int c = 0; c < 3; ++c, dst += 8 * kMomThreads, pr += plane) {
+                    copy4_hint(dst, pr, pol_stream);
+                    if (two) copy4_hint(dst + 4, pr + 1, pol_stream);
+                }
+            }
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+#pragma unroll
+    for (int row = 0; row < D; ++row) issue(row);
     if (by == 0 && cx == 0 && warp == 0) {
         // the frame reference the models are expressed in (used by the solve and apply)
         __shared__ float s_ref[NS];
@@ -92,77 +177,42 @@ __device__ __forceinline__ void stage_moments(const FastArgs &a, int by, int cx)
         __syncwarp();
         if (lane < NS) a.shift[lane] = s_ref[lane];
     }
-    const int x = cx * 512 + 2 * tid;  // this thread's columns x, x + 1
-    const size_t plane = (size_t)a.Hi * a.Wi;
-    const int y0 = by * F, y1 = min(y0 + F, a.Hi);
     // the block's reference: its top-left input pixel (column x of lane (lane & ~(LPB-1)))
-    float ref[NS];
-    {
-        const size_t off0 = (size_t)y0 * a.Wi + min(x, a.Wi - 1);
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(D - 1) : "memory");
+    float ref[NS], acc[C::NCH];
 #pragma unroll
-        for (int k = 0; k < Q; ++k) ref[k] = __ldg(a.guide + k * plane + off0);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) ref[Q + c] = __ldg(a.rad + c * plane + off0);
-#pragma unroll
-        for (int k = 0; k < NS; ++k) ref[k] = __shfl_sync(0xffffffffu, ref[k], lane & ~(LPB - 1));
-    }
-    float acc[C::NCH];
+    for (int k = 0; k < NS; ++k) ref[k] = __shfl_sync(0xffffffffu, mine[k * kMomThreads].x, lane & ~(LPB - 1));
 #pragma unroll
     for (int c = 0; c < C::NCH; ++c) acc[c] = 0.f;
-    if (x < a.Wi) {
-        // with an even width, x + 1 < Wi and the 8-byte loads are aligned (x even, planes
-        // 16-byte aligned)
-        const bool vec = (a.Wi & 1) == 0;
-        const bool two = x + 1 < a.Wi;
-        const uint64_t pol_keep = l2_policy_keep(), pol_stream = l2_policy_stream();
+#pragma unroll 1
+    for (int row = 0; row < rows; ++row) {
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(D - 1) : "memory");
+        const float2 *src = mine + (row % D) * NS * kMomThreads;
+        float v0[NS], v1[NS];
 #pragma unroll
-        for (int yy = 0; yy < F; ++yy) {
-            const int y = y0 + yy;
-            if (y >= y1) break;
-            const size_t off = (size_t)y * a.Wi + x;
-            float v0[NS], v1[NS];
-            if (vec) {
-#pragma unroll
-                for (int k = 0; k < Q; ++k) {
-                    const float2 g = ld_f2_hint(a.guide + k * plane + off, pol_keep);
-                    v0[k] = g.x - ref[k];
-                    v1[k] = g.y - ref[k];
-                }
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const float2 g = ld_f2_hint(a.rad + c * plane + off, pol_stream);
-                    v0[Q + c] = g.x - ref[Q + c];
-                    v1[Q + c] = g.y - ref[Q + c];
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < Q; ++k) {
-                    v0[k] = __ldg(a.guide + k * plane + off) - ref[k];
-                    v1[k] = two ? __ldg(a.guide + k * plane + off + 1) - ref[k] : 0.f;
-                }
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    v0[Q + c] = __ldg(a.rad + c * plane + off) - ref[Q + c];
-                    v1[Q + c] = two ? __ldg(a.rad + c * plane + off + 1) - ref[Q + c] : 0.f;
-                }
-            }
-            moments_all<Q>(acc, v0, std::make_integer_sequence<int, C::NCH>{});
-            moments_all<Q>(acc, v1, std::make_integer_sequence<int, C::NCH>{});
+        for (int k = 0; k < NS; ++k) {
+            const float2 g = src[k * kMomThreads];
+            v0[k] = g.x - ref[k];
+            v1[k] = two ? g.y - ref[k] : 0.f;
         }
+        issue(row + D);
+        moments_all<Q>(acc, v0, std::make_integer_sequence<int, C::NCH>{});
+        moments_all<Q>(acc, v1, std::make_integer_sequence<int, C::NCH>{});
     }
-    // reduce over the LPB lanes of each block (blocks never straddle a warp: 32 % LPB == 0)
+    if (!in) {  // columns past the image: lanes of a block that starts inside it add nothing
 #pragma unroll
-    for (int ch = 0; ch < C::NCH; ++ch)
+        for (int c = 0; c < C::NCH; ++c) acc[c] = 0.f;
+    }
+    // blocks never straddle a warp (32 % LPB == 0); a block's first column is that of its first lane
+    const int sub = lane & (LPB - 1), bx = (x - 2 * sub) / F;
+    const bool block_in = x - 2 * sub < a.Wi;
+    const size_t bplane = (size_t)a.Hb * a.Wb;
+    float *dst = a.blk + (size_t)by * a.Wb + bx;
+    fold_store<C::NCH, 1, LPB>(acc, lane, 0, block_in ? C::NCH : 0, dst, bplane);
+    if (block_in) {
 #pragma unroll
-        for (int o = 1; o < LPB; o <<= 1) acc[ch] += __shfl_xor_sync(0xffffffffu, acc[ch], o);
-    if ((lane & (LPB - 1)) == 0 && x < a.Wi) {
-        const int bx = x / F;
-        const size_t bplane = (size_t)a.Hb * a.Wb;
-        const size_t boff = (size_t)by * a.Wb + bx;
-#pragma unroll
-        for (int ch = 0; ch < C::NCH; ++ch) a.blk[ch * bplane + boff] = acc[ch];
-#pragma unroll
-        for (int k = 0; k < NS; ++k) a.blk[(C::NCH + k) * bplane + boff] = ref[k];
+        for (int k = 0; k < NS; ++k)
+            if ((k & (LPB - 1)) == sub) dst[(C::NCH + k) * bplane] = ref[k];
     }
 }
 
@@ -171,33 +221,35 @@ __device__ __forceinline__ float block_len(int b, int F, int n) { return (float)
 
 // acc += w * (sums of block b re-expressed relative to another reference), given
 // d = ref_b - ref_target for the Q + 3 input slots and the block's pixel count nb:
-//   sum (v + d) = L + nb d,   sum (v + d)(v' + d') = S + L d' + d L' + nb d d'.
+//   G = sum (v + d) = L + nb d,   sum (v + d)(v' + d') = S + L' d + G d'.
+// p: channel 0 of the block; the other channels follow stride apart, read in order.
 template <int Q>
-__device__ __forceinline__ void accumulate_shifted(float (&acc)[Chan<Q>::NCH], const float *src, size_t stride,
+__device__ __forceinline__ void accumulate_shifted(float (&acc)[Chan<Q>::NCH], const float *p, size_t stride,
                                                    const float (&d)[Q + 3], float nb, float w)
 {
     using C = Chan<Q>;
-    float L[Q + 3];
+    static_assert(C::X0 == 0 && C::XX0 == Q + 3 && C::XY0 == C::XX0 + C::NXX, "channels in order");
+    float L[Q + 3], G[Q + 3];
 #pragma unroll
-    for (int k = 0; k < Q + 3; ++k) L[k] = src[(C::X0 + k) * stride];  // X0..Y0+2 are the linear sums
+    for (int k = 0; k < Q + 3; ++k, p += stride) L[k] = *p;  // X0..Y0+2 are the linear sums
 #pragma unroll
-    for (int k = 0; k < Q + 3; ++k) acc[C::X0 + k] = fmaf(w, fmaf(nb, d[k], L[k]), acc[C::X0 + k]);
-#pragma unroll
-    for (int i = 0; i < Q; ++i)
-#pragma unroll
-        for (int j = 0; j < Q; ++j)
-            if (j >= i) {
-                const int ch = C::xx(i, j);
-                const float t = fmaf(nb * d[i], d[j], fmaf(L[i], d[j], fmaf(d[i], L[j], src[ch * stride])));
-                acc[ch] = fmaf(w, t, acc[ch]);
-            }
+    for (int k = 0; k < Q + 3; ++k) {
+        G[k] = fmaf(nb, d[k], L[k]);
+        acc[C::X0 + k] = fmaf(w, G[k], acc[C::X0 + k]);
+    }
 #pragma unroll
     for (int i = 0; i < Q; ++i)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
+        for (int j = i; j < Q; ++j, p += stride) {
+            const int ch = C::xx(i, j);
+            acc[ch] = fmaf(w, fmaf(G[i], d[j], fmaf(d[i], L[j], *p)), acc[ch]);
+        }
+#pragma unroll
+    for (int i = 0; i < Q; ++i)
+#pragma unroll
+        for (int c = 0; c < 3; ++c, p += stride) {
             const int ch = C::xy(i, c);
-            const float t = fmaf(nb * d[i], d[Q + c], fmaf(L[i], d[Q + c], fmaf(d[i], L[Q + c], src[ch * stride])));
-            acc[ch] = fmaf(w, t, acc[ch]);
+            acc[ch] = fmaf(w, fmaf(G[i], d[Q + c], fmaf(d[i], L[Q + c], *p)), acc[ch]);
         }
 }
 
@@ -289,6 +341,23 @@ __device__ __forceinline__ bool solve_appendix(const float *Sp, int VS, float n,
         bv[c] = b;
     }
     return low;
+}
+
+template <int Q>
+__device__ __forceinline__ void store_model(float *dst, const float (&A)[Q][3], const float (&b)[3])
+{
+    using M = Model<Q>;
+    float m[M::CS];
+#pragma unroll
+    for (int k = 0; k < M::CS; ++k) m[k] = 0.f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        m[c] = b[c];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) m[M::at(c, i)] = A[i][c];
+    }
+#pragma unroll
+    for (int k = 0; k < M::CS; k += 4) *reinterpret_cast<float4 *>(dst + k) = make_float4(m[k], m[k + 1], m[k + 2], m[k + 3]);
 }
 
 // 3. vertical Gaussian + per-block solve; S: this thread's column of a [NCH][stride] buffer
@@ -405,16 +474,10 @@ __device__ __forceinline__ void stage_blur_v_solve(const FastArgs &a, size_t k, 
     // the model was fitted relative to this block's reference; re-express the bias
     // relative to the frame reference the apply step uses
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        float bb = bv[c] + (rk[Q + c] - a.shift[Q + c]);
+    for (int c = 0; c < 3; ++c)
 #pragma unroll
-        for (int i = 0; i < Q; ++i) bb = fmaf(-A[i][c], rk[i] - a.shift[i], bb);
-        a.coef[c * bplane + k] = bb;
-    }
-#pragma unroll
-    for (int i = 0; i < Q; ++i)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) a.coef[(3 * (i + 1) + c) * bplane + k] = A[i][c];
+        for (int i = 0; i < Q; ++i) bv[c] = fmaf(-A[i][c], rk[i] - a.shift[i], i == 0 ? bv[c] + (rk[Q + c] - a.shift[Q + c]) : bv[c]);
+    store_model<Q>(a.coef + k * Model<Q>::CS, A, bv);
 }
 
 // 3'. Tangents of the block models with respect to the Gaussian's sigma and the
@@ -535,7 +598,7 @@ __device__ __forceinline__ void stage_blur_v_tangent(const FastArgs &a, size_t k
                 R[i][c] = r;
             }
         dev::chol_solve3<Q>(L, inv_d, R, da);
-        float *dc = a.dcoef + (size_t)t * 3 * (Q + 1) * bplane;
+        float dbv[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             float db = t == 0 ? dmuy[c] : 0.f;
@@ -546,10 +609,22 @@ __device__ __forceinline__ void stage_blur_v_tangent(const FastArgs &a, size_t k
                 if (t == 0) db = fmaf(-A[i][c], dmu[i], db);
                 db = fmaf(-da[i][c], rk[i] - a.shift[i], db);  // re-expressed relative to the frame reference
             }
-            dc[c * bplane + k] = db;
-#pragma unroll
-            for (int i = 0; i < Q; ++i) dc[(3 * (i + 1) + c) * bplane + k] = da[i][c];
+            dbv[c] = db;
         }
+        store_model<Q>(a.dcoef + ((size_t)t * bplane + k) * Model<Q>::CS, da, dbv);
+    }
+}
+
+template <int Q>
+__device__ __forceinline__ void load_model(float (&m)[Model<Q>::CS], const float *src)
+{
+#pragma unroll
+    for (int k = 0; k < Model<Q>::CS; k += 4) {
+        const float4 v = __ldg(reinterpret_cast<const float4 *>(src + k));
+        m[k] = v.x;
+        m[k + 1] = v.y;
+        m[k + 2] = v.z;
+        m[k + 3] = v.w;
     }
 }
 
@@ -561,9 +636,8 @@ __device__ __forceinline__ void stage_blur_v_tangent(const FastArgs &a, size_t k
 template <int Q>
 __device__ __forceinline__ void stage_apply(const FastArgs &a, size_t t)
 {
-    constexpr int NC = 3 * (Q + 1);
+    using M = Model<Q>;
     const size_t oplane = (size_t)a.Ho * a.Wo;
-    const size_t bplane = (size_t)a.Hb * a.Wb;
     const int P = a.F * a.s, den = 2 * P;
     const int nruns = a.Wo / P + 2;
     const size_t total = (size_t)a.Ho * nruns;
@@ -580,17 +654,17 @@ __device__ __forceinline__ void stage_apply(const FastArgs &a, size_t t)
         // corner models: left values and right-minus-left differences of the two block rows
         // (interpolated horizontally, then vertically, per pixel: the same order and the same
         // roundings as the TMA apply kernel, so both paths agree bit for bit)
-        float l0[NC], d0[NC], l1[NC], d1[NC];
+        float l0[M::CS], d0[M::CS], l1[M::CS], d1[M::CS];
         {
-            const size_t bl0 = (size_t)i0 * a.Wb + jl, bl1 = (size_t)i1 * a.Wb + jl;
-            const size_t br0 = (size_t)i0 * a.Wb + jr, br1 = (size_t)i1 * a.Wb + jr;
+            const float *row0 = a.coef + (size_t)i0 * a.Wb * M::CS, *row1 = a.coef + (size_t)i1 * a.Wb * M::CS;
+            load_model<Q>(l0, row0 + (size_t)jl * M::CS);
+            load_model<Q>(d0, row0 + (size_t)jr * M::CS);
+            load_model<Q>(l1, row1 + (size_t)jl * M::CS);
+            load_model<Q>(d1, row1 + (size_t)jr * M::CS);
 #pragma unroll
-            for (int k = 0; k < NC; ++k) {
-                const float *pl = a.coef + k * bplane;
-                l0[k] = __ldg(pl + bl0);
-                l1[k] = __ldg(pl + bl1);
-                d0[k] = __ldg(pl + br0) - l0[k];
-                d1[k] = __ldg(pl + br1) - l1[k];
+            for (int k = 0; k < M::CS; ++k) {
+                d0[k] -= l0[k];
+                d1[k] -= l1[k];
             }
         }
         float sh[Q + 3];
@@ -624,15 +698,17 @@ __device__ __forceinline__ void stage_apply(const FastArgs &a, size_t t)
                 const float fx = fminf(fmaxf((float)(nx - (r - 1) * den) / (float)den, 0.f), 1.f);
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
+                    // even and odd guides in two sums, as the pairs of the TMA apply
                     float top = fmaf(fx, d0[c], l0[c]);
-                    float acc = fmaf(fy, fmaf(fx, d1[c], l1[c]) - top, top);
+                    const float bias = fmaf(fy, fmaf(fx, d1[c], l1[c]) - top, top);
+                    float sum[2] = {0.f, 0.f};
 #pragma unroll
                     for (int i = 0; i < Q; ++i) {
-                        const int k = 3 * (i + 1) + c;
+                        const int k = M::at(c, i);
                         top = fmaf(fx, d0[k], l0[k]);
-                        acc = fmaf(fmaf(fy, fmaf(fx, d1[k], l1[k]) - top, top), z[i][u] - sh[i], acc);
+                        sum[i & 1] = fmaf(fmaf(fy, fmaf(fx, d1[k], l1[k]) - top, top), z[i][u] - sh[i], sum[i & 1]);
                     }
-                    o[c][u] = acc + sh[Q + c];
+                    o[c][u] = (bias + (sum[0] + sum[1])) + sh[Q + c];
                 }
             }
             if (vec) {
@@ -652,11 +728,8 @@ __device__ __forceinline__ void stage_apply(const FastArgs &a, size_t t)
     }
 }
 
-// Work-item counts of each stage for one frame (256 threads per item).
-__host__ __device__ inline int moment_chunks(int Wi) { return (Wi + 511) / 512; }
-inline size_t items_moments(const FastArgs &a) { return (size_t)a.Hb * moment_chunks(a.Wi); }
-inline size_t items_blocks(const FastArgs &a) { return ((size_t)a.Hb * a.Wb + 255) / 256; }
-inline size_t items_apply(const FastArgs &a) { return ((size_t)a.Ho * (a.Wo / (a.F * a.s) + 2) + 255) / 256; }
+// Input columns of a row are dealt to CTAs of stage 1 in chunks of two per thread.
+__host__ __device__ inline int moment_chunks(int Wi) { return (Wi + 2 * kMomThreads - 1) / (2 * kMomThreads); }
 
 }  // namespace fast
 }  // namespace flr

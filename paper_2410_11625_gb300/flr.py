@@ -377,7 +377,7 @@ class FastFLR:
         _check(load_library().flr_fast_reserve_batch(self._h, len(frames), arr), "flr_fast_reserve_batch")
 
     def denoise_batch(self, frames, stream=None):
-        """One persistent launch over every frame: list of (guide, radiance, map_guide, out)."""
+        """The four stages, each in one launch over every frame: list of (guide, radiance, map_guide, out)."""
         import torch
         arr = self._frames(frames)
         if stream is None:

@@ -3,7 +3,7 @@ frames of mixed sizes (Sec. 3.2.1) with model guides enhanced by the network (Se
 
 One step: for every group of same-size frames, the network's forward pass over the group's
 half-resolution inputs (guides and noisy radiance, concatenated channel-wise) gives the
-enhanced model guides; then ONE persistent cooperative fast-FLR launch fits every frame's
+enhanced model guides; then one batched fast-FLR pass (four launches) fits every frame's
 block models on its enhanced guides and half-resolution radiance and applies them to its
 full-resolution map guides.  The whole step is captured once in a CUDA graph and replayed.
 Launch arrangement only: every step runs in libflr.so's kernels.
