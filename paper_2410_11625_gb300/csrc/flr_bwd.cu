@@ -102,10 +102,22 @@ __global__ void __launch_bounds__(kBThreads) box_sum_kernel(const float *__restr
 }
 
 // The same clipped box sum over many planes with TMA staging (rows 16-byte aligned): a CTA
-// walks the planes [p0, p1) of one 64 x 32 output tile, p0 = blockIdx.z * per_cta; each plane's
+// walks the planes [p0, p1) of one 64 x 64 output tile, p0 = blockIdx.z * per_cta; each plane's
 // tile + halo arrives by one TMA box copy (the copy engine zero-fills outside the image) into
 // a double-buffered ring, so the next plane loads while the current one is summed.  Waits are
 // bounded (1 s).
+//
+// Bound by DRAM: the three calls of a 1080p backward pass (Q = 8) read and write 122 planes of
+// 8.3 MB, 298 us at the measured copy rate; they take 324 us.  The form before this was bound by
+// instruction issue (64 x 32 tiles, a second buffer for the horizontal sums, one column per
+// thread: 38 instructions per value, 68% of the issue slots, 372 us).  Ten warps of
+// eight rows each cover the 80 staged rows of radius 8 exactly; a warp's eight rows are its own,
+// so the horizontal sums replace their operands in place after a warp-wide barrier (which also
+// leaves room for three CTAs per SM); the vertical sums take two columns per thread, packed.
+// Each sum adds the same values in the same order as that form did: a run of 16 columns (8 rows)
+// from a multiple of 16 (8) on starts from its full window and slides.
+constexpr int kTH = 64, kTThreads = 320;
+
 struct alignas(128) BoxKArgs {
     CUtensorMap tm;  // [nplanes][H][W] float32, box (TS, THh, 1)
     float *out;
@@ -114,118 +126,146 @@ struct alignas(128) BoxKArgs {
 };
 
 struct BoxGeom {
-    int RCA, TWa, THh, TS, HS;
-    __host__ __device__ BoxGeom(int rad)
+    int RCA, TWa, THh, TS;
+    __host__ __device__ constexpr BoxGeom(int rad)
+        : RCA((rad + 3) & ~3),        // staged columns start 16-byte aligned
+          TWa(kBW + 2 * ((rad + 3) & ~3)),
+          THh(kTH + 2 * rad),
+          TS(kBW + 2 * ((rad + 3) & ~3) + 4)  // row stride = 4 (mod 8) floats: conflict-free 128-bit phases
     {
-        RCA = (rad + 3) & ~3;  // staged columns start 16-byte aligned
-        TWa = kBW + 2 * RCA;
-        THh = kBH + 2 * rad;
-        TS = TWa + 4;          // row stride = 4 (mod 8) floats: conflict-free 128-bit phases
-        HS = kBW + 1;
     }
-    __host__ __device__ int tile_floats() const { return (THh * TS + 31) / 32 * 32; }
-    __host__ __device__ size_t floats() const { return 32 + (size_t)2 * tile_floats() + (size_t)THh * HS + 8; }
+    __host__ __device__ constexpr int tile_floats() const { return (THh * TS + 31) / 32 * 32; }
+    __host__ __device__ constexpr size_t floats() const { return 32 + (size_t)2 * tile_floats() + 8; }
 };
 
 constexpr unsigned long long kBoxTimeoutNs = 1000000000ull;
 
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+
+// RT: the radius at compile time, or -1 (k.rad).  Radius 8 forms a window's first sum in four
+// interleaved parts, every other radius from left to right.
 template <int RT>
-__global__ void __launch_bounds__(kBThreads, 4) box_sum_tma_kernel(const __grid_constant__ BoxKArgs k)
+__global__ void __launch_bounds__(kTThreads, 3) box_sum_tma_kernel(const __grid_constant__ BoxKArgs k)
 {
     extern __shared__ __align__(16) float sm[];
     const int rad = RT >= 0 ? RT : k.rad;
     const BoxGeom g(rad);
     float *base = sm + (((128 - (tma::smem_addr(sm) & 127)) & 127) >> 2);
-    float *T0 = base, *T1 = base + g.tile_floats();
-    float *Hb = T1 + g.tile_floats();
-    uint64_t *bar = reinterpret_cast<uint64_t *>(Hb + ((g.THh * g.HS + 1) & ~1));
+    uint64_t *bar = reinterpret_cast<uint64_t *>(base + 2 * g.tile_floats());
     __shared__ int s_abort;
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int tx0 = blockIdx.x * kBW, ty0 = blockIdx.y * kBH;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tx0 = blockIdx.x * kBW, ty0 = blockIdx.y * kTH;
     const size_t plane = (size_t)k.H * k.W;
     const int p0 = blockIdx.z * k.per_cta, np = min(k.per_cta, k.nplanes - p0);  // p below counts from p0
-    auto stage = [&](float *T, int p) {
-        if (tid == 0) {
-            uint64_t *b = bar + (p & 1);
-            tma::mbar_expect_tx(b, (unsigned)(g.THh * g.TS * 4));
-            tma::load_3d(T, &k.tm, tx0 - g.RCA, ty0 - rad, p0 + p, b);
-        }
+    auto stage = [&](int p) {
+        uint64_t *b = bar + (p & 1);
+        tma::mbar_expect_tx(b, (unsigned)(g.THh * g.TS * 4));
+        tma::load_3d(base + (p & 1) * g.tile_floats(), &k.tm, tx0 - g.RCA, ty0 - rad, p0 + p, b);
     };
     if (tid == 0) {
         s_abort = 0;
         tma::mbar_init(bar, 1);
         tma::mbar_init(bar + 1, 1);
         tma::mbar_init_fence();
+        stage(0);
     }
     __syncthreads();
-    stage(T0, 0);
-    const int x = tid % kBW, run = tid / kBW;
-    const int gx = tx0 + x;
-    for (int p = 0; p < np; ++p) {
-        float *Tc = (p & 1) ? T1 : T0;
-        if (p + 1 < np) stage((p & 1) ? T0 : T1, p + 1);
+    // vertical sums: a warp takes a run of 8 rows, a lane two columns
+    const int gx = tx0 + 2 * lane, gy = ty0 + 8 * warp;
+    const int vrows = warp < kTH / 8 && gx < k.W ? min(8, k.H - gy) : 0;
+    float *dst = k.out + (size_t)p0 * plane + (size_t)gy * k.W + gx;
+    for (int p = 0; p < np; ++p, dst += plane) {
+        float *T = base + (p & 1) * g.tile_floats();
+        if (tid == 0 && p + 1 < np) stage(p + 1);
         if (!tma::wait_warp(bar + (p & 1), (uint32_t)((p >> 1) & 1), kBoxTimeoutNs) && lane == 0) {
             s_abort = 1;
             if (k.status) atomicExch(k.status, 1);
         }
-        __syncthreads();
+        // horizontal sums in place: 16 outputs per lane, eight rows per warp (lanes 0-7 take
+        // consecutive rows: 16-byte accesses at row stride 4 mod 8 floats, distinct banks)
+        for (int row = warp * 8 + (lane & 7); row - (lane & 7) < g.THh; row += kTThreads / 4) {
+            const bool in = row < g.THh;
+            float *q = T + row * g.TS + (lane >> 3) * 16;
+            float o[16];
+            if (in) {
+                if constexpr (RT >= 0) {
+                    constexpr int RCA = (RT + 3) & ~3, XO = RCA - RT, N = 16 + 2 * RCA;
+                    float v[N];
+#pragma unroll
+                    for (int kk = 0; kk < N; kk += 4) {
+                        const float4 f = *reinterpret_cast<const float4 *>(q + kk);
+                        v[kk] = f.x;
+                        v[kk + 1] = f.y;
+                        v[kk + 2] = f.z;
+                        v[kk + 3] = f.w;
+                    }
+                    float s;
+                    if constexpr (RT == 8) {
+                        float s4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                        for (int kk = 0; kk <= 2 * RT; ++kk) s4[kk & 3] += v[XO + kk];
+                        s = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+                    } else {
+                        s = 0.f;
+#pragma unroll
+                        for (int kk = 0; kk <= 2 * RT; ++kk) s += v[XO + kk];
+                    }
+                    o[0] = s;
+#pragma unroll
+                    for (int t = 1; t < 16; ++t) {
+                        s += v[XO + t + 2 * RT] - v[XO + t - 1];
+                        o[t] = s;
+                    }
+                } else {
+                    const float *qq = q + (g.RCA - rad);
+                    float s = 0.f;
+                    for (int kk = 0; kk <= 2 * rad; ++kk) s += qq[kk];
+                    o[0] = s;
+#pragma unroll
+                    for (int t = 1; t < 16; ++t) {
+                        s += qq[t + 2 * rad] - qq[t - 1];
+                        o[t] = s;
+                    }
+                }
+            }
+            __syncwarp();  // the row's operands are read
+            if (in) {
+#pragma unroll
+                for (int t = 0; t < 16; t += 4) *reinterpret_cast<float4 *>(q + t) = make_float4(o[t], o[t + 1], o[t + 2], o[t + 3]);
+            }
+        }
+        __syncthreads();  // horizontal sums complete
         if (s_abort) {  // let a copy still in flight land before the CTA exits, then stop
             if (p + 1 < np && tid < 32)
                 tma::wait_warp(bar + ((p + 1) & 1), (uint32_t)(((p + 1) >> 1) & 1), kBoxTimeoutNs);
             return;
         }
-        // horizontal sums: 16 outputs per item, operands in registers; consecutive lanes take
-        // consecutive rows (16-byte loads at row stride 4 mod 8 floats: distinct banks)
-        for (int item = tid; item < g.THh * 4; item += kBThreads) {
-            const int xr = (item / g.THh) * 16, row = item % g.THh;
-            const float *q = Tc + row * g.TS + xr;
-            float *h = Hb + row * g.HS + xr;
-            if constexpr (RT >= 0) {
-                constexpr int RCA = (RT + 3) & ~3, XO = RCA - RT, N = 16 + 2 * RCA;
-                float v[N];
+        if (vrows > 0) {
+            const float2 *q = reinterpret_cast<const float2 *>(T + (warp * 8) * g.TS) + lane;
+            const int st = g.TS / 2;
+            float2 first[7], s = make_float2(0.f, 0.f);
+            if constexpr (RT >= 4) {
 #pragma unroll
-                for (int kk = 0; kk < N; kk += 4) {
-                    const float4 f = *reinterpret_cast<const float4 *>(q + kk);
-                    v[kk] = f.x;
-                    v[kk + 1] = f.y;
-                    v[kk + 2] = f.z;
-                    v[kk + 3] = f.w;
-                }
-                float s4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int kk = 0; kk <= 2 * RT; ++kk) s4[kk & 3] += v[XO + kk];
-                float s = (s4[0] + s4[1]) + (s4[2] + s4[3]);
-                h[0] = s;
-#pragma unroll
-                for (int t = 1; t < 16; ++t) {
-                    s += v[XO + t + 2 * RT] - v[XO + t - 1];
-                    h[t] = s;
+                for (int kk = 0; kk <= 2 * RT; ++kk) {
+                    const float2 f = q[kk * st];
+                    if (kk < 7) first[kk < 7 ? kk : 0] = f;
+                    s = __fadd2_rn(s, f);
                 }
             } else {
-                const float *qq = q + (g.RCA - rad);
-                float s = 0.f;
-                for (int kk = 0; kk <= 2 * rad; ++kk) s += qq[kk];
-                h[0] = s;
+                for (int kk = 0; kk <= 2 * rad; ++kk) s = __fadd2_rn(s, q[kk * st]);
+            }
+            float *d = dst;
 #pragma unroll
-                for (int t = 1; t < 16; ++t) {
-                    s += qq[t + 2 * rad] - qq[t - 1];
-                    h[t] = s;
+            for (int t = 0; t < 8; ++t, d += k.W) {
+                if (t > 0) {
+                    const float2 old = RT >= 4 ? first[t - 1] : q[(t - 1) * st];
+                    s = __fadd2_rn(s, sub2(q[(t + 2 * rad) * st], old));
                 }
+                if (t < vrows) *reinterpret_cast<float2 *>(d) = s;
             }
         }
-        __syncthreads();  // Hb complete; Tc may be refilled from here on
-        if (tid == 0) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        // vertical sums: thread = (column, run of 8 rows)
-        const float *q = Hb + (run * 8) * g.HS + x;
-        float s = 0.f;
-        for (int kk = 0; kk <= 2 * rad; ++kk) s += q[kk * g.HS];
-        float *dst = k.out + (size_t)(p0 + p) * plane;
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            if (t > 0) s += q[(t + 2 * rad) * g.HS] - q[(t - 1) * g.HS];
-            const int gy = ty0 + run * 8 + t;
-            if (gx < k.W && gy < k.H) dst[(size_t)gy * k.W + gx] = s;
-        }
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        __syncthreads();  // this buffer may be refilled from here on
     }
 }
 
@@ -414,12 +454,12 @@ cudaError_t launch_box_sum_tma(const BoxKArgs &k, cudaStream_t st)
     const size_t smem = sizeof(float) * g.floats();
     cudaError_t e = cudaFuncSetAttribute(box_sum_tma_kernel<RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    // four CTAs per SM need most of the unified L1 / shared array as shared memory
+    // three CTAs per SM need most of the unified L1 / shared array as shared memory
     e = cudaFuncSetAttribute(box_sum_tma_kernel<RT>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
-    dim3 grid((k.W + kBW - 1) / kBW, (k.H + kBH - 1) / kBH, (k.nplanes + k.per_cta - 1) / k.per_cta);
-    box_sum_tma_kernel<RT><<<grid, kBThreads, smem, st>>>(k);
+    dim3 grid((k.W + kBW - 1) / kBW, (k.H + kTH - 1) / kTH, (k.nplanes + k.per_cta - 1) / k.per_cta);
+    box_sum_tma_kernel<RT><<<grid, kTThreads, smem, st>>>(k);
     return cudaGetLastError();
 }
 
@@ -436,15 +476,15 @@ cudaError_t launch_box_sum(const float *in, float *out, int nplanes, int H, int 
             k.rad = rad;
             k.nplanes = nplanes;
             k.status = status;
-            // Planes per CTA: about eight waves of four CTAs per SM, so that the last wave
+            // Planes per CTA: about eight waves of three CTAs per SM, so that the last wave
             // costs little, and one plane per CTA on frames with fewer tile-planes than that.
             // One CTA walking every plane of a tile left a 128 x 128 frame on 8 SMs (its three
             // box sums 105 us, split 10 us) and a 1080p frame with a second wave two thirds
             // full (the backward pass 1.066 ms, split 1.029 ms).
-            const long long tiles = (long long)((W + kBW - 1) / kBW) * ((H + kBH - 1) / kBH);
-            const long long target = 8LL * 4 * sm_count();
+            const long long tiles = (long long)((W + kBW - 1) / kBW) * ((H + kTH - 1) / kTH);
+            const long long target = 8LL * 3 * sm_count();
             k.per_cta = (int)std::min<long long>(nplanes, std::max<long long>(1, tiles * nplanes / target));
-            return rad == 8 ? launch_box_sum_tma<8>(k, st) : launch_box_sum_tma<-1>(k, st);
+            return rad == 8 ? launch_box_sum_tma<8>(k, st) : rad == 5 ? launch_box_sum_tma<5>(k, st) : launch_box_sum_tma<-1>(k, st);
         }
     }
     const size_t smem = sizeof(float) * ((size_t)(kBH + 2 * rad) * (kBW + 2 * rad + 1) + (size_t)(kBH + 2 * rad) * (kBW + 1));
