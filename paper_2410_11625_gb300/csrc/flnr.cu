@@ -798,6 +798,12 @@ __global__ void __launch_bounds__(WsGeom<CIN, COUT, KS, NT>::THREADS) conv_tail_
 // The products are those of the convolution on the concatenated map; only their order of
 // accumulation differs.  Roles and waits as conv_ws_kernel; the MMA lane issues the four
 // classes of a stage into one of two accumulator sets (4 * COUT columns each).
+// Bound by the number of MMAs: reading the 128 x 16 operand A costs about 50 clocks whatever N is
+// up to 64, and the four classes' 36 taps x (CA + CB)/16 of them took 71 us for d0a and 54 us for
+// d1a of a 1920x1080 pass.  The two classes (a, 0) and (a, 1) read position (t, u) for taps
+// dx = u + 1 and dx = u, whose weights lie side by side in shared memory ([dy][chunk][2 - dx]), so
+// one MMA of N = 2 COUT serves both: 24 instead of 36 per channel step, in the same order for
+// each class.
 template <int CA, int CB, int COUT, int NBUF>
 struct UpGeom {
     static constexpr int SH = 18, SW = 10;                       // staged rows and columns
@@ -871,10 +877,10 @@ __global__ void __launch_bounds__(kWsThreads) conv_up_kernel(const __grid_consta
     __syncthreads();  // tensor memory allocated
     pdl::trigger();
     pdl::wait();
-    // weights: global [tap][COUT][CA + CB] -> shared [tap][c8][COUT][8] (lo chunks first)
+    // weights: global [tap][COUT][CA + CB] -> shared [dy][c8][2 - dx][COUT][8] (lo chunks first)
     for (int i = tid; i < 9 * COUT * C8; i += kWsThreads) {
         const int c8 = i % C8, row = i / C8, tap = row / COUT, co = row % COUT;
-        cp_async16(sw + ((tap * C8 + c8) * COUT + co) * 16, a.w + (size_t)row * (CA + CB) + c8 * 8, true);
+        cp_async16(sw + ((((tap / 3) * C8 + c8) * 3 + 2 - tap % 3) * COUT + co) * 16, a.w + (size_t)row * (CA + CB) + c8 * 8, true);
     }
     cp_async_commit();
     cp_async_wait<0>();
@@ -921,9 +927,9 @@ __global__ void __launch_bounds__(kWsThreads) conv_up_kernel(const __grid_consta
         }
     } else if (warp == 5) {
         if (lane == 0) {  // MMA issuer
-            constexpr uint32_t idesc = umma_idesc(COUT);
+            constexpr uint32_t idesc1 = umma_idesc(COUT), idesc2 = umma_idesc(2 * COUT);
             const uint64_t adesc0 = umma_sdesc(smem_u32(sx0), PS, SW * 16);
-            const uint64_t bdesc0 = umma_sdesc(smem_u32(sw), COUT * 16, 128);
+            const uint64_t bdesc0 = umma_sdesc(smem_u32(sw), 3 * COUT * 16, 128);
             for (int j = 0; j < mine; ++j) {
                 const int st = j % NBUF, acc = j & 1;
                 if (!mbar_wait_thread(smem_u32(full + st), (uint32_t)((j / NBUF) & 1))) {
@@ -938,24 +944,26 @@ __global__ void __launch_bounds__(kWsThreads) conv_up_kernel(const __grid_consta
                 asm volatile("tcgen05.fence::after_thread_sync;\n");
                 const uint64_t ab = adesc0 + (uint64_t)((st * G::XBYTES) >> 4);
 #pragma unroll
-                for (int cls = 0; cls < 4; ++cls) {
-                    const uint32_t d = tmem + (uint32_t)((acc * 4 + cls) * COUT);
+                for (int ca = 0; ca < 2; ++ca) {
+                    const uint32_t d0 = tmem + (uint32_t)((acc * 4 + 2 * ca) * COUT);
 #pragma unroll
-                    for (int tap = 0; tap < 9; ++tap) {
-                        const int t = (cls >> 1) + tap / 3 - 1, u = (cls & 1) + tap % 3 - 1;  // -1 .. 2
+                    for (int pos = 0; pos < 12; ++pos) {
+                        const int dy = pos / 4, t = ca + dy - 1, u = pos % 4 - 1;  // t, u: -1 .. 2
                         const int oy = t >> 1, ox = u >> 1, pp = (t & 1) * 2 + (u & 1);
-                        const int pos = ((oy + 1) * SW + (ox + 1)) * 16;
+                        const int at = ((oy + 1) * SW + (ox + 1)) * 16;
+                        const bool both = u == 0 || u == 1;  // classes b = 0 (dx = u + 1) and 1 (dx = u)
+                        const uint32_t d = d0 + (u == 2 ? COUT : 0);
+                        const int tap0 = u == -1 ? 2 : u == 0 ? 1 : 0;  // 2 - dx of the first class
 #pragma unroll
-                        for (int kk = 0; kk < CA8 / 2; ++kk) {
-                            const uint32_t aoff = (uint32_t)((2 * kk * PS + pos) >> 4);
-                            const uint32_t boff = (uint32_t)(((tap * C8 + 2 * kk) * COUT * 16) >> 4);
-                            umma_bf16(d, ab + aoff, bdesc0 + boff, idesc, (tap | kk) ? 1u : 0u);
-                        }
-#pragma unroll
-                        for (int kk = 0; kk < CB8 / 2; ++kk) {
-                            const uint32_t aoff = (uint32_t)(((CA8 + pp * CB8 + 2 * kk) * PS + pos) >> 4);
-                            const uint32_t boff = (uint32_t)(((tap * C8 + CA8 + 2 * kk) * COUT * 16) >> 4);
-                            umma_bf16(d, ab + aoff, bdesc0 + boff, idesc, 1u);
+                        for (int kk = 0; kk < C8 / 2; ++kk) {
+                            const uint32_t aoff = (uint32_t)(((kk < CA8 / 2 ? 2 * kk : CA8 + pp * CB8 + 2 * kk - CA8) * PS + at) >> 4);
+                            const uint64_t b = bdesc0 + (uint32_t)((((dy * C8 + 2 * kk) * 3 + tap0) * COUT * 16) >> 4);
+                            if (dy == 0 && u == 0 && kk == 0) {  // class b = 1 starts here
+                                umma_bf16(d, ab + aoff, b, idesc1, 1u);
+                                umma_bf16(d + COUT, ab + aoff, b + (uint32_t)(COUT * 16 >> 4), idesc1, 0u);
+                            } else {
+                                umma_bf16(d, ab + aoff, b, both ? idesc2 : idesc1, (pos | kk) ? 1u : 0u);
+                            }
                         }
                     }
                 }
