@@ -166,13 +166,14 @@ int grow(flr_handle *h, int H, int W)
         if (cudaMalloc(&h->d_flags, px * sizeof(int)) != cudaSuccess) return FLR_ERR_NOMEM;
         h->flag_cap = (int)px;
     }
-    if (h->p.coef_radius > 0 && h->coef_px < px) {
+    const size_t coef_px = (size_t)H * flr::coef_pitch(W);
+    if (h->p.coef_radius > 0 && h->coef_px < coef_px) {
         if (h->d_coef) cudaFree(h->d_coef);
         h->d_coef = nullptr;
         h->coef_px = 0;
-        if (cudaMalloc(&h->d_coef, px * (size_t)(h->p.q + 1) * 3 * sizeof(float)) != cudaSuccess)
+        if (cudaMalloc(&h->d_coef, coef_px * (size_t)(h->p.q + 1) * 3 * sizeof(float)) != cudaSuccess)
             return FLR_ERR_NOMEM;
-        h->coef_px = px;
+        h->coef_px = coef_px;
     }
     return FLR_OK;
 }
@@ -423,6 +424,7 @@ int flr_denoise(flr_handle *h, const float *guide, const float *map_guide, const
     fa.rad = radiance;
     fa.out = out;
     fa.coef = h->d_coef;
+    fa.coef_pitch = flr::coef_pitch(W);
     fa.H = H;
     fa.W = W;
     fa.r = h->p.radius;
@@ -454,6 +456,7 @@ int flr_denoise(flr_handle *h, const float *guide, const float *map_guide, const
         da.shift = h->d_shift;
         da.out = out;
         da.coef = h->d_coef;
+        da.coef_pitch = flr::coef_pitch(W);
         da.H = H;
         da.W = W;
         da.r = h->p.radius;
@@ -471,6 +474,7 @@ int flr_denoise(flr_handle *h, const float *guide, const float *map_guide, const
     if (h->p.coef_radius > 0) {
         flr::ApplyArgs aa;
         aa.coef = h->d_coef;
+        aa.coef_pitch = flr::coef_pitch(W);
         aa.map_guide = map_guide ? map_guide : guide;
         aa.shift = h->d_shift;
         aa.out = out;
@@ -718,6 +722,7 @@ int flr_denoise_host(flr_handle *h, const float *guide, const float *map_guide,
         fa.rad = dr;
         fa.out = dout;
         fa.coef = h->d_coef;
+        fa.coef_pitch = flr::coef_pitch(W);
         fa.H = H;
         fa.W = W;
         fa.r = r;
@@ -749,6 +754,7 @@ int flr_denoise_host(flr_handle *h, const float *guide, const float *map_guide,
             da.shift = h->d_shift;
             da.out = dout;
             da.coef = h->d_coef;
+            da.coef_pitch = flr::coef_pitch(W);
             da.H = H;
             da.W = W;
             da.r = r;
@@ -768,6 +774,7 @@ int flr_denoise_host(flr_handle *h, const float *guide, const float *map_guide,
         if (rc > 0) {  // averaged models applied to rows [o_k, o_k+1)
             flr::ApplyArgs aa;
             aa.coef = h->d_coef;
+            aa.coef_pitch = flr::coef_pitch(W);
             aa.map_guide = map_guide ? dm : dg;
             aa.shift = h->d_shift;
             aa.out = dout;

@@ -48,12 +48,14 @@ __global__ void __launch_bounds__(kDThreads) flr_fp64_kernel(const Fp64Args a)
             }
             if (bad && a.nonfinite) atomicAdd(a.nonfinite, (unsigned long long)bad);
         } else {
+            const int pitch = a.coef_pitch ? a.coef_pitch : a.W;
+            const size_t cplane = (size_t)a.H * pitch, coff = (size_t)(idx / a.W) * pitch + idx % a.W;
 #pragma unroll
-            for (int c = 0; c < 3; ++c) a.coef[c * plane + idx] = (float)bv[c];
+            for (int c = 0; c < 3; ++c) a.coef[c * cplane + coff] = (float)bv[c];
 #pragma unroll
             for (int i = 0; i < Q; ++i)
 #pragma unroll
-                for (int c = 0; c < 3; ++c) a.coef[(3 * (i + 1) + c) * plane + idx] = (float)A[i][c];
+                for (int c = 0; c < 3; ++c) a.coef[(3 * (i + 1) + c) * cplane + coff] = (float)A[i][c];
         }
     }
 }

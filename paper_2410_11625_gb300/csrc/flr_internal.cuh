@@ -102,8 +102,9 @@ constexpr int kShiftSamples = 16;  // the shifts are means over a 16 x 16 sample
 struct FwdArgs {
     const float *guide, *map_guide, *rad;
     float *out;   // [3][H][W] written when rc == 0
-    float *coef;  // [(Q+1)*3][H][W] per-pixel models written when rc > 0
+    float *coef;  // [(Q+1)*3][H][coef_pitch] per-pixel models written when rc > 0
     int H, W, r, rc;
+    int coef_pitch = 0;  // floats per row of coef (0: W)
     float eps, tau;
     int TH;                          // rows per segment (a multiple of kB)
     unsigned long long *flag_count;  // device counter of flagged pixels
@@ -122,10 +123,16 @@ struct FwdArgs {
     int row_lo = 0, row_hi = -1, ref_rows = 0;
 };
 
+// Floats per row of the coefficient planes: W rounded up to 16 bytes, so that the apply stages its
+// tiles by TMA at every width (1277 x 719, q = 6, rc = 6: 123 us with 4-byte copies).  Not below 16
+// columns, where the padding would multiply the planes.
+__host__ __device__ inline int coef_pitch(int W) { return W >= 16 ? (W + 3) & ~3 : W; }
+
 struct ApplyArgs {
-    const float *coef, *map_guide, *shift;
+    const float *coef, *map_guide, *shift;  // coef: [(Q+1)*3][H][coef_pitch]
     float *out;
     int H, W, rc;
+    int coef_pitch;
     int *status = nullptr;  // set to 1 if a bounded device wait ran out (may be NULL)
     int row_lo = 0, row_hi = -1;  // output rows [row_lo, row_hi) (row_hi < 0: to H)
     unsigned long long *nonfinite = nullptr;  // count of non-finite output values (may be NULL)
@@ -135,6 +142,7 @@ struct Fp64Args {
     const float *guide, *map_guide, *rad, *shift;
     float *out, *coef;
     int H, W, r, rc;
+    int coef_pitch = 0;  // as FwdArgs
     int force_coef;  // write the model to the coefficient planes even when rc == 0
     double eps;
     const unsigned long long *flag_count;

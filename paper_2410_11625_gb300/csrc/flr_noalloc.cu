@@ -134,6 +134,9 @@ extern "C" int flr_denoise_noalloc(const flr_params *p, const float *guide, cons
     }
 
     auto *coef = (float *)big;
+    // padded rows where the array has room for them
+    const size_t padded = (size_t)H * flr::coef_pitch(W) * (size_t)(q + 1) * 3 * sizeof(float);
+    const int pitch = padded <= kBigBytes ? flr::coef_pitch(W) : W;
     const size_t smem = flr::fwd_smem_bytes(q, p->radius);
     if (flr::fwd_prepare(q, p->radius, smem) != cudaSuccess) return FLR_ERR_CUDA;
     flr::FwdArgs fa;
@@ -142,6 +145,7 @@ extern "C" int flr_denoise_noalloc(const flr_params *p, const float *guide, cons
     fa.rad = radiance;
     fa.out = out;
     fa.coef = coef;
+    fa.coef_pitch = pitch;
     fa.H = H;
     fa.W = W;
     fa.r = p->radius;
@@ -169,6 +173,7 @@ extern "C" int flr_denoise_noalloc(const flr_params *p, const float *guide, cons
         da.shift = shift;
         da.out = out;
         da.coef = coef;
+        da.coef_pitch = pitch;
         da.H = H;
         da.W = W;
         da.r = p->radius;
@@ -184,6 +189,7 @@ extern "C" int flr_denoise_noalloc(const flr_params *p, const float *guide, cons
     if (p->coef_radius > 0) {
         flr::ApplyArgs aa;
         aa.coef = coef;
+        aa.coef_pitch = pitch;
         aa.map_guide = map_guide ? map_guide : guide;
         aa.shift = shift;
         aa.out = out;
