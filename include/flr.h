@@ -95,6 +95,15 @@ int flr_destroy(flr_handle *h);
 int flr_reserve(flr_handle *h, int H, int W);
 
 /*
+ * Tell a handle that n handles' calls run at the same time, each on its own stream (the crops
+ * of a training step): later flr_denoise calls of this one plan their launches for 1/n of the
+ * device, so that the calls run side by side.  Only the split of the work changes; 1 is the
+ * default.
+ * Call it before flr_reserve (the workspace depends on the plan).  Errors: FLR_ERR_ARG.
+ */
+int flr_set_concurrency(flr_handle *h, int n);
+
+/*
  * FLR forward pass on device images (Sec. 3.1-3.2, Appendix; see the file header).
  *   guide      [q][H][W]  guides X the per-pixel models are fitted on
  *   map_guide  [q][H][W]  guides z the models are applied to, or NULL to use `guide`

@@ -108,6 +108,7 @@ struct flr_handle {
     flr_params p;
     int device = 0;
     int n_sm = 0;
+    int plan_sm = 0;  // SMs that a forward call's launches are planned for (flr_set_concurrency)
     unsigned long long *d_count = nullptr;  // [0] flagged pixels, [1] non-finite output values
     int *d_status = nullptr;                // set by a kernel whose bounded wait ran out
     float *d_shift = nullptr;               // frame reference shift, Q+3 floats
@@ -221,7 +222,7 @@ int grow_fused(flr_handle *h, const FusedPlan &pl)
 int run_fused(flr_handle *h, const float *guide, const float *map_guide, const float *radiance, float *out, int H,
               int W, int row_lo, int row_hi, cudaStream_t s)
 {
-    const FusedPlan pl = fused_plan(row_hi - row_lo, W, h->p.radius, h->p.coef_radius, h->n_sm);
+    const FusedPlan pl = fused_plan(row_hi - row_lo, W, h->p.radius, h->p.coef_radius, h->plan_sm);
     int st = grow_fused(h, pl);
     if (st != FLR_OK) return st;
     flr::FusedArgs fa;
@@ -335,6 +336,7 @@ int flr_create(const flr_params *params, flr_handle **out)
     h->p = *params;
     cudaError_t e = cudaGetDevice(&h->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->n_sm, cudaDevAttrMultiProcessorCount, h->device);
+    h->plan_sm = h->n_sm;
     if (e == cudaSuccess) e = cudaMalloc(&h->d_count, 2 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMalloc(&h->d_shift, sizeof(float) * (FLR_MAX_Q + 3));
     if (e == cudaSuccess) e = cudaMemset(h->d_count, 0, 2 * sizeof(unsigned long long));
@@ -389,8 +391,20 @@ int flr_reserve(flr_handle *h, int H, int W)
 {
     if (!h || H <= 0 || W <= 0) return FLR_ERR_ARG;
     if (flr::fused_supported(h->p.q, h->p.radius, h->p.coef_radius) && W % 4 == 0)
-        return grow_fused(h, fused_plan(H, W, h->p.radius, h->p.coef_radius, h->n_sm));
+        return grow_fused(h, fused_plan(H, W, h->p.radius, h->p.coef_radius, h->plan_sm));
     return grow(h, H, W);
+}
+
+// 16 crops of 128 x 128, each on a stream of its own: planned for the whole chip, a crop's fused
+// kernel is 64 CTAs of 4 rows that each walk 32 rows of warm-up, 16 x 64 CTAs in seven waves of 40 us
+// (a training step 1337 us); planned for 9 SMs it is 8 CTAs of 32 rows, all 16 crops in one wave of
+// 80 us (1174 us).  The backward pass keeps its split: its gradients follow the rounding of the window
+// sums to 1e-4 of their scale.
+int flr_set_concurrency(flr_handle *h, int n)
+{
+    if (!h || n < 1) return FLR_ERR_ARG;
+    h->plan_sm = std::max(1, h->n_sm / n);
+    return FLR_OK;
 }
 
 int flr_denoise(flr_handle *h, const float *guide, const float *map_guide, const float *radiance,
@@ -431,7 +445,7 @@ int flr_denoise(flr_handle *h, const float *guide, const float *map_guide, const
     fa.rc = h->p.coef_radius;
     fa.eps = h->p.eps;
     fa.tau = h->p.pivot_ratio;
-    fa.TH = choose_segment_rows(H, W, h->p.radius, h->n_sm);
+    fa.TH = choose_segment_rows(H, W, h->p.radius, h->plan_sm);
     fa.flag_count = h->d_count;
     fa.flag_list = h->d_flags;
     fa.flag_cap = h->flag_cap;
@@ -467,7 +481,7 @@ int flr_denoise(flr_handle *h, const float *guide, const float *map_guide, const
         da.flag_cap = h->flag_cap;
         da.force_coef = 0;
         da.nonfinite = h->d_count + 1;
-        FLR_CUDA(flr::launch_fp64(q, da, h->n_sm, s), "fp64 re-solve launch");
+        FLR_CUDA(flr::launch_fp64(q, da, h->plan_sm, s), "fp64 re-solve launch");
         ++h->n_fp64;
     }
     FLR_CUDA(mark(h, s), "timing event");
@@ -729,7 +743,7 @@ int flr_denoise_host(flr_handle *h, const float *guide, const float *map_guide,
         fa.rc = rc;
         fa.eps = h->p.eps;
         fa.tau = h->p.pivot_ratio;
-        fa.TH = choose_segment_rows(c[k + 1] - c[k], W, r, h->n_sm);
+        fa.TH = choose_segment_rows(c[k + 1] - c[k], W, r, h->plan_sm);
         fa.flag_count = h->d_count;
         fa.flag_list = h->d_flags;
         fa.flag_cap = h->flag_cap;
@@ -766,7 +780,7 @@ int flr_denoise_host(flr_handle *h, const float *guide, const float *map_guide,
             da.force_coef = 0;
             da.nonfinite = h->d_count + 1;
             da.flag_start = h->d_fstart;  // only this band's flags
-            FLR_CUDA(flr::launch_fp64(q, da, h->n_sm, s), "fp64 re-solve launch");
+            FLR_CUDA(flr::launch_fp64(q, da, h->plan_sm, s), "fp64 re-solve launch");
             FLR_CUDA(cudaMemcpyAsync(h->d_fstart, h->d_count, sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s),
                      "re-solve index");
             ++h->n_fp64;

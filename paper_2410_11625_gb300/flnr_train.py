@@ -104,6 +104,7 @@ class Trainer:
         # captured in a graph; `flr` is a separate handle for evaluation at other sizes.
         self.flrs = [_flr.FLR(q=8, radius=radius, eps=eps) for _ in range(batch)]
         for f in self.flrs:
+            f.set_concurrency(batch)
             f.reserve(crop, crop)
         self.flr = _flr.FLR(q=8, radius=radius, eps=eps)
         self.streams = [torch.cuda.Stream() for _ in range(batch)]

@@ -20,7 +20,7 @@ EXPORTS = ("flr_create", "flr_destroy", "flr_reserve", "flr_denoise", "flr_denoi
            "flr_denoise_host_async", "flr_host_wait",
            "flr_get_stats", "flr_get_kernel_times", "flr_status_string", "flr_last_cuda_error",
            "flr_denoise_noalloc", "flr_backward", "flr_fast_create", "flr_fast_destroy",
-           "flr_fast_denoise", "flr_fast_get_stats", "flr_fast_param_grad", "flr_denoise_batch", "flr_fast_reserve_batch",
+           "flr_set_concurrency", "flr_fast_denoise", "flr_fast_get_stats", "flr_fast_param_grad", "flr_denoise_batch", "flr_fast_reserve_batch",
            "flr_fast_denoise_batch", "flr_fast_batch_status", "flr_barrier_selftest",
            "flr_mbarrier_selftest", "flr_host_band_plan",
            "flnr_param_count", "flnr_create", "flnr_destroy", "flnr_set_weights", "flnr_get_weights",
@@ -93,6 +93,7 @@ def load_library():
     lib.flr_create.argtypes = [ctypes.POINTER(FlrParams), ctypes.POINTER(ctypes.c_void_p)]
     lib.flr_destroy.argtypes = [vp]
     lib.flr_reserve.argtypes = [vp, ip, ip]
+    lib.flr_set_concurrency.argtypes = [vp, ip]
     lib.flr_denoise.argtypes = [vp, fp, fp, fp, fp, ip, ip, vp]
     lib.flr_denoise_host.argtypes = [vp, fp, fp, fp, fp, ip, ip, vp]
     lib.flr_denoise_host_async.argtypes = [vp, fp, fp, fp, fp, ip, ip, vp]
@@ -127,7 +128,7 @@ def load_library():
     lib.flr_status_string.restype = ctypes.c_char_p
     lib.flr_last_cuda_error.argtypes = []
     lib.flr_last_cuda_error.restype = ctypes.c_char_p
-    for name in ("flr_create", "flr_destroy", "flr_reserve", "flr_denoise", "flr_denoise_host",
+    for name in ("flr_create", "flr_destroy", "flr_reserve", "flr_set_concurrency", "flr_denoise", "flr_denoise_host",
                  "flr_denoise_host_async", "flr_host_wait", "flr_get_stats", "flr_get_kernel_times"):
         getattr(lib, name).restype = ctypes.c_int
     _lib = lib
@@ -187,6 +188,11 @@ class FLR:
 
     def reserve(self, H, W):
         _check(load_library().flr_reserve(self._h, int(H), int(W)), "flr_reserve")
+
+    def set_concurrency(self, n):
+        """n handles' calls run at the same time, each on its own stream: this handle's later
+        launches are planned for 1/n of the device.  Call it before reserve."""
+        _check(load_library().flr_set_concurrency(self._h, int(n)), "flr_set_concurrency")
 
     def denoise(self, guide, radiance, map_guide=None, out=None, stream=None):
         """Device FLR: guide [q,H,W], radiance [3,H,W] CUDA float32 -> out [3,H,W]."""
