@@ -1,12 +1,12 @@
 // flr_bwd.cu -- kernels of the FLR backward pass that are not the per-pixel adjoint solve
-// (that one is the forward kernel in adjoint mode, flr_fwd.cu).  sm_103a.
+// (that one is the forward kernel in adjoint mode, flr_fwd_kernel.cuh).  sm_103a.
 //
 // The backward pass is the reverse-mode derivative of the forward's steps (the paper
 // trains through FLR by backpropagation, Sec. 3.2-3.3; it prints no adjoint).  With
 // g = dL/dI and m_i the size of the clipped averaging window T'_i:
 //   fields    F_i = (1, z_i - s) g_i^T / m_i                       (adjoint of the apply)
 //   G(A_k)    = sum_{i in T'_k} F_i                                (adjoint of the average)
-//   adjoint   per pixel k: the moment gradients GS_k               (flr_fwd.cu, ADJ = true)
+//   adjoint   per pixel k: the moment gradients GS_k               (flr_fwd_kernel.cuh, ADJ = true)
 //   BS_j      = sum_{k in T_j} GS_k                                (adjoint of the window sums)
 //   contract  dx_j = BS_x + 2 BS_xx (x_j - s) + BS_xy (y_j - s_y)
 //             dy_j = BS_y + BS_xy^T (x_j - s)
