@@ -329,12 +329,19 @@ __device__ __forceinline__ void tc_store(const ConvArgs &a, float (&v)[COUT], co
 // accumulator rows of their TMEM lane quarter, release the accumulator, and run the epilogue
 // (with several tiles per stage eight warps: the sigmoid of the head keeps four busy longer than
 // the MMAs take; o0 + o1 at 1920x1080 101 us with four, 81 us with eight).
-// The operand layouts are those described above.  A stage covers NT MMA tiles side by side
-// (16 rows x 8 NT pixels): one halo and one hand-over of the barriers for NT accumulators, which
-// pays where there are enough stages to go round (conv_ws_launch).  Every wait is bounded.
+// A stage covers NT row phases of 8 columns (16 NT rows x 8 pixels, issue_phases; a 1x1 layer NT
+// tiles of 16 rows x 8 pixels side by side): one halo and one hand-over of the barriers for NT accumulators, which pays where there are enough stages to
+// go round (conv_ws_launch).  Every wait is bounded.
 template <int CIN, int COUT, int KS, int NT>
 struct WsGeom {
-    static constexpr int TH = 16, TW = 8 * NT, P = KS / 2, SH = TH + 2 * P, SW = TW + 2 * P, C8 = CIN / 8;
+    // NT row phases of 8 columns, or (1x1: no row is read twice, and long rows cost TMA fewer
+    // requests; 16 -> 16 at 16 x 128^2 19.4 us against 21.1) NT tiles side by side
+    static constexpr bool PHASES = KS > 1;
+    static constexpr int STEP = PHASES ? NT : 1;  // rows between an accumulator's 8-row groups
+    static constexpr int TH = PHASES ? 16 * NT : 16, TW = PHASES ? 8 : 8 * NT;
+    static constexpr int P = KS / 2, SH = TH + 2 * P, SW = TW + 2 * P, C8 = CIN / 8;
+    // one MMA for the up to KS row phases that read a staged row (N <= 256)
+    static constexpr bool MERGE = PHASES && NT > 1 && KS * COUT <= 256;
     static constexpr int NBUF = NT == 1 ? 4 : (C8 <= 2 ? 3 : 2);
     static constexpr int PS = (SH * SW * 16 + 127) / 128 * 128;
     static constexpr int XBYTES = C8 * PS;
@@ -356,6 +363,53 @@ __device__ __forceinline__ void load_planes(uint32_t dst, const CUtensorMap *tm,
     for (int k = 0; k < C8; ++k) {
         if (layout == kNHWC) tma_load_4d(dst + k * PS, tm, k * 8, x, y, n, bar);
         else tma_load_4d(dst + k * PS, tm, 4 * x, y, k, n, bar);  // 32-bit elements: four per pixel
+    }
+}
+
+// The MMAs of one stage.  Row phase t of a stage is its output rows t, t + NT, t + 2 NT, ...: 16
+// rows x 8 pixels, the M = 128 rows of an operand whose 8-row groups lie NT staged rows apart.  Staged
+// row rho + NT g is then read by phase t = rho - ky for tap row ky, so the same operand A serves up to
+// KS phases, whose accumulators and weights ([kx][chunk][KS - 1 - ky][COUT]) lie side by side: one
+// MMA of N = KS COUT instead of KS of N = COUT.  An MMA costs about 50 clocks whatever N is up to
+// 64 and little more up to 200 (operand A is read from shared memory at 128 bytes per clock), and
+// a 16 -> 16 layer spent 36 of them on 512 pixels (tiles side by side), now 21.  Each accumulator
+// still takes its taps in the order (ky, kx, channels).  1920x1080 forward pass 428 us before, 417
+// us so; gradients of 16 x 128^2 562 and 549 us.
+template <class G, int CIN, int COUT, int KS, int NT>
+__device__ __forceinline__ void issue_phases(uint32_t d0, uint64_t ab, uint64_t bdesc0)
+{
+    constexpr int C8 = G::C8, SW = G::SW, PS = G::PS;
+    if constexpr (!G::PHASES) {
+#pragma unroll
+        for (int t = 0; t < NT; ++t)
+#pragma unroll
+            for (int kk = 0; kk < C8 / 2; ++kk)
+                umma_bf16(d0 + (uint32_t)(t * COUT), ab + (uint32_t)((2 * kk * PS + 8 * t * 16) >> 4),
+                          bdesc0 + (uint32_t)((2 * kk * COUT * 16) >> 4), umma_idesc(COUT), kk ? 1u : 0u);
+        return;
+    }
+#pragma unroll
+    for (int rho = 0; rho < NT + KS - 1; ++rho) {
+        const int lo = rho - KS + 1 > 0 ? rho - KS + 1 : 0, hi = rho < NT - 1 ? rho : NT - 1;  // phases that read rho
+#pragma unroll
+        for (int kx = 0; kx < KS; ++kx) {
+#pragma unroll
+            for (int kk = 0; kk < C8 / 2; ++kk) {
+                const uint64_t a = ab + (uint32_t)((2 * kk * PS + (rho * SW + kx) * 16) >> 4);
+                // weights of phase t: tap row rho - t
+                auto b = [&](int t) { return bdesc0 + (uint32_t)((((kx * C8 + 2 * kk) * KS + KS - 1 - (rho - t)) * COUT * 16) >> 4); };
+                auto d = [&](int t) { return d0 + (uint32_t)(t * COUT); };
+                const bool starts = rho < NT && (kx | kk) == 0;  // phase rho begins here
+                if constexpr (G::MERGE) {
+                    const int n = hi - lo + (starts ? 0 : 1);
+                    if (n > 0) umma_bf16(d(lo), a, b(lo), umma_idesc(n * COUT), 1u);
+                    if (starts) umma_bf16(d(rho), a, b(rho), umma_idesc(COUT), 0u);
+                } else {
+#pragma unroll
+                    for (int t = lo; t <= hi; ++t) umma_bf16(d(t), a, b(t), umma_idesc(COUT), starts && t == rho ? 0u : 1u);
+                }
+            }
+        }
     }
 }
 
@@ -404,7 +458,7 @@ __global__ void __launch_bounds__(WsGeom<CIN, COUT, KS, NT>::THREADS) conv_ws_ke
     pdl::wait();
     for (int i = tid; i < KS * KS * COUT * C8; i += G::THREADS) {
         const int c8 = i % C8, row = i / C8, tap = row / COUT, co = row % COUT;
-        cp_async16(sw + ((tap * C8 + c8) * COUT + co) * 16, a.w + (size_t)row * CIN + c8 * 8, true);
+        cp_async16(sw + (((tap % KS * C8 + c8) * KS + KS - 1 - tap / KS) * COUT + co) * 16, a.w + (size_t)row * CIN + c8 * 8, true);
     }
     cp_async_commit();
     cp_async_wait<0>();
@@ -443,9 +497,8 @@ __global__ void __launch_bounds__(WsGeom<CIN, COUT, KS, NT>::THREADS) conv_ws_ke
         }
     } else if (warp == G::EW + 1) {
         if (lane == 0) {  // MMA issuer
-            constexpr uint32_t idesc = umma_idesc(COUT);
-            const uint64_t adesc0 = umma_sdesc(smem_u32(sx0), PS, SW * 16);
-            const uint64_t bdesc0 = umma_sdesc(smem_u32(sw), COUT * 16, 128);
+            const uint64_t adesc0 = umma_sdesc(smem_u32(sx0), PS, G::STEP * SW * 16);
+            const uint64_t bdesc0 = umma_sdesc(smem_u32(sw), KS * COUT * 16, 128);
             for (int j = 0; j < mine; ++j) {
                 const int st = j % NBUF, acc = j & 1;
                 if (!mbar_wait_thread(smem_u32(full + st), (uint32_t)((j / NBUF) & 1))) {
@@ -459,19 +512,7 @@ __global__ void __launch_bounds__(WsGeom<CIN, COUT, KS, NT>::THREADS) conv_ws_ke
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;\n");
                 const uint64_t ab = adesc0 + (uint64_t)((st * G::XBYTES) >> 4);
-#pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                    const uint32_t d = tmem + (uint32_t)((acc * NT + t) * COUT);
-#pragma unroll
-                    for (int tap = 0; tap < KS * KS; ++tap) {
-#pragma unroll
-                        for (int kk = 0; kk < C8 / 2; ++kk) {
-                            const uint32_t aoff = (uint32_t)((2 * kk * PS + ((tap / KS) * SW + tap % KS + 8 * t) * 16) >> 4);
-                            const uint32_t boff = (uint32_t)(((tap * C8 + 2 * kk) * COUT * 16) >> 4);
-                            umma_bf16(d, ab + aoff, bdesc0 + boff, idesc, (tap | kk) ? 1u : 0u);
-                        }
-                    }
-                }
+                issue_phases<G, CIN, COUT, KS, NT>(tmem + (uint32_t)(acc * NT * COUT), ab, bdesc0);
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
                     smem_u32(empty + st)));
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
@@ -499,7 +540,8 @@ __global__ void __launch_bounds__(WsGeom<CIN, COUT, KS, NT>::THREADS) conv_ws_ke
                     __syncwarp();
                     if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(acce + acc)) : "memory");
                 }
-                tc_store<COUT, ACT, OUTM, MASK>(a, v, bias, n, ty0 + 4 * (warp & 3) + (lane >> 3), tx0 + 8 * t + (lane & 7));
+                tc_store<COUT, ACT, OUTM, MASK>(a, v, bias, n, ty0 + G::STEP * (4 * (warp & 3) + (lane >> 3)) + (G::PHASES ? t : 0),
+                         tx0 + (G::PHASES ? 0 : 8 * t) + (lane & 7));
             }
         }
     }
@@ -601,7 +643,7 @@ __global__ void __launch_bounds__(WsGeom<CIN, COUT, KS, NT>::THREADS) conv_tail_
     pdl::wait();
     for (int i = tid; i < KS * KS * COUT * C8; i += G::THREADS) {
         const int c8 = i % C8, row = i / C8, tap = row / COUT, co = row % COUT;
-        cp_async16(sw + ((tap * C8 + c8) * COUT + co) * 16, a.w + (size_t)row * CIN + c8 * 8, true);
+        cp_async16(sw + (((tap % KS * C8 + c8) * KS + KS - 1 - tap / KS) * COUT + co) * 16, a.w + (size_t)row * CIN + c8 * 8, true);
     }
     if (args.w2_kept && blockIdx.x == 0) {
         for (int i = tid; i < COUT2 * COUT; i += G::THREADS) args.w2_kept[i] = a2.w[i];
@@ -649,9 +691,9 @@ __global__ void __launch_bounds__(WsGeom<CIN, COUT, KS, NT>::THREADS) conv_tail_
         }
     } else if (warp == G::EW + 1) {
         if (lane == 0) {  // MMA issuer
-            constexpr uint32_t idesc = umma_idesc(COUT), idesc2 = umma_idesc(COUT2);
-            const uint64_t adesc0 = umma_sdesc(smem_u32(sx0), PS, SW * 16);
-            const uint64_t bdesc0 = umma_sdesc(smem_u32(sw), COUT * 16, 128);
+            constexpr uint32_t idesc2 = umma_idesc(COUT2);
+            const uint64_t adesc0 = umma_sdesc(smem_u32(sx0), PS, G::STEP * SW * 16);
+            const uint64_t bdesc0 = umma_sdesc(smem_u32(sw), KS * COUT * 16, 128);
             const uint64_t a2desc0 = umma_sdesc(smem_u32(sa2), 128 * 16, 128);
             const uint64_t b2desc0 = umma_sdesc(smem_u32(sw2), COUT2 * 16, 128);
             // the 1x1 of tile t: its A operand written, its accumulator slot drained
@@ -687,19 +729,7 @@ __global__ void __launch_bounds__(WsGeom<CIN, COUT, KS, NT>::THREADS) conv_tail_
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;\n");
                 const uint64_t ab = adesc0 + (uint64_t)((st * G::XBYTES) >> 4);
-#pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                    const uint32_t d = tmem + (uint32_t)((acc * NT + t) * COUT);
-#pragma unroll
-                    for (int tap = 0; tap < KS * KS; ++tap) {
-#pragma unroll
-                        for (int kk = 0; kk < C8 / 2; ++kk) {
-                            const uint32_t aoff = (uint32_t)((2 * kk * PS + ((tap / KS) * SW + tap % KS + 8 * t) * 16) >> 4);
-                            const uint32_t boff = (uint32_t)(((tap * C8 + 2 * kk) * COUT * 16) >> 4);
-                            umma_bf16(d, ab + aoff, bdesc0 + boff, idesc, (tap | kk) ? 1u : 0u);
-                        }
-                    }
-                }
+                issue_phases<G, CIN, COUT, KS, NT>(tmem + (uint32_t)(acc * NT * COUT), ab, bdesc0);
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
                     smem_u32(empty + st)));
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
@@ -731,7 +761,8 @@ __global__ void __launch_bounds__(WsGeom<CIN, COUT, KS, NT>::THREADS) conv_tail_
                     __syncwarp();
                     if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(acc2e + sl)) : "memory");
                 }
-                tc_store<COUT2, ACT2, OUTM2, false>(a2, v2, bias2, n, ty0 + 4 * (warp & 3) + (lane >> 3), tx0 + 8 * i + (lane & 7));
+                tc_store<COUT2, ACT2, OUTM2, false>(a2, v2, bias2, n, ty0 + G::STEP * (4 * (warp & 3) + (lane >> 3)) + (G::PHASES ? i : 0),
+                         tx0 + (G::PHASES ? 0 : 8 * i) + (lane & 7));
             }
             return true;
         };
@@ -753,7 +784,8 @@ __global__ void __launch_bounds__(WsGeom<CIN, COUT, KS, NT>::THREADS) conv_tail_
                     __syncwarp();
                     if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(acce + acc)) : "memory");
                 }
-                const int yy = ty0 + 4 * (warp & 3) + (lane >> 3), xx = tx0 + 8 * t + (lane & 7);
+                const int yy = ty0 + G::STEP * (4 * (warp & 3) + (lane >> 3)) + (G::PHASES ? t : 0);
+                const int xx = tx0 + (G::PHASES ? 0 : 8 * t) + (lane & 7);
                 const bool in = yy < a.H && xx < a.W;
                 size_t yc = 0;
                 bf16 *yp = a.y ? a.y + pixel_at(a.ly, COUT, a.H, a.W, n, yy, xx, &yc) : nullptr;
@@ -1937,9 +1969,9 @@ cudaError_t resident(K kern, int threads, size_t smem, int cols, Resident &out)
 
 // Stages of a map of N images.  NT tiles per stage share a halo, a hand-over of the barriers and
 // eight epilogue warps; they are taken as soon as half the SMs get a stage (a 1920x1080 forward
-// pass takes 472 us with several tiles per stage and 516 us with one, forward and backward over
-// 16 x 128^2 572 and 621 us); smaller maps would leave the chip idle.
-long long stages(int N, int H, int W, int tw) { return (long long)N * ((H + 15) / 16) * ((W + tw - 1) / tw); }
+// pass took 472 us with several tiles per stage and 516 us with one, forward and backward over
+// 16 x 128^2 572 and 621 us, both before the row phases); smaller maps would leave the chip idle.
+long long stages(int N, int H, int W, int th, int tw) { return (long long)N * ((H + th - 1) / th) * ((W + tw - 1) / tw); }
 
 // Launch of the warp-specialised convolution with NT tiles per stage; when only asked, *fits
 // reports whether that many per stage is the better choice.
@@ -1953,7 +1985,7 @@ cudaError_t conv_ws_launch_nt(const ConvArgs &a, bool ask, bool *fits, cudaStrea
     static Resident res;
     cudaError_t e = resident(kern, G::THREADS, smem, G::COLS, res);
     if (e != cudaSuccess) return e;
-    const long long ntiles = stages(a.N, a.H, a.W, G::TW), cap = (long long)res.per_sm * res.n_sm;
+    const long long ntiles = stages(a.N, a.H, a.W, G::TH, G::TW), cap = (long long)res.per_sm * res.n_sm;
     if (ask) {
         *fits = 2 * ntiles >= res.n_sm;
         return cudaSuccess;
@@ -2011,7 +2043,7 @@ cudaError_t conv_tail_launch_nt(const ConvArgs &c, const ConvArgs &c2, bf16 *w2_
     static Resident res;
     cudaError_t e = resident(kern, G::THREADS, smem, T::COLS, res);
     if (e != cudaSuccess) return e;
-    const long long ntiles = stages(c.N, c.H, c.W, G::TW), cap = (long long)res.per_sm * res.n_sm;
+    const long long ntiles = stages(c.N, c.H, c.W, G::TH, G::TW), cap = (long long)res.per_sm * res.n_sm;
     if (ask) {
         *fits = 2 * ntiles >= res.n_sm;
         return cudaSuccess;
@@ -2050,7 +2082,7 @@ cudaError_t conv_up_launch(const ConvArgs &a, cudaStream_t st)
     cudaError_t e = resident(kern, kWsThreads, smem, G::COLS, res);
     if (e != cudaSuccess) return e;
     if ((a.H | a.W) & 1) return cudaErrorInvalidValue;
-    const long long ntiles = stages(a.N, a.H / 2, a.W / 2, 8), cap = (long long)res.per_sm * res.n_sm;
+    const long long ntiles = stages(a.N, a.H / 2, a.W / 2, 16, 8), cap = (long long)res.per_sm * res.n_sm;
     if (ntiles <= 0) return cudaSuccess;
     UpArgs ua;
     std::memset(&ua, 0, sizeof(ua));
@@ -2075,7 +2107,7 @@ cudaError_t conv_s2_launch(const ConvArgs &a, cudaStream_t st)
     cudaError_t e = resident(kern, kWsThreads, smem, G::COLS, res);
     if (e != cudaSuccess) return e;
     if ((a.H | a.W) & 1) return cudaErrorInvalidValue;
-    const long long ntiles = stages(a.N, a.H / 2, a.W / 2, G::TW), cap = (long long)res.per_sm * res.n_sm;
+    const long long ntiles = stages(a.N, a.H / 2, a.W / 2, 16, G::TW), cap = (long long)res.per_sm * res.n_sm;
     if (ntiles <= 0) return cudaSuccess;
     S2Args sa;
     std::memset(&sa, 0, sizeof(sa));
@@ -2109,7 +2141,7 @@ cudaError_t wgrad_launch(const bf16 *x, const bf16 *dz, int layout, int N, int H
     static Resident res;
     cudaError_t e = resident(kern, kWgThreads, smem, G::COLS, res);
     if (e != cudaSuccess) return e;
-    const long long ntiles = stages(N, H, W, 8);
+    const long long ntiles = stages(N, H, W, 16, 8);
     const int slots = n_sm / G::NG > 0 ? n_sm / G::NG : 1;
     const int slices = (int)(ntiles < slots ? ntiles : slots);
     WgradArgs a;
