@@ -50,6 +50,7 @@
 #include "flr_fp64_model.cuh"
 #include "flr_internal.cuh"
 #include "flr_tmem.cuh"
+#include "pdl.cuh"
 #include "tma.cuh"
 
 namespace flr {
@@ -358,6 +359,7 @@ __global__ void __launch_bounds__(kThreads, 1) flr_fused_kernel(const __grid_con
     const int y1 = min(y0 + a.TH, row_hi);
     const int cta = blockIdx.y * gridDim.x + blockIdx.x;
     if (y0 >= y1) {  // a segment past the last row (not produced by the host plan)
+        pdl::wait();
         if (tid == 0) a.list_count[cta] = 0;
         return;
     }
@@ -384,6 +386,7 @@ __global__ void __launch_bounds__(kThreads, 1) flr_fused_kernel(const __grid_con
         for (int i = 0; i < kStages + 3; ++i) tma::mbar_init(bar + i, 1);
         tma::mbar_init_fence();
     }
+    pdl::wait();  // the inputs and the zeroed counters
     // the CTA's reference shift: mean of a 16 x 16 sample grid of its input region
     if (warp == 1)
         dev::sample_mean<Q>(s_sh, a.guide, a.rad, H, W, max(0, m_lo - R), min(H, m_hi + R), max(0, x0 - RC - R),
@@ -775,6 +778,7 @@ __global__ void __launch_bounds__(kFixThreads) flr_fused_fix_kernel(const FusedA
     __shared__ float s_sh[NS];
     __shared__ unsigned long long s_cnt[2];
     const int cta = blockIdx.y * gridDim.x + blockIdx.x;
+    pdl::wait();
     const int n = a.list_count[cta];
     if (n == 0) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -889,8 +893,7 @@ cudaError_t launch_qr(const FusedArgs &a, dim3 grid, cudaStream_t st)
         tma::encode_planes_f32(&ka.tz, a.map_guide ? a.map_guide : a.guide, a.W, a.H, Q, G::TW, kB, Q) !=
             cudaSuccess)
         return cudaErrorInvalidValue;
-    flr_fused_kernel<Q, R, RC><<<grid, kThreads, G::SMEM, st>>>(ka);
-    return cudaGetLastError();
+    return pdl::launch(flr_fused_kernel<Q, R, RC>, grid, kThreads, G::SMEM, st, ka);
 }
 
 }  // namespace fused
@@ -917,8 +920,7 @@ cudaError_t launch_fused(int q, const FusedArgs &a, dim3 grid, cudaStream_t st)
 cudaError_t launch_fused_fix(int q, const FusedArgs &a, dim3 grid, cudaStream_t st)
 {
     if (q != 8) return cudaErrorInvalidValue;
-    fused::flr_fused_fix_kernel<8><<<grid, fused::kFixThreads, 0, st>>>(a);
-    return cudaGetLastError();
+    return pdl::launch(fused::flr_fused_fix_kernel<8>, grid, fused::kFixThreads, 0, st, a);
 }
 
 }  // namespace flr
