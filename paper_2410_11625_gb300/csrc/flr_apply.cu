@@ -26,6 +26,7 @@
 
 #include "flr.h"
 #include "flr_internal.cuh"
+#include "pdl.cuh"
 #include "tma.cuh"
 
 namespace flr {
@@ -123,6 +124,7 @@ __global__ void __launch_bounds__(kAThreads, 2) flr_apply_kernel(const __grid_co
         }
     }
     __syncthreads();
+    pdl::wait();
     stage(0);
     // vertical sums and accumulation: warps 0 to 7 take a run of 8 rows each, a lane two columns
     const int gx = tx0 + 2 * lane, gy = ty0 + kARun * warp;
@@ -271,8 +273,7 @@ cudaError_t launch_apply_rc(int q, const ApplyArgs &a, cudaStream_t st)
                   tma::encode_planes_f32(&ka.tm, a.coef, a.W, a.H, 3 * (q + 1), g.TS, g.THh, 1, a.coef_pitch) == cudaSuccess)
                      ? 1
                      : 0;
-    flr_apply_kernel<RC><<<grid, kAThreads, smem, st>>>(ka);
-    return cudaGetLastError();
+    return pdl::launch(flr_apply_kernel<RC>, grid, kAThreads, smem, st, ka);
 }
 
 }  // namespace

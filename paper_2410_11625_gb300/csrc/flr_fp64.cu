@@ -11,6 +11,7 @@
 // reduces the sums.  Rarely run, so it is written for clarity rather than speed.
 #include "flr_fp64_model.cuh"
 #include "flr_internal.cuh"
+#include "pdl.cuh"
 
 namespace flr {
 namespace {
@@ -20,6 +21,7 @@ constexpr int kDThreads = 128;
 template <int Q>
 __global__ void __launch_bounds__(kDThreads) flr_fp64_kernel(const Fp64Args a)
 {
+    pdl::wait();
     const int lane = threadIdx.x & 31;
     const int gw = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int nw = (int)((gridDim.x * blockDim.x) >> 5);
@@ -63,8 +65,7 @@ __global__ void __launch_bounds__(kDThreads) flr_fp64_kernel(const Fp64Args a)
 template <int Q>
 cudaError_t launch_fp64_q(const Fp64Args &a, int n_sm, cudaStream_t st)
 {
-    flr_fp64_kernel<Q><<<2 * n_sm, kDThreads, 0, st>>>(a);
-    return cudaGetLastError();
+    return pdl::launch(flr_fp64_kernel<Q>, dim3(2 * n_sm), kDThreads, 0, st, a);
 }
 
 }  // namespace

@@ -2,6 +2,7 @@
 // adjoint kernel (flr_fwd_kernel.cuh) over the guide count.
 #include "flr_fwd.cuh"
 #include "flr_internal.cuh"
+#include "pdl.cuh"
 
 namespace flr {
 namespace {
@@ -15,6 +16,7 @@ template <int Q>
 __global__ void __launch_bounds__(32 * (Q + 3)) frame_shift_kernel(const float *guide, const float *rad, int H, int W,
                                                                     int ref_rows, float *shift_out)
 {
+    pdl::wait();
     constexpr int NS = kShiftSamples;
     const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int yb = ref_rows > 0 ? min(ref_rows, H) : H;
@@ -62,8 +64,8 @@ cudaError_t launch_adj(int q, const FwdArgs &a, dim3 grid, size_t smem, cudaStre
 cudaError_t launch_frame_shift(int q, const float *guide, const float *rad, int H, int W, int ref_rows, float *shift_out,
                                cudaStream_t st)
 {
-    FLR_Q_DISPATCH(q, frame_shift_kernel<QQ><<<1, 32 * (QQ + 3), 0, st>>>(guide, rad, H, W, ref_rows, shift_out);
-                   return cudaGetLastError());
+    FLR_Q_DISPATCH(q, return pdl::launch(frame_shift_kernel<QQ>, dim3(1), 32 * (QQ + 3), 0, st, guide, rad, H, W, ref_rows,
+                                         shift_out));
     return cudaErrorInvalidValue;
 }
 

@@ -46,6 +46,7 @@
 #include "flr_fwd.cuh"
 #include "flr_internal.cuh"
 #include "flr_tmem.cuh"
+#include "pdl.cuh"
 #include "tma.cuh"
 
 namespace flr {
@@ -399,6 +400,7 @@ __global__ void __launch_bounds__(kThreads, 1) flr_fwd_kernel(const __grid_const
     const int first_row = y0 - r;  // first input row summed by this segment
     int yv = y0 - 2 * r;           // first virtual row: the walkers start from an empty window
     int nstaged = 0;               // stage_batch calls so far (mbarrier phase)
+    pdl::wait();
     stage_batch<Q>(stage, gm, ka, bar, r, yv, x0, warp, lane);
     ++nstaged;
 
@@ -625,8 +627,7 @@ cudaError_t launch_fwd_qr(const FwdArgs &a, dim3 grid, size_t smem, cudaStream_t
                          tma::encode_planes_f32(&ka.tr, a.rad, a.W, a.H, 3, gm.WSt, kB, 3) == cudaSuccess
                      ? 1
                      : 0;
-    flr_fwd_kernel<Q, RT, ADJ><<<grid, kThreads, smem, st>>>(ka);
-    return cudaGetLastError();
+    return pdl::launch(flr_fwd_kernel<Q, RT, ADJ>, grid, kThreads, smem, st, ka);
 }
 
 // The dynamic shared memory a kernel instance may use is a per-device attribute shared by
