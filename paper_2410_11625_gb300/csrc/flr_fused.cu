@@ -205,7 +205,7 @@ __device__ __forceinline__ void walk_rows(float2 (&E)[Groups<Q>::MAXG], float2 (
 // n D = XY - L_y mu^T (the same a as M^{-1} D).  model_factor centres and factors n M, column by
 // column with the trailing matrix updated at once, so that consecutive instructions are
 // independent; low0/low1: whether a Cholesky pivot ratio d_j / (n M)_jj fell to tau or below.
-// model_rhs solves for one colour.
+// model_rhs solves for the three colours side by side.
 template <int Q>
 struct Factor {
     float2 nmu[Q], L[Q * (Q - 1) / 2], inv_d[Q];  // minus the guide means, strict lower triangle, 1 / L_jj
@@ -893,6 +893,8 @@ cudaError_t launch_qr(const FusedArgs &a, dim3 grid, cudaStream_t st)
         tma::encode_planes_f32(&ka.tz, a.map_guide ? a.map_guide : a.guide, a.W, a.H, Q, G::TW, kB, Q) !=
             cudaSuccess)
         return cudaErrorInvalidValue;
+    // dependent launches here and below, with no early trigger (a waiting CTA of the successor would
+    // take an SM from another stream's fused kernel): 256 x 256 41.0 -> 38.7 us, 1920x1080 299.2 -> 296.5
     return pdl::launch(flr_fused_kernel<Q, R, RC>, grid, kThreads, G::SMEM, st, ka);
 }
 
