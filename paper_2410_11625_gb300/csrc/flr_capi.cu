@@ -526,7 +526,8 @@ int flr_backward(flr_handle *h, const float *guide, const float *map_guide, cons
         h->bwd = nullptr;
         h->bwd_px = 0;
         const size_t planes = 3 * (size_t)(3 * (FLR_MAX_Q + 1)) + 2 * (size_t)(FLR_MAX_Q + 3 + FLR_MAX_Q * (FLR_MAX_Q + 1) / 2 + 3 * FLR_MAX_Q);
-        if (cudaMalloc(&h->bwd, px * planes * sizeof(float)) != cudaSuccess) return FLR_ERR_NOMEM;
+        // and one double, 8-byte aligned, for an eps gradient that the caller does not ask for
+        if (cudaMalloc(&h->bwd, px * planes * sizeof(float) + 2 * sizeof(double)) != cudaSuccess) return FLR_ERR_NOMEM;
         h->bwd_px = px;
     }
     float *Acoef = h->bwd;                 // per-pixel models A_k
@@ -594,9 +595,7 @@ int flr_backward(flr_handle *h, const float *guide, const float *map_guide, cons
     // 3. per-pixel adjoint solve (moments recomputed) -> GS, d/d eps
     if (grad_eps) FLR_CUDA(cudaMemsetAsync(grad_eps, 0, sizeof(double), s), "backward: reset eps gradient");
     double *geps = grad_eps;
-    if (!geps) {
-        geps = (double *)(BS + (size_t)nch * px);  // unused slot at the end of the workspace
-    }
+    if (!geps) geps = (double *)(((uintptr_t)(BS + (size_t)nch * px) + 7) & ~(uintptr_t)7);  // after the planes
     fa.gA = gA;
     fa.gS = GS;
     fa.geps = geps;
