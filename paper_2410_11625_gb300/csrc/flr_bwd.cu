@@ -29,12 +29,13 @@ constexpr int kBW = 64, kBH = 32, kBThreads = 256;
 
 template <int Q>
 __global__ void bwd_fields_kernel(const float *__restrict__ g, const float *__restrict__ z,
-                                  const float *__restrict__ shift, float *__restrict__ F, int H, int W, int rc)
+                                  const float *__restrict__ shift, float *__restrict__ F, int H, int W, int pitch, int rc)
 {
     pdl::wait();
     const size_t plane = (size_t)H * W;
     for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < plane; p += (size_t)gridDim.x * blockDim.x) {
         const int y = (int)(p / W), x = (int)(p % W);
+        const size_t fplane = (size_t)H * pitch, fp = (size_t)y * pitch + x;
         float inv_m = 1.f;
         if (rc > 0) {
             const float ny = (float)(min(y + rc, H - 1) - max(y - rc, 0) + 1);
@@ -45,20 +46,20 @@ __global__ void bwd_fields_kernel(const float *__restrict__ g, const float *__re
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             gc[c] = g[c * plane + p] * inv_m;
-            F[c * plane + p] = gc[c];
+            F[c * fplane + fp] = gc[c];
         }
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             const float zi = z[i * plane + p] - shift[i];
 #pragma unroll
-            for (int c = 0; c < 3; ++c) F[(3 * (i + 1) + c) * plane + p] = zi * gc[c];
+            for (int c = 0; c < 3; ++c) F[(3 * (i + 1) + c) * fplane + fp] = zi * gc[c];
         }
     }
 }
 
 // out[plane] = sum over the clipped radius-rad window of in[plane]; blockIdx.z = plane.
 __global__ void __launch_bounds__(kBThreads) box_sum_kernel(const float *__restrict__ in, float *__restrict__ out,
-                                                           int H, int W, int rad)
+                                                           int H, int W, int pitch, int rad)
 {
     pdl::wait();
     extern __shared__ float sm[];
@@ -66,7 +67,7 @@ __global__ void __launch_bounds__(kBThreads) box_sum_kernel(const float *__restr
     const int TS = TWh + 1, HS = kBW + 1;
     float *T = sm;
     float *Hb = T + THh * TS;
-    const size_t plane = (size_t)H * W;
+    const size_t plane = (size_t)H * pitch;
     const float *src = in + (size_t)blockIdx.z * plane;
     float *dst = out + (size_t)blockIdx.z * plane;
     const int tx0 = blockIdx.x * kBW, ty0 = blockIdx.y * kBH;
@@ -75,7 +76,7 @@ __global__ void __launch_bounds__(kBThreads) box_sum_kernel(const float *__restr
         const int sy = ty0 - rad + row;
         for (int col = lane; col < TWh; col += 32) {
             const int sx = tx0 - rad + col;
-            T[row * TS + col] = (sy >= 0 && sy < H && sx >= 0 && sx < W) ? __ldg(src + (size_t)sy * W + sx) : 0.f;
+            T[row * TS + col] = (sy >= 0 && sy < H && sx >= 0 && sx < W) ? __ldg(src + (size_t)sy * pitch + sx) : 0.f;
         }
     }
     __syncthreads();
@@ -102,15 +103,18 @@ __global__ void __launch_bounds__(kBThreads) box_sum_kernel(const float *__restr
     for (int t = 0; t < 8; ++t) {
         if (t > 0) s += q[(t + 2 * rad) * HS] - q[(t - 1) * HS];
         const int gy = ty0 + run * 8 + t;
-        if (gx < W && gy < H) dst[(size_t)gy * W + gx] = s;
+        if (gx < W && gy < H) dst[(size_t)gy * pitch + gx] = s;
     }
 }
 
-// The same clipped box sum over many planes with TMA staging (rows 16-byte aligned): a CTA
+// The same clipped box sum over many planes with TMA staging (row pitch a multiple of 16 bytes): a CTA
 // walks the planes [p0, p1) of one 64 x 64 output tile, p0 = blockIdx.z * per_cta; each plane's
 // tile + halo arrives by one TMA box copy (the copy engine zero-fills outside the image) into
 // a double-buffered ring, so the next plane loads while the current one is summed.  Waits are
 // bounded (1 s).
+//
+// The planes' rows are padded to 16 bytes (coef_pitch), so that every width from 16 on comes this
+// way: backward 1919 x 1080, r = rc = 8, 1827 us at first, 1088 us so (same bits).
 //
 // Bound by DRAM: the three calls of a 1080p backward pass (Q = 8) read and write 122 planes of
 // 8.3 MB, 298 us at the measured copy rate; they take 324 us.  The form before this was bound by
@@ -126,7 +130,7 @@ constexpr int kTH = 64, kTThreads = 320;
 struct alignas(128) BoxKArgs {
     CUtensorMap tm;  // [nplanes][H][W] float32, box (TS, THh, 1)
     float *out;
-    int H, W, rad, nplanes, per_cta;
+    int H, W, pitch, rad, nplanes, per_cta;
     int *status;
 };
 
@@ -147,9 +151,10 @@ constexpr unsigned long long kBoxTimeoutNs = 1000000000ull;
 
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 
-// RT: the radius at compile time, or -1 (k.rad).  Radius 8 forms a window's first sum in four
-// interleaved parts, every other radius from left to right.
-template <int RT>
+// RT: the radius at compile time, or -1 (k.rad).  PARTS: a window's first horizontal sum in four
+// interleaved parts (radius 8 at widths that are multiples of 4), else from left to right: each
+// width keeps the order of additions it has always had, which the gradients follow.
+template <int RT, bool PARTS>
 __global__ void __launch_bounds__(kTThreads, 3) box_sum_tma_kernel(const __grid_constant__ BoxKArgs k)
 {
     extern __shared__ __align__(16) float sm[];
@@ -160,7 +165,7 @@ __global__ void __launch_bounds__(kTThreads, 3) box_sum_tma_kernel(const __grid_
     __shared__ int s_abort;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tx0 = blockIdx.x * kBW, ty0 = blockIdx.y * kTH;
-    const size_t plane = (size_t)k.H * k.W;
+    const size_t plane = (size_t)k.H * k.pitch;
     const int p0 = blockIdx.z * k.per_cta, np = min(k.per_cta, k.nplanes - p0);  // p below counts from p0
     auto stage = [&](int p) {
         uint64_t *b = bar + (p & 1);
@@ -179,7 +184,7 @@ __global__ void __launch_bounds__(kTThreads, 3) box_sum_tma_kernel(const __grid_
     // vertical sums: a warp takes a run of 8 rows, a lane two columns
     const int gx = tx0 + 2 * lane, gy = ty0 + 8 * warp;
     const int vrows = warp < kTH / 8 && gx < k.W ? min(8, k.H - gy) : 0;
-    float *dst = k.out + (size_t)p0 * plane + (size_t)gy * k.W + gx;
+    float *dst = k.out + (size_t)p0 * plane + (size_t)gy * k.pitch + gx;
     for (int p = 0; p < np; ++p, dst += plane) {
         float *T = base + (p & 1) * g.tile_floats();
         if (tid == 0 && p + 1 < np) stage(p + 1);
@@ -206,7 +211,7 @@ __global__ void __launch_bounds__(kTThreads, 3) box_sum_tma_kernel(const __grid_
                         v[kk + 3] = f.w;
                     }
                     float s;
-                    if constexpr (RT == 8) {
+                    if constexpr (PARTS) {
                         float s4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                         for (int kk = 0; kk <= 2 * RT; ++kk) s4[kk & 3] += v[XO + kk];
@@ -262,7 +267,7 @@ __global__ void __launch_bounds__(kTThreads, 3) box_sum_tma_kernel(const __grid_
             }
             float *d = dst;
 #pragma unroll
-            for (int t = 0; t < 8; ++t, d += k.W) {
+            for (int t = 0; t < 8; ++t, d += k.pitch) {
                 if (t > 0) {
                     const float2 old = RT >= 4 ? first[t - 1] : q[(t - 1) * st];
                     s = __fadd2_rn(s, sub2(q[(t + 2 * rad) * st], old));
@@ -284,6 +289,7 @@ __global__ void __launch_bounds__(256) bwd_contract_kernel(const BwdArgs a)
     const size_t plane = (size_t)H * W;
     for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < plane; p += (size_t)gridDim.x * blockDim.x) {
         const int y = (int)(p / W), x = (int)(p % W);
+        const size_t bplane = (size_t)H * a.pitch, bp = (size_t)y * a.pitch + x;  // of BS and BA
         // every input of this pixel is read once, up front (the outputs may not alias them)
         float xs[Q], ys[3], gc[3];
 #pragma unroll
@@ -302,15 +308,15 @@ __global__ void __launch_bounds__(256) bwd_contract_kernel(const BwdArgs a)
         const float *BS = a.BS;
         float bxx[C::NXX];
 #pragma unroll
-        for (int t = 0; t < C::NXX; ++t) bxx[t] = __ldg(BS + (C::XX0 + t) * plane + p);
+        for (int t = 0; t < C::NXX; ++t) bxx[t] = __ldg(BS + (C::XX0 + t) * bplane + bp);
         float bxy[Q][3];
 #pragma unroll
         for (int i = 0; i < Q; ++i)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) bxy[i][c] = __ldg(BS + C::xy(i, c) * plane + p);
+            for (int c = 0; c < 3; ++c) bxy[i][c] = __ldg(BS + C::xy(i, c) * bplane + bp);
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            float d = __ldg(BS + (C::X0 + i) * plane + p);
+            float d = __ldg(BS + (C::X0 + i) * bplane + bp);
 #pragma unroll
             for (int j = 0; j < Q; ++j) {
                 const int t = (i <= j ? C::xx(i, j) : C::xx(j, i)) - C::XX0;
@@ -321,7 +327,7 @@ __global__ void __launch_bounds__(256) bwd_contract_kernel(const BwdArgs a)
             // the applied guide: dz_i = sum_c Abar[i][c] g_c
             float dz = 0.f;
 #pragma unroll
-            for (int c = 0; c < 3; ++c) dz = fmaf(__ldg(a.BA + (3 * (i + 1) + c) * plane + p), gc[c], dz);
+            for (int c = 0; c < 3; ++c) dz = fmaf(__ldg(a.BA + (3 * (i + 1) + c) * bplane + bp), gc[c], dz);
             dz *= inv_m;
             if (a.separate_map) {
                 a.grad_guide[i * plane + p] = d;
@@ -332,7 +338,7 @@ __global__ void __launch_bounds__(256) bwd_contract_kernel(const BwdArgs a)
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            float d = __ldg(BS + (C::Y0 + c) * plane + p);
+            float d = __ldg(BS + (C::Y0 + c) * bplane + bp);
 #pragma unroll
             for (int i = 0; i < Q; ++i) d = fmaf(bxy[i][c], xs[i], d);
             a.grad_rad[c * plane + p] = d;
@@ -438,47 +444,49 @@ int elem_grid(size_t n) { return (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 
 }  // namespace
 
 cudaError_t launch_bwd_fields(int q, const float *g, const float *z, const float *shift, float *F, int H, int W,
-                              int rc, cudaStream_t st)
+                              int pitch, int rc, cudaStream_t st)
 {
     const int grid = elem_grid((size_t)H * W);
     switch (q) {
-    case 1: return pdl::launch(bwd_fields_kernel<1>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, rc);
-    case 2: return pdl::launch(bwd_fields_kernel<2>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, rc);
-    case 3: return pdl::launch(bwd_fields_kernel<3>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, rc);
-    case 4: return pdl::launch(bwd_fields_kernel<4>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, rc);
-    case 5: return pdl::launch(bwd_fields_kernel<5>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, rc);
-    case 6: return pdl::launch(bwd_fields_kernel<6>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, rc);
-    case 7: return pdl::launch(bwd_fields_kernel<7>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, rc);
-    case 8: return pdl::launch(bwd_fields_kernel<8>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, rc);
+    case 1: return pdl::launch(bwd_fields_kernel<1>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, pitch, rc);
+    case 2: return pdl::launch(bwd_fields_kernel<2>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, pitch, rc);
+    case 3: return pdl::launch(bwd_fields_kernel<3>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, pitch, rc);
+    case 4: return pdl::launch(bwd_fields_kernel<4>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, pitch, rc);
+    case 5: return pdl::launch(bwd_fields_kernel<5>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, pitch, rc);
+    case 6: return pdl::launch(bwd_fields_kernel<6>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, pitch, rc);
+    case 7: return pdl::launch(bwd_fields_kernel<7>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, pitch, rc);
+    case 8: return pdl::launch(bwd_fields_kernel<8>, dim3(grid), 256, 0, st, g, z, shift, F, H, W, pitch, rc);
     default: return cudaErrorInvalidValue;
     }
 }
 
-template <int RT>
+template <int RT, bool PARTS>
 cudaError_t launch_box_sum_tma(const BoxKArgs &k, cudaStream_t st)
 {
     const BoxGeom g(k.rad);
     const size_t smem = sizeof(float) * g.floats();
-    cudaError_t e = cudaFuncSetAttribute(box_sum_tma_kernel<RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(box_sum_tma_kernel<RT, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // three CTAs per SM need most of the unified L1 / shared array as shared memory
-    e = cudaFuncSetAttribute(box_sum_tma_kernel<RT>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    e = cudaFuncSetAttribute(box_sum_tma_kernel<RT, PARTS>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     dim3 grid((k.W + kBW - 1) / kBW, (k.H + kTH - 1) / kTH, (k.nplanes + k.per_cta - 1) / k.per_cta);
-    return pdl::launch(box_sum_tma_kernel<RT>, grid, kTThreads, smem, st, k);
+    return pdl::launch(box_sum_tma_kernel<RT, PARTS>, grid, kTThreads, smem, st, k);
 }
 
-cudaError_t launch_box_sum(const float *in, float *out, int nplanes, int H, int W, int rad, cudaStream_t st, int *status)
+cudaError_t launch_box_sum(const float *in, float *out, int nplanes, int H, int W, int pitch, int rad, cudaStream_t st,
+                           int *status)
 {
-    if ((W & 3) == 0 && ((uintptr_t)in & 15) == 0 && nplanes > 0) {
+    if ((pitch & 3) == 0 && ((uintptr_t)in & 15) == 0 && nplanes > 0) {
         BoxKArgs k;
         std::memset(&k, 0, sizeof(k));
         const BoxGeom g(rad);
-        if (tma::encode_planes_f32(&k.tm, in, W, H, nplanes, g.TS, g.THh, 1) == cudaSuccess) {
+        if (tma::encode_planes_f32(&k.tm, in, W, H, nplanes, g.TS, g.THh, 1, pitch) == cudaSuccess) {
             k.out = out;
             k.H = H;
             k.W = W;
+            k.pitch = pitch;
             k.rad = rad;
             k.nplanes = nplanes;
             k.status = status;
@@ -490,14 +498,15 @@ cudaError_t launch_box_sum(const float *in, float *out, int nplanes, int H, int 
             const long long tiles = (long long)((W + kBW - 1) / kBW) * ((H + kTH - 1) / kTH);
             const long long target = 8LL * 3 * sm_count();
             k.per_cta = (int)std::min<long long>(nplanes, std::max<long long>(1, tiles * nplanes / target));
-            return rad == 8 ? launch_box_sum_tma<8>(k, st) : rad == 5 ? launch_box_sum_tma<5>(k, st) : launch_box_sum_tma<-1>(k, st);
+            if (rad == 8) return (W & 3) == 0 ? launch_box_sum_tma<8, true>(k, st) : launch_box_sum_tma<8, false>(k, st);
+            return rad == 5 ? launch_box_sum_tma<5, false>(k, st) : launch_box_sum_tma<-1, false>(k, st);
         }
     }
     const size_t smem = sizeof(float) * ((size_t)(kBH + 2 * rad) * (kBW + 2 * rad + 1) + (size_t)(kBH + 2 * rad) * (kBW + 1));
     cudaError_t e = cudaFuncSetAttribute(box_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((W + kBW - 1) / kBW, (H + kBH - 1) / kBH, nplanes);
-    return pdl::launch(box_sum_kernel, grid, kBThreads, smem, st, in, out, H, W, rad);
+    return pdl::launch(box_sum_kernel, grid, kBThreads, smem, st, in, out, H, W, pitch, rad);
 }
 
 cudaError_t launch_bwd_contract(int q, const BwdArgs &a, cudaStream_t st)

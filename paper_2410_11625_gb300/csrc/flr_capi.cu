@@ -518,7 +518,9 @@ int flr_backward(flr_handle *h, const float *guide, const float *map_guide, cons
     const int q = h->p.q;
     const int nch = q + 3 + q * (q + 1) / 2 + 3 * q;
     const int ncf = 3 * (q + 1);
-    const size_t px = (size_t)H * W;
+    // the workspace's planes have padded rows, so that the box sums stage them by TMA at every width
+    const int pitch = flr::coef_pitch(W);
+    const size_t px = (size_t)H * pitch;
     int st = grow(h, H, W);
     if (st != FLR_OK) return st;
     if (h->bwd_px < px || !h->bwd) {
@@ -548,6 +550,7 @@ int flr_backward(flr_handle *h, const float *guide, const float *map_guide, cons
     fa.rad = radiance;
     fa.out = nullptr;
     fa.coef = Acoef;
+    fa.coef_pitch = pitch;
     fa.H = H;
     fa.W = W;
     fa.r = r;
@@ -574,6 +577,7 @@ int flr_backward(flr_handle *h, const float *guide, const float *map_guide, cons
         da.shift = h->d_shift;
         da.out = nullptr;
         da.coef = Acoef;
+        da.coef_pitch = pitch;
         da.H = H;
         da.W = W;
         da.r = r;
@@ -586,10 +590,10 @@ int flr_backward(flr_handle *h, const float *guide, const float *map_guide, cons
     }
     // 2. adjoint of the apply and of the average: G(A_k)
     const float *z = map_guide ? map_guide : guide;
-    FLR_CUDA(flr::launch_bwd_fields(q, grad_out, z, h->d_shift, F, H, W, rc, s), "backward: fields launch");
+    FLR_CUDA(flr::launch_bwd_fields(q, grad_out, z, h->d_shift, F, H, W, pitch, rc, s), "backward: fields launch");
     const float *gA = F;
     if (rc > 0) {
-        FLR_CUDA(flr::launch_box_sum(F, GA, ncf, H, W, rc, s, h->d_status), "backward: average adjoint launch");
+        FLR_CUDA(flr::launch_box_sum(F, GA, ncf, H, W, pitch, rc, s, h->d_status), "backward: average adjoint launch");
         gA = GA;
     }
     // 3. per-pixel adjoint solve (moments recomputed) -> GS, d/d eps
@@ -607,10 +611,10 @@ int flr_backward(flr_handle *h, const float *guide, const float *map_guide, cons
     FLR_CUDA(flr::launch_adj(q, fa, grid, h->adj_smem, s), "backward: adjoint kernel launch");
     if (fp64_fix) FLR_CUDA(flr::launch_fp64(q, da, h->n_sm, s), "backward: fp64 re-solve launch");
     // 4. adjoint of the window sums, the averaged models for the applied guide, contraction
-    FLR_CUDA(flr::launch_box_sum(GS, BS, nch, H, W, r, s, h->d_status), "backward: window-sum adjoint launch");
+    FLR_CUDA(flr::launch_box_sum(GS, BS, nch, H, W, pitch, r, s, h->d_status), "backward: window-sum adjoint launch");
     const float *BA = Acoef;
     if (rc > 0) {  // the averaged a (planes 3 .. ncf - 1); the contraction reads no averaged bias
-        FLR_CUDA(flr::launch_box_sum(Acoef + 3 * px, F + 3 * px, ncf - 3, H, W, rc, s, h->d_status),
+        FLR_CUDA(flr::launch_box_sum(Acoef + 3 * px, F + 3 * px, ncf - 3, H, W, pitch, rc, s, h->d_status),
                  "backward: model average launch");
         BA = F;
     }
@@ -626,6 +630,7 @@ int flr_backward(flr_handle *h, const float *guide, const float *map_guide, cons
     ba.grad_rad = grad_radiance;
     ba.H = H;
     ba.W = W;
+    ba.pitch = pitch;
     ba.rc = rc;
     ba.separate_map = map_guide != nullptr;
     FLR_CUDA(flr::launch_bwd_contract(q, ba, s), "backward: contraction launch");

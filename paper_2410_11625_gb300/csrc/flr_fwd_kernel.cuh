@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(kThreads, 1) flr_fwd_kernel(const __grid_const
                 const int cpitch = a.coef_pitch ? a.coef_pitch : W;
                 const size_t cplane = (size_t)H * cpitch, coff = (size_t)yc * cpitch + xc;
                 if constexpr (ADJ) {
-                    geps_acc += adjoint_pixel<Q>(A, mu, muy, L, inv_d, ny * nx, a.gA, a.gS, plane, off,
+                    geps_acc += adjoint_pixel<Q>(A, mu, muy, L, inv_d, ny * nx, a.gA, a.gS, cplane, coff,
                                                  s_cta, s_ref);
                     if (a.coef) {  // the model itself (for the backward's averaged models)
 #pragma unroll

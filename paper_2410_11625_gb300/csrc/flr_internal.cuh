@@ -113,8 +113,8 @@ struct FwdArgs {
     float *shift_out;  // frame reference shift (Q+3 floats), written by block (0, 0)
     int force_coef;    // write the coefficient planes even when rc == 0 (backward pass)
     // adjoint mode only: G(A_k) planes in, per-pixel moment gradients out, d/d eps
-    const float *gA;   // [(Q+1)*3][H][W]: row 0 = G(b_k), rows 1..Q = G(a_k)
-    float *gS;         // [NCH][H][W] in moment-channel order (see Chan)
+    const float *gA;   // [(Q+1)*3][H][coef_pitch]: row 0 = G(b_k), rows 1..Q = G(a_k)
+    float *gS;         // [NCH][H][coef_pitch] in moment-channel order (see Chan)
     double *geps;      // accumulated d L / d eps
     int *status = nullptr;  // set to 1 if a bounded device wait ran out (may be NULL)
     unsigned long long *nonfinite = nullptr;  // count of non-finite output values (may be NULL)
@@ -158,6 +158,7 @@ struct BwdArgs {
     const float *BA;                       // [(Q+1)*3] box-summed (rc > 0) or raw models
     float *grad_guide, *grad_map, *grad_rad;
     int H, W, rc;
+    int pitch;                             // floats per row of BS and BA
     int separate_map;                      // the map guide is not the model guide
 };
 
@@ -206,8 +207,9 @@ cudaError_t fwd_prepare(int q, int r, size_t smem);
 cudaError_t launch_apply(int q, const ApplyArgs &a, cudaStream_t st);
 cudaError_t launch_fp64(int q, const Fp64Args &a, int n_sm, cudaStream_t st);
 cudaError_t launch_bwd_fields(int q, const float *g, const float *z, const float *shift, float *F, int H, int W,
-                              int rc, cudaStream_t st);
-cudaError_t launch_box_sum(const float *in, float *out, int nplanes, int H, int W, int rad, cudaStream_t st,
+                              int pitch, int rc, cudaStream_t st);
+// in, out: [nplanes][H][pitch] floats; columns W .. pitch - 1 are not read (and may be written)
+cudaError_t launch_box_sum(const float *in, float *out, int nplanes, int H, int W, int pitch, int rad, cudaStream_t st,
                            int *status = nullptr);
 cudaError_t launch_bwd_contract(int q, const BwdArgs &a, cudaStream_t st);
 // the frame reference shift of the forward kernel (Q + 3 floats), by itself
