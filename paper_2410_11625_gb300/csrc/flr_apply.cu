@@ -23,6 +23,7 @@
 // without the padding come by 4-byte asynchronous copies.  719 x 1277, q = 6, rc = 6: 43 us (123 us
 // before: 64 x 32 tiles, one column per thread, sums of run-time radius, 4-byte copies).
 #include <cstring>
+#include <type_traits>
 
 #include "flr.h"
 #include "flr_internal.cuh"
@@ -256,11 +257,8 @@ cudaError_t launch_apply_rc(int q, const ApplyArgs &a, cudaStream_t st)
 {
     constexpr ApplyGeom g(RC);
     constexpr size_t smem = sizeof(float) * g.floats();
-    cudaError_t e = cudaFuncSetAttribute(flr_apply_kernel<RC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     // two CTAs per SM need most of the unified L1 / shared array
-    e = cudaFuncSetAttribute(flr_apply_kernel<RC>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
+    cudaError_t e = pdl::allow_smem<std::integral_constant<int, RC>>(flr_apply_kernel<RC>, smem, true);
     if (e != cudaSuccess) return e;
     const int rows = (a.row_hi < 0 ? a.H : a.row_hi) - a.row_lo;
     if (rows <= 0) return cudaSuccess;

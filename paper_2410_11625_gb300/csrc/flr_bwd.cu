@@ -16,8 +16,11 @@
 // Every launch here is a dependent one (pdl.cuh) without an early trigger, as those of the unfused
 // forward path: backward 1920x1080 957 -> 946 us, 719 x 1277 forward, q = 6, 151 -> 146 us.
 #include <algorithm>
+#include <atomic>
 #include <cstring>
+#include <type_traits>
 
+#include "flr.h"
 #include "flr_internal.cuh"
 #include "pdl.cuh"
 #include "tma.cuh"
@@ -114,7 +117,7 @@ __global__ void __launch_bounds__(kBThreads) box_sum_kernel(const float *__restr
 // bounded (1 s).
 //
 // The planes' rows are padded to 16 bytes (coef_pitch), so that every width from 16 on comes this
-// way: backward 1919 x 1080, r = rc = 8, 1827 us at first, 1088 us so (same bits).
+// way: backward 1919 x 1080, r = rc = 8, 1827 us at first, 1089 us so (same bits).
 //
 // Bound by DRAM: the three calls of a 1080p backward pass (Q = 8) read and write 122 planes of
 // 8.3 MB, 298 us at the measured copy rate; they take 324 us.  The form before this was bound by
@@ -361,30 +364,52 @@ __device__ __forceinline__ float4 fma4(float4 a, float4 b, float4 c)
     return make_float4(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y), fmaf(a.z, b.z, c.z), fmaf(a.w, b.w, c.w));
 }
 
-template <int Q>
+// The caller's images: 16-byte rows (ALIGNED), or row by row of any width, n of the four pixels inside
+template <bool ALIGNED>
+__device__ __forceinline__ float4 ld4u(const float *p, int n)
+{
+    if (ALIGNED) return ld4(p);
+    return make_float4(__ldg(p), n > 1 ? __ldg(p + 1) : 0.f, n > 2 ? __ldg(p + 2) : 0.f, n > 3 ? __ldg(p + 3) : 0.f);
+}
+template <bool ALIGNED>
+__device__ __forceinline__ void st4u(float *p, float4 v, int n)
+{
+    if (ALIGNED) {
+        st4(p, v);
+        return;
+    }
+    p[0] = v.x;
+    if (n > 1) p[1] = v.y;
+    if (n > 2) p[2] = v.z;
+    if (n > 3) p[3] = v.w;
+}
+
+template <int Q, bool ALIGNED>
 __global__ void __launch_bounds__(256) bwd_contract4_kernel(const BwdArgs a)
 {
     using C = Chan<Q>;
     pdl::wait();
     const int H = a.H, W = a.W;
     const size_t plane = (size_t)H * W;
-    const size_t nq = plane / 4;
+    // BS and BA have padded rows of a.pitch floats (a.pitch = W when ALIGNED)
+    const int quads = a.pitch / 4;
+    const size_t bplane = (size_t)H * a.pitch, nq = (size_t)H * quads;
     for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += (size_t)gridDim.x * blockDim.x) {
-        const size_t p = 4 * q;
-        const int y = (int)(p / W), x0 = (int)(p % W);
+        const int y = (int)(q / quads), x0 = 4 * (int)(q % quads), n = W - x0;
+        const size_t p = (size_t)y * W + x0, bp = 4 * q;
         float4 xs[Q], ys[3], gc[3];
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            const float4 v = ld4(a.guide + i * plane + p);
+            const float4 v = ld4u<ALIGNED>(a.guide + i * plane + p, n);
             const float s = a.shift[i];
             xs[i] = make_float4(v.x - s, v.y - s, v.z - s, v.w - s);
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const float4 v = ld4(a.rad + c * plane + p);
+            const float4 v = ld4u<ALIGNED>(a.rad + c * plane + p, n);
             const float s = a.shift[Q + c];
             ys[c] = make_float4(v.x - s, v.y - s, v.z - s, v.w - s);
-            gc[c] = ld4(a.g + c * plane + p);
+            gc[c] = ld4u<ALIGNED>(a.g + c * plane + p, n);
         }
         float inv_m[4] = {1.f, 1.f, 1.f, 1.f};
         if (a.rc > 0) {
@@ -401,41 +426,44 @@ __global__ void __launch_bounds__(256) bwd_contract4_kernel(const BwdArgs a)
         const int one = blockIdx.y;
 #pragma unroll 1
         for (int i = all ? 0 : min(one, Q); i < (all ? Q : min(one + 1, Q)); ++i) {  // one channel's 15 planes in flight
-            float4 d = ld4(BS + (C::X0 + i) * plane + p);
+            float4 d = ld4(BS + (C::X0 + i) * bplane + bp);
 #pragma unroll
             for (int j = 0; j < Q; ++j) {
                 const int t = (i <= j ? C::xx(i, j) : C::xx(j, i));
-                const float4 b = ld4(BS + t * plane + p);
+                const float4 b = ld4(BS + t * bplane + bp);
                 d = fma4(make_float4(2.f * b.x, 2.f * b.y, 2.f * b.z, 2.f * b.w), xs[j], d);
             }
 #pragma unroll
-            for (int c = 0; c < 3; ++c) d = fma4(ld4(BS + C::xy(i, c) * plane + p), ys[c], d);
+            for (int c = 0; c < 3; ++c) d = fma4(ld4(BS + C::xy(i, c) * bplane + bp), ys[c], d);
             float4 dz = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) dz = fma4(ld4(a.BA + (3 * (i + 1) + c) * plane + p), gc[c], dz);
+            for (int c = 0; c < 3; ++c) dz = fma4(ld4(a.BA + (3 * (i + 1) + c) * bplane + bp), gc[c], dz);
             dz = make_float4(dz.x * inv_m[0], dz.y * inv_m[1], dz.z * inv_m[2], dz.w * inv_m[3]);
             if (a.separate_map) {
-                st4(a.grad_guide + i * plane + p, d);
-                if (a.grad_map) st4(a.grad_map + i * plane + p, dz);
+                st4u<ALIGNED>(a.grad_guide + i * plane + p, d, n);
+                if (a.grad_map) st4u<ALIGNED>(a.grad_map + i * plane + p, dz, n);
             } else {
-                st4(a.grad_guide + i * plane + p, make_float4(d.x + dz.x, d.y + dz.y, d.z + dz.z, d.w + dz.w));
+                st4u<ALIGNED>(a.grad_guide + i * plane + p, make_float4(d.x + dz.x, d.y + dz.y, d.z + dz.z, d.w + dz.w), n);
             }
         }
 #pragma unroll 1
         for (int c = all ? 0 : max(one - Q, 0); c < (all ? 3 : one - Q + 1); ++c) {
-            float4 d = ld4(BS + (C::Y0 + c) * plane + p);
+            float4 d = ld4(BS + (C::Y0 + c) * bplane + bp);
 #pragma unroll
-            for (int i = 0; i < Q; ++i) d = fma4(ld4(BS + C::xy(i, c) * plane + p), xs[i], d);
-            st4(a.grad_rad + c * plane + p, d);
+            for (int i = 0; i < Q; ++i) d = fma4(ld4(BS + C::xy(i, c) * bplane + bp), xs[i], d);
+            st4u<ALIGNED>(a.grad_rad + c * plane + p, d, n);
         }
     }
 }
 
 int sm_count()
 {
+    static std::atomic<int> known[64];
     int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return 1;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    if (dev >= 0 && dev < 64 && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
+    if (dev >= 0 && dev < 64) known[dev].store(n, std::memory_order_relaxed);
     return n;
 }
 
@@ -465,11 +493,10 @@ cudaError_t launch_box_sum_tma(const BoxKArgs &k, cudaStream_t st)
 {
     const BoxGeom g(k.rad);
     const size_t smem = sizeof(float) * g.floats();
-    cudaError_t e = cudaFuncSetAttribute(box_sum_tma_kernel<RT, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     // three CTAs per SM need most of the unified L1 / shared array as shared memory
-    e = cudaFuncSetAttribute(box_sum_tma_kernel<RT, PARTS>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
+    const BoxGeom most(RT >= 0 ? RT : 16);
+    static_assert(FLR_MAX_RADIUS == 16 && FLR_MAX_COEF_RADIUS == 16, "radii known at run time");
+    cudaError_t e = pdl::allow_smem<std::integral_constant<int, 2 * RT + PARTS>>(box_sum_tma_kernel<RT, PARTS>, sizeof(float) * most.floats(), true);
     if (e != cudaSuccess) return e;
     dim3 grid((k.W + kBW - 1) / kBW, (k.H + kTH - 1) / kTH, (k.nplanes + k.per_cta - 1) / k.per_cta);
     return pdl::launch(box_sum_tma_kernel<RT, PARTS>, grid, kTThreads, smem, st, k);
@@ -512,21 +539,25 @@ cudaError_t launch_box_sum(const float *in, float *out, int nplanes, int H, int 
 cudaError_t launch_bwd_contract(int q, const BwdArgs &a, cudaStream_t st)
 {
     auto al = [](const void *p) { return ((uintptr_t)p & 15) == 0; };
-    if ((a.W & 3) == 0 && al(a.guide) && al(a.rad) && al(a.g) && al(a.BS) && al(a.BA) && al(a.grad_guide) &&
-        al(a.grad_map) && al(a.grad_rad)) {
+    if ((a.pitch & 3) == 0 && al(a.BS) && al(a.BA)) {
         // one thread per four pixels; below two CTAs per SM (about 311k pixels, whose planes fit
-        // in L2) also one output channel per thread: 128 x 128 takes 14.8 us without, 4.0 us with
-        const int ctas = (int)(((size_t)a.H * a.W / 4 + 255) / 256);
+        // in L2) also one output channel per thread: 128 x 128 takes 14.8 us without, 4.0 us with.
+        // Images whose rows are not 16-byte aligned are read and written by single values beside the
+        // workspace's 16-byte loads (backward 1919 x 1080: 1052 us, with one thread per pixel 1089).
+        const bool aligned = (a.W & 3) == 0 && al(a.guide) && al(a.rad) && al(a.g) && al(a.grad_guide) && al(a.grad_map) &&
+                             al(a.grad_rad);
+        const int ctas = (int)(((size_t)a.H * (a.pitch / 4) + 255) / 256);
         const dim3 grid4(ctas, ctas < 2 * sm_count() ? q + 3 : 1);
+        auto launch = [&](auto with, auto without) { return pdl::launch(aligned ? with : without, grid4, 256, 0, st, a); };
         switch (q) {
-        case 1: return pdl::launch(bwd_contract4_kernel<1>, grid4, 256, 0, st, a);
-        case 2: return pdl::launch(bwd_contract4_kernel<2>, grid4, 256, 0, st, a);
-        case 3: return pdl::launch(bwd_contract4_kernel<3>, grid4, 256, 0, st, a);
-        case 4: return pdl::launch(bwd_contract4_kernel<4>, grid4, 256, 0, st, a);
-        case 5: return pdl::launch(bwd_contract4_kernel<5>, grid4, 256, 0, st, a);
-        case 6: return pdl::launch(bwd_contract4_kernel<6>, grid4, 256, 0, st, a);
-        case 7: return pdl::launch(bwd_contract4_kernel<7>, grid4, 256, 0, st, a);
-        case 8: return pdl::launch(bwd_contract4_kernel<8>, grid4, 256, 0, st, a);
+        case 1: return launch(bwd_contract4_kernel<1, true>, bwd_contract4_kernel<1, false>);
+        case 2: return launch(bwd_contract4_kernel<2, true>, bwd_contract4_kernel<2, false>);
+        case 3: return launch(bwd_contract4_kernel<3, true>, bwd_contract4_kernel<3, false>);
+        case 4: return launch(bwd_contract4_kernel<4, true>, bwd_contract4_kernel<4, false>);
+        case 5: return launch(bwd_contract4_kernel<5, true>, bwd_contract4_kernel<5, false>);
+        case 6: return launch(bwd_contract4_kernel<6, true>, bwd_contract4_kernel<6, false>);
+        case 7: return launch(bwd_contract4_kernel<7, true>, bwd_contract4_kernel<7, false>);
+        case 8: return launch(bwd_contract4_kernel<8, true>, bwd_contract4_kernel<8, false>);
         default: return cudaErrorInvalidValue;
         }
     }
