@@ -632,7 +632,8 @@ __device__ __forceinline__ void load_model(float (&m)[Model<Q>::CS], const float
 // pixels apart, so the P pixels of run r, [P r - P/2, P r + P/2), all interpolate between
 // block columns r - 1 and r (clamped at the edges): one thread per (output row, run) loads
 // the 4 x (Q+1) x 3 corner coefficients once, interpolates them vertically once, and
-// streams the run (vector loads and stores when the run is aligned and inside the image).
+// streams the run (vector loads and stores when the run is inside the image and starts on a
+// 16-byte boundary: column P r - P/2 is a multiple of 4 for every r only where P is one of 8).
 template <int Q>
 __device__ __forceinline__ void stage_apply(const FastArgs &a, size_t t)
 {
@@ -671,7 +672,7 @@ __device__ __forceinline__ void stage_apply(const FastArgs &a, size_t t)
 #pragma unroll
         for (int k = 0; k < Q + 3; ++k) sh[k] = a.shift[k];
         const size_t row = (size_t)yo * a.Wo;
-        const bool vec = (a.Wo & 3) == 0 && (P & 3) == 0 && xs >= 0 && xs + P <= a.Wo;
+        const bool vec = (a.Wo & 3) == 0 && (P & 7) == 0 && xs >= 0 && xs + P <= a.Wo;
         for (int x0 = 0; x0 < P; x0 += 4) {
             float o[3][4];
             float z[Q][4];

@@ -1,0 +1,54 @@
+"""The last stage's runs of P = factor * scale output pixels start at column P r - P/2: a 16-byte
+boundary only where P is a multiple of 8.  Cells of 4 pixels (parameter gradients take the runs at
+every P) and of 12, 20 and 28 (too wide for the tiled last stage), on output rows that are
+16-byte aligned themselves, against the FP64 oracle at the bars of test_flr_fast_gpu, whose
+derivation does not depend on P; a batch of such frames equals the single calls bit for bit."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from helpers import to_dev
+from test_flr_fast_gpu import check, flr  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("factor,scale,H,W", [(4, 3, 60, 100), (2, 6, 31, 52), (4, 5, 40, 64), (4, 7, 25, 40), (8, 3, 32, 48)])
+def test_wide_cells(flr, factor, scale, H, W):  # noqa: F811
+    g, y = synth.render(4, H, W)
+    z, _ = synth.render(4, H * scale, W * scale)
+    check(flr, g, y, z=z, scale=scale, factor=factor, rms_bar=True)
+
+
+@pytest.mark.parametrize("factor,scale,H,W", [(4, 1, 96, 160), (2, 2, 48, 80), (4, 3, 32, 48), (2, 1, 49, 80)])
+def test_parameter_gradients(flr, factor, scale, H, W):  # noqa: F811
+    import torch
+    g, y = synth.render(12, H, W)
+    z = synth.render(12, H * scale, W * scale)[0] if scale > 1 else None
+    kw = dict(factor=factor, sigma_blocks=1.1, taps=3, eps=2e-3, map_guide=z, scale=scale)
+    out = oracle.flr_fast(g, y, **kw)
+    G = (out - 0.9 * np.mean(out, axis=(1, 2), keepdims=True)).astype(np.float32)
+    ref = oracle.flr_fast_param_grads(g, y, G, **kw)
+    f = flr.FastFLR(q=8, factor=factor, scale=scale, sigma=1.1, taps=3, eps=2e-3)
+    got = f.param_grad(to_dev(g), to_dev(y), to_dev(G), map_guide=None if z is None else to_dev(z))
+    torch.cuda.synchronize()
+    got = got.cpu().numpy()
+    f.close()
+    for t, name in enumerate(["sigma", "eps"]):
+        assert abs(got[t] - ref[name]) <= 1e-4 * abs(ref[name]), (name, got[t], ref[name])
+
+
+def test_batch_of_wide_cells(flr):  # noqa: F811
+    import torch
+    f = flr.FastFLR(q=8, factor=4, scale=3)
+    frames = []
+    for k, (H, W) in enumerate([(20, 36), (17, 40), (23, 37)]):
+        g, y = synth.random_frame(60 + k, H, W, 8)
+        z, _ = synth.random_frame(70 + k, 3 * H, 3 * W, 8)
+        frames.append((to_dev(g), to_dev(y), to_dev(z), torch.full((3, 3 * H, 3 * W), float("nan"), device="cuda")))
+    f.denoise_batch(frames)
+    assert f.batch_status() == 0
+    for g, y, z, o in frames:
+        assert torch.equal(f.denoise(g, y, map_guide=z), o)
+    f.close()
