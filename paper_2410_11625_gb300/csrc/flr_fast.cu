@@ -102,13 +102,47 @@ __global__ void __launch_bounds__(kBlurThreads, 2) blur_v_solve_kernel(const __g
                                 kBlurThreads);
 }
 
+// Stage 4 for frames whose rows do not start on 16-byte boundaries, cells of more than 8 rows and
+// the parameter gradients: as apply_tma_kernel below, with plain loads of the map guide.  One item
+// per CTA: kFW output columns of up to kApplyRows rows of a cell row (a cell has up to 64).
+// Coalesced in every access, four CTAs per SM, the loads of two rows in flight per thread.  With one
+// thread per run of P pixels of a row (each reading its four block-major models for that row
+// alone) four 1080x1919 frames took 470 us, so 250; 16 frames of 540x960 from 270x480, F = 8, 348
+// and 144; one 1080x1919 frame 119 and 72.
+constexpr int kFW = 128, kApplyRows = 8;
+
+__host__ __device__ inline int apply_parts(int P) { return (P + kApplyRows - 1) / kApplyRows; }
+
 template <int Q, int N>
-__global__ void __launch_bounds__(256) fast_apply_kernel(const __grid_constant__ FrameTable<N> t)
+__global__ void __launch_bounds__(kFW, 4) fast_apply_kernel(const __grid_constant__ FrameTable<N> t)
 {
+    using M = fast::Model<Q>;
+    const int f = frame_of(t, 3, blockIdx.x);
+    const FastArgs &a = t.f[f];
+    const int P = a.F * a.s, ncx = (a.Wo + kFW - 1) / kFW, parts = apply_parts(P);
+    const int local = (int)(blockIdx.x - t.off[3][f]), cx = local % ncx, part = local / ncx % parts, ci = local / ncx / parts;
+    const int x = cx * kFW + (int)threadIdx.x, ya = P * ci - P / 2;
+    const int t0 = max(kApplyRows * part, -ya), t1 = min(min(kApplyRows * (part + 1), P), a.Ho - ya);
     pdl::wait();
-    for (unsigned item = blockIdx.x; item < t.off[3][t.n]; item += gridDim.x) {
-        const int f = frame_of(t, 3, item);
-        fast::stage_apply<Q>(t.f[f], (size_t)(item - t.off[3][f]) * 256 + threadIdx.x);
+    if (x >= a.Wo || t0 >= t1) return;
+    float2 top[M::CS / 2], dtb[M::CS / 2], nsh[M::QE / 2];
+    float shr[3];
+    const size_t oplane = (size_t)a.Ho * a.Wo, off = (size_t)(ya + t0) * a.Wo + x;
+    const float *zp = a.map_guide + off;
+    float *out = a.out + off;
+    const int i0 = fast::column_models<Q>(a, P, x, ya, top, dtb);
+    fast::load_reference<Q>(a, nsh, shr);
+    for (int r = t0; r < t1; r += 2, zp += 2 * (size_t)a.Wo, out += 2 * (size_t)a.Wo) {
+        const bool two = r + 1 < t1;
+        float z0[Q], z1[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            z0[i] = __ldg(zp + i * oplane);
+            z1[i] = two ? __ldg(zp + i * oplane + a.Wo) : 0.f;
+        }
+        fast::apply_pixel<Q>(a, P, ya + r, i0, top, dtb, nsh, shr, [&](int i) { return z0[i]; }, out, oplane);
+        if (two)
+            fast::apply_pixel<Q>(a, P, ya + r + 1, i0, top, dtb, nsh, shr, [&](int i) { return z1[i]; }, out + a.Wo, oplane);
     }
 }
 
@@ -158,7 +192,6 @@ __global__ void __launch_bounds__(256) dot_final_kernel(const double *part, doub
 // computed), so the bytes in flight do not depend on registers per thread.  The copy
 // engine zero-fills outside the image.  Waits are bounded (1 s) and report through the
 // status word.
-constexpr int kFW = 128;
 constexpr unsigned long long kFastTimeoutNs = 1000000000ull;
 
 template <int N>
@@ -172,25 +205,21 @@ __device__ __forceinline__ float *align128(float *p)
     return p + (((128 - (tma::smem_addr(p) & 127)) & 127) >> 2);
 }
 
-// Stage 4 with TMA: item (cell row i, column chunk cx).  Cell row i is the P = F s output
-// rows [P i - P/2, P i + P/2), which all interpolate between the same two block rows; the
-// item loads those rows of the Q map-guide planes.  Thread t owns output column kFW cx + t:
-// it interpolates its corner models horizontally once per item (top and bottom block row),
-// while the item's rows are still on their way, then for each row vertically, and applies them,
-// two guides per instruction (packed FP32).  The coordinates are the exact rational ones of
-// fast::stage_apply.  PC: P known at compile time (the weights' divisions become products), or 0.
+// Stage 4 with TMA: item (cell row i, column chunk cx), the P rows of the Q map-guide planes.  The
+// corner models are interpolated horizontally while the item's rows are still on their way.  PC: P
+// known at compile time (the weights' divisions become products), or 0.
 template <int Q, int N, int PC>
 __global__ void __launch_bounds__(kFW, 3) apply_tma_kernel(const __grid_constant__ FastKArgs<N> k)
 {
     using M = fast::Model<Q>;
-    constexpr int PMAX = 8, STAGE = Q * PMAX * kFW, CS = M::CS, QE = M::QE;
+    constexpr int PMAX = 8, STAGE = Q * PMAX * kFW;
     extern __shared__ __align__(16) float smem[];
     float *base = align128(smem);
     uint64_t *bar = reinterpret_cast<uint64_t *>(base + 2 * STAGE);
     __shared__ int s_abort;
     const int tid = threadIdx.x, lane = tid & 31;
     const unsigned nitems = k.t.off[3][k.t.n];
-    const int P = PC ? PC : k.t.f[0].F * k.t.f[0].s, den = 2 * P;  // the handle's: the same for every frame
+    const int P = PC ? PC : k.t.f[0].F * k.t.f[0].s;  // the handle's: the same for every frame
     int *status = k.t.f[0].status;
     if (tid == 0) {
         s_abort = 0;
@@ -223,39 +252,10 @@ __global__ void __launch_bounds__(kFW, 3) apply_tma_kernel(const __grid_constant
         const int ci = local / ncx, cx = local % ncx;
         const int x = min(cx * kFW + tid, a.Wo - 1);
         const int ya = P * ci - P / 2;       // first output row of the cell (may be < 0)
-        // block rows of the cell (the same for all its rows)
-        const int ny0 = min(max(2 * max(ya, 0) + 1 - P, 0), (a.Hb - 1) * den);
-        const int i0 = min(ny0 / den, max(a.Hb - 2, 0)), i1 = min(i0 + 1, a.Hb - 1);
-        float2 top[CS / 2], dtb[CS / 2];  // horizontally interpolated top row, bottom minus top
-        {
-            // block columns and weight of this column
-            const int r = (x + P / 2) / P;
-            const int jl = min(max(r - 1, 0), a.Wb - 1), jr = min(max(r, 0), a.Wb - 1);
-            const int nx = min(max(2 * x + 1 - P, 0), (a.Wb - 1) * den);
-            const float fx = fminf(fmaxf((float)(nx - (r - 1) * den) / (float)den, 0.f), 1.f);
-            const float4 *l0 = reinterpret_cast<const float4 *>(a.coef + ((size_t)i0 * a.Wb + jl) * CS);
-            const float4 *l1 = reinterpret_cast<const float4 *>(a.coef + ((size_t)i1 * a.Wb + jl) * CS);
-            const int step = (jr - jl) * (CS / 4);
-            const float2 fx2 = make_float2(fx, fx), minus = make_float2(-1.f, -1.f);
-#pragma unroll
-            for (int c = 0; c < CS / 4; ++c) {
-                const float4 tl = __ldg(l0 + c), tr = __ldg(l0 + step + c), bl = __ldg(l1 + c), br = __ldg(l1 + step + c);
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const float2 t0 = h ? make_float2(tl.z, tl.w) : make_float2(tl.x, tl.y);
-                    const float2 t1 = h ? make_float2(tr.z, tr.w) : make_float2(tr.x, tr.y);
-                    const float2 b0 = h ? make_float2(bl.z, bl.w) : make_float2(bl.x, bl.y);
-                    const float2 b1 = h ? make_float2(br.z, br.w) : make_float2(br.x, br.y);
-                    const float2 tp = __ffma2_rn(fx2, __ffma2_rn(t0, minus, t1), t0);
-                    top[2 * c + h] = tp;
-                    dtb[2 * c + h] = __ffma2_rn(tp, minus, __ffma2_rn(fx2, __ffma2_rn(b0, minus, b1), b0));
-                }
-            }
-        }
-        float2 nsh[QE / 2];  // minus the frame reference, in pairs
-#pragma unroll
-        for (int i = 0; i < QE; i += 2) nsh[i / 2] = make_float2(-a.shift[i], i + 1 < Q ? -a.shift[i + 1] : 0.f);
-        const float shr[3] = {a.shift[Q], a.shift[Q + 1], a.shift[Q + 2]};
+        float2 top[M::CS / 2], dtb[M::CS / 2], nsh[M::QE / 2];
+        float shr[3];
+        const int i0 = fast::column_models<Q>(a, P, x, ya, top, dtb);
+        fast::load_reference<Q>(a, nsh, shr);
         if (!tma::wait_warp(bar + st, (uint32_t)((it >> 1) & 1), kFastTimeoutNs) && lane == 0) {
             s_abort = 1;
             if (status) atomicExch(status, 1);
@@ -268,27 +268,8 @@ __global__ void __launch_bounds__(kFW, 3) apply_tma_kernel(const __grid_constant
             const int t0 = max(-ya, 0), t1 = min(P, a.Ho - ya);
             float *out = a.out + (size_t)(ya + t0) * a.Wo + x;
 #pragma unroll 2
-            for (int t = t0; t < t1; ++t, out += a.Wo) {
-                const int ny = min(max(2 * (ya + t) + 1 - P, 0), (a.Hb - 1) * den);
-                const float fy = (float)(ny - i0 * den) / (float)den;
-                const float2 fy2 = make_float2(fy, fy), one = make_float2(1.f, 1.f);
-                float2 z[QE / 2], o2[3];
-#pragma unroll
-                for (int i = 0; i < QE; i += 2)
-                    z[i / 2] = __ffma2_rn(make_float2(T[(i * P + t) * kFW], i + 1 < Q ? T[((i + 1) * P + t) * kFW] : 0.f),
-                                          one, nsh[i / 2]);
-                float bias[3] = {fmaf(fy, dtb[0].x, top[0].x), fmaf(fy, dtb[0].y, top[0].y), fmaf(fy, dtb[1].x, top[1].x)};
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    o2[c] = make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int i = 0; i < QE; i += 2) {
-                        const int m = M::at(c, i) / 2;
-                        o2[c] = __ffma2_rn(__ffma2_rn(fy2, dtb[m], top[m]), z[i / 2], o2[c]);
-                    }
-                    __stcs(out + c * oplane, (bias[c] + (o2[c].x + o2[c].y)) + shr[c]);  // streamed: not kept in L2
-                }
-            }
+            for (int t = t0; t < t1; ++t, out += a.Wo)
+                fast::apply_pixel<Q>(a, P, ya + t, i0, top, dtb, nsh, shr, [&](int i) { return T[(i * P + t) * kFW]; }, out, oplane);
         }
         __syncthreads();  // stage st is read; the next iteration may refill it
     }
@@ -350,17 +331,15 @@ cudaError_t launch_moments_f(const FrameTable<N> &t, cudaStream_t st)
     }
 }
 
-// One thread per output-row run, any row alignment and any P: the frames of t, whose stage-4
-// items are counted here.
+// Any row alignment and any P: the frames of t, whose stage-4 items are counted here.
 template <int Q, int N>
-cudaError_t launch_apply_runs(FrameTable<N> &t, cudaStream_t st)
+cudaError_t launch_apply_plain(FrameTable<N> &t, cudaStream_t st)
 {
     for (int i = 0; i < t.n; ++i) {
-        const size_t runs = (size_t)t.f[i].Ho * (t.f[i].Wo / (t.f[i].F * t.f[i].s) + 2);
-        t.off[3][i + 1] = t.off[3][i] + (unsigned)((runs + 255) / 256);
+        const FastArgs &a = t.f[i];
+        t.off[3][i + 1] = t.off[3][i] + (unsigned)(a.Hb + 1) * apply_parts(a.F * a.s) * ((a.Wo + kFW - 1) / kFW);
     }
-    const unsigned ctas = t.off[3][t.n];
-    return pdl::launch(fast_apply_kernel<Q, N>, dim3(ctas < 16384 ? ctas : 16384), 256, 0, st, t);
+    return pdl::launch(fast_apply_kernel<Q, N>, dim3(t.off[3][t.n]), kFW, 0, st, t);
 }
 
 // Stage 4.  Frames whose rows start on 16-byte boundaries, with P <= 8, take the TMA kernel; the
@@ -398,7 +377,7 @@ cudaError_t launch_apply_fast(const FrameTable<N> &all, cudaStream_t st)
         if (e != cudaSuccess || nr == 0) return e;
     }
     fill_table(rest, nr, run_f, all.count, all.status);
-    return launch_apply_runs<Q>(rest, st);
+    return launch_apply_plain<Q>(rest, st);
 }
 
 // The four stages over n frames: each launch may start while its predecessor drains (pdl.cuh),
@@ -457,7 +436,7 @@ cudaError_t launch_param_grad_q(const FastArgs &a, unsigned long long *count, fl
         tp.f[0].coef = a.dcoef + (size_t)p * nb * fast::Model<Q>::CS;
         tp.f[0].shift = tshift;
         tp.f[0].out = dout;
-        if ((e = launch_apply_runs<Q>(tp, st)) != cudaSuccess) return e;
+        if ((e = launch_apply_plain<Q>(tp, st)) != cudaSuccess) return e;
         dot_partial_kernel<<<kDotBlocks, 256, 0, st>>>(dout, grad_out, npx, part);
         dot_final_kernel<<<1, kDotBlocks, 0, st>>>(part, grad + p);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;

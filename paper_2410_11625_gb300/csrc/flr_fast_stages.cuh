@@ -615,117 +615,85 @@ __device__ __forceinline__ void stage_blur_v_tangent(const FastArgs &a, size_t k
     }
 }
 
+// 4. bilinear interpolation of the block models + apply.  Block centres are P = F s output pixels
+// apart, so the output rows [P i - P/2, P i + P/2) of cell row i interpolate between the same two
+// block rows: a thread takes one output column of a cell row and interpolates its four corner
+// models horizontally once, then each row's model vertically, two guides per instruction (packed
+// FP32).
+//
+// column_models: the models of output column x, the cell row beginning at output row ya (< 0 for
+// the first): the upper block row's, and lower minus upper.  Returns the upper block row.
 template <int Q>
-__device__ __forceinline__ void load_model(float (&m)[Model<Q>::CS], const float *src)
+__device__ __forceinline__ int column_models(const FastArgs &a, int P, int x, int ya, float2 (&top)[Model<Q>::CS / 2],
+                                             float2 (&dtb)[Model<Q>::CS / 2])
 {
+    constexpr int CS = Model<Q>::CS;
+    const int den = 2 * P;
+    // block rows of the cell (the same for all its rows)
+    const int ny0 = min(max(2 * max(ya, 0) + 1 - P, 0), (a.Hb - 1) * den);
+    const int i0 = min(ny0 / den, max(a.Hb - 2, 0)), i1 = min(i0 + 1, a.Hb - 1);
+    // block columns and weight of this column (exact rational coordinate (2 x + 1 - P) / (2 P))
+    const int r = (x + P / 2) / P;
+    const int jl = min(max(r - 1, 0), a.Wb - 1), jr = min(max(r, 0), a.Wb - 1);
+    const int nx = min(max(2 * x + 1 - P, 0), (a.Wb - 1) * den);
+    const float fx = fminf(fmaxf((float)(nx - (r - 1) * den) / (float)den, 0.f), 1.f);
+    const float4 *l0 = reinterpret_cast<const float4 *>(a.coef + ((size_t)i0 * a.Wb + jl) * CS);
+    const float4 *l1 = reinterpret_cast<const float4 *>(a.coef + ((size_t)i1 * a.Wb + jl) * CS);
+    const int step = (jr - jl) * (CS / 4);
+    const float2 fx2 = make_float2(fx, fx), minus = make_float2(-1.f, -1.f);
 #pragma unroll
-    for (int k = 0; k < Model<Q>::CS; k += 4) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(src + k));
-        m[k] = v.x;
-        m[k + 1] = v.y;
-        m[k + 2] = v.z;
-        m[k + 3] = v.w;
+    for (int c = 0; c < CS / 4; ++c) {
+        const float4 tl = __ldg(l0 + c), tr = __ldg(l0 + step + c), bl = __ldg(l1 + c), br = __ldg(l1 + step + c);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float2 t0 = h ? make_float2(tl.z, tl.w) : make_float2(tl.x, tl.y);
+            const float2 t1 = h ? make_float2(tr.z, tr.w) : make_float2(tr.x, tr.y);
+            const float2 b0 = h ? make_float2(bl.z, bl.w) : make_float2(bl.x, bl.y);
+            const float2 b1 = h ? make_float2(br.z, br.w) : make_float2(br.x, br.y);
+            const float2 tp = __ffma2_rn(fx2, __ffma2_rn(t0, minus, t1), t0);
+            top[2 * c + h] = tp;
+            dtb[2 * c + h] = __ffma2_rn(tp, minus, __ffma2_rn(fx2, __ffma2_rn(b0, minus, b1), b0));
+        }
     }
+    return i0;
 }
 
-// 4. bilinear interpolation of the block models + apply.  Block centres are P = F s output
-// pixels apart, so the P pixels of run r, [P r - P/2, P r + P/2), all interpolate between
-// block columns r - 1 and r (clamped at the edges): one thread per (output row, run) loads
-// the 4 x (Q+1) x 3 corner coefficients once, interpolates them vertically once, and
-// streams the run (vector loads and stores when the run is inside the image and starts on a
-// 16-byte boundary: column P r - P/2 is a multiple of 4 for every r only where P is one of 8).
+// The frame reference: minus the guides' in pairs, and the radiance's
 template <int Q>
-__device__ __forceinline__ void stage_apply(const FastArgs &a, size_t t)
+__device__ __forceinline__ void load_reference(const FastArgs &a, float2 (&nsh)[Model<Q>::QE / 2], float (&shr)[3])
+{
+#pragma unroll
+    for (int i = 0; i < Model<Q>::QE; i += 2) nsh[i / 2] = make_float2(-a.shift[i], i + 1 < Q ? -a.shift[i + 1] : 0.f);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) shr[c] = a.shift[Q + c];
+}
+
+// apply_pixel: the model of output row y of that column, applied to the map guide z(i), i < Q, into
+// out[c * oplane]
+template <int Q, class Z>
+__device__ __forceinline__ void apply_pixel(const FastArgs &a, int P, int y, int i0, const float2 (&top)[Model<Q>::CS / 2],
+                                            const float2 (&dtb)[Model<Q>::CS / 2], const float2 (&nsh)[Model<Q>::QE / 2],
+                                            const float (&shr)[3], Z z, float *out, size_t oplane)
 {
     using M = Model<Q>;
-    const size_t oplane = (size_t)a.Ho * a.Wo;
-    const int P = a.F * a.s, den = 2 * P;
-    const int nruns = a.Wo / P + 2;
-    const size_t total = (size_t)a.Ho * nruns;
-    if (t >= total) return;
-    {
-        const int yo = (int)(t / nruns), r = (int)(t % nruns);
-        const int xs = P * r - P / 2;
-        if (xs >= a.Wo) return;
-        // rows: i0, i1, fy (exact rational coordinate (2 yo + 1 - P) / (2 P))
-        int ny = min(max(2 * yo + 1 - P, 0), (a.Hb - 1) * den);
-        const int i0 = min(ny / den, max(a.Hb - 2, 0)), i1 = min(i0 + 1, a.Hb - 1);
-        const float fy = (float)(ny - i0 * den) / (float)den;
-        const int jl = min(max(r - 1, 0), a.Wb - 1), jr = min(max(r, 0), a.Wb - 1);
-        // corner models: left values and right-minus-left differences of the two block rows
-        // (interpolated horizontally, then vertically, per pixel: the same order and the same
-        // roundings as the TMA apply kernel, so both paths agree bit for bit)
-        float l0[M::CS], d0[M::CS], l1[M::CS], d1[M::CS];
-        {
-            const float *row0 = a.coef + (size_t)i0 * a.Wb * M::CS, *row1 = a.coef + (size_t)i1 * a.Wb * M::CS;
-            load_model<Q>(l0, row0 + (size_t)jl * M::CS);
-            load_model<Q>(d0, row0 + (size_t)jr * M::CS);
-            load_model<Q>(l1, row1 + (size_t)jl * M::CS);
-            load_model<Q>(d1, row1 + (size_t)jr * M::CS);
+    const int den = 2 * P;
+    const int ny = min(max(2 * y + 1 - P, 0), (a.Hb - 1) * den);
+    const float fy = (float)(ny - i0 * den) / (float)den;
+    const float2 fy2 = make_float2(fy, fy), one = make_float2(1.f, 1.f);
+    float2 zs[M::QE / 2], o2[3];
 #pragma unroll
-            for (int k = 0; k < M::CS; ++k) {
-                d0[k] -= l0[k];
-                d1[k] -= l1[k];
-            }
+    for (int i = 0; i < M::QE; i += 2)
+        zs[i / 2] = __ffma2_rn(make_float2(z(i), i + 1 < Q ? z(i + 1) : 0.f), one, nsh[i / 2]);
+    float bias[3] = {fmaf(fy, dtb[0].x, top[0].x), fmaf(fy, dtb[0].y, top[0].y), fmaf(fy, dtb[1].x, top[1].x)};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        o2[c] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < M::QE; i += 2) {
+            const int m = M::at(c, i) / 2;
+            o2[c] = __ffma2_rn(__ffma2_rn(fy2, dtb[m], top[m]), zs[i / 2], o2[c]);
         }
-        float sh[Q + 3];
-#pragma unroll
-        for (int k = 0; k < Q + 3; ++k) sh[k] = a.shift[k];
-        const size_t row = (size_t)yo * a.Wo;
-        const bool vec = (a.Wo & 3) == 0 && (P & 7) == 0 && xs >= 0 && xs + P <= a.Wo;
-        for (int x0 = 0; x0 < P; x0 += 4) {
-            float o[3][4];
-            float z[Q][4];
-            const int xb = xs + x0;
-            if (vec) {
-#pragma unroll
-                for (int i = 0; i < Q; ++i) {
-                    const float4 v = __ldg(reinterpret_cast<const float4 *>(a.map_guide + i * oplane + row + xb));
-                    z[i][0] = v.x; z[i][1] = v.y; z[i][2] = v.z; z[i][3] = v.w;
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < Q; ++i)
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int x = xb + u;
-                        z[i][u] = (x >= 0 && x < a.Wo && x0 + u < P) ? __ldg(a.map_guide + i * oplane + row + x) : 0.f;
-                    }
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int x = xb + u;
-                int nx = min(max(2 * x + 1 - P, 0), (a.Wb - 1) * den);
-                const float fx = fminf(fmaxf((float)(nx - (r - 1) * den) / (float)den, 0.f), 1.f);
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    // even and odd guides in two sums, as the pairs of the TMA apply
-                    float top = fmaf(fx, d0[c], l0[c]);
-                    const float bias = fmaf(fy, fmaf(fx, d1[c], l1[c]) - top, top);
-                    float sum[2] = {0.f, 0.f};
-#pragma unroll
-                    for (int i = 0; i < Q; ++i) {
-                        const int k = M::at(c, i);
-                        top = fmaf(fx, d0[k], l0[k]);
-                        sum[i & 1] = fmaf(fmaf(fy, fmaf(fx, d1[k], l1[k]) - top, top), z[i][u] - sh[i], sum[i & 1]);
-                    }
-                    o[c][u] = (bias + (sum[0] + sum[1])) + sh[Q + c];
-                }
-            }
-            if (vec) {
-#pragma unroll
-                for (int c = 0; c < 3; ++c)
-                    *reinterpret_cast<float4 *>(a.out + c * oplane + row + xb) = make_float4(o[c][0], o[c][1], o[c][2], o[c][3]);
-            } else {
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int x = xb + u;
-                    if (x >= 0 && x < a.Wo && x0 + u < P)
-#pragma unroll
-                        for (int c = 0; c < 3; ++c) a.out[c * oplane + row + x] = o[c][u];
-                }
-            }
-        }
+        __stcs(out + c * oplane, (bias[c] + (o2[c].x + o2[c].y)) + shr[c]);  // streamed: not kept in L2
     }
 }
 
