@@ -332,7 +332,7 @@ typedef struct flr_frame {
 } flr_frame;
 
 #define FLR_MAX_BATCH 16
-#define FLR_BATCH_TIMEOUT 1 /* device status word value after a barrier wait ran out */
+#define FLR_BATCH_TIMEOUT 1 /* device status word value after a wait ran out */
 
 /*
  * The per-pixel FLR pass (flr_denoise, Sec. 3.1-3.2) over n frames of any sizes, in order, on
@@ -375,6 +375,16 @@ int flr_barrier_selftest(int ctas, unsigned long long timeout_ns, int *status);
  * involved.  Not a paper operation.  Errors: FLR_ERR_ARG, FLR_ERR_NOMEM, FLR_ERR_CUDA.
  */
 int flr_mbarrier_selftest(int ctas, unsigned long long timeout_ns, int *status);
+
+/*
+ * Self-test of the fast path's last stage when its waits run out: the kernel runs on a small
+ * frame of its own, first with waits that give up at once while two copies per CTA are in
+ * flight (they land before the CTA exits), then as ever.  *status receives bit 0 if the first
+ * pass recorded the timeout and bit 1 if the second one recorded any or gave a wrong output
+ * (a failure); so 1 is a pass.  No fault is involved.  Not a paper operation.
+ * Errors: FLR_ERR_ARG, FLR_ERR_NOMEM, FLR_ERR_CUDA.
+ */
+int flr_fast_abort_selftest(int *status);
 
 /*
  * FLNR (Sec. 3.3, "Fast Local Neural Regression"): a U-Net maps the guides and the noisy

@@ -25,6 +25,7 @@
 #include <cstring>
 #include <new>
 #include <utility>
+#include <vector>
 
 #include "flr.h"
 #include "flr_fast_stages.cuh"
@@ -198,6 +199,7 @@ template <int N>
 struct alignas(128) FastKArgs {
     CUtensorMap t0[N];  // map-guide planes [Q][Ho][Wo], box (kFW, P, Q)
     FrameTable<N> t;
+    unsigned long long wait_ns;  // limit of a wait for a copy (0: gives up at once, the self-test)
 };
 
 __device__ __forceinline__ float *align128(float *p)
@@ -256,12 +258,18 @@ __global__ void __launch_bounds__(kFW, 3) apply_tma_kernel(const __grid_constant
         float shr[3];
         const int i0 = fast::column_models<Q>(a, P, x, ya, top, dtb);
         fast::load_reference<Q>(a, nsh, shr);
-        if (!tma::wait_warp(bar + st, (uint32_t)((it >> 1) & 1), kFastTimeoutNs) && lane == 0) {
+        if (!(k.wait_ns && tma::wait_warp(bar + st, (uint32_t)((it >> 1) & 1), k.wait_ns)) && lane == 0) {
             s_abort = 1;
             if (status) atomicExch(status, 1);
         }
         __syncthreads();
-        if (s_abort) break;
+        if (s_abort) {  // let the copies in flight, this item's and the next one's, land before the CTA exits
+            if (tid < 32) {
+                tma::wait_warp(bar + st, (uint32_t)((it >> 1) & 1), kFastTimeoutNs);
+                if (item + gridDim.x < nitems) tma::wait_warp(bar + (st ^ 1), (uint32_t)(((it + 1) >> 1) & 1), kFastTimeoutNs);
+            }
+            break;
+        }
         const float *T = base + st * STAGE + tid;  // [Q][P][kFW]
         if (cx * kFW + tid < a.Wo) {
             const size_t oplane = (size_t)a.Ho * a.Wo;
@@ -352,6 +360,7 @@ cudaError_t launch_apply_fast(const FrameTable<N> &all, cudaStream_t st)
     FastArgs tma_f[N], run_f[N];
     int nt = 0, nr = 0;
     std::memset(&k, 0, sizeof(k));
+    k.wait_ns = kFastTimeoutNs;
     for (int i = 0; i < all.n; ++i) {
         const FastArgs &a = all.f[i];
         const int P = a.F * a.s;
@@ -511,6 +520,55 @@ __global__ void mbarrier_selftest_kernel(int *status, unsigned long long timeout
         if (!done0) atomicOr(status, 1);
         if (!done1) atomicOr(status, 2);
     }
+}
+
+// Self-test of apply_tma_kernel's way out: a frame of zero models on four CTAs of nine items each,
+// once with waits that give up at once, so that every CTA leaves with two copies in flight, and
+// once with the ordinary limit into an output of NaNs.
+cudaError_t abort_selftest(int *result)
+{
+    constexpr int Q = 8, F = 8, H = 64, W = 512, Hb = H / F, Wb = W / F, CS = fast::Model<Q>::CS;
+    constexpr size_t px = (size_t)H * W, nz = Q * px, nc = (size_t)Hb * Wb * CS, total = nz + nc + 32 + 3 * px;
+    float *buf = nullptr;
+    cudaError_t e = cudaMalloc(&buf, total * sizeof(float));
+    if (e != cudaSuccess) return e;
+    FastKArgs<1> k;
+    std::memset(&k, 0, sizeof(k));
+    FastArgs a = {};
+    a.map_guide = buf;
+    a.coef = buf + nz;
+    a.shift = a.coef + nc;
+    a.status = (int *)(a.shift + 16);
+    a.out = a.shift + 32;
+    a.Hi = a.Ho = H;
+    a.Wi = a.Wo = W;
+    a.Hb = Hb;
+    a.Wb = Wb;
+    a.F = F;
+    a.s = 1;
+    fill_table(k.t, 1, &a, (unsigned long long *)nullptr, (int *)nullptr);
+    k.t.off[3][1] = (Hb + 1) * (W / kFW);
+    const size_t smem = apply_tma_smem<Q>();
+    e = tma::encode_planes_f32(&k.t0[0], a.map_guide, W, H, Q, kFW, F, Q);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(apply_tma_kernel<Q, 1, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    std::vector<float> out(3 * px);
+    *result = 0;
+    for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
+        int status = 0;
+        k.wait_ns = pass ? kFastTimeoutNs : 0;
+        e = cudaMemset(buf, 0, (nz + nc + 32) * sizeof(float));
+        if (e == cudaSuccess) e = cudaMemset(a.out, 0xff, 3 * px * sizeof(float));
+        if (e == cudaSuccess) e = pdl::launch(apply_tma_kernel<Q, 1, 8>, dim3(4), kFW, smem, (cudaStream_t)0, k);
+        if (e == cudaSuccess) e = cudaMemcpy(&status, a.status, sizeof(int), cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess) e = cudaMemcpy(out.data(), a.out, 3 * px * sizeof(float), cudaMemcpyDeviceToHost);
+        bool zero = true;
+        for (float v : out) zero &= v == 0.f;
+        if (pass == 0 && status != 0) *result |= 1;
+        if (pass == 1 && (status != 0 || !zero)) *result |= 2;
+    }
+    cudaFree(buf);
+    return e;
 }
 
 thread_local char g_fast_err[256] = "no error";
@@ -786,6 +844,13 @@ int flr_mbarrier_selftest(int ctas, unsigned long long timeout_ns, int *status)
     if (e == cudaSuccess) e = cudaMemcpy(status, d, sizeof(int), cudaMemcpyDeviceToHost);
     cudaFree(d);
     return e == cudaSuccess ? FLR_OK : FLR_ERR_CUDA;
+}
+
+int flr_fast_abort_selftest(int *status)
+{
+    if (!status) return FLR_ERR_ARG;
+    const cudaError_t e = flr::abort_selftest(status);
+    return e == cudaSuccess ? FLR_OK : e == cudaErrorMemoryAllocation ? FLR_ERR_NOMEM : FLR_ERR_CUDA;
 }
 
 int flr_fast_param_grad(flr_fast_handle *h, const float *guide, const float *map_guide, const float *radiance,

@@ -22,7 +22,7 @@ EXPORTS = ("flr_create", "flr_destroy", "flr_reserve", "flr_denoise", "flr_denoi
            "flr_denoise_noalloc", "flr_backward", "flr_fast_create", "flr_fast_destroy",
            "flr_set_concurrency", "flr_fast_denoise", "flr_fast_get_stats", "flr_fast_param_grad", "flr_denoise_batch", "flr_fast_reserve_batch",
            "flr_fast_denoise_batch", "flr_fast_batch_status", "flr_barrier_selftest",
-           "flr_mbarrier_selftest", "flr_host_band_plan",
+           "flr_mbarrier_selftest", "flr_fast_abort_selftest", "flr_host_band_plan",
            "flnr_param_count", "flnr_create", "flnr_destroy", "flnr_set_weights", "flnr_get_weights",
            "flnr_get_state", "flnr_set_state",
            "flnr_guide_forward", "flnr_guide_backward", "flnr_zero_grads", "flnr_get_grads",
@@ -117,8 +117,10 @@ def load_library():
     lib.flr_fast_batch_status.argtypes = [vp]
     lib.flr_barrier_selftest.argtypes = [ip, ctypes.c_ulonglong, ctypes.POINTER(ctypes.c_int)]
     lib.flr_mbarrier_selftest.argtypes = [ip, ctypes.c_ulonglong, ctypes.POINTER(ctypes.c_int)]
+    lib.flr_fast_abort_selftest.argtypes = [ctypes.POINTER(ctypes.c_int)]
     for name in ("flr_denoise_batch", "flr_fast_reserve_batch", "flr_fast_denoise_batch",
-                 "flr_fast_batch_status", "flr_barrier_selftest", "flr_mbarrier_selftest"):
+                 "flr_fast_batch_status", "flr_barrier_selftest", "flr_mbarrier_selftest",
+                 "flr_fast_abort_selftest"):
         getattr(lib, name).restype = ctypes.c_int
     lib.flr_fp32_fma_peak.argtypes = [ip, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double)]
     lib.flr_fp32_fma_peak.restype = ctypes.c_int
@@ -425,6 +427,14 @@ def mbarrier_selftest(ctas=4, timeout_ns=20_000_000):
     st = ctypes.c_int(0)
     _check(load_library().flr_mbarrier_selftest(int(ctas), ctypes.c_ulonglong(timeout_ns), ctypes.byref(st)),
            "flr_mbarrier_selftest")
+    return st.value
+
+
+def fast_abort_selftest():
+    """Status word of flr_fast_abort_selftest (1 = the pass whose waits gave up recorded it and
+    the pass after it was right)."""
+    st = ctypes.c_int(0)
+    _check(load_library().flr_fast_abort_selftest(ctypes.byref(st)), "flr_fast_abort_selftest")
     return st.value
 
 
