@@ -29,31 +29,36 @@ def _lib():
     global _bound
     lib = _flr.load_library()
     if not _bound:
-        vp, ip = ctypes.c_void_p, ctypes.c_int
-        lib.flnr_param_count.restype = ctypes.c_size_t
-        lib.flnr_param_count.argtypes = [ip]
-        lib.flnr_create.argtypes = [ip, ip, ctypes.POINTER(ctypes.c_void_p)]
-        lib.flnr_destroy.argtypes = [vp]
-        lib.flnr_set_weights.argtypes = [vp, vp, ctypes.c_size_t]
-        lib.flnr_get_weights.argtypes = [vp, vp, ctypes.c_size_t]
-        lib.flnr_get_grads.argtypes = [vp, vp, ctypes.c_size_t]
-        lib.flnr_get_state.argtypes = [vp, vp, ctypes.c_size_t]
-        lib.flnr_set_state.argtypes = [vp, vp, ctypes.c_size_t]
-        lib.flnr_guide_forward.argtypes = [vp, vp, vp, ip, ip, ip, vp]
-        lib.flnr_guide_backward.argtypes = [vp, vp, vp, vp]
-        lib.flnr_zero_grads.argtypes = [vp, vp]
-        lib.flnr_adam_step.argtypes = [vp, ctypes.c_float, ctypes.c_float, ctypes.c_float, ctypes.c_float, ip, vp]
-        lib.flnr_l1_loss.argtypes = [vp, vp, vp, vp, ctypes.c_size_t, vp]
-        lib.flnr_smape_loss.argtypes = [vp, vp, vp, vp, ctypes.c_size_t, ctypes.c_float, vp]
-        lib.flnr_layer.argtypes = [vp, ip, ip, vp, vp, vp, vp, ip, ip, ip, vp]
-        lib.flnr_status.argtypes = [vp]
-        for name in ("flnr_create", "flnr_destroy", "flnr_set_weights", "flnr_get_weights", "flnr_get_grads",
-                     "flnr_get_state", "flnr_set_state", "flnr_guide_forward", "flnr_guide_backward",
-                     "flnr_zero_grads", "flnr_adam_step",
-                     "flnr_l1_loss", "flnr_smape_loss", "flnr_layer", "flnr_status"):
-            getattr(lib, name).restype = ctypes.c_int
-        _bound = True
+        with _flr._lib_lock:
+            _bind(lib)
+            _bound = True
     return lib
+
+
+def _bind(lib):
+    vp, ip = ctypes.c_void_p, ctypes.c_int
+    lib.flnr_param_count.restype = ctypes.c_size_t
+    lib.flnr_param_count.argtypes = [ip]
+    lib.flnr_create.argtypes = [ip, ip, ctypes.POINTER(ctypes.c_void_p)]
+    lib.flnr_destroy.argtypes = [vp]
+    lib.flnr_set_weights.argtypes = [vp, vp, ctypes.c_size_t]
+    lib.flnr_get_weights.argtypes = [vp, vp, ctypes.c_size_t]
+    lib.flnr_get_grads.argtypes = [vp, vp, ctypes.c_size_t]
+    lib.flnr_get_state.argtypes = [vp, vp, ctypes.c_size_t]
+    lib.flnr_set_state.argtypes = [vp, vp, ctypes.c_size_t]
+    lib.flnr_guide_forward.argtypes = [vp, vp, vp, ip, ip, ip, vp]
+    lib.flnr_guide_backward.argtypes = [vp, vp, vp, vp]
+    lib.flnr_zero_grads.argtypes = [vp, vp]
+    lib.flnr_adam_step.argtypes = [vp, ctypes.c_float, ctypes.c_float, ctypes.c_float, ctypes.c_float, ip, vp]
+    lib.flnr_l1_loss.argtypes = [vp, vp, vp, vp, ctypes.c_size_t, vp]
+    lib.flnr_smape_loss.argtypes = [vp, vp, vp, vp, ctypes.c_size_t, ctypes.c_float, vp]
+    lib.flnr_layer.argtypes = [vp, ip, ip, vp, vp, vp, vp, ip, ip, ip, vp]
+    lib.flnr_status.argtypes = [vp]
+    for name in ("flnr_create", "flnr_destroy", "flnr_set_weights", "flnr_get_weights", "flnr_get_grads",
+                 "flnr_get_state", "flnr_set_state", "flnr_guide_forward", "flnr_guide_backward",
+                 "flnr_zero_grads", "flnr_adam_step",
+                 "flnr_l1_loss", "flnr_smape_loss", "flnr_layer", "flnr_status"):
+        getattr(lib, name).restype = ctypes.c_int
 
 
 def init_weights(seed=0, outputs=8):

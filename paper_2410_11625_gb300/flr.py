@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import threading
 
 from . import _build
 
@@ -74,6 +75,7 @@ class FlrError(RuntimeError):
 
 
 _lib = None
+_lib_lock = threading.Lock()  # held while the library is loaded and its functions' types are set
 
 
 def library_path() -> str:
@@ -81,10 +83,18 @@ def library_path() -> str:
 
 
 def load_library():
-    """Load libflr.so (built by ``paper_2410_11625_gb300.build()``); raises if absent."""
+    """Load libflr.so (built by ``paper_2410_11625_gb300.build()``); raises if absent.  One object
+    for every thread: another one would have functions without types, whose addresses ctypes
+    cuts to 32 bits."""
     global _lib
-    if _lib is not None:
-        return _lib
+    if _lib is None:
+        with _lib_lock:
+            if _lib is None:
+                _lib = _load()
+    return _lib
+
+
+def _load():
     path = _build.LIBPATH
     if not os.path.exists(path):
         raise FileNotFoundError(f"{path} is missing: run paper_2410_11625_gb300.build() first")
@@ -133,7 +143,6 @@ def load_library():
     for name in ("flr_create", "flr_destroy", "flr_reserve", "flr_set_concurrency", "flr_denoise", "flr_denoise_host",
                  "flr_denoise_host_async", "flr_host_wait", "flr_get_stats", "flr_get_kernel_times"):
         getattr(lib, name).restype = ctypes.c_int
-    _lib = lib
     return lib
 
 
