@@ -34,6 +34,7 @@
 
 #include "flr.h"
 #include "pdl.cuh"
+#include "tma.cuh"
 
 namespace flnr {
 namespace {
@@ -1808,24 +1809,10 @@ int egrid(size_t n) { return (int)((n + 255) / 256 < 8192 ? (n + 255) / 256 : 81
 
 // ---------------------------------------------------------------------------------------
 // Launch helpers for the template instantiations the network uses.
-// cuTensorMapEncodeTiled through the runtime's driver entry point (no link to libcuda)
-PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder()
-{
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    if (!fn) {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }
-    return fn;
-}
-
 // 4-D map of an NHWC bf16 tensor [N][H][W][C]: box (8 channels, bw, bh, 1), zero fill outside
 cudaError_t make_tmap(CUtensorMap *m, const void *base, int C, int W, int H, int N, int bw, int bh)
 {
-    PFN_cuTensorMapEncodeTiled_v12000 fn = tmap_encoder();
+    PFN_cuTensorMapEncodeTiled_v12000 fn = tma::encoder();
     if (!fn) return cudaErrorNotSupported;
     const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
     const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)W * C * 2, (cuuint64_t)H * W * C * 2};
@@ -1842,7 +1829,7 @@ cudaError_t make_tmap(CUtensorMap *m, const void *base, int C, int W, int H, int
 // N); box (8, bw, 1, bh, 1).  The start channel b * C + 8k selects column parity b, chunk k.
 cudaError_t make_tmap_parity(CUtensorMap *m, const void *base, int C, int W, int H, int N, int bw, int bh)
 {
-    PFN_cuTensorMapEncodeTiled_v12000 fn = tmap_encoder();
+    PFN_cuTensorMapEncodeTiled_v12000 fn = tma::encoder();
     if (!fn) return cudaErrorNotSupported;
     const cuuint64_t dims[5] = {(cuuint64_t)2 * C, (cuuint64_t)W / 2, 2, (cuuint64_t)H / 2, (cuuint64_t)N};
     const cuuint64_t strides[4] = {(cuuint64_t)C * 4, (cuuint64_t)W * C * 2, (cuuint64_t)W * C * 4,
@@ -1859,7 +1846,7 @@ cudaError_t make_tmap_parity(CUtensorMap *m, const void *base, int C, int W, int
 // columns x bh rows of one plane, zero fill outside
 cudaError_t make_tmap_planes(CUtensorMap *m, const void *base, int P, int W, int H, int N, int bw, int bh)
 {
-    PFN_cuTensorMapEncodeTiled_v12000 fn = tmap_encoder();
+    PFN_cuTensorMapEncodeTiled_v12000 fn = tma::encoder();
     if (!fn) return cudaErrorNotSupported;
     const cuuint64_t row = (cuuint64_t)W * 16;
     const cuuint64_t dims[4] = {(cuuint64_t)4 * W, (cuuint64_t)H, (cuuint64_t)P, (cuuint64_t)N};
@@ -1877,7 +1864,7 @@ cudaError_t make_tmap_planes(CUtensorMap *m, const void *base, int P, int W, int
 // (8, bw, 1, bh, 1).  The start value 8 b selects column parity b.
 cudaError_t make_tmap_pairs(CUtensorMap *m, const void *base, int C, int W, int H, int N, int bw, int bh)
 {
-    PFN_cuTensorMapEncodeTiled_v12000 fn = tmap_encoder();
+    PFN_cuTensorMapEncodeTiled_v12000 fn = tma::encoder();
     if (!fn) return cudaErrorNotSupported;
     const cuuint64_t row = (cuuint64_t)W * 16;
     const cuuint64_t dims[5] = {16, (cuuint64_t)W / 2, 2, (cuuint64_t)H / 2, (cuuint64_t)(C / 8) * N};
@@ -1895,7 +1882,7 @@ cudaError_t make_tmap_pairs(CUtensorMap *m, const void *base, int C, int W, int 
 // (W, H: the plane's size).
 cudaError_t make_tmap_rows(CUtensorMap *m, int layout, const void *base, int C, int W, int H, int N, int bw, int bh)
 {
-    PFN_cuTensorMapEncodeTiled_v12000 fn = tmap_encoder();
+    PFN_cuTensorMapEncodeTiled_v12000 fn = tma::encoder();
     if (!fn) return cudaErrorNotSupported;
     const cuuint64_t w = W, h = H, n = N, c8 = C / 8, row = w * 16;
     const cuuint32_t es[5] = {1, 1, 1, 1, 1}, b4 = 4 * bw, bb = bw, hh = bh, cc = C / 8;
@@ -1940,31 +1927,35 @@ constexpr size_t tc_smem(int smem, int cols, int threads)
 struct Resident {
     int per_sm = 0, n_sm = 0;
 };
+// known: the kernel's own, so that it is asked once per device.
 template <class K>
-cudaError_t resident(K kern, int threads, size_t smem, int cols, Resident &out)
+cudaError_t resident(PerDevice<Resident> &known, K kern, int threads, size_t smem, int cols, Resident &out)
 {
-    if (out.per_sm > 0) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    cudaFuncAttributes fa;
-    if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
-    int dev = 0, n_sm = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    // registers are split over the SM's four sub-partitions: warps per sub-partition first
-    const int regs_per_warp = (fa.numRegs * 32 + 255) / 256 * 256;
-    const int by_regs = (4 * (16384 / regs_per_warp)) / (threads / 32);
-    const int by_smem = kSmemPerSm / ((int)smem + (int)fa.sharedSizeBytes + kReservedPerCta);
-    int r = kThreadsPerSm / threads;
-    r = r < by_regs ? r : by_regs;
-    r = r < by_smem ? r : by_smem;
-    r = r < 512 / cols ? r : 512 / cols;
-    if (r < 1) return cudaErrorInvalidConfiguration;
-    out.n_sm = n_sm;
-    out.per_sm = r;
-    return cudaSuccess;
+    int dev = 0;
+    const cudaError_t ed = cudaGetDevice(&dev);
+    if (ed != cudaSuccess) return ed;
+    return known.get(dev, [&](Resident &v) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+        if (e != cudaSuccess) return e;
+        cudaFuncAttributes fa;
+        if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
+        int n_sm = 0;
+        if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        // registers are split over the SM's four sub-partitions: warps per sub-partition first
+        const int regs_per_warp = (fa.numRegs * 32 + 255) / 256 * 256;
+        const int by_regs = (4 * (16384 / regs_per_warp)) / (threads / 32);
+        const int by_smem = kSmemPerSm / ((int)smem + (int)fa.sharedSizeBytes + kReservedPerCta);
+        int r = kThreadsPerSm / threads;
+        r = r < by_regs ? r : by_regs;
+        r = r < by_smem ? r : by_smem;
+        r = r < 512 / cols ? r : 512 / cols;
+        if (r < 1) return cudaErrorInvalidConfiguration;
+        v.n_sm = n_sm;
+        v.per_sm = r;
+        return cudaSuccess;
+    }, out);
 }
 
 // Stages of a map of N images.  NT tiles per stage share a halo, a hand-over of the barriers and
@@ -1982,8 +1973,9 @@ cudaError_t conv_ws_launch_nt(const ConvArgs &a, bool ask, bool *fits, cudaStrea
     constexpr size_t smem = tc_smem(G::SMEM, G::COLS, G::THREADS);
     static_assert(smem <= 227 * 1024, "warp-specialised conv tile does not fit in shared memory");
     auto kern = conv_ws_kernel<CIN, COUT, KS, ACT, OUTM, MASK, NT>;
-    static Resident res;
-    cudaError_t e = resident(kern, G::THREADS, smem, G::COLS, res);
+    static PerDevice<Resident> known;
+    Resident res;
+    cudaError_t e = resident(known, kern, G::THREADS, smem, G::COLS, res);
     if (e != cudaSuccess) return e;
     const long long ntiles = stages(a.N, a.H, a.W, G::TH, G::TW), cap = (long long)res.per_sm * res.n_sm;
     if (ask) {
@@ -2040,8 +2032,9 @@ cudaError_t conv_tail_launch_nt(const ConvArgs &c, const ConvArgs &c2, bf16 *w2_
     constexpr size_t smem = tc_smem(T::SMEM, T::COLS, G::THREADS);
     static_assert(smem <= 227 * 1024, "fused conv stage does not fit in shared memory");
     auto kern = conv_tail_kernel<CIN, COUT, KS, COUT2, ACT2, OUTM2, NT>;
-    static Resident res;
-    cudaError_t e = resident(kern, G::THREADS, smem, T::COLS, res);
+    static PerDevice<Resident> known;
+    Resident res;
+    cudaError_t e = resident(known, kern, G::THREADS, smem, T::COLS, res);
     if (e != cudaSuccess) return e;
     const long long ntiles = stages(c.N, c.H, c.W, G::TH, G::TW), cap = (long long)res.per_sm * res.n_sm;
     if (ask) {
@@ -2078,8 +2071,9 @@ cudaError_t conv_up_launch(const ConvArgs &a, cudaStream_t st)
     constexpr size_t smem = tc_smem(G::SMEM, G::COLS, kWsThreads);
     static_assert(smem <= 227 * 1024, "decoder conv stage does not fit in shared memory");
     auto kern = conv_up_kernel<CA, CB, COUT, NBUF>;
-    static Resident res;
-    cudaError_t e = resident(kern, kWsThreads, smem, G::COLS, res);
+    static PerDevice<Resident> known;
+    Resident res;
+    cudaError_t e = resident(known, kern, kWsThreads, smem, G::COLS, res);
     if (e != cudaSuccess) return e;
     if ((a.H | a.W) & 1) return cudaErrorInvalidValue;
     const long long ntiles = stages(a.N, a.H / 2, a.W / 2, 16, 8), cap = (long long)res.per_sm * res.n_sm;
@@ -2103,8 +2097,9 @@ cudaError_t conv_s2_launch(const ConvArgs &a, cudaStream_t st)
     constexpr size_t smem = tc_smem(G::SMEM, G::COLS, kWsThreads);
     static_assert(smem <= 227 * 1024, "stride-2 conv stage does not fit in shared memory");
     auto kern = conv_s2_kernel<CIN, COUT, NBUF>;
-    static Resident res;
-    cudaError_t e = resident(kern, kWsThreads, smem, G::COLS, res);
+    static PerDevice<Resident> known;
+    Resident res;
+    cudaError_t e = resident(known, kern, kWsThreads, smem, G::COLS, res);
     if (e != cudaSuccess) return e;
     if ((a.H | a.W) & 1) return cudaErrorInvalidValue;
     const long long ntiles = stages(a.N, a.H / 2, a.W / 2, 16, G::TW), cap = (long long)res.per_sm * res.n_sm;
@@ -2138,8 +2133,9 @@ cudaError_t wgrad_launch(const bf16 *x, const bf16 *dz, int layout, int N, int H
     constexpr size_t smem = tc_smem(G::SMEM, G::COLS, kWgThreads);
     static_assert(smem <= 227 * 1024, "weight-gradient tile does not fit in shared memory");
     auto kern = wgrad_tc_kernel<CIN, COUT, KS, MODE>;
-    static Resident res;
-    cudaError_t e = resident(kern, kWgThreads, smem, G::COLS, res);
+    static PerDevice<Resident> known;
+    Resident res;
+    cudaError_t e = resident(known, kern, kWgThreads, smem, G::COLS, res);
     if (e != cudaSuccess) return e;
     const long long ntiles = stages(N, H, W, 16, 8);
     const int slots = n_sm / G::NG > 0 ? n_sm / G::NG : 1;

@@ -16,7 +16,6 @@
 // Every launch here is a dependent one (pdl.cuh) without an early trigger, as those of the unfused
 // forward path: backward 1920x1080 957 -> 946 us, 719 x 1277 forward, q = 6, 151 -> 146 us.
 #include <algorithm>
-#include <atomic>
 #include <cstring>
 #include <type_traits>
 
@@ -456,17 +455,6 @@ __global__ void __launch_bounds__(256) bwd_contract4_kernel(const BwdArgs a)
     }
 }
 
-int sm_count()
-{
-    static std::atomic<int> known[64];
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-    if (dev >= 0 && dev < 64 && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
-    if (dev >= 0 && dev < 64) known[dev].store(n, std::memory_order_relaxed);
-    return n;
-}
-
 int elem_grid(size_t n) { return (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096); }
 
 }  // namespace
@@ -523,7 +511,7 @@ cudaError_t launch_box_sum(const float *in, float *out, int nplanes, int H, int 
             // box sums 105 us, split 10 us) and a 1080p frame with a second wave two thirds
             // full (the backward pass 1.066 ms, split 1.029 ms).
             const long long tiles = (long long)((W + kBW - 1) / kBW) * ((H + kTH - 1) / kTH);
-            const long long target = 8LL * 3 * sm_count();
+            const long long target = 8LL * 3 * pdl::sm_count();
             k.per_cta = (int)std::min<long long>(nplanes, std::max<long long>(1, tiles * nplanes / target));
             if (rad == 8) return (W & 3) == 0 ? launch_box_sum_tma<8, true>(k, st) : launch_box_sum_tma<8, false>(k, st);
             return rad == 5 ? launch_box_sum_tma<5, false>(k, st) : launch_box_sum_tma<-1, false>(k, st);
@@ -547,7 +535,7 @@ cudaError_t launch_bwd_contract(int q, const BwdArgs &a, cudaStream_t st)
         const bool aligned = (a.W & 3) == 0 && al(a.guide) && al(a.rad) && al(a.g) && al(a.grad_guide) && al(a.grad_map) &&
                              al(a.grad_rad);
         const int ctas = (int)(((size_t)a.H * (a.pitch / 4) + 255) / 256);
-        const dim3 grid4(ctas, ctas < 2 * sm_count() ? q + 3 : 1);
+        const dim3 grid4(ctas, ctas < 2 * pdl::sm_count() ? q + 3 : 1);
         auto launch = [&](auto with, auto without) { return pdl::launch(aligned ? with : without, grid4, 256, 0, st, a); };
         switch (q) {
         case 1: return launch(bwd_contract4_kernel<1, true>, bwd_contract4_kernel<1, false>);

@@ -289,17 +289,6 @@ size_t apply_tma_smem()
     return 128 + sizeof(float) * 2 * (size_t)Q * 8 * kFW + 16;
 }
 
-int fast_n_sm()
-{
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            n = 1;
-    }
-    return n;
-}
-
 // Table of the frames f[0..n) with the CTAs of stages 1 to 3; stage 4's items are its launch's.
 template <int N>
 void fill_table(FrameTable<N> &t, int n, const FastArgs *f, unsigned long long *count, int *status)
@@ -318,11 +307,15 @@ void fill_table(FrameTable<N> &t, int n, const FastArgs *f, unsigned long long *
     }
 }
 
+// Names a kernel instance for pdl::allow_smem
+template <int KIND, int... I>
+struct KernelTag {};
+
 template <int Q, int F, int N>
 cudaError_t launch_moments(const FrameTable<N> &t, cudaStream_t st)
 {
     constexpr size_t smem = fast::moments_smem<Q>();
-    const cudaError_t e = cudaFuncSetAttribute(block_moments_kernel<Q, F, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = pdl::allow_smem<KernelTag<0, Q, F, N>>(block_moments_kernel<Q, F, N>, smem, false);
     if (e != cudaSuccess) return e;
     block_moments_kernel<Q, F, N><<<t.off[0][t.n], fast::kMomThreads, smem, st>>>(t);
     return cudaGetLastError();
@@ -375,13 +368,12 @@ cudaError_t launch_apply_fast(const FrameTable<N> &all, cudaStream_t st)
         for (int i = 0; i < nt; ++i)
             k.t.off[3][i + 1] = k.t.off[3][i] + (unsigned)((tma_f[i].Hb + 1) * ((tma_f[i].Wo + kFW - 1) / kFW));
         const size_t smem = apply_tma_smem<Q>();
-        auto kern = tma_f[0].F * tma_f[0].s == 8 ? apply_tma_kernel<Q, N, 8> : apply_tma_kernel<Q, N, 0>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
+        const bool cell8 = tma_f[0].F * tma_f[0].s == 8;
+        auto kern = cell8 ? apply_tma_kernel<Q, N, 8> : apply_tma_kernel<Q, N, 0>;
         // three CTAs per SM need the whole unified L1 / shared array as shared memory
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+        cudaError_t e = cell8 ? pdl::allow_smem<KernelTag<1, Q, N, 8>>(kern, smem, true) : pdl::allow_smem<KernelTag<1, Q, N, 0>>(kern, smem, true);
         if (e != cudaSuccess) return e;
-        const unsigned nitems = k.t.off[3][nt], most = 3 * (unsigned)fast_n_sm();  // three CTAs per SM
+        const unsigned nitems = k.t.off[3][nt], most = 3 * (unsigned)pdl::sm_count();  // three CTAs per SM
         e = pdl::launch(kern, dim3(nitems < most ? nitems : most), kFW, smem, st, k);
         if (e != cudaSuccess || nr == 0) return e;
     }
@@ -426,13 +418,7 @@ cudaError_t launch_param_grad_q(const FastArgs &a, unsigned long long *count, fl
     std::memcpy(td.f[0].w, a.wd, sizeof(a.wd));
     if ((e = pdl::launch(blur_h_kernel<Q, 1>, dim3(t.off[1][1]), kBlurThreads, 0, st, td)) != cudaSuccess) return e;
     const size_t smem = sizeof(float) * 2 * Chan<Q>::NCH * 128;
-    static bool attr_set = false;
-    if (!attr_set) {
-        if ((e = cudaFuncSetAttribute(blur_v_tangent_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-            cudaSuccess)
-            return e;
-        attr_set = true;
-    }
+    if ((e = pdl::allow_smem<KernelTag<2, Q>>(blur_v_tangent_kernel<Q>, smem, false)) != cudaSuccess) return e;
     blur_v_tangent_kernel<Q><<<gb, 128, smem, st>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // the frame reference the moments wrote, with the radiance offset zero: a tangent of the
@@ -551,7 +537,7 @@ cudaError_t abort_selftest(int *result)
     const size_t smem = apply_tma_smem<Q>();
     e = tma::encode_planes_f32(&k.t0[0], a.map_guide, W, H, Q, kFW, F, Q);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(apply_tma_kernel<Q, 1, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = pdl::allow_smem<KernelTag<1, Q, 1, 8>>(apply_tma_kernel<Q, 1, 8>, smem, true);
     std::vector<float> out(3 * px);
     *result = 0;
     for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {

@@ -9,8 +9,9 @@
 
 #include <cuda_runtime.h>
 
-#include <atomic>
 #include <utility>
+
+#include "device_cache.h"
 
 namespace pdl {
 
@@ -40,16 +41,28 @@ cudaError_t launch(void (*kern)(P...), dim3 grid, int threads, size_t smem, cuda
 template <class Tag, class K>
 cudaError_t allow_smem(K kern, size_t bytes, bool max_carveout)
 {
-    static std::atomic<bool> done[64];
+    static PerDevice<bool> done;
     int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    bool set = false;
+    const cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64 && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess && max_carveout)
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-    if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev].store(true, std::memory_order_release);
-    return e;
+    return done.get(dev, [&](bool &d) {
+        cudaError_t f = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (f == cudaSuccess && max_carveout)
+            f = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+        d = f == cudaSuccess;
+        return f;
+    }, set);
+}
+
+// SMs of the current device (1 if the device cannot be asked)
+inline int sm_count()
+{
+    static PerDevice<int> known;
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    const cudaError_t e = known.get(dev, [&](int &v) { return cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev); }, n);
+    return e == cudaSuccess && n > 0 ? n : 1;
 }
 
 }  // namespace pdl

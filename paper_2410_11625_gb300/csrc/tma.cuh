@@ -8,18 +8,23 @@
 #include <cudaTypedefs.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace tma {
 
 // cuTensorMapEncodeTiled, looked up once (no link against libcuda)
 inline PFN_cuTensorMapEncodeTiled_v12000 encoder()
 {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
+    static std::atomic<PFN_cuTensorMapEncodeTiled_v12000> known{nullptr};
+    PFN_cuTensorMapEncodeTiled_v12000 fn = known.load(std::memory_order_acquire);
     if (!fn) {
         void *p = nullptr;
         cudaDriverEntryPointQueryResult q;
         if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
+            q == cudaDriverEntryPointSuccess) {
             fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+            known.store(fn, std::memory_order_release);
+        }
     }
     return fn;
 }
