@@ -151,15 +151,20 @@ def _check(status, what):
         raise FlrError(status, what)
 
 
-def _dev_ptr(t, name, shape):
+def _dev_addr(t, name, shape):
+    """The device address of a contiguous float32 CUDA tensor of that shape (a tuple)."""
     import torch
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype != torch.float32 or not t.is_contiguous():
         raise TypeError(f"{name} must be contiguous float32")
-    if tuple(t.shape) != tuple(shape):
+    if t.shape != shape:
         raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+def _dev_ptr(t, name, shape):
+    return ctypes.c_void_p(_dev_addr(t, name, shape))
 
 
 def _host_ptr(a, name, shape):
@@ -291,10 +296,10 @@ class FLR:
         import torch
         arr = (FlrFrame * len(frames))()
         for i, (g, y, z, o) in enumerate(frames):
-            H, W = int(y.shape[-2]), int(y.shape[-1])
-            arr[i] = FlrFrame(_dev_ptr(g, "guide", (self.q, H, W)).value,
-                              None if z is None else _dev_ptr(z, "map_guide", (self.q, H, W)).value,
-                              _dev_ptr(y, "radiance", (3, H, W)).value, _dev_ptr(o, "out", (3, H, W)).value, H, W)
+            H, W = y.shape[-2:]
+            arr[i] = FlrFrame(_dev_addr(g, "guide", (self.q, H, W)),
+                              None if z is None else _dev_addr(z, "map_guide", (self.q, H, W)),
+                              _dev_addr(y, "radiance", (3, H, W)), _dev_addr(o, "out", (3, H, W)), H, W)
         if stream is None:
             stream = torch.cuda.current_stream(frames[0][1].device)
         _check(load_library().flr_denoise_batch(self._h, len(frames), arr, ctypes.c_void_p(stream.cuda_stream)),
@@ -380,12 +385,11 @@ class FastFLR:
     def _frames(self, frames):
         arr = (FlrFrame * len(frames))()
         for i, (g, y, z, o) in enumerate(frames):
-            Hi, Wi = int(y.shape[-2]), int(y.shape[-1])
+            Hi, Wi = y.shape[-2:]
             Ho, Wo = Hi * self.scale, Wi * self.scale
-            arr[i] = FlrFrame(_dev_ptr(g, "guide", (self.q, Hi, Wi)).value,
-                              None if z is None else _dev_ptr(z, "map_guide", (self.q, Ho, Wo)).value,
-                              _dev_ptr(y, "radiance", (3, Hi, Wi)).value,
-                              _dev_ptr(o, "out", (3, Ho, Wo)).value, Hi, Wi)
+            arr[i] = FlrFrame(_dev_addr(g, "guide", (self.q, Hi, Wi)),
+                              None if z is None else _dev_addr(z, "map_guide", (self.q, Ho, Wo)),
+                              _dev_addr(y, "radiance", (3, Hi, Wi)), _dev_addr(o, "out", (3, Ho, Wo)), Hi, Wi)
         return arr
 
     def reserve_batch(self, frames):
