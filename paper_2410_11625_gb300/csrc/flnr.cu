@@ -237,6 +237,23 @@ __device__ __forceinline__ bool mbar_wait_thread(uint32_t mbar, uint32_t parity)
     }
 }
 
+// bounded wait of a whole warp, every lane polling and the branches decided by votes: the code after
+// it stays one path
+__device__ __forceinline__ bool mbar_wait_vote(uint32_t mbar, uint32_t parity)
+{
+    const unsigned long long t0 = global_ns();
+    for (;;) {
+        uint32_t done;
+        asm volatile(
+            "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 20000;\nselp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(done)
+            : "r"(mbar), "r"(parity)
+            : "memory");
+        if (__all_sync(0xffffffffu, done != 0)) return true;
+        if (__any_sync(0xffffffffu, global_ns() - t0 > kTcTimeoutNs)) return false;
+    }
+}
+
 // Epilogue pieces shared by the tensor-core kernels.  tc_load_acc: one accumulator row (an
 // output pixel) from the warp's TMEM lane quarter, COUT columns from `taddr` on.
 template <int COUT>
@@ -1279,7 +1296,11 @@ __global__ void __launch_bounds__(kWsThreads) conv_s2_kernel(const __grid_consta
 // of D that nothing reads.
 // A tile is 16 rows x 8 pixels, K = 128.  A CTA walks tiles blockIdx.x, + gridDim.x, ...: one lane
 // loads them by TMA into a ring, one lane issues a tile's MMAs, warp 3 adds up the bias gradient
-// from the staged dz, and the accumulators stay in tensor memory to the end.  Where nine taps do
+// from the staged dz.  The tensor cores do not round their accumulations to nearest: a chain of n of
+// them is off by up to n units in the last place, all in one direction.  So the accumulators start
+// again with every tile (8 MMAs), and summing warps, one per 16 rows of D, add a tile's sums to
+// FP32 sums of their own in registers (the 16 rows over all 32 lanes, as C fragments), unit by unit
+// (WgGeom) while the MMAs of the next units run.  Where nine taps do
 // not fit (CIN = 64, 96), blockIdx.y takes a column of taps each.  MODE 1 is the stride-2 layer:
 // dz at the output's size and x as parity planes (conv_s2_kernel's taps: rows ky = 0 and 2 of
 // parity 1, ky = 1 of parity 0), so that no product is spent on dropped positions.  Every CTA
@@ -1311,13 +1332,22 @@ struct WgGeom {
     static constexpr int NBUF = 4 * STAGE <= 150 * 1024 ? 4 : 2;
     static constexpr int TMA_BYTES = NXP * XH * RP + O8 * DP;
     static constexpr int PAD = (8 - O8) * DP;  // the 64 rows of A reach past the last stage
-    static constexpr int SMEM = 128 + NBUF * STAGE + PAD + (2 * NBUF + 1) * 8 + 16;
-    static constexpr int COLS = tmem_cols<KXN * KS * CIN>();
     static constexpr int CTOT = TAPS * CIN + 8;  // columns of a partial: (kx, ky, channel), then the bias
     // tap rows of one MMA: MODE 0 as many as N = 256 holds; MODE 1 rows 0 and 2, then row 1
     static constexpr int KYN = KS == 1 ? 1 : MODE ? 2 : (3 * CIN <= 256 ? 3 : 2);
+    // units: the accumulators of one MMA (tap column, group of tap rows), each handed over by itself
+    static constexpr int NSG = (KS + KYN - 1) / KYN, U = KXN * NSG;
+    static constexpr int DCOLS = KXN * KS * CIN;   // accumulator columns of a tile
+    static constexpr int SETS = U == 1 ? 2 : 1;    // a lone unit has two sets, so that the MMAs need not wait
+    static constexpr int CHAIN = NG > 1 ? 1 : 2;   // tiles that the tensor cores accumulate
+    static constexpr int COLS = tmem_cols<SETS * DCOLS>();
+    __host__ __device__ static constexpr int unit_col(int u) { return ((u / NSG) * KS + (u % NSG) * KYN) * CIN; }
+    __host__ __device__ static constexpr int unit_len(int u) { return (KS - (u % NSG) * KYN < KYN ? KS - (u % NSG) * KYN : KYN) * CIN; }
+    // summing warps: one per 16 rows of D, two where one's half of the columns fills its registers
+    static constexpr int EW = COUT / 16, EH = DCOLS > 288 ? 2 : 1;
+    static constexpr int THREADS = 32 * (EH == 1 ? 4 + EW : 12);
+    static constexpr int SMEM = 128 + NBUF * STAGE + PAD + (2 * NBUF + 2 * U * SETS) * 8 + 16;
 };
-constexpr int kWgThreads = 128;
 
 // instruction descriptor, kind::f16: D FP32, A and B BF16, both MN-major, M = 64, N = n
 __host__ __device__ constexpr uint32_t umma_idesc_mn64(int n)
@@ -1325,43 +1355,76 @@ __host__ __device__ constexpr uint32_t umma_idesc_mn64(int n)
     return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(64 >> 4) << 24);
 }
 
-// The MMAs of one staged tile, tap columns [kx0, kx0 + KXN)
+// The MMAs of unit u of one staged tile (tap columns from kx0 on) into the accumulators at `set`
 template <int CIN, int COUT, int KS, int MODE>
-__device__ __forceinline__ void wgrad_mmas(uint32_t stage, uint32_t tmem, int kx0, bool first)
+__device__ __forceinline__ void wgrad_mmas(const int u, uint32_t stage, uint32_t set, int kx0, bool first)
 {
     using G = WgGeom<CIN, COUT, KS, MODE>;
     // MN-major, no swizzle: LBO between K groups (8 pixels), SBO between groups of 8 channels
     const uint64_t ad0 = umma_sdesc(stage + G::NXP * G::XP, 128, G::DP);
     const uint64_t bd0 = umma_sdesc(stage, G::RP, G::XW * 16);
+    const int s = u % G::NSG * G::KYN;  // first slot of the column (MODE 1: ky = 0, 2, 1)
+    const int kx = kx0 + u / G::NSG;
+    uint32_t off;
+    if (MODE) off = (uint32_t)((2 * (s == 0) + (kx != 1)) * G::XP + (s != 0) * G::RP + (kx != 0) * 16);
+    else off = (uint32_t)(s * G::RP + kx * 16);
+    const uint32_t idesc = umma_idesc_mn64(G::unit_len(u));
 #pragma unroll
-    for (int k = 0; k < G::KXN; ++k) {
-        const int kx = kx0 + k;
-#pragma unroll
-        for (int s = 0; s < KS; s += G::KYN) {  // slots s .. of the column (MODE 1: ky = 0, 2, 1)
-            constexpr int kyn = G::KYN;
-            const int ns = KS - s < kyn ? KS - s : kyn;
-            uint32_t off;
-            if (MODE) off = (uint32_t)((2 * (s == 0) + (kx != 1)) * G::XP + (s != 0) * G::RP + (kx != 0) * 16);
-            else off = (uint32_t)(s * G::RP + kx * 16);
-            const uint32_t idesc = umma_idesc_mn64(ns * CIN), d = tmem + (uint32_t)((k * KS + s) * CIN);
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks)
-                umma_bf16(d, ad0 + (uint64_t)((ks * 256) >> 4), bd0 + (uint64_t)((off + 2 * ks * G::RP) >> 4), idesc,
-                          (first && ks == 0) ? 0u : 1u);
-        }
+    for (int ks = 0; ks < 8; ++ks)
+        umma_bf16(set + G::unit_col(u), ad0 + (uint64_t)((ks * 256) >> 4), bd0 + (uint64_t)((off + 2 * ks * G::RP) >> 4), idesc,
+                  first && ks == 0 ? 0u : 1u);
+}
+
+// 16 lanes x 8 N columns of the warp's TMEM lane quarter, as C fragments: of block b (8 columns)
+// v[4 b], v[4 b + 1] are row lane / 4, columns 2 (lane % 4) and + 1, v[4 b + 2], v[4 b + 3] row lane / 4 + 8
+template <int N>
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t *r)
+{
+    if constexpr (N >= 4) {
+        asm volatile(
+            "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+              "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+            : "r"(taddr));
+        if constexpr (N > 4) tmem_ld_frag<N - 4>(taddr + 32, r + 16);
+    } else if constexpr (N >= 2) {
+        asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                     : "r"(taddr));
+        if constexpr (N > 2) tmem_ld_frag<N - 2>(taddr + 16, r + 8);
+    } else {
+        asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];\n"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                     : "r"(taddr));
     }
 }
 
-template <int CIN, int COUT, int KS, int MODE>
-__global__ void __launch_bounds__(kWgThreads) wgrad_tc_kernel(const __grid_constant__ WgradArgs a)
+// acc += the LEN columns at taddr (16 lanes), up to 48 columns in flight
+template <int LEN>
+__device__ __forceinline__ void add_frags(float *acc, uint32_t taddr)
+{
+    constexpr int B = LEN % 48 == 0 ? 48 : LEN % 32 == 0 ? 32 : LEN % 24 == 0 ? 24 : 16;
+    static_assert(LEN % B == 0 && B % 8 == 0, "columns in blocks of eight");
+#pragma unroll
+    for (int c = 0; c < LEN; c += B) {
+        uint32_t r[B / 2];
+        tmem_ld_frag<B / 8>(taddr + (uint32_t)c, r);
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n");
+#pragma unroll
+        for (int i = 0; i < B / 2; ++i) acc[c / 2 + i] += __uint_as_float(r[i]);
+    }
+}
+
+template <int CIN, int COUT, int KS, int MODE, int... UN>
+__device__ __forceinline__ void wgrad_body(const WgradArgs &a, std::integer_sequence<int, UN...>)
 {
     using G = WgGeom<CIN, COUT, KS, MODE>;
     static_assert(CIN % 16 == 0 && COUT % 16 == 0 && COUT <= 64 && (MODE == 0 || KS == 3), "UMMA shape");
-    constexpr int NBUF = G::NBUF;
+    constexpr int NBUF = G::NBUF, SETS = G::SETS, CHAIN = G::CHAIN;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char *base = smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127);
     uint64_t *full = reinterpret_cast<uint64_t *>(base + NBUF * G::STAGE + G::PAD);
-    uint64_t *empty = full + NBUF, *done = empty + NBUF;
+    uint64_t *empty = full + NBUF, *ufull = empty + NBUF, *uempty = ufull + G::U * SETS;  // [U][SETS]
     __shared__ uint32_t s_tmem;
     __shared__ int s_issued, s_consumed, s_fail;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1378,7 +1441,10 @@ __global__ void __launch_bounds__(kWgThreads) wgrad_tc_kernel(const __grid_const
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(full + i)));
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 2;\n" ::"r"(smem_u32(empty + i)));  // MMAs, bias warp
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(done)));
+        for (int i = 0; i < G::U * SETS; ++i) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(ufull + i)));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(uempty + i)), "r"(G::EW * G::EH));
+        }
         asm volatile("fence.mbarrier_init.release.cluster;\n");
         s_issued = s_consumed = s_fail = 0;
     }
@@ -1389,6 +1455,10 @@ __global__ void __launch_bounds__(kWgThreads) wgrad_tc_kernel(const __grid_const
     pdl::trigger();
     pdl::wait();
 
+    // summing warps: quarter and half of the columns; acc: the sums over this CTA's tiles
+    const int quarter = warp & 3, half = (warp - 4) >> 2;
+    const bool sums = warp >= 4 && quarter < G::EW && half < G::EH;
+    float acc[G::DCOLS / G::EH / 2];
     if (warp == 1 && lane == 0) {  // producer
         for (int j = 0; j < mine; ++j) {
             const int st = j % NBUF;
@@ -1414,40 +1484,76 @@ __global__ void __launch_bounds__(kWgThreads) wgrad_tc_kernel(const __grid_const
     } else if (warp == 2 && lane == 0) {  // MMA issuer
         int j = 0;
         for (; j < mine; ++j) {
-            const int st = j % NBUF;
+            const int st = j % NBUF, chain = j / CHAIN, set = chain % SETS;
+            const bool first = j % CHAIN == 0, last = (j + 1) % CHAIN == 0 || j + 1 == mine;
             if (!mbar_wait_thread(smem_u32(full + st), (uint32_t)((j / NBUF) & 1))) {
                 s_fail = 1;
                 break;
             }
             s_consumed = j + 1;
             asm volatile("tcgen05.fence::after_thread_sync;\n");
-            wgrad_mmas<CIN, COUT, KS, MODE>(smem_u32(base + st * G::STAGE), tmem, G::NG > 1 ? (int)blockIdx.y : 0, j == 0);
+            bool ok = true;
+            const uint32_t stage = smem_u32(base + st * G::STAGE), d = tmem + set * G::DCOLS;
+            const int kx0 = G::NG > 1 ? (int)blockIdx.y : 0;
+            if (first) {
+#pragma unroll
+                for (int u = 0; u < G::U; ++u) {
+                    if (chain >= SETS) {
+                        ok &= mbar_wait_thread(smem_u32(uempty + u * SETS + set), (uint32_t)((chain / SETS - 1) & 1));
+                        asm volatile("tcgen05.fence::after_thread_sync;\n");
+                    }
+                    wgrad_mmas<CIN, COUT, KS, MODE>(u, stage, d, kx0, true);
+                    if (last) asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                        smem_u32(ufull + u * SETS + set)));
+                }
+            } else {
+#pragma unroll
+                for (int u = 0; u < G::U; ++u) {
+                    wgrad_mmas<CIN, COUT, KS, MODE>(u, stage, d, kx0, false);
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                        smem_u32(ufull + u * SETS + set)));
+                }
+            }
+            if (!ok) {
+                s_fail = 1;
+                break;
+            }
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
                 smem_u32(empty + st)));
         }
-        if (mine > 0 && j == mine)
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_u32(done)));
+        // the last stages' commits have arrived before the CTA exits
+        for (int i = mine > NBUF ? mine - NBUF : 0; j == mine && i < mine; ++i)
+            if (!mbar_wait_thread(smem_u32(empty + i % NBUF), (uint32_t)((i / NBUF) & 1))) s_fail = 1;
     } else if (warp == 3) {  // bias gradient: LP lanes per 8-channel chunk of dz, every LP-th pixel each
         constexpr int LP = 32 / G::O8;
         const int o8 = lane / LP, l = lane % LP;
-        float acc[8] = {};
+        float bsum[8] = {};  // over the tiles; a tile's own sums in two, even and odd steps
         for (int j = 0; j < mine; ++j) {
             const int st = j % NBUF;
-            if (!mbar_wait_warp(smem_u32(full + st), (uint32_t)((j / NBUF) & 1))) {
+            if (!mbar_wait_vote(smem_u32(full + st), (uint32_t)((j / NBUF) & 1))) {
                 if (lane == 0) s_fail = 1;
                 break;
             }
             if (blockIdx.y == 0) {
                 const uint4 *dz = reinterpret_cast<const uint4 *>(base + st * G::STAGE + G::NXP * G::XP + o8 * G::DP) + l;
+                float2 t[2][4] = {};
 #pragma unroll
-                for (int p = 0; p < 128 / LP; ++p) {
-                    const uint4 v = dz[p * LP];
-                    const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
+                for (int p0 = 0; p0 < 128 / LP; p0 += 8) {
+                    uint4 v[8];  // eight loads in flight
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        acc[2 * i] += __low2float(h[i]);
-                        acc[2 * i + 1] += __high2float(h[i]);
+                    for (int p = 0; p < 8; ++p) v[p] = dz[(p0 + p) * LP];
+#pragma unroll
+                    for (int p = 0; p < 8; ++p) {
+                        const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v[p]);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) t[p & 1][i] = __fadd2_rn(t[p & 1][i], __bfloat1622float2(h[i]));
                     }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float2 u = __fadd2_rn(t[0][i], t[1][i]);
+                    bsum[2 * i] += u.x;
+                    bsum[2 * i + 1] += u.y;
                 }
             }
             __syncwarp();
@@ -1457,36 +1563,54 @@ __global__ void __launch_bounds__(kWgThreads) wgrad_tc_kernel(const __grid_const
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
 #pragma unroll
-                for (int o = LP / 2; o > 0; o >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
-                if (l == 0) a.part[((size_t)blockIdx.x * COUT + o8 * 8 + i) * G::CTOT + G::TAPS * CIN] = acc[i];
+                for (int o = LP / 2; o > 0; o >>= 1) bsum[i] += __shfl_xor_sync(0xffffffffu, bsum[i], o);
+                if (l == 0) a.part[((size_t)blockIdx.x * COUT + o8 * 8 + i) * G::CTOT + G::TAPS * CIN] = bsum[i];
             }
         }
+    } else if (sums) {
+#pragma unroll
+        for (int i = 0; i < G::DCOLS / G::EH / 2; ++i) acc[i] = 0.f;
+        bool ok = true;
+        for (int j = 0; j < (mine + CHAIN - 1) / CHAIN && ok; ++j) {
+            const int set = j % SETS;
+            auto unit = [&](auto un) {
+                constexpr int u = decltype(un)::value, len = G::unit_len(u) / G::EH;
+                if (!ok) return;
+                if (!mbar_wait_vote(smem_u32(ufull + u * SETS + set), (uint32_t)((j / SETS) & 1))) {
+                    ok = false;
+                    return;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;\n");
+                add_frags<len>(acc + G::unit_col(u) / G::EH / 2,
+                               tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(set * G::DCOLS + G::unit_col(u) + half * len));
+                asm volatile("tcgen05.fence::before_thread_sync;\n");
+                __syncwarp();
+                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(uempty + u * SETS + set)) : "memory");
+            };
+            (unit(std::integral_constant<int, UN>{}), ...);
+        }
+        if (!ok && lane == 0) s_fail = 1;
     }
     __syncwarp();
-    __syncthreads();  // the issuing lanes are through
-    if (!s_fail && mine > 0 && !mbar_wait_warp(smem_u32(done), 0u)) {
-        if (lane == 0) s_fail = 1;
-    }
-    __syncthreads();
+    __syncthreads();  // every role is through: the sums hold every tile, or a wait ran out
     if (s_fail) {
         if (tid == 0 && a.status) atomicExch(a.status, FLNR_STATUS_TIMEOUT);
         if (tid == 32)  // let copies still in flight land before the CTA exits
             for (int j = s_consumed; j < s_issued; ++j) mbar_wait_thread(smem_u32(full + j % NBUF), (uint32_t)((j / NBUF) & 1));
-    } else if (16 * warp < COUT) {
+    } else if (sums) {
         // M = 64: rows 16 w .. 16 w + 15 in lanes 0-15 of lane quarter w
-        asm volatile("tcgen05.fence::after_thread_sync;\n");
-        float *dst = a.part + ((size_t)blockIdx.x * COUT + 16 * warp + lane) * G::CTOT + blockIdx.y * (G::KXN * KS * CIN);
-#pragma unroll 1
-        for (int c = 0; c < G::KXN * KS * CIN; c += 16) {
-            float v[16] = {};
-            if (mine > 0) tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c, v);
-            asm volatile("tcgen05.wait::ld.sync.aligned;\n");
-            if (lane < 16) {
+        float *dst = a.part + ((size_t)blockIdx.x * COUT + 16 * quarter + lane / 4) * G::CTOT + blockIdx.y * G::DCOLS + 2 * (lane & 3);
+        auto unit = [&](auto un) {
+            constexpr int u = decltype(un)::value, len = G::unit_len(u) / G::EH;
+            const float *v = acc + G::unit_col(u) / G::EH / 2;
+            float *d = dst + G::unit_col(u) + half * len;
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    *reinterpret_cast<float4 *>(dst + c + 4 * j) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+            for (int b = 0; b < len / 8; ++b) {
+                *reinterpret_cast<float2 *>(d + 8 * b) = make_float2(v[4 * b], v[4 * b + 1]);
+                *reinterpret_cast<float2 *>(d + 8 * b + 8 * G::CTOT) = make_float2(v[4 * b + 2], v[4 * b + 3]);
             }
-        }
+        };
+        (unit(std::integral_constant<int, UN>{}), ...);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
     __syncthreads();
@@ -1496,10 +1620,16 @@ __global__ void __launch_bounds__(kWgThreads) wgrad_tc_kernel(const __grid_const
     }
 }
 
+template <int CIN, int COUT, int KS, int MODE>
+__global__ void __launch_bounds__(WgGeom<CIN, COUT, KS, MODE>::THREADS) wgrad_tc_kernel(const __grid_constant__ WgradArgs a)
+{
+    wgrad_body<CIN, COUT, KS, MODE>(a, std::make_integer_sequence<int, WgGeom<CIN, COUT, KS, MODE>::U>{});
+}
+
 // The layers' partials into the FP32 master gradients, one launch for all of them: element f of
 // a layer is (o, column) of its slices [slices][COUT][CTOT]; 32 consecutive elements per CTA
-// (coalesced), sixteen warps take slices w, w + 16, ... in turn and their sums are added in warp
-// order, so the result is the same every run.  Padding channels are skipped.
+// (coalesced), sixteen warps take slices w, w + 16, ... and their sums are added, in a fixed order, so
+// the result is the same every run.  Padding channels are skipped.
 struct RedLayer {
     const float *part;
     float *gw, *gb;
@@ -1533,15 +1663,21 @@ __global__ void __launch_bounds__(32 * kRedWarps) wgrad_reduce_kernel(const __gr
                 const int jj = j + u * kRedWarps;
                 v[u] = jj < l.slices ? __ldg(p + (size_t)jj * total) : 0.f;
             }
-#pragma unroll
-            for (int u = 0; u < NB; ++u) s += v[u];
+            // in pairs, here and below: half the rounding of a chain
+            s += (((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]))) + (v[8] + v[9]);
         }
     }
     s_sum[w][lane] = s;
     __syncthreads();
     if (w != 0 || f >= total) return;
+    float v[kRedWarps];
 #pragma unroll
-    for (int u = 1; u < kRedWarps; ++u) s += s_sum[u][lane];
+    for (int u = 0; u < kRedWarps; ++u) v[u] = s_sum[u][lane];
+#pragma unroll
+    for (int n = kRedWarps / 2; n > 0; n /= 2)
+#pragma unroll
+        for (int u = 0; u < n; ++u) v[u] += v[u + n];
+    s = v[0];
     const int o = f / ctot, c = f % ctot;
     if (o >= l.cout_true) return;
     if (c == taps * l.cin) {
@@ -2130,12 +2266,12 @@ cudaError_t wgrad_launch(const bf16 *x, const bf16 *dz, int layout, int N, int H
                          int n_sm, int *status, cudaStream_t st)
 {
     using G = WgGeom<CIN, COUT, KS, MODE>;
-    constexpr size_t smem = tc_smem(G::SMEM, G::COLS, kWgThreads);
+    constexpr size_t smem = tc_smem(G::SMEM, G::COLS, G::THREADS);
     static_assert(smem <= 227 * 1024, "weight-gradient tile does not fit in shared memory");
     auto kern = wgrad_tc_kernel<CIN, COUT, KS, MODE>;
     static PerDevice<Resident> known;
     Resident res;
-    cudaError_t e = resident(known, kern, kWgThreads, smem, G::COLS, res);
+    cudaError_t e = resident(known, kern, G::THREADS, smem, G::COLS, res);
     if (e != cudaSuccess) return e;
     const long long ntiles = stages(N, H, W, 16, 8);
     const int slots = n_sm / G::NG > 0 ? n_sm / G::NG : 1;
@@ -2152,7 +2288,7 @@ cudaError_t wgrad_launch(const bf16 *x, const bf16 *dz, int layout, int N, int H
     if ((e = make_tmap_tile(&a.tdz, layout, dz, COUT, W, H, N, 8, 16)) != cudaSuccess) return e;
     ra.l[ra.n++] = RedLayer{d.part, d.gw, d.gb, slices, COUT, CIN, KS, MODE, d.cin_true, d.cout_true, ra.blocks};
     ra.blocks += (COUT * G::CTOT + 31) / 32;
-    return pdl::launch(kern, dim3(slices, G::NG), kWgThreads, smem, st, a);
+    return pdl::launch(kern, dim3(slices, G::NG), G::THREADS, smem, st, a);
 }
 
 cudaError_t wgrad_reduce(const RedArgs &ra, cudaStream_t st)
