@@ -1298,9 +1298,11 @@ __global__ void __launch_bounds__(kWsThreads) conv_s2_kernel(const __grid_consta
 // loads them by TMA into a ring, one lane issues a tile's MMAs, warp 3 adds up the bias gradient
 // from the staged dz.  The tensor cores do not round their accumulations to nearest: a chain of n of
 // them is off by up to n units in the last place, all in one direction.  So the accumulators start
-// again with every tile (8 MMAs), and summing warps, one per 16 rows of D, add a tile's sums to
+// again every CHAIN tiles, and summing warps, one per 16 rows of D, add a chain's sums to
 // FP32 sums of their own in registers (the 16 rows over all 32 lanes, as C fragments), unit by unit
-// (WgGeom) while the MMAs of the next units run.  Where nine taps do
+// (WgGeom) while the MMAs of the next units run.  Operands of one sign, error over the sum, 16 -> 16
+// channels: one chain per CTA 3.4e-6 on a 16 x 128^2 batch and 6.5e-5 at 1920x1080, two tiles 2.5e-7
+// on both, one tile 1.1e-7.  Backward pass of 16 x 128^2: 373 us with one chain, 378 with two tiles.  Where nine taps do
 // not fit (CIN = 64, 96), blockIdx.y takes a column of taps each.  MODE 1 is the stride-2 layer:
 // dz at the output's size and x as parity planes (conv_s2_kernel's taps: rows ky = 0 and 2 of
 // parity 1, ky = 1 of parity 0), so that no product is spent on dropped positions.  Every CTA
@@ -1308,8 +1310,8 @@ __global__ void __launch_bounds__(kWsThreads) conv_s2_kernel(const __grid_consta
 // slices in a fixed order.
 // The form before built both operands with ldmatrix and shared stores from NHWC pixels and took
 // its bias sums in kernels of their own: the backward pass of a 16 x 128^2 batch spent 343 us in
-// weight gradients, 158 us in bias gradients and 110 us in twelve reductions; now 145 us with the bias and one reduction
-// of 27 us.
+// weight gradients, 158 us in bias gradients and 110 us in twelve reductions; now about 150 us with the
+// bias and one reduction of 27 us.
 struct alignas(128) WgradArgs {
     CUtensorMap tx, tdz;
     float *part;  // [gridDim.x][COUT][KS^2 CIN + 8]
@@ -1318,10 +1320,15 @@ struct alignas(128) WgradArgs {
     int *status;
 };
 
+// Groups of tap columns that a layer's gradient is split into: the accumulators of one fit in tensor memory
+__host__ __device__ constexpr int wgrad_groups(int cin, int ks) { return ks * ks * cin > 512 ? ks : 1; }
+// Slices of a layer's partials: one CTA per SM and tap group
+constexpr int wgrad_slots(int n_sm, int groups) { return n_sm / groups > 0 ? n_sm / groups : 1; }
+
 template <int CIN, int COUT, int KS, int MODE>
 struct WgGeom {
     static constexpr int P = KS / 2, C8 = CIN / 8, O8 = COUT / 8, TAPS = KS * KS;
-    static constexpr int NG = TAPS * CIN > 512 ? KS : 1;  // tap columns split over blockIdx.y
+    static constexpr int NG = wgrad_groups(CIN, KS);      // tap columns split over blockIdx.y
     static constexpr int KXN = KS / NG;                   // tap columns per CTA
     static constexpr int XH = MODE ? 17 : 16 + 2 * P, XW = MODE ? 9 : 8 + 2 * P;  // staged rows and columns
     static constexpr int RP = C8 * XW * 16;                                       // one row, all chunks
@@ -2274,7 +2281,7 @@ cudaError_t wgrad_launch(const bf16 *x, const bf16 *dz, int layout, int N, int H
     cudaError_t e = resident(known, kern, G::THREADS, smem, G::COLS, res);
     if (e != cudaSuccess) return e;
     const long long ntiles = stages(N, H, W, 16, 8);
-    const int slots = n_sm / G::NG > 0 ? n_sm / G::NG : 1;
+    const int slots = wgrad_slots(n_sm, G::NG);
     const int slices = (int)(ntiles < slots ? ntiles : slots);
     WgradArgs a;
     std::memset(&a, 0, sizeof(a));
@@ -2420,12 +2427,13 @@ int flnr_create(int max_pixels, int outputs, flnr_net **out)
     st |= nalloc(n, &n->gskip0, P * 16) | nalloc(n, &n->gskip1, P2 * 32);
     st |= nalloc(n, &n->head_w, 16 * 16) | nalloc(n, &n->head_b, 16);
     st |= nalloc(n, &n->status, 1);
-    // partial gradients: one slice per SM of each layer's [Cout][k k Cin + 8] sums
+    // partial gradients: the slices of each layer's [Cout][k k Cin + 8] sums (47 MB on 152 SMs)
     size_t wp = 0;
     for (int l = 0; l < flnr::kNL; ++l) {
         const auto &d = flnr::kLayers[l];
+        const int cin = flnr::pad16(d.cin), slots = flnr::wgrad_slots(n->n_sm, flnr::wgrad_groups(cin, d.k));
         n->wpart_off[l] = wp;
-        wp += (size_t)n->n_sm * flnr::pad16(d.cout) * (d.k * d.k * flnr::pad16(d.cin) + 8);
+        wp += (size_t)slots * flnr::pad16(d.cout) * (d.k * d.k * cin + 8);
     }
     st |= nalloc(n, &n->wpart, wp);
     if (st != FLR_OK) {
