@@ -23,6 +23,14 @@ def test_wide_cells(flr, factor, scale, H, W):  # noqa: F811
     check(flr, g, y, z=z, scale=scale, factor=factor, rms_bar=True)
 
 
+@pytest.mark.parametrize("factor,scale,H,W", [(2, 1, 49, 80), (4, 1, 40, 260), (2, 2, 33, 62), (2, 3, 20, 128)])
+def test_small_cells(flr, factor, scale, H, W):  # noqa: F811
+    """Cells of 2, 4 and 6 pixels in the tiled form."""
+    g, y = synth.random_frame(40 + H, H, W, 8)
+    z = synth.random_frame(41 + H, H * scale, W * scale, 8)[0] if scale > 1 else None
+    check(flr, g, y, z=z, scale=scale, factor=factor, rms_bar=scale > 1)
+
+
 @pytest.mark.parametrize("factor,scale,H,W", [(4, 1, 96, 160), (2, 2, 48, 80), (4, 3, 32, 48), (2, 1, 49, 80)])
 def test_parameter_gradients(flr, factor, scale, H, W):  # noqa: F811
     import torch
