@@ -51,7 +51,8 @@ constexpr LayerDef kLayers[kNL] = {
 __host__ __device__ constexpr int pad16(int c) { return (c + 15) / 16 * 16; }
 
 // ---------------------------------------------------------------------------------------
-// Every launch is a programmatic dependent one (pdl.cuh).  The network is a chain of short
+// Every launch of the passes is a programmatic dependent one (pdl.cuh); the weights' conversion, Adam
+// and the losses are ordinary.  The network is a chain of short
 // kernels, each reading what the one before wrote, and at 16 x 128^2 a training pass lost 120 us
 // of 690 between them.  A kernel that allocates tensor memory triggers after its allocation: its
 // successor's CTAs, which may be resident beside it and hold columns while they wait, then cannot

@@ -348,8 +348,8 @@ __global__ void __launch_bounds__(256) bwd_contract_kernel(const BwdArgs a)
     }
 }
 
-// The same contraction for four consecutive pixels of a row per thread (W a multiple of 4,
-// every plane 16-byte aligned): one 16-byte load per plane and four pixels instead of four
+// The same contraction for four consecutive pixels of a row per thread (workspace rows a multiple
+// of 16 bytes; ALIGNED: the images' too): one 16-byte load per plane and four pixels instead of four
 // 4-byte loads, and each output channel's gradient formed from its own planes in turn, so
 // that a thread holds four pixels' inputs and one channel's operands at a time.  Every
 // pixel's arithmetic (operands, order of the fused multiply-adds) is that of

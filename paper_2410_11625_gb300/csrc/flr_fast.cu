@@ -317,6 +317,7 @@ cudaError_t launch_moments(const FrameTable<N> &t, cudaStream_t st)
     constexpr size_t smem = fast::moments_smem<Q>();
     const cudaError_t e = pdl::allow_smem<KernelTag<0, Q, F, N>>(block_moments_kernel<Q, F, N>, smem, false);
     if (e != cudaSuccess) return e;
+    // an ordinary launch, not a dependent one: apply_tma_kernel reads the map guide before its wait
     block_moments_kernel<Q, F, N><<<t.off[0][t.n], fast::kMomThreads, smem, st>>>(t);
     return cudaGetLastError();
 }

@@ -215,7 +215,6 @@ cudaError_t launch_bwd_contract(int q, const BwdArgs &a, cudaStream_t st);
 // the frame reference shift of the forward kernel (Q + 3 floats), by itself
 cudaError_t launch_frame_shift(int q, const float *guide, const float *rad, int H, int W, int ref_rows, float *shift_out,
                                cudaStream_t st);
-namespace fast { struct FastArgs; }
 cudaError_t launch_barrier_selftest(unsigned *count, unsigned *gen, unsigned expected, int *status,
                                     unsigned long long timeout_ns, int grid, cudaStream_t st);
 

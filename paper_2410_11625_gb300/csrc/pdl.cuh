@@ -3,8 +3,12 @@
 // A kernel launched with pdl::launch may start when every CTA of its predecessor has called
 // pdl::trigger (or exited); it must call pdl::wait, which returns when the predecessor has
 // finished and its writes are visible, before it touches global memory.  Only set-up (barriers,
-// tensor memory, index arithmetic) runs ahead.  Every CTA of a kernel that triggers calls wait
-// itself, so a finished predecessor implies that its own predecessors have finished.
+// tensor memory, index arithmetic) runs ahead.  Every CTA of a dependent kernel that triggers calls
+// wait itself, so a finished predecessor implies that its own predecessors have finished.
+// One chain differs: the first stage of fast FLR is an ordinary launch that triggers without
+// waiting.  It starts when everything before the call is complete, so the last stage may read the
+// caller's map guide ahead of its wait; were the first stage a dependent launch, that read would race
+// with the map guide's producer.
 #pragma once
 
 #include <cuda_runtime.h>
